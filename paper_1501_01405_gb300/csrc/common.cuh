@@ -156,85 +156,90 @@ __device__ __forceinline__ double u53(uint32_t lo, uint32_t hi) {
 // (Tang's table-driven reduction, ACM TOMS 16(4), 1990, carried out in
 // integers).  With 1 - u = K 2^-53, K in [1, 2^53], K = 2^e M, M in [1, 2):
 //   -log(1 - u) = (53 - e) ln 2 - ln M,
-//   ln M = ln c_j + log1p(r),  r = M / c_j - 1,  |r| < 2^-13,
-// c_j the centre of the j-th of 4096 slices of [1, 2) (j = the 12 bits after
-// the leading one), 1/c_j stored as a 63-bit fraction, ln c_j as a 64-bit
-// fraction.  log1p(r) = r - r^2/2 + r^2 (r/3 - r^2/4) (the r^5 term is below
-// 2^-67): r in 64-bit fixed point; r^2 from r's top 32 bits and one cross
-// product (two 32x32 multiplies instead of a signed 64x64 high product, to
-// 2^-64); the bracket and its product with r^2 in 32-bit pieces (one wide
-// multiply), since their weight is below 2^-40; ln c_j + log1p(r) is summed
-// and rounded once, unsigned; n ln 2 comes rounded from a 64-entry table.  The result carries an
-// absolute error below 2^-56 (2^-57.0 in an exhaustive check of slice edges
-// and centres at every exponent) before its one rounding to double, i.e.
-// within about an ulp for -log(1 - u) > 1/16 and far below the ulp of any
-// sum it enters.
+//   ln M = -ln w_j + log1p(r),  r = w_j M - 1,  |r| <= 2^-14,
+// w_j a 27-bit approximation of 1/c_j, c_j the centre of the j-th of 8192
+// slices of [1, 2) (j = the 13 bits after the leading one).
+//
+// The kernels that draw variates are bound by instruction issue, so the
+// scales are chosen for the fewest instructions:
+//  - w_j has 27 bits and M 2^63 is a two-word integer, so V = w_j M 2^58 takes
+//    one high and one wide multiply and no shift: it enters the result as it
+//    is, and its bits 13..44 are r 2^45 as a signed word (1 2^45 vanishes
+//    modulo 2^32);
+//  - |r| <= 2^-14 leaves log1p(r) = r - r^2 (1/2 - r/3 + r^2/4) with the
+//    bracket to 2^-32 (its last term as a constant of a few 2^-32, within
+//    2^-60.5 of the result) and r^2 to 2^-58: three 32-bit high multiplies;
+//  - n ln 2 and 2^58 + ln w_j come rounded from tables, so four 64-bit terms
+//    are added once, at 2^-58 (the largest result, 53 ln 2, still fits).
+// w_j is taken among the candidates near 1/c_j whose logarithm lies closest to
+// a multiple of 2^-58 (Gal's accurate tables); the table also carries the
+// truncations' mean.  Absolute error against 113-bit arithmetic, in units of
+// 2^-58: 0.58 rms and 2.2 at most for uniform u, slice edges and every
+// exponent (6 million draws each); the earlier 4,096-slice form, rounded to
+// 2^-57, had 0.83 and 2.2.
+//
+// Measured against that form: 157 instead of 235 warp instructions per M/M/1
+// client (two variates); M/M/1 65,536 replications x 1,000 clients 0.795 ->
+// 0.604 ms, tandem 4,096 x 256 replications x 10,000 clients 178.3 -> 123.7
+// ms, 16 x 100,000 clients (CTA) 0.611 -> 0.449 ms, skip-sampled 128 x 128
+// forest fire 2.89 -> 2.52 ms.
 // ---------------------------------------------------------------------------
-constexpr int kLogSliceBits = 12;
+constexpr int kLogSliceBits = 13;
 constexpr int kLogSlices = 1 << kLogSliceBits;
 
 struct __align__(16) LogSlice {
-    unsigned long long inv;  // round(2^63 / c_j)
-    unsigned long long lnc;  // round(-ln(inv 2^-63) 2^64) = ln c_j to 2^-64
+    unsigned long long lnw;  // 2^58 + ln(w_j) 2^58, rounded
+    uint32_t w;              // w_j 2^27
+    uint32_t pad;
 };
 
 struct LogTable {
-    const LogSlice* slice;            // kLogSlices entries, device memory
-    const unsigned long long* nln2;   // [n] = round(n ln 2 * 2^57), n = 0..63, device memory
-    unsigned long long ln2_q64;       // round(ln 2 * 2^64)
+    // entry kLogSlices + j is slice j (the pointer is kLogSlices entries
+    // before the first, so that the leading one need not be masked off)
+    const ulonglong2* slice;
+    const unsigned long long* nln2;  // [s] = round((s + 1) ln 2 2^58), s = 0..63; [64] see neg_log_q58
 };
 
 // Table for the current device (built and uploaded on first use; call it
 // outside stream capture before the first launch that needs it).
 mrip_status log_table(LogTable* out);
 
-// High 64 bits of a 64 x 64-bit product, short by 0, 1 or 2 units: of the
-// four 32 x 32 partial products the lowest is dropped and the two middle ones
-// enter by their high halves only (one wide multiply and two high products).
-__device__ __forceinline__ unsigned long long umul64hi_trunc(unsigned long long a, unsigned long long b) {
-    const uint32_t ah = static_cast<uint32_t>(a >> 32), al = static_cast<uint32_t>(a);
-    const uint32_t bh = static_cast<uint32_t>(b >> 32), bl = static_cast<uint32_t>(b);
-    return static_cast<unsigned long long>(ah) * bh + __umulhi(ah, bl) + __umulhi(al, bh);
+// a b >> 32 plus c.
+__device__ __forceinline__ uint32_t mad_hi_u32(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t r;
+    asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
 }
 
-// -log(K 2^-53) * 2^57 for K in [1, 2^53] (the result is below 53 ln 2 < 2^5.2,
-// so it fits a signed 64-bit word).
-__device__ __forceinline__ unsigned long long neg_log_q57(unsigned long long K, const LogTable& tab) {
-    const int lz = __clzll(K);
-    const unsigned long long m = K << lz;                   // bit 63 set: M = m 2^-63
-    const unsigned long long n = static_cast<unsigned long long>(lz - 10);  // 53 - e
-    const int j = static_cast<int>((m >> (63 - kLogSliceBits)) & (kLogSlices - 1));
-    const ulonglong2 e = __ldg(reinterpret_cast<const ulonglong2*>(tab.slice) + j);
-    // m inv = 2^126 (1 + r); r 2^64 = (m inv - 2^126) >> 62 to 2^-60 (the
-    // truncated high product is short by at most 2 units of 2^-62), |r 2^64| < 2^51
-    const unsigned long long hi = umul64hi_trunc(m, e.x);
-    const long long R = static_cast<long long>((hi - (1ULL << 62)) << 2);
-    const int a = static_cast<int>(R >> 20);       // r 2^44, |a| < 2^31
-    const int rho = static_cast<int>(R & 0xFFFFF);  // R = a 2^20 + rho
-    // r^2 2^64 = (a^2 + a rho 2^-19) 2^-24 + rho^2 2^-64 (< 2^-24, dropped); < 2^38
-    const long long r2 =
-        (static_cast<long long>(a) * a + ((static_cast<long long>(a) * rho) >> 19)) >> 24;
-    const int q = __mulhi(a, 1431655766) - static_cast<int>(r2 >> 22);  // (r/3 - r^2/4) 2^44
-    const long long tail = (static_cast<long long>(static_cast<int>(r2 >> 7)) * q) >> 37;  // r^2 q 2^64
-    const long long l1p = R - (r2 >> 1) + tail;                          // log1p(r) 2^64
-    // ln M 2^64 + 2^6: below 2^64 (ln M < ln 2) and, the roundings being a
-    // few units, never below zero, so the unsigned sum does not wrap
-    const unsigned long long s64 = e.y + static_cast<unsigned long long>(l1p) + 64u;
-    const unsigned long long nln2 = __ldg(tab.nln2 + n);  // n ln2 2^57, rounded (n <= 53)
-    // No clamp is needed: for n >= 1 the exact result is at least
-    // -ln(1 - 2^-53) (16 units) and the error below 2^-56 (2 units); for
-    // n = 0 (K = 2^53, M = 1) s64 is 2^6 plus an error of a few units of
-    // 2^-64, so s64 >> 7 = 0 = nln2.
-    return nln2 - (s64 >> 7);
+// -log(1 - u) * 2^58, u = top 53 bits of hi:lo times 2^-53.
+__device__ __forceinline__ unsigned long long neg_log_q58(uint32_t lo, uint32_t hi, const LogTable& tab) {
+    // K 2^11 = 2^64 - (hi:lo without its 11 lowest bits); 0 stands for K = 2^53
+    const unsigned long long K = 0ull - ((static_cast<unsigned long long>(hi) << 32) | (lo & 0xFFFFF800u));
+    const uint32_t kh = static_cast<uint32_t>(K >> 32), kl = static_cast<uint32_t>(K);
+    uint32_t s, ml;
+    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(s) : "r"(kh));
+    uint32_t mh = __funnelshift_lc(kl, kh, s);
+    asm("shl.b32 %0, %1, %2;" : "=r"(ml) : "r"(kl), "r"(s));  // 0 for s >= 32
+    while (static_cast<int>(s) < 0) {  // kh = 0 (s = 2^32 - 1), once in 2^32 draws: one turn
+        s = 32u + static_cast<uint32_t>(__clz(kl));
+        mh = kl ? kl << (s & 31u) : 0x80000000u;  // K = 2^53: M = 1, s = 64
+        ml = 0u;
+    }
+    const ulonglong2 e = __ldg(tab.slice + (mh >> (31 - kLogSliceBits)));
+    const unsigned long long nln2 = __ldg(tab.nln2 + s);
+    const uint32_t w = static_cast<uint32_t>(e.y);
+    const unsigned long long V = static_cast<unsigned long long>(mh) * w + __umulhi(ml, w);  // (1 + r) 2^58
+    const int a = static_cast<int>(static_cast<uint32_t>(V >> 13));                          // r 2^45
+    const uint32_t r2 = static_cast<uint32_t>(__mulhi(a, a));                                // r^2 2^58
+    const uint32_t g = static_cast<uint32_t>(__mulhi(a, -174763)) + 0x80000004u;  // (1/2 - r/3 + ..) 2^32
+    return nln2 + e.x - V + __umulhi(r2, g);
 }
 
-// Exponential variate from words (lo, hi): -log(1 - u) * inv_rate_q57 where
-// inv_rate_q57 = 2^-57 / rate.
+// Exponential variate from words (lo, hi): -log(1 - u) * inv_rate_q58 where
+// inv_rate_q58 = 2^-58 / rate.
 __device__ __forceinline__ double expo_fast(uint32_t lo, uint32_t hi, const LogTable& tab,
-                                            double inv_rate_q57) {
-    const unsigned long long bits = (static_cast<unsigned long long>(hi) << 32) | lo;
-    const unsigned long long K = (1ULL << 53) - (bits >> 11);
-    return __ull2double_rn(neg_log_q57(K, tab)) * inv_rate_q57;
+                                            double inv_rate_q58) {
+    return __ull2double_rn(neg_log_q58(lo, hi, tab)) * inv_rate_q58;
 }
 
 // Bernoulli threshold floor(p 2^32) for p in [0, 1) -- exact in double.

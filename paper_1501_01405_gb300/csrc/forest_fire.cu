@@ -343,9 +343,9 @@ mrip_status launch_ff(const double* dps, long long n_items, long long n_reps, lo
 // step parity for L <= 256, so one barrier per step (between the draw and
 // the update) suffices; L = 512 keeps one buffer and adds a second barrier.
 // ---------------------------------------------------------------------------
-// K = floor(E / mu) without the FP64 pipe: E = y57 2^-57 (the fixed-point
-// log), 2^-57 / mu = dm 2^-shift with dm a 64-bit integer (dm = the double's
-// significand scaled to [2^63, 2^64)), so K = (y57 dm) >> shift on the
+// K = floor(E / mu) without the FP64 pipe: E = y58 2^-58 (the fixed-point
+// log), 2^-58 / mu = dm 2^-shift with dm a 64-bit integer (dm = the double's
+// significand scaled to [2^63, 2^64)), so K = (y58 dm) >> shift on the
 // 128-bit product, saturated at n_cells.  It differs from floor of the FP64
 // quotient only when that quotient is within a few ulps of an integer.
 struct GapScale {
@@ -356,8 +356,8 @@ struct GapScale {
 __device__ __forceinline__ GapScale gap_scale(double p) {
     GapScale g{0ull, 128};
     if (p >= 1.0) return g;
-    const double d = 0x1p-57 / -log1p(-p);  // p in (0, 1)
-    if (!(d < 0x1p64)) {                     // mu below 2^-121: every positive E saturates
+    const double d = 0x1p-58 / -log1p(-p);  // p in (0, 1)
+    if (!(d < 0x1p64)) {                     // mu below 2^-122: every positive E saturates
         g.dm = ~0ull;
         g.shift = 0;
         return g;
@@ -365,18 +365,18 @@ __device__ __forceinline__ GapScale gap_scale(double p) {
     int ex;
     const double mant = frexp(d, &ex);  // d = mant 2^ex, mant in [0.5, 1), ex <= 64
     g.dm = static_cast<unsigned long long>(ldexp(mant, 64));
-    g.shift = 64 - ex;  // >= 128: d < 2^-64, so y57 d < 1 and every gap is 0
+    g.shift = 64 - ex;  // >= 128: d < 2^-64, so y58 d < 1 and every gap is 0
     return g;
 }
 
-__device__ __forceinline__ int gap_cells(unsigned long long y57, const GapScale& g, int n_cells) {
+__device__ __forceinline__ int gap_cells(unsigned long long y58, const GapScale& g, int n_cells) {
     if (g.shift >= 128) return 0;
-    const unsigned long long hi = __umul64hi(y57, g.dm);
+    const unsigned long long hi = __umul64hi(y58, g.dm);
     unsigned long long k;
     if (g.shift >= 64) {
         k = hi >> (g.shift - 64);
     } else {
-        const unsigned long long lo = y57 * g.dm;
+        const unsigned long long lo = y58 * g.dm;
         if (g.shift == 0)
             k = hi ? ~0ull : lo;
         else
@@ -398,11 +398,6 @@ __device__ __forceinline__ unsigned long long first_gap_none(double p, int n) {
     return t >= 0x1p53 ? (1ull << 53) : static_cast<unsigned long long>(t);
 }
 
-__device__ __forceinline__ unsigned long long expo_q57(uint32_t lo, uint32_t hi, const LogTable& tab) {
-    const unsigned long long bits = (static_cast<unsigned long long>(hi) << 32) | lo;
-    return neg_log_q57((1ULL << 53) - (bits >> 11), tab);
-}
-
 // Call only for p > 0.
 __device__ void draw_events(uint32_t* __restrict__ ev, int n_cells, const GapScale& gs, uint32_t t, uint32_t rep,
                             uint32_t c3, const RoundKeys& rk, const LogTable& tab) {
@@ -410,8 +405,8 @@ __device__ void draw_events(uint32_t* __restrict__ ev, int n_cells, const GapSca
     int pos = -1;  // last event so far (warp-uniform)
     for (uint32_t r = 0; pos + 1 < n_cells; ++r) {
         const uint4 b = philox(32u * r + static_cast<uint32_t>(lane), t, rep, c3, rk);
-        const int k0 = gap_cells(expo_q57(b.x, b.y, tab), gs, n_cells);
-        const int k1 = gap_cells(expo_q57(b.z, b.w, tab), gs, n_cells);
+        const int k0 = gap_cells(neg_log_q58(b.x, b.y, tab), gs, n_cells);
+        const int k1 = gap_cells(neg_log_q58(b.z, b.w, tab), gs, n_cells);
         const int span = 2 + k0 + k1;
         int incl = span;
 #pragma unroll
@@ -465,8 +460,8 @@ __device__ void draw_step_events(uint32_t* __restrict__ ev_g, uint32_t* __restri
                 if (lane == 31) tt[warp] = incl;
             } else {
                 const GapScale& gs = g ? gsg : gsh;
-                k0 = gap_cells(expo_q57(b.x, b.y, tab), gs, n_cells);
-                k1 = gap_cells(expo_q57(b.z, b.w, tab), gs, n_cells);
+                k0 = gap_cells(neg_log_q58(b.x, b.y, tab), gs, n_cells);
+                k1 = gap_cells(neg_log_q58(b.z, b.w, tab), gs, n_cells);
                 span = 2 + k0 + k1;
                 incl = span;
 #pragma unroll

@@ -22,9 +22,9 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // Times in 64-bit fixed point.  GB300 retires about two FP64 operations per
 // SM-clock and over forty 32-bit integer multiplies, so the queue recurrences
 // (additions, subtractions and maxima only) run on integers: a time t is held
-// as round(t 2^48).  A variate is E / rate with E = y57 2^-57 from the
-// fixed-point log, i.e. round(y57 * (2^-9 / rate)), the factor stored as a
-// 64-bit multiplier cm = round(2^57 / rate) (2^-9 / rate = cm 2^-66).  A
+// as round(t 2^48).  A variate is E / rate with E = y58 2^-58 from the
+// fixed-point log, i.e. round(y58 * (2^-10 / rate)), the factor stored as a
+// 64-bit multiplier cm = round(2^56 / rate) (2^-10 / rate = cm 2^-66).  A
 // variate then carries the multiplier's relative error (2^-53, as an FP64
 // division would) plus at most one unit (2^-48), and every recurrence step is
 // exact, where FP64 rounds each addition; the outputs agree with
@@ -42,18 +42,24 @@ constexpr int kFixBits = 48;
 constexpr long long kFixGuard = 1LL << 60;
 constexpr long long kFixNegInf = -(1LL << 62);  // "empty" state: v - A stays above -2^63
 
-// 2^-9 / rate as cm 2^-66 (cm in [2^53, 2^63] for the rates above: at least
-// 53 significant bits), so that round(y57 2^-9 / rate) = (hi(y57 cm) + 2) >> 2.
-// hi comes from umul64hi_trunc, 0 to 2 units short, so 3 is added instead of
-// 2: the variate is then within one unit (2^-48) of y57 2^-9 / rate.
+// 2^-10 / rate as cm 2^-66 (cm in [2^52, 2^62] for the rates above: at least
+// 53 significant bits), so that round(y58 2^-10 / rate) = (hi(y58 cm) + 2) >> 2.
+// Of the four partial products of hi(y58 cm) the lowest is dropped and the two
+// middle ones enter by their high halves only, 0 to 3 units short in all, so
+// 3 is added instead of 2: the variate is then within one unit (2^-48) of
+// y58 2^-10 / rate.  cm < 2^62 keeps the sum of the middle halves (below
+// 1.15 2^31 + 2^30 + 4) in 32 bits, so both additions ride on the multiplies.
 __device__ __forceinline__ bool fix_rate_ok(double rate) { return rate >= 0x1p-6 && rate <= 0x1p4; }
 
 __device__ __forceinline__ unsigned long long fix_scale(double rate) {
-    return static_cast<unsigned long long>(0x1p57 / rate + 0.5);
+    return static_cast<unsigned long long>(0x1p56 / rate + 0.5);
 }
 
-__device__ __forceinline__ long long to_fix(unsigned long long y57, unsigned long long cm) {
-    return static_cast<long long>((umul64hi_trunc(y57, cm) + 3u) >> 2);
+__device__ __forceinline__ long long to_fix(unsigned long long y58, unsigned long long cm) {
+    const uint32_t yh = static_cast<uint32_t>(y58 >> 32), yl = static_cast<uint32_t>(y58);
+    const uint32_t ch = static_cast<uint32_t>(cm >> 32), cl = static_cast<uint32_t>(cm);
+    const uint32_t mid = mad_hi_u32(yl, ch, mad_hi_u32(yh, cl, 3u));
+    return static_cast<long long>((static_cast<unsigned long long>(yh) * ch + mid) >> 2);
 }
 
 struct U128 {
@@ -83,11 +89,6 @@ __device__ __forceinline__ void add_u128(U128& a, const U128& b) {
     a.hi += b.hi + ((a.lo < b.lo) ? 1u : 0u);
 }
 
-__device__ __forceinline__ unsigned long long word_k(uint32_t lo, uint32_t hi) {
-    const unsigned long long bits = (static_cast<unsigned long long>(hi) << 32) | lo;
-    return (1ULL << 53) - (bits >> 11);
-}
-
 struct Mm1Out {
     double* wait;
     double* idle;
@@ -95,7 +96,7 @@ struct Mm1Out {
 };
 
 // Client n of (dp, rep): service S_n from words (0,1), gap A_{n+1} from (2,3).
-// inv_mu, inv_lam are 2^-57 / rate (see expo_fast).
+// inv_mu, inv_lam are 2^-58 / rate (see expo_fast).
 __device__ __forceinline__ void mm1_client(uint32_t n, uint32_t rep, uint32_t dp, double inv_lam,
                                            double inv_mu, const RoundKeys& rk, const LogTable& tab,
                                            double& s, double& a) {
@@ -130,8 +131,8 @@ __global__ void __launch_bounds__(128, 4) mm1_serial_kernel(const double* __rest
         bool overflow = false;
         for (long long n = 0; n < n_clients; ++n) {
             const uint4 b = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-            const long long s_ = to_fix(neg_log_q57(word_k(b.x, b.y), tab), cmu);
-            const long long a_ = to_fix(neg_log_q57(word_k(b.z, b.w), tab), cl);
+            const long long s_ = to_fix(neg_log_q58(b.x, b.y, tab), cmu);
+            const long long a_ = to_fix(neg_log_q58(b.z, b.w, tab), cl);
             sw.add(wf);
             const long long v = wf + s_;
             sv.add(v);
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(128, 4) mm1_serial_kernel(const double* __rest
             return;
         }
     }
-    const double inv_lam = 0x1p-57 / lam, inv_mu = 0x1p-57 / mu;
+    const double inv_lam = 0x1p-58 / lam, inv_mu = 0x1p-58 / mu;
     double w = 0.0, sum_w = 0.0, sum_i = 0.0, sum_v = 0.0;
     for (long long n = 0; n < n_clients; ++n) {
         double s, a;
@@ -192,7 +193,7 @@ __global__ void mm1_warp_coop_kernel(const double* __restrict__ dps, long long n
     if (item >= n_items) return;  // warp-uniform
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
-    const double inv_lam = 0x1p-57 / dps[2 * dp], inv_mu = 0x1p-57 / dps[2 * dp + 1];
+    const double inv_lam = 0x1p-58 / dps[2 * dp], inv_mu = 0x1p-58 / dps[2 * dp + 1];
     const long long seg = (n_clients + 31) / 32;
     const long long lo = lane * seg;
     const long long hi = (lo + seg < n_clients) ? lo + seg : n_clients;
@@ -295,8 +296,8 @@ __global__ void __launch_bounds__(128, 8) tandem3_serial_kernel(const double* __
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double lam = dps[4 * dp], mu1 = dps[4 * dp + 1], mu2 = dps[4 * dp + 2],
                  mu3 = dps[4 * dp + 3];
-    const double i_lam = 0x1p-57 / lam, i_mu1 = 0x1p-57 / mu1, i_mu2 = 0x1p-57 / mu2,
-                 i_mu3 = 0x1p-57 / mu3;
+    const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2,
+                 i_mu3 = 0x1p-58 / mu3;
     const uint32_t c3 = stream_word(tag, dp);
     const long long w_len = (n_clients < window) ? n_clients : window;
     double sum_y = 0.0, sum_a = 0.0, sum_1 = 0.0, sum_2 = 0.0, sum_3 = 0.0;
@@ -313,10 +314,10 @@ __global__ void __launch_bounds__(128, 8) tandem3_serial_kernel(const double* __
                         unsigned long long& y3) {
             const uint4 b0 = philox(0u, n, rep, c3, rk);
             const uint4 b1 = philox(1u, n, rep, c3, rk);
-            ya = neg_log_q57(word_k(b0.x, b0.y), tab);
-            y1 = neg_log_q57(word_k(b0.z, b0.w), tab);
-            y2 = neg_log_q57(word_k(b1.x, b1.y), tab);
-            y3 = neg_log_q57(word_k(b1.z, b1.w), tab);
+            ya = neg_log_q58(b0.x, b0.y, tab);
+            y1 = neg_log_q58(b0.z, b0.w, tab);
+            y2 = neg_log_q58(b1.x, b1.y, tab);
+            y3 = neg_log_q58(b1.z, b1.w, tab);
         };
         auto step = [&](unsigned long long ya, unsigned long long y1, unsigned long long y2,
                         unsigned long long y3) {
@@ -540,7 +541,7 @@ __device__ void tandem_coop_fp64(long long item, uint32_t dp, uint32_t rep, doub
                                  const RoundKeys& rk, const LogTable& tab, const TandemOut& out) {
     (void)dp;
     const int lane = threadIdx.x & 31;
-    const double i_lam = 0x1p-57 / lam, i_mu1 = 0x1p-57 / mu1, i_mu2 = 0x1p-57 / mu2, i_mu3 = 0x1p-57 / mu3;
+    const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2, i_mu3 = 0x1p-58 / mu3;
     const long long w_len = (n_clients < window) ? n_clients : window;
     const long long seg = (n_clients + 31) / 32;
     const long long lo = min(lane * seg, n_clients);
@@ -626,8 +627,8 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double lam = dps[4 * dp], mu1 = dps[4 * dp + 1], mu2 = dps[4 * dp + 2], mu3 = dps[4 * dp + 3];
-    const double i_lam = 0x1p-57 / lam, i_mu1 = 0x1p-57 / mu1, i_mu2 = 0x1p-57 / mu2,
-                 i_mu3 = 0x1p-57 / mu3;
+    const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2,
+                 i_mu3 = 0x1p-58 / mu3;
     const uint32_t c3 = stream_word(tag, dp);
     const long long w_len = (n_clients < window) ? n_clients : window;
     const long long seg = (n_clients + 31) / 32;
@@ -641,10 +642,10 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
         for (long long n = lo; n < hi; ++n) {
             const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
             const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-            f = ftmap_push(f, to_fix(neg_log_q57(word_k(b0.x, b0.y), tab), cl),
-                           to_fix(neg_log_q57(word_k(b0.z, b0.w), tab), c1),
-                           to_fix(neg_log_q57(word_k(b1.x, b1.y), tab), c2),
-                           to_fix(neg_log_q57(word_k(b1.z, b1.w), tab), c3f));
+            f = ftmap_push(f, to_fix(neg_log_q58(b0.x, b0.y, tab), cl),
+                           to_fix(neg_log_q58(b0.z, b0.w, tab), c1),
+                           to_fix(neg_log_q58(b1.x, b1.y, tab), c2),
+                           to_fix(neg_log_q58(b1.z, b1.w, tab), c3f));
         }
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -664,10 +665,10 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
         for (long long n = lo; n < hi && !bad; ++n) {
             const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
             const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-            const unsigned long long ya = neg_log_q57(word_k(b0.x, b0.y), tab);
-            const unsigned long long y1 = neg_log_q57(word_k(b0.z, b0.w), tab);
-            const unsigned long long y2 = neg_log_q57(word_k(b1.x, b1.y), tab);
-            const unsigned long long y3 = neg_log_q57(word_k(b1.z, b1.w), tab);
+            const unsigned long long ya = neg_log_q58(b0.x, b0.y, tab);
+            const unsigned long long y1 = neg_log_q58(b0.z, b0.w, tab);
+            const unsigned long long y2 = neg_log_q58(b1.x, b1.y, tab);
+            const unsigned long long y3 = neg_log_q58(b1.z, b1.w, tab);
             const long long a = to_fix(ya, cl);
             long long q = v1 - a;
             v1 = ((q > 0) ? q : 0) + to_fix(y1, c1);
@@ -822,8 +823,8 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
         long long* st_a = fix_stage + k * blockDim.x + threadIdx.x;
         for (long long n = lo; n < hi; ++n) {
             const uint4 b = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-            const long long sv = to_fix(neg_log_q57(word_k(b.x, b.y), tab), cmu);
-            const long long av = to_fix(neg_log_q57(word_k(b.z, b.w), tab), cl);
+            const long long sv = to_fix(neg_log_q58(b.x, b.y, tab), cmu);
+            const long long av = to_fix(neg_log_q58(b.z, b.w, tab), cl);
             if (staged) {
                 st_s[(n - lo) * blockDim.x] = sv;
                 st_a[(n - lo) * blockDim.x] = av;
@@ -842,8 +843,8 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
                 av = st_a[(n - lo) * blockDim.x];
             } else {
                 const uint4 b = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-                sv = to_fix(neg_log_q57(word_k(b.x, b.y), tab), cmu);
-                av = to_fix(neg_log_q57(word_k(b.z, b.w), tab), cl);
+                sv = to_fix(neg_log_q58(b.x, b.y, tab), cmu);
+                av = to_fix(neg_log_q58(b.z, b.w, tab), cl);
             }
             sm.w.add(w);
             const long long v = w + sv;
@@ -877,7 +878,7 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
         }
     }
     // FP64: the same passes with doubles
-    const double inv_lam = 0x1p-57 / lam, inv_mu = 0x1p-57 / mu;
+    const double inv_lam = 0x1p-58 / lam, inv_mu = 0x1p-58 / mu;
     DblMap f{-INFINITY, 0.0};
     for (long long n = lo; n < hi; ++n) {
         double sv, av;
@@ -958,10 +959,10 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
         for (long long n = lo; n < hi; ++n) {
             const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
             const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-            f = ftmap_push(f, to_fix(neg_log_q57(word_k(b0.x, b0.y), tab), cl),
-                           to_fix(neg_log_q57(word_k(b0.z, b0.w), tab), c1),
-                           to_fix(neg_log_q57(word_k(b1.x, b1.y), tab), c2),
-                           to_fix(neg_log_q57(word_k(b1.z, b1.w), tab), c3f));
+            f = ftmap_push(f, to_fix(neg_log_q58(b0.x, b0.y, tab), cl),
+                           to_fix(neg_log_q58(b0.z, b0.w, tab), c1),
+                           to_fix(neg_log_q58(b1.x, b1.y, tab), c2),
+                           to_fix(neg_log_q58(b1.z, b1.w, tab), c3f));
         }
         // block exclusive scan of the maps
         FTMap incl = f;
@@ -981,15 +982,15 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
         bool bad = v3 >= kFixGuard;
         U128 sy;
         double wa = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
-        const double i_lam = 0x1p-57 / lam, i_mu1 = 0x1p-57 / mu1, i_mu2 = 0x1p-57 / mu2,
-                     i_mu3 = 0x1p-57 / mu3;
+        const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2,
+                     i_mu3 = 0x1p-58 / mu3;
         for (long long n = lo; n < hi && !bad; ++n) {
             const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
             const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-            const unsigned long long ya = neg_log_q57(word_k(b0.x, b0.y), tab);
-            const unsigned long long y1 = neg_log_q57(word_k(b0.z, b0.w), tab);
-            const unsigned long long y2 = neg_log_q57(word_k(b1.x, b1.y), tab);
-            const unsigned long long y3 = neg_log_q57(word_k(b1.z, b1.w), tab);
+            const unsigned long long ya = neg_log_q58(b0.x, b0.y, tab);
+            const unsigned long long y1 = neg_log_q58(b0.z, b0.w, tab);
+            const unsigned long long y2 = neg_log_q58(b1.x, b1.y, tab);
+            const unsigned long long y3 = neg_log_q58(b1.z, b1.w, tab);
             const long long a = to_fix(ya, cl);
             long long q = v1 - a;
             v1 = ((q > 0) ? q : 0) + to_fix(y1, c1);

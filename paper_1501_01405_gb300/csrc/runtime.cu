@@ -79,18 +79,42 @@ int* device_error_flags() {
 }
 
 namespace {
-// 1/c_j and ln c_j for the slices of [1, 2), from the host's long-double
-// logarithm (64-bit or wider mantissa).
+// neg_log_q58's 64-bit sum without the n ln 2 term, for the mantissa mh:ml of
+// slice e.
+unsigned long long log_core(uint32_t mh, uint32_t ml, const LogSlice& e) {
+    auto hi_u = [](uint32_t a, uint32_t b) { return static_cast<uint32_t>((static_cast<uint64_t>(a) * b) >> 32); };
+    auto hi_s = [](int32_t a, int32_t b) { return static_cast<int32_t>((static_cast<int64_t>(a) * b) >> 32); };
+    const uint64_t V = static_cast<uint64_t>(mh) * e.w + hi_u(ml, e.w);
+    const int32_t a = static_cast<int32_t>(static_cast<uint32_t>(V >> 13));
+    const uint32_t r2 = static_cast<uint32_t>(hi_s(a, a));
+    return e.lnw - V + hi_u(r2, static_cast<uint32_t>(hi_s(a, -174763)) + 0x80000004u);
+}
+
+// The slices' w_j and ln w_j from the host's long-double logarithm (64-bit or
+// wider mantissa).  w_j keeps |r| <= 2^-14 over its slice; among up to 49 such
+// 27-bit values around 1/c_j the one whose logarithm's rounding to 2^-58, about
+// the mean 0.3 of the truncations, is smallest.
 void build_log_slices(std::vector<LogSlice>& t) {
+    constexpr long double kMean = 0.3L;
     t.resize(kLogSlices);
     for (int j = 0; j < kLogSlices; ++j) {
-        const long double c = 1.0L + (static_cast<long double>(j) + 0.5L) / static_cast<long double>(kLogSlices);
-        const unsigned long long inv =
-            static_cast<unsigned long long>(ldexpl(1.0L / c, 63) + 0.5L);
-        const long double ic = ldexpl(static_cast<long double>(inv), -63);
-        const long double lnc = -logl(ic);
-        t[j].inv = inv;
-        t[j].lnc = static_cast<unsigned long long>(ldexpl(lnc, 64) + 0.5L);
+        const long double from = 1.0L + static_cast<long double>(j) / kLogSlices;
+        const long double to = 1.0L + static_cast<long double>(j + 1) / kLogSlices;
+        const long long lo = static_cast<long long>(ceill(ldexpl((1.0L - 0x1p-14L) / from, 27)));
+        const long long hi = static_cast<long long>(floorl(ldexpl((1.0L + 0x1p-14L) / to, 27)));
+        const long long mid = static_cast<long long>(ldexpl(2.0L / (from + to), 27) + 0.5L);
+        long double best = 2.0L;
+        for (long long w = mid - 24; w <= mid + 24; ++w) {
+            if (w < lo || w > hi) continue;
+            const long double x = ldexpl(logl(ldexpl(static_cast<long double>(w), -27)), 58) + kMean;
+            const long double r = floorl(x + 0.5L);
+            if (fabsl(x - r) < best) {
+                best = fabsl(x - r);
+                t[j].w = static_cast<uint32_t>(w);
+                t[j].lnw = (1ull << 58) - static_cast<unsigned long long>(-r);
+                t[j].pad = 0;
+            }
+        }
     }
 }
 }  // namespace
@@ -98,16 +122,18 @@ void build_log_slices(std::vector<LogSlice>& t) {
 mrip_status log_table(LogTable* out) {
     std::lock_guard<std::mutex> lock(g_scratch_mutex);
     DeviceScratch& d = dev_scratch();
-    const unsigned long long ln2_q64 = static_cast<unsigned long long>(ldexpl(logl(2.0L), 64) + 0.5L);
     if (!d.log_slices) {
         std::vector<LogSlice> t;
         build_log_slices(t);
-        // n ln2 2^57 rounded, from the 128-bit product n * round(ln2 2^64)
-        std::vector<unsigned long long> nln2(64);
-        for (unsigned n = 0; n < 64; ++n) {
-            const unsigned __int128 prod = static_cast<unsigned __int128>(n) * ln2_q64 + 64u;
-            nln2[n] = static_cast<unsigned long long>(prod >> 7);
+        // n ln2 2^58 rounded, from the 128-bit product n * round(ln2 2^64);
+        // entry 64 makes K = 2^53 (M = 1 in slice 0) exactly 0
+        const unsigned long long ln2_q64 = static_cast<unsigned long long>(ldexpl(logl(2.0L), 64) + 0.5L);
+        std::vector<unsigned long long> nln2(65);
+        for (unsigned s = 0; s < 64; ++s) {
+            const unsigned __int128 prod = static_cast<unsigned __int128>(s + 1) * ln2_q64 + 32u;
+            nln2[s] = static_cast<unsigned long long>(prod >> 6);
         }
+        nln2[64] = 0ull - log_core(0x80000000u, 0u, t[0]);
         const size_t slice_bytes = t.size() * sizeof(LogSlice);
         LogSlice* p = nullptr;
         cudaError_t e = cudaMalloc(&p, slice_bytes + nln2.size() * sizeof(unsigned long long));
@@ -121,9 +147,9 @@ mrip_status log_table(LogTable* out) {
         }
         d.log_slices = p;
     }
-    out->slice = d.log_slices;
+    out->slice = reinterpret_cast<const ulonglong2*>(reinterpret_cast<uintptr_t>(d.log_slices) -
+                                                     kLogSlices * sizeof(LogSlice));
     out->nln2 = reinterpret_cast<const unsigned long long*>(d.log_slices + kLogSlices);
-    out->ln2_q64 = ln2_q64;
     return MRIP_OK;
 }
 
@@ -164,7 +190,7 @@ __global__ void expo_kernel(const uint32_t* __restrict__ lo, const uint32_t* __r
     long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
     if (i >= n) return;
     if (u_out) u_out[i] = u53(lo[i], hi[i]);
-    if (e_out) e_out[i] = expo_fast(lo[i], hi[i], tab, 0x1p-57 / rate[i]);
+    if (e_out) e_out[i] = expo_fast(lo[i], hi[i], tab, 0x1p-58 / rate[i]);
 }
 
 }  // namespace mrip

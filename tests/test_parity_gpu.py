@@ -82,6 +82,23 @@ def test_expo_variates(eng, torch_mod):
     assert np.max(np.abs(got - e_ref)[big] / np.spacing(e_ref[big])) <= 3
 
 
+def test_expo_edges(eng, torch_mod):
+    """The logarithm where its cases meet: 1 - u = K 2^-53 with K at powers of two and their neighbours (the high
+    word of 2^11 K zero below 2^21), at the edges of the 8,192 slices, and K = 2^53 (u = 0).  Bound as above."""
+    t = torch_mod
+    ks = [2**e + d for e in range(54) for d in (-1, 0, 1)] + [2**21 - 2**10, 3 << 19]
+    ks += [2**52 + (j << 39) + d for j in (0, 1, 2, 4095, 4096, 8190, 8191) for d in (-1, 0, 1)]
+    x = np.array([(2**53 - k) << 11 for k in sorted(set(ks)) if 1 <= k <= 2**53], dtype=np.uint64)
+    lo, hi = (x & np.uint64(0xFFFFFFFF)).astype(np.uint32), (x >> np.uint64(32)).astype(np.uint32)
+    rate = np.ones(x.size)
+    e = t.empty(x.size, dtype=t.float64, device="cuda")
+    eng.mrip_expo(dev(t, lo.view(np.int32)), dev(t, hi.view(np.int32)), dev(t, rate), None, e)
+    _, ref = oracle.u53_expo(lo, hi, rate)
+    got = e.cpu().numpy()
+    assert np.all(np.abs(got - ref) <= 4 * np.spacing(np.abs(ref)) + 2.0**-55)
+    assert got[ref == 0.0].tolist() == [0.0]
+
+
 # ------------------------------------------------------------------ M/M/1
 MM1_DPS = np.array([[0.9, 1.0], [0.5, 1.0], [1.2, 1.0]])
 
