@@ -148,6 +148,67 @@ __device__ __forceinline__ double u53(uint32_t lo, uint32_t hi) {
     return __ull2double_rn(bits >> 11) * 0x1p-53;
 }
 
+// Counters (c0, c1, rep, c3) of one replication with a small c0 and a running
+// c1 (the queues' clients, the walks' and pi's blocks).  Three of the first six
+// products do not depend on c1: round 1's products (of c0 <= 1, whose high
+// half is 0, and of rep), round 2's product of word 2 and round 3's product of
+// word 0.  RowKey holds what they leave, once per replication: 16 (c0 = 0) or
+// 31 (the pair c0 = 0, 1, which shares round 2's product) products per client
+// remain of 20 or 40, same words.  (With the recurrences' sums and
+// maxima as carry chains and sign masks: M/M/1 65,536 x 1,000 clients 0.604 ->
+// 0.569 ms, tandem 4,096 x 256 x 10,000 clients 123.7 -> 122.7 ms; part of it
+// the compiler had already hoisted.)
+struct RowKey {
+    uint32_t h;     // word 0 after round 1, without c1
+    uint32_t u;     // word 1 after round 2, with round 3's key
+    uint32_t t, l;  // round 3's product of word 0: high half with its key, low half
+};
+
+__device__ __forceinline__ RowKey row_key(uint32_t rep, uint32_t c3, const RoundKeys& rk) {
+    RowKey r;
+    uint32_t hi, lo, w0;
+    mul_wide_u32(0xCD9E8D57u, rep, hi, lo);
+    r.h = hi ^ rk.k0[0];
+    w0 = lo ^ rk.k0[1];
+    mul_wide_u32(0xCD9E8D57u, c3 ^ rk.k1[0], hi, lo);
+    w0 ^= hi;
+    r.u = lo ^ rk.k0[2];
+    mul_wide_u32(0xD2511F53u, w0, hi, lo);
+    r.t = hi ^ rk.k1[2];
+    r.l = lo;
+    return r;
+}
+
+// Rounds 3 to 10 of block (kC0, c1), c0 = kC0 = 0 or 1; (p_hi, p_lo) is round
+// 2's product 0xD2511F53 * (r.h ^ c1), the same for both.
+template <uint32_t kC0>
+__device__ __forceinline__ uint4 row_rounds(const RowKey& r, uint32_t p_hi, uint32_t p_lo, const RoundKeys& rk) {
+    static_assert(kC0 <= 1, "0xD2511F53 * c0 must fit its low half");
+    uint32_t x0, x1, x2, x3, hi;
+    mul_wide_u32(0xCD9E8D57u, p_hi ^ (kC0 * 0xD2511F53u) ^ rk.k1[1], hi, x1);
+    x0 = hi ^ r.u;
+    x2 = r.t ^ p_lo;
+    x3 = r.l;
+#pragma unroll
+    for (int i = 3; i < 10; ++i) philox_round(x0, x1, x2, x3, rk.k0[i], rk.k1[i]);
+    return make_uint4(x0, x1, x2, x3);
+}
+
+// philox(0, c1, rep, c3) from the replication's row key.
+__device__ __forceinline__ uint4 philox_row(const RowKey& r, uint32_t c1, const RoundKeys& rk) {
+    uint32_t hi, lo;
+    mul_wide_u32(0xD2511F53u, r.h ^ c1, hi, lo);
+    return row_rounds<0>(r, hi, lo, rk);
+}
+
+// philox(0, c1, rep, c3) and philox(1, c1, rep, c3).
+__device__ __forceinline__ void philox_row2(const RowKey& r, uint32_t c1, const RoundKeys& rk, uint4& b0, uint4& b1) {
+    uint32_t hi, lo;
+    mul_wide_u32(0xD2511F53u, r.h ^ c1, hi, lo);
+    b0 = row_rounds<0>(r, hi, lo, rk);
+    b1 = row_rounds<1>(r, hi, lo, rk);
+}
+
 // ---------------------------------------------------------------------------
 // Exponential variates without the FP64 log.
 //
@@ -166,15 +227,16 @@ __device__ __forceinline__ double u53(uint32_t lo, uint32_t hi) {
 //    one high and one wide multiply and no shift: it enters the result as it
 //    is, and its bits 13..44 are r 2^45 as a signed word (1 2^45 vanishes
 //    modulo 2^32);
-//  - |r| <= 2^-14 leaves log1p(r) = r - r^2 (1/2 - r/3 + r^2/4) with the
-//    bracket to 2^-32 (its last term as a constant of a few 2^-32, within
-//    2^-60.5 of the result) and r^2 to 2^-58: three 32-bit high multiplies;
+//  - |r| <= 2^-14 leaves log1p(r) = r - r^2/2 + r^3/3 - r^4/4: r^2 to 2^-58 is
+//    one 32-bit high multiply; the last two terms (below 2^-42) are FP32, on
+//    the half of the FMA pipe that integer multiplies cannot use, and rounded
+//    to an integer by an added 1.5 2^23;
 //  - n ln 2 and 2^58 + ln w_j come rounded from tables, so four 64-bit terms
 //    are added once, at 2^-58 (the largest result, 53 ln 2, still fits).
 // w_j is taken among the candidates near 1/c_j whose logarithm lies closest to
 // a multiple of 2^-58 (Gal's accurate tables); the table also carries the
 // truncations' mean.  Absolute error against 113-bit arithmetic, in units of
-// 2^-58: 0.58 rms and 2.2 at most for uniform u, slice edges and every
+// 2^-58: 0.58 rms and 2.04 at most over uniform u, slice edges and every
 // exponent (6 million draws each); the earlier 4,096-slice form, rounded to
 // 2^-57, had 0.83 and 2.2.
 //
@@ -182,7 +244,10 @@ __device__ __forceinline__ double u53(uint32_t lo, uint32_t hi) {
 // client (two variates); M/M/1 65,536 replications x 1,000 clients 0.795 ->
 // 0.604 ms, tandem 4,096 x 256 replications x 10,000 clients 178.3 -> 123.7
 // ms, 16 x 100,000 clients (CTA) 0.611 -> 0.449 ms, skip-sampled 128 x 128
-// forest fire 2.89 -> 2.52 ms.
+// forest fire 2.89 -> 2.52 ms.  That moved the limit to the FMA-heavy pipe (78 %
+// busy on the tandem); the FP32 tail, n ln 2 from shared memory (no 64-bit
+// address multiply) and carry-chain adds (on the other pipe) take the M/M/1
+// row on from 0.569 to 0.531 ms and the tandem's from 121.2 to 119.0.
 // ---------------------------------------------------------------------------
 constexpr int kLogSliceBits = 13;
 constexpr int kLogSlices = 1 << kLogSliceBits;
@@ -198,11 +263,31 @@ struct LogTable {
     // before the first, so that the leading one need not be masked off)
     const ulonglong2* slice;
     const unsigned long long* nln2;  // [s] = round((s + 1) ln 2 2^58), s = 0..63; [64] see neg_log_q58
+    uint32_t nln2_shared;            // the same table in the CTA's shared memory (stage_nln2)
 };
+constexpr int kLogExponents = 65;
+// coefficients of the FP32 tail in a = r 2^45, result in half units of 2^-58
+constexpr float kLogR3 = -0x1p-76f / 3.0f, kLogR4 = 0x1p-123f, kLogMagic = 12582912.0f;  // 1.5 2^23
+constexpr uint32_t kLogMagicBits = 0x4B400000u;
 
 // Table for the current device (built and uploaded on first use; call it
 // outside stream capture before the first launch that needs it).
 mrip_status log_table(LogTable* out);
+
+// The CTA's copy of the n ln 2 table, for neg_log_q58<true> (every thread calls;
+// ends with a barrier).
+__device__ __forceinline__ void stage_nln2(LogTable& tab, unsigned long long (&buf)[kLogExponents]) {
+    for (int i = threadIdx.x; i < kLogExponents; i += blockDim.x) buf[i] = tab.nln2[i];
+    tab.nln2_shared = static_cast<uint32_t>(__cvta_generic_to_shared(buf));
+    __syncthreads();
+}
+
+// hi:lo + c as an explicit carry chain (both adds on the integer ALU; a plain
+// 64-bit add may be put on the multiply pipe).
+__device__ __forceinline__ unsigned long long add_carry(uint32_t lo, uint32_t hi, uint32_t c) {
+    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(lo), "+r"(hi) : "r"(c));
+    return (static_cast<unsigned long long>(hi) << 32) | lo;
+}
 
 // a b >> 32 plus c.
 __device__ __forceinline__ uint32_t mad_hi_u32(uint32_t a, uint32_t b, uint32_t c) {
@@ -211,7 +296,9 @@ __device__ __forceinline__ uint32_t mad_hi_u32(uint32_t a, uint32_t b, uint32_t 
     return r;
 }
 
-// -log(1 - u) * 2^58, u = top 53 bits of hi:lo times 2^-53.
+// -log(1 - u) * 2^58, u = top 53 bits of hi:lo times 2^-53.  kShared: n ln 2
+// from the copy stage_nln2 made.
+template <bool kShared>
 __device__ __forceinline__ unsigned long long neg_log_q58(uint32_t lo, uint32_t hi, const LogTable& tab) {
     // K 2^11 = 2^64 - (hi:lo without its 11 lowest bits); 0 stands for K = 2^53
     const unsigned long long K = 0ull - ((static_cast<unsigned long long>(hi) << 32) | (lo & 0xFFFFF800u));
@@ -226,20 +313,28 @@ __device__ __forceinline__ unsigned long long neg_log_q58(uint32_t lo, uint32_t 
         ml = 0u;
     }
     const ulonglong2 e = __ldg(tab.slice + (mh >> (31 - kLogSliceBits)));
-    const unsigned long long nln2 = __ldg(tab.nln2 + s);
+    unsigned long long nln2;
+    if constexpr (kShared)
+        asm("ld.shared.u64 %0, [%1];" : "=l"(nln2) : "r"(tab.nln2_shared + 8u * s));
+    else
+        nln2 = __ldg(tab.nln2 + s);
     const uint32_t w = static_cast<uint32_t>(e.y);
-    const unsigned long long V = static_cast<unsigned long long>(mh) * w + __umulhi(ml, w);  // (1 + r) 2^58
-    const int a = static_cast<int>(static_cast<uint32_t>(V >> 13));                          // r 2^45
-    const uint32_t r2 = static_cast<uint32_t>(__mulhi(a, a));                                // r^2 2^58
-    const uint32_t g = static_cast<uint32_t>(__mulhi(a, -174763)) + 0x80000004u;  // (1/2 - r/3 + ..) 2^32
-    return nln2 + e.x - V + __umulhi(r2, g);
+    uint32_t v_hi, v_lo;
+    mul_wide_u32(mh, w, v_hi, v_lo);
+    const unsigned long long V = add_carry(v_lo, v_hi, __umulhi(ml, w));  // (1 + r) 2^58
+    const int a = static_cast<int>(static_cast<uint32_t>(V >> 13));       // r 2^45
+    const uint32_t r2 = static_cast<uint32_t>(__mulhi(a, a));             // r^2 2^58
+    const float f = __int2float_rn(a);
+    const float tail = __fmaf_rn(f * f * f, __fmaf_rn(f, kLogR4, kLogR3), kLogMagic);  // -2 r^3/3 + r^4/2
+    return nln2 + e.x - V + ((r2 + (__float_as_uint(tail) - kLogMagicBits)) >> 1);
 }
 
 // Exponential variate from words (lo, hi): -log(1 - u) * inv_rate_q58 where
 // inv_rate_q58 = 2^-58 / rate.
+template <bool kShared>
 __device__ __forceinline__ double expo_fast(uint32_t lo, uint32_t hi, const LogTable& tab,
                                             double inv_rate_q58) {
-    return __ull2double_rn(neg_log_q58(lo, hi, tab)) * inv_rate_q58;
+    return __ull2double_rn(neg_log_q58<kShared>(lo, hi, tab)) * inv_rate_q58;
 }
 
 // Bernoulli threshold floor(p 2^32) for p in [0, 1) -- exact in double.

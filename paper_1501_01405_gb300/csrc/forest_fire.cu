@@ -405,8 +405,8 @@ __device__ void draw_events(uint32_t* __restrict__ ev, int n_cells, const GapSca
     int pos = -1;  // last event so far (warp-uniform)
     for (uint32_t r = 0; pos + 1 < n_cells; ++r) {
         const uint4 b = philox(32u * r + static_cast<uint32_t>(lane), t, rep, c3, rk);
-        const int k0 = gap_cells(neg_log_q58(b.x, b.y, tab), gs, n_cells);
-        const int k1 = gap_cells(neg_log_q58(b.z, b.w, tab), gs, n_cells);
+        const int k0 = gap_cells(neg_log_q58<false>(b.x, b.y, tab), gs, n_cells);
+        const int k1 = gap_cells(neg_log_q58<false>(b.z, b.w, tab), gs, n_cells);
         const int span = 2 + k0 + k1;
         int incl = span;
 #pragma unroll
@@ -460,8 +460,8 @@ __device__ void draw_step_events(uint32_t* __restrict__ ev_g, uint32_t* __restri
                 if (lane == 31) tt[warp] = incl;
             } else {
                 const GapScale& gs = g ? gsg : gsh;
-                k0 = gap_cells(neg_log_q58(b.x, b.y, tab), gs, n_cells);
-                k1 = gap_cells(neg_log_q58(b.z, b.w, tab), gs, n_cells);
+                k0 = gap_cells(neg_log_q58<false>(b.x, b.y, tab), gs, n_cells);
+                k1 = gap_cells(neg_log_q58<false>(b.z, b.w, tab), gs, n_cells);
                 span = 2 + k0 + k1;
                 incl = span;
 #pragma unroll

@@ -48,7 +48,7 @@ constexpr long long kFixNegInf = -(1LL << 62);  // "empty" state: v - A stays ab
 // middle ones enter by their high halves only, 0 to 3 units short in all, so
 // 3 is added instead of 2: the variate is then within one unit (2^-48) of
 // y58 2^-10 / rate.  cm < 2^62 keeps the sum of the middle halves (below
-// 1.15 2^31 + 2^30 + 4) in 32 bits, so both additions ride on the multiplies.
+// 1.15 2^31 + 2^30 + 4) in 32 bits, so the first additions ride on the multiplies.
 __device__ __forceinline__ bool fix_rate_ok(double rate) { return rate >= 0x1p-6 && rate <= 0x1p4; }
 
 __device__ __forceinline__ unsigned long long fix_scale(double rate) {
@@ -59,35 +59,42 @@ __device__ __forceinline__ long long to_fix(unsigned long long y58, unsigned lon
     const uint32_t yh = static_cast<uint32_t>(y58 >> 32), yl = static_cast<uint32_t>(y58);
     const uint32_t ch = static_cast<uint32_t>(cm >> 32), cl = static_cast<uint32_t>(cm);
     const uint32_t mid = mad_hi_u32(yl, ch, mad_hi_u32(yh, cl, 3u));
-    return static_cast<long long>((static_cast<unsigned long long>(yh) * ch + mid) >> 2);
+    uint32_t p_hi, p_lo;
+    mul_wide_u32(yh, ch, p_hi, p_lo);
+    return static_cast<long long>(add_carry(p_lo, p_hi, mid) >> 2);
 }
 
-struct U128 {
-    unsigned long long lo = 0, hi = 0;
-    __device__ __forceinline__ void add(long long v) {  // v >= 0
-        const unsigned long long u = static_cast<unsigned long long>(v);
-        lo += u;
-        hi += (lo < u) ? 1u : 0u;
+// Sum of up to 2^32 values below 2^61: 96 bits (one carry chain of three adds).
+struct U96 {
+    unsigned long long lo = 0;
+    uint32_t hi = 0;
+    __device__ __forceinline__ void add(unsigned long long v) { add(v, 0u); }
+    __device__ __forceinline__ void add(unsigned long long v, uint32_t v_hi) {
+        uint32_t l0 = static_cast<uint32_t>(lo), l1 = static_cast<uint32_t>(lo >> 32);
+        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+            : "+r"(l0), "+r"(l1), "+r"(hi)
+            : "r"(static_cast<uint32_t>(v)), "r"(static_cast<uint32_t>(v >> 32)), "r"(v_hi));
+        lo = (static_cast<unsigned long long>(l1) << 32) | l0;
     }
     __device__ __forceinline__ double to_double() const {  // value 2^-48
         return static_cast<double>(hi) * 0x1p16 + static_cast<double>(lo) * 0x1p-48;
     }
 };
 
+// max(x, 0) from the sign alone.
+__device__ __forceinline__ long long relu64(long long x) { return x & ~(x >> 63); }
+
 constexpr long long kSat = 1LL << 61;
 
 __device__ __forceinline__ long long sat61(long long x) { return x > kSat ? kSat : (x < -kSat ? -kSat : x); }
 
-__device__ __forceinline__ U128 shfl_down_u128(const U128& x, int off) {
-    U128 r;
+__device__ __forceinline__ U96 shfl_down_u96(const U96& x, int off) {
+    U96 r;
     r.lo = __shfl_down_sync(kFull, x.lo, off);
     r.hi = __shfl_down_sync(kFull, x.hi, off);
     return r;
 }
-__device__ __forceinline__ void add_u128(U128& a, const U128& b) {
-    a.lo += b.lo;
-    a.hi += b.hi + ((a.lo < b.lo) ? 1u : 0u);
-}
+__device__ __forceinline__ void add_u96(U96& a, const U96& b) { a.add(b.lo, b.hi); }
 
 struct Mm1Out {
     double* wait;
@@ -95,22 +102,26 @@ struct Mm1Out {
     double* system;
 };
 
-// Client n of (dp, rep): service S_n from words (0,1), gap A_{n+1} from (2,3).
+// Client n of a replication: service S_n from words (0,1), gap A_{n+1} from (2,3).
 // inv_mu, inv_lam are 2^-58 / rate (see expo_fast).
-__device__ __forceinline__ void mm1_client(uint32_t n, uint32_t rep, uint32_t dp, double inv_lam,
+template <bool kShared>
+__device__ __forceinline__ void mm1_client(uint32_t n, const RowKey& row, double inv_lam,
                                            double inv_mu, const RoundKeys& rk, const LogTable& tab,
                                            double& s, double& a) {
-    const uint4 b = philox(0u, n, rep, stream_word(0u, dp), rk);
-    s = expo_fast(b.x, b.y, tab, inv_mu);
-    a = expo_fast(b.z, b.w, tab, inv_lam);
+    const uint4 b = philox_row(row, n, rk);
+    s = expo_fast<kShared>(b.x, b.y, tab, inv_mu);
+    a = expo_fast<kShared>(b.z, b.w, tab, inv_lam);
 }
 
-// (A minimum of four CTAs per SM rather than eight: the same 64 registers,
-// but 0.80 instead of 0.83 ms for 2^16 replications of 1,000 clients.)
+// (A minimum of four CTAs per SM; 1, 3, 6 and 8 take the same time, 0.569 ms
+// for 2^16 replications of 1,000 clients before the FP32 tail of the
+// logarithm: 13.5 warps per SM are latency-bound at any budget.)
 template <bool kLane0Only>
 __global__ void __launch_bounds__(128, 4) mm1_serial_kernel(const double* __restrict__ dps, long long n_items,
                                   long long n_reps, long long rep0, long long n_clients,
                                   const __grid_constant__ RoundKeys rk, LogTable tab, Mm1Out out) {
+    __shared__ unsigned long long nln2[kLogExponents];
+    stage_nln2(tab, nln2);
     long long item;
     if (kLane0Only) {
         if ((threadIdx.x & 31) != 0) return;
@@ -123,22 +134,24 @@ __global__ void __launch_bounds__(128, 4) mm1_serial_kernel(const double* __rest
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double lam = dps[2 * dp], mu = dps[2 * dp + 1];
     const double inv = static_cast<double>(n_clients);
+    const RowKey row = row_key(rep, stream_word(0u, dp), rk);
     if (fix_rate_ok(lam) && fix_rate_ok(mu)) {  // 48-bit fixed-point times
         const unsigned long long cl = fix_scale(lam), cmu = fix_scale(mu);
-        const uint32_t c3 = stream_word(0u, dp);
         long long wf = 0;
-        U128 sw, si, sv;
+        U96 sw, si, sv;
         bool overflow = false;
-        for (long long n = 0; n < n_clients; ++n) {
-            const uint4 b = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-            const long long s_ = to_fix(neg_log_q58(b.x, b.y, tab), cmu);
-            const long long a_ = to_fix(neg_log_q58(b.z, b.w, tab), cl);
+        // (client indices are 32-bit: n_clients < 2^32, the counter word c1)
+        const uint32_t nc = static_cast<uint32_t>(n_clients);
+        for (uint32_t n = 0; n < nc; ++n) {
+            const uint4 b = philox_row(row, static_cast<uint32_t>(n), rk);
+            const long long s_ = to_fix(neg_log_q58<true>(b.x, b.y, tab), cmu);
+            const long long a_ = to_fix(neg_log_q58<true>(b.z, b.w, tab), cl);
             sw.add(wf);
             const long long v = wf + s_;
             sv.add(v);
             const long long t = v - a_;
-            si.add(t < 0 ? -t : 0);
-            wf = t > 0 ? t : 0;
+            wf = relu64(t);
+            si.add(wf - t);  // max(0, -t)
             if (wf >= kFixGuard) {
                 overflow = true;
                 break;
@@ -155,7 +168,7 @@ __global__ void __launch_bounds__(128, 4) mm1_serial_kernel(const double* __rest
     double w = 0.0, sum_w = 0.0, sum_i = 0.0, sum_v = 0.0;
     for (long long n = 0; n < n_clients; ++n) {
         double s, a;
-        mm1_client(static_cast<uint32_t>(n), rep, dp, inv_lam, inv_mu, rk, tab, s, a);
+        mm1_client<true>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, s, a);
         sum_w += w;
         const double v = w + s;
         sum_v += v;
@@ -194,6 +207,7 @@ __global__ void mm1_warp_coop_kernel(const double* __restrict__ dps, long long n
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double inv_lam = 0x1p-58 / dps[2 * dp], inv_mu = 0x1p-58 / dps[2 * dp + 1];
+    const RowKey row = row_key(rep, stream_word(0u, dp), rk);
     const long long seg = (n_clients + 31) / 32;
     const long long lo = lane * seg;
     const long long hi = (lo + seg < n_clients) ? lo + seg : n_clients;
@@ -209,7 +223,7 @@ __global__ void mm1_warp_coop_kernel(const double* __restrict__ dps, long long n
     MaxPlus f{-INFINITY, 0.0};
     for (long long n = lo; n < hi; ++n) {
         double s, a;
-        mm1_client(static_cast<uint32_t>(n), rep, dp, inv_lam, inv_mu, rk, tab, s, a);
+        mm1_client<false>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, s, a);
         if (staged) {
             s_buf[(n - lo) * 32 + lane] = s;
             a_buf[(n - lo) * 32 + lane] = a;
@@ -240,7 +254,7 @@ __global__ void mm1_warp_coop_kernel(const double* __restrict__ dps, long long n
             s = s_buf[(n - lo) * 32 + lane];
             a = a_buf[(n - lo) * 32 + lane];
         } else {
-            mm1_client(static_cast<uint32_t>(n), rep, dp, inv_lam, inv_mu, rk, tab, s, a);
+            mm1_client<false>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, s, a);
         }
         sum_w += w;
         const double v = w + s;
@@ -278,12 +292,28 @@ struct TandemOut {
     long long plane;  // plane stride = n_items
 };
 
+// One client in fixed point: v_j <- max(v_j - a, v'_{j-1}) + s_j (v'_0 = 0), the
+// maximum as v'_{j-1} + max(v_j - a - v'_{j-1}, 0): three-input adds and a sign
+// mask instead of a two-word compare and two selects.  Every state is at
+// least kFixNegInf and below 2^62, so no difference overflows.
+__device__ __forceinline__ void tandem_step(long long& v1, long long& v2, long long& v3, long long a, long long s1,
+                                            long long s2, long long s3) {
+    v1 = relu64(v1 - a) + s1;
+    v2 = v1 + s2 + relu64(v2 - a - v1);
+    v3 = v2 + s3 + relu64(v3 - a - v2);
+}
+
+// Five CTAs per SM (96 registers, nothing spilled): 121.2 ms for 4,096 x 256
+// replications of 10,000 clients against 124.1, 122.2, 122.1 and 122.7 at 4, 6, 7 and
+// 8 (104 bytes spilled).
 template <bool kLane0Only>
-__global__ void __launch_bounds__(128, 8) tandem3_serial_kernel(const double* __restrict__ dps, long long n_items,
+__global__ void __launch_bounds__(128, 5) tandem3_serial_kernel(const double* __restrict__ dps, long long n_items,
                                       long long n_reps, long long rep0, long long n_clients,
                                       long long window, uint32_t tag,
                                       const __grid_constant__ RoundKeys rk, LogTable tab,
                                       TandemOut out) {
+    __shared__ unsigned long long nln2[kLogExponents];
+    stage_nln2(tab, nln2);
     long long item;
     if (kLane0Only) {
         if ((threadIdx.x & 31) != 0) return;
@@ -298,7 +328,7 @@ __global__ void __launch_bounds__(128, 8) tandem3_serial_kernel(const double* __
                  mu3 = dps[4 * dp + 3];
     const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2,
                  i_mu3 = 0x1p-58 / mu3;
-    const uint32_t c3 = stream_word(tag, dp);
+    const RowKey row = row_key(rep, stream_word(tag, dp), rk);
     const long long w_len = (n_clients < window) ? n_clients : window;
     double sum_y = 0.0, sum_a = 0.0, sum_1 = 0.0, sum_2 = 0.0, sum_3 = 0.0;
     bool fixed_done = false;
@@ -306,28 +336,22 @@ __global__ void __launch_bounds__(128, 8) tandem3_serial_kernel(const double* __
         const unsigned long long fl = fix_scale(lam), f1 = fix_scale(mu1), f2 = fix_scale(mu2),
                                  f3 = fix_scale(mu3);
         long long v1 = kFixNegInf, v2 = kFixNegInf, v3 = kFixNegInf;
-        U128 sy;
+        U96 sy;
         double wa = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
         bool overflow = false;
         // client n's four log values; then one step of the recurrence
         auto logs = [&](uint32_t n, unsigned long long& ya, unsigned long long& y1, unsigned long long& y2,
                         unsigned long long& y3) {
-            const uint4 b0 = philox(0u, n, rep, c3, rk);
-            const uint4 b1 = philox(1u, n, rep, c3, rk);
-            ya = neg_log_q58(b0.x, b0.y, tab);
-            y1 = neg_log_q58(b0.z, b0.w, tab);
-            y2 = neg_log_q58(b1.x, b1.y, tab);
-            y3 = neg_log_q58(b1.z, b1.w, tab);
+            uint4 b0, b1;
+            philox_row2(row, n, rk, b0, b1);
+            ya = neg_log_q58<true>(b0.x, b0.y, tab);
+            y1 = neg_log_q58<true>(b0.z, b0.w, tab);
+            y2 = neg_log_q58<true>(b1.x, b1.y, tab);
+            y3 = neg_log_q58<true>(b1.z, b1.w, tab);
         };
         auto step = [&](unsigned long long ya, unsigned long long y1, unsigned long long y2,
                         unsigned long long y3) {
-            const long long a = to_fix(ya, fl);
-            long long q = v1 - a;
-            v1 = ((q > 0) ? q : 0) + to_fix(y1, f1);
-            q = v2 - a;
-            v2 = ((q > v1) ? q : v1) + to_fix(y2, f2);
-            q = v3 - a;
-            v3 = ((q > v2) ? q : v2) + to_fix(y3, f3);
+            tandem_step(v1, v2, v3, to_fix(ya, fl), to_fix(y1, f1), to_fix(y2, f2), to_fix(y3, f3));
             sy.add(v3);
             return v3 < kFixGuard;
         };
@@ -364,12 +388,12 @@ __global__ void __launch_bounds__(128, 8) tandem3_serial_kernel(const double* __
     }
     double v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY;
     for (long long n = 0; !fixed_done && n < n_clients; ++n) {
-        const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-        const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-        const double a = expo_fast(b0.x, b0.y, tab, i_lam);
-        const double s1 = expo_fast(b0.z, b0.w, tab, i_mu1);
-        const double s2 = expo_fast(b1.x, b1.y, tab, i_mu2);
-        const double s3 = expo_fast(b1.z, b1.w, tab, i_mu3);
+        uint4 b0, b1;
+        philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
+        const double a = expo_fast<true>(b0.x, b0.y, tab, i_lam);
+        const double s1 = expo_fast<true>(b0.z, b0.w, tab, i_mu1);
+        const double s2 = expo_fast<true>(b1.x, b1.y, tab, i_mu2);
+        const double s3 = expo_fast<true>(b1.z, b1.w, tab, i_mu3);
         double q = v1 - a;
         v1 = ((q > 0.0) ? q : 0.0) + s1;
         q = v2 - a;
@@ -467,14 +491,13 @@ struct TandemClient {
     double a, s1, s2, s3;
 };
 
-__device__ __forceinline__ TandemClient tandem_client(uint32_t n, uint32_t rep, uint32_t c3,
-                                                      const RoundKeys& rk, const LogTable& tab,
+__device__ __forceinline__ TandemClient tandem_client(uint32_t n, const RowKey& row, const RoundKeys& rk, const LogTable& tab,
                                                       double i_lam, double i_mu1, double i_mu2,
                                                       double i_mu3) {
-    const uint4 b0 = philox(0u, n, rep, c3, rk);
-    const uint4 b1 = philox(1u, n, rep, c3, rk);
-    return TandemClient{expo_fast(b0.x, b0.y, tab, i_lam), expo_fast(b0.z, b0.w, tab, i_mu1),
-                        expo_fast(b1.x, b1.y, tab, i_mu2), expo_fast(b1.z, b1.w, tab, i_mu3)};
+    uint4 b0, b1;
+    philox_row2(row, n, rk, b0, b1);
+    return TandemClient{expo_fast<false>(b0.x, b0.y, tab, i_lam), expo_fast<false>(b0.z, b0.w, tab, i_mu1),
+                        expo_fast<false>(b1.x, b1.y, tab, i_mu2), expo_fast<false>(b1.z, b1.w, tab, i_mu3)};
 }
 
 // The same maps in 48-bit fixed point, every sum saturated at +-2^61 (the
@@ -536,11 +559,10 @@ __device__ __forceinline__ FTMap ftmap_shfl_up(const FTMap& m, int off) {
 
 // FP64 warp scan of one replication (the fallback of the fixed-point paths):
 // lane l takes the l-th of 32 contiguous client segments.
-__device__ void tandem_coop_fp64(long long item, uint32_t dp, uint32_t rep, double lam, double mu1, double mu2,
-                                 double mu3, long long n_clients, long long window, uint32_t c3,
+__device__ void tandem_coop_fp64(long long item, double lam, double mu1, double mu2,
+                                 double mu3, long long n_clients, long long window, const RowKey& row,
                                  const RoundKeys& rk, const LogTable& tab, const TandemOut& out) {
-    (void)dp;
-    const int lane = threadIdx.x & 31;
+        const int lane = threadIdx.x & 31;
     const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2, i_mu3 = 0x1p-58 / mu3;
     const long long w_len = (n_clients < window) ? n_clients : window;
     const long long seg = (n_clients + 31) / 32;
@@ -549,7 +571,7 @@ __device__ void tandem_coop_fp64(long long item, uint32_t dp, uint32_t rep, doub
     // pass 1: this segment's map
     TMap f = tmap_identity();
     for (long long n = lo; n < hi; ++n) {
-        const TandemClient k = tandem_client(static_cast<uint32_t>(n), rep, c3, rk, tab, i_lam, i_mu1, i_mu2, i_mu3);
+        const TandemClient k = tandem_client(static_cast<uint32_t>(n), row, rk, tab, i_lam, i_mu1, i_mu2, i_mu3);
         f = tmap_push(f, k.a, k.s1, k.s2, k.s3);
     }
     // inclusive scan over lanes, then the previous lane's prefix is the entry map
@@ -569,7 +591,7 @@ __device__ void tandem_coop_fp64(long long item, uint32_t dp, uint32_t rep, doub
     // pass 2: replay the segment with the plain recurrence
     double sum_y = 0.0, sum_a = 0.0, sum_1 = 0.0, sum_2 = 0.0, sum_3 = 0.0;
     for (long long n = lo; n < hi; ++n) {
-        const TandemClient k = tandem_client(static_cast<uint32_t>(n), rep, c3, rk, tab, i_lam, i_mu1, i_mu2, i_mu3);
+        const TandemClient k = tandem_client(static_cast<uint32_t>(n), row, rk, tab, i_lam, i_mu1, i_mu2, i_mu3);
         double q = v1 - k.a;
         v1 = ((q > 0.0) ? q : 0.0) + k.s1;
         q = v2 - k.a;
@@ -629,7 +651,7 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
     const double lam = dps[4 * dp], mu1 = dps[4 * dp + 1], mu2 = dps[4 * dp + 2], mu3 = dps[4 * dp + 3];
     const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2,
                  i_mu3 = 0x1p-58 / mu3;
-    const uint32_t c3 = stream_word(tag, dp);
+    const RowKey row = row_key(rep, stream_word(tag, dp), rk);
     const long long w_len = (n_clients < window) ? n_clients : window;
     const long long seg = (n_clients + 31) / 32;
     const long long lo = min(lane * seg, n_clients);
@@ -640,12 +662,12 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
                                  c3f = fix_scale(mu3);
         FTMap f = ftmap_identity();
         for (long long n = lo; n < hi; ++n) {
-            const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-            const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-            f = ftmap_push(f, to_fix(neg_log_q58(b0.x, b0.y, tab), cl),
-                           to_fix(neg_log_q58(b0.z, b0.w, tab), c1),
-                           to_fix(neg_log_q58(b1.x, b1.y, tab), c2),
-                           to_fix(neg_log_q58(b1.z, b1.w, tab), c3f));
+            uint4 b0, b1;
+            philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
+            f = ftmap_push(f, to_fix(neg_log_q58<false>(b0.x, b0.y, tab), cl),
+                           to_fix(neg_log_q58<false>(b0.z, b0.w, tab), c1),
+                           to_fix(neg_log_q58<false>(b1.x, b1.y, tab), c2),
+                           to_fix(neg_log_q58<false>(b1.z, b1.w, tab), c3f));
         }
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -660,22 +682,16 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
             v3 = excl.c3;
         }
         bool bad = v3 >= kFixGuard;
-        U128 sy;
+        U96 sy;
         double wa = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
         for (long long n = lo; n < hi && !bad; ++n) {
-            const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-            const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-            const unsigned long long ya = neg_log_q58(b0.x, b0.y, tab);
-            const unsigned long long y1 = neg_log_q58(b0.z, b0.w, tab);
-            const unsigned long long y2 = neg_log_q58(b1.x, b1.y, tab);
-            const unsigned long long y3 = neg_log_q58(b1.z, b1.w, tab);
-            const long long a = to_fix(ya, cl);
-            long long q = v1 - a;
-            v1 = ((q > 0) ? q : 0) + to_fix(y1, c1);
-            q = v2 - a;
-            v2 = ((q > v1) ? q : v1) + to_fix(y2, c2);
-            q = v3 - a;
-            v3 = ((q > v2) ? q : v2) + to_fix(y3, c3f);
+            uint4 b0, b1;
+            philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
+            const unsigned long long ya = neg_log_q58<false>(b0.x, b0.y, tab);
+            const unsigned long long y1 = neg_log_q58<false>(b0.z, b0.w, tab);
+            const unsigned long long y2 = neg_log_q58<false>(b1.x, b1.y, tab);
+            const unsigned long long y3 = neg_log_q58<false>(b1.z, b1.w, tab);
+            tandem_step(v1, v2, v3, to_fix(ya, cl), to_fix(y1, c1), to_fix(y2, c2), to_fix(y3, c3f));
             sy.add(v3);
             if (n < w_len) {
                 wa += __ull2double_rn(ya) * i_lam;
@@ -688,13 +704,13 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
         if (!__any_sync(kFull, bad)) {
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {  // lane-ordered tree (integers: exact)
-                const U128 oy = shfl_down_u128(sy, off);
+                const U96 oy = shfl_down_u96(sy, off);
                 const double oa = __shfl_down_sync(kFull, wa, off);
                 const double o1 = __shfl_down_sync(kFull, w1, off);
                 const double o2 = __shfl_down_sync(kFull, w2, off);
                 const double o3 = __shfl_down_sync(kFull, w3, off);
                 if ((lane & (2 * off - 1)) == 0) {
-                    add_u128(sy, oy);
+                    add_u96(sy, oy);
                     wa += oa;
                     w1 += o1;
                     w2 += o2;
@@ -721,7 +737,7 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
     }
 
     // FP64
-    tandem_coop_fp64(item, dp, rep, lam, mu1, mu2, mu3, n_clients, window, c3, rk, tab, out);
+    tandem_coop_fp64(item, lam, mu1, mu2, mu3, n_clients, window, row, rk, tab, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -779,8 +795,8 @@ __device__ Map block_exclusive_map(Map f, Map identity, Map* smem, Compose compo
     return compose(before, excl);
 }
 
-struct Mm1Sums128 {
-    U128 w, i, v;
+struct Mm1Sums {
+    U96 w, i, v;
 };
 
 
@@ -791,14 +807,14 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
     extern __shared__ long long fix_stage[];  // [client - lo][thread] x (S, A) when staged
     __shared__ FixMap fmaps[32];
     __shared__ DblMap dmaps[32];
-    __shared__ U128 part[3][32];
+    __shared__ U96 part[3][32];
     __shared__ double dpart[3][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const long long item = blockIdx.x;
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double lam = dps[2 * dp], mu = dps[2 * dp + 1];
-    const uint32_t c3 = stream_word(0u, dp);
+    const RowKey row = row_key(rep, stream_word(0u, dp), rk);
     const long long k = (n_clients + blockDim.x - 1) / blockDim.x;
     const long long lo = min(static_cast<long long>(threadIdx.x) * k, n_clients);
     const long long hi = min(lo + k, n_clients);
@@ -822,9 +838,9 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
         long long* st_s = fix_stage + threadIdx.x;
         long long* st_a = fix_stage + k * blockDim.x + threadIdx.x;
         for (long long n = lo; n < hi; ++n) {
-            const uint4 b = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-            const long long sv = to_fix(neg_log_q58(b.x, b.y, tab), cmu);
-            const long long av = to_fix(neg_log_q58(b.z, b.w, tab), cl);
+            const uint4 b = philox_row(row, static_cast<uint32_t>(n), rk);
+            const long long sv = to_fix(neg_log_q58<false>(b.x, b.y, tab), cmu);
+            const long long av = to_fix(neg_log_q58<false>(b.z, b.w, tab), cl);
             if (staged) {
                 st_s[(n - lo) * blockDim.x] = sv;
                 st_a[(n - lo) * blockDim.x] = av;
@@ -835,32 +851,32 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
         long long w = pre.c > pre.d ? pre.c : pre.d;  // map at W_0 = 0
         if (threadIdx.x == 0) w = 0;
         bool bad = w >= kFixGuard;
-        Mm1Sums128 sm;
+        Mm1Sums sm;
         for (long long n = lo; n < hi && !bad; ++n) {
             long long sv, av;
             if (staged) {
                 sv = st_s[(n - lo) * blockDim.x];
                 av = st_a[(n - lo) * blockDim.x];
             } else {
-                const uint4 b = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-                sv = to_fix(neg_log_q58(b.x, b.y, tab), cmu);
-                av = to_fix(neg_log_q58(b.z, b.w, tab), cl);
+                const uint4 b = philox_row(row, static_cast<uint32_t>(n), rk);
+                sv = to_fix(neg_log_q58<false>(b.x, b.y, tab), cmu);
+                av = to_fix(neg_log_q58<false>(b.z, b.w, tab), cl);
             }
             sm.w.add(w);
             const long long v = w + sv;
             sm.v.add(v);
             const long long t = v - av;
-            sm.i.add(t < 0 ? -t : 0);
-            w = t > 0 ? t : 0;
+            w = relu64(t);
+            sm.i.add(w - t);  // max(0, -t)
             bad = w >= kFixGuard;
         }
         fixed_ok = !__syncthreads_or(bad);
         if (fixed_ok) {
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) {
-                add_u128(sm.w, shfl_down_u128(sm.w, off));
-                add_u128(sm.i, shfl_down_u128(sm.i, off));
-                add_u128(sm.v, shfl_down_u128(sm.v, off));
+                add_u96(sm.w, shfl_down_u96(sm.w, off));
+                add_u96(sm.i, shfl_down_u96(sm.i, off));
+                add_u96(sm.v, shfl_down_u96(sm.v, off));
             }
             if (lane == 0) {
                 part[0][warp] = sm.w;
@@ -869,8 +885,8 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
             }
             __syncthreads();
             if (threadIdx.x < 3) {
-                U128 tot;
-                for (int x = 0; x < nwarp; ++x) add_u128(tot, part[threadIdx.x][x]);
+                U96 tot;
+                for (int x = 0; x < nwarp; ++x) add_u96(tot, part[threadIdx.x][x]);
                 double* dst = threadIdx.x == 0 ? out.wait : threadIdx.x == 1 ? out.idle : out.system;
                 if (dst) dst[item] = tot.to_double() / inv_n;
             }
@@ -882,7 +898,7 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
     DblMap f{-INFINITY, 0.0};
     for (long long n = lo; n < hi; ++n) {
         double sv, av;
-        mm1_client(static_cast<uint32_t>(n), rep, dp, inv_lam, inv_mu, rk, tab, sv, av);
+        mm1_client<false>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, sv, av);
         f = dcompose(f, DblMap{0.0, sv - av});
     }
     const DblMap pre = block_exclusive_map(f, DblMap{-INFINITY, 0.0}, dmaps, dcompose);
@@ -891,7 +907,7 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
     double sw = 0.0, si = 0.0, sv_sum = 0.0;
     for (long long n = lo; n < hi; ++n) {
         double sv, av;
-        mm1_client(static_cast<uint32_t>(n), rep, dp, inv_lam, inv_mu, rk, tab, sv, av);
+        mm1_client<false>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, sv, av);
         sw += w;
         const double v = w + sv;
         sv_sum += v;
@@ -930,7 +946,7 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
 // (FTMap) is composed in pass 1, a block scan (warp shuffles, then the warp
 // totals in order) gives every thread the map of all clients before it, and
 // pass 2 replays its clients from that entry state.  Sojourn sums are exact
-// 128-bit integers; the early-window sums FP64 in a fixed order.  Rates
+// 96-bit integers; the early-window sums FP64 in a fixed order.  Rates
 // outside the fixed-point range or a sojourn past 2^12 hand the replication
 // to the FP64 warp scan (warp 0).
 // ---------------------------------------------------------------------------
@@ -939,14 +955,14 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
                                                            uint32_t tag, const __grid_constant__ RoundKeys rk,
                                                            LogTable tab, TandemOut out) {
     __shared__ FTMap wmap[32];
-    __shared__ U128 wy[32];
+    __shared__ U96 wy[32];
     __shared__ double wsum[4][32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarp = blockDim.x >> 5;
     const long long item = blockIdx.x;
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double lam = dps[4 * dp], mu1 = dps[4 * dp + 1], mu2 = dps[4 * dp + 2], mu3 = dps[4 * dp + 3];
-    const uint32_t c3 = stream_word(tag, dp);
+    const RowKey row = row_key(rep, stream_word(tag, dp), rk);
     const long long w_len = (n_clients < window) ? n_clients : window;
     const long long k = (n_clients + blockDim.x - 1) / blockDim.x;
     const long long lo = min(static_cast<long long>(t) * k, n_clients);
@@ -957,12 +973,12 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
                                  c3f = fix_scale(mu3);
         FTMap f = ftmap_identity();
         for (long long n = lo; n < hi; ++n) {
-            const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-            const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-            f = ftmap_push(f, to_fix(neg_log_q58(b0.x, b0.y, tab), cl),
-                           to_fix(neg_log_q58(b0.z, b0.w, tab), c1),
-                           to_fix(neg_log_q58(b1.x, b1.y, tab), c2),
-                           to_fix(neg_log_q58(b1.z, b1.w, tab), c3f));
+            uint4 b0, b1;
+            philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
+            f = ftmap_push(f, to_fix(neg_log_q58<false>(b0.x, b0.y, tab), cl),
+                           to_fix(neg_log_q58<false>(b0.z, b0.w, tab), c1),
+                           to_fix(neg_log_q58<false>(b1.x, b1.y, tab), c2),
+                           to_fix(neg_log_q58<false>(b1.z, b1.w, tab), c3f));
         }
         // block exclusive scan of the maps
         FTMap incl = f;
@@ -980,24 +996,18 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
         pre = ftmap_compose(pre, excl);
         long long v1 = pre.c1, v2 = pre.c2, v3 = pre.c3;  // -2^61 for the first thread: empty
         bool bad = v3 >= kFixGuard;
-        U128 sy;
+        U96 sy;
         double wa = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
         const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2,
                      i_mu3 = 0x1p-58 / mu3;
         for (long long n = lo; n < hi && !bad; ++n) {
-            const uint4 b0 = philox(0u, static_cast<uint32_t>(n), rep, c3, rk);
-            const uint4 b1 = philox(1u, static_cast<uint32_t>(n), rep, c3, rk);
-            const unsigned long long ya = neg_log_q58(b0.x, b0.y, tab);
-            const unsigned long long y1 = neg_log_q58(b0.z, b0.w, tab);
-            const unsigned long long y2 = neg_log_q58(b1.x, b1.y, tab);
-            const unsigned long long y3 = neg_log_q58(b1.z, b1.w, tab);
-            const long long a = to_fix(ya, cl);
-            long long q = v1 - a;
-            v1 = ((q > 0) ? q : 0) + to_fix(y1, c1);
-            q = v2 - a;
-            v2 = ((q > v1) ? q : v1) + to_fix(y2, c2);
-            q = v3 - a;
-            v3 = ((q > v2) ? q : v2) + to_fix(y3, c3f);
+            uint4 b0, b1;
+            philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
+            const unsigned long long ya = neg_log_q58<false>(b0.x, b0.y, tab);
+            const unsigned long long y1 = neg_log_q58<false>(b0.z, b0.w, tab);
+            const unsigned long long y2 = neg_log_q58<false>(b1.x, b1.y, tab);
+            const unsigned long long y3 = neg_log_q58<false>(b1.z, b1.w, tab);
+            tandem_step(v1, v2, v3, to_fix(ya, cl), to_fix(y1, c1), to_fix(y2, c2), to_fix(y3, c3f));
             sy.add(v3);
             if (n < w_len) {
                 wa += __ull2double_rn(ya) * i_lam;
@@ -1010,13 +1020,13 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
         if (!__syncthreads_or(bad)) {
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {  // lane-ordered tree (integers: exact)
-                const U128 oy = shfl_down_u128(sy, off);
+                const U96 oy = shfl_down_u96(sy, off);
                 const double oa = __shfl_down_sync(kFull, wa, off);
                 const double o1 = __shfl_down_sync(kFull, w1, off);
                 const double o2 = __shfl_down_sync(kFull, w2, off);
                 const double o3 = __shfl_down_sync(kFull, w3, off);
                 if ((lane & (2 * off - 1)) == 0) {
-                    add_u128(sy, oy);
+                    add_u96(sy, oy);
                     wa += oa;
                     w1 += o1;
                     w2 += o2;
@@ -1032,10 +1042,10 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
             }
             __syncthreads();
             if (t == 0) {
-                U128 ty;
+                U96 ty;
                 double sa = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
                 for (int w = 0; w < nwarp; ++w) {
-                    add_u128(ty, wy[w]);
+                    add_u96(ty, wy[w]);
                     sa += wsum[0][w];
                     s1 += wsum[1][w];
                     s2 += wsum[2][w];
@@ -1059,7 +1069,7 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
             return;
         }
     }
-    if (warp == 0) tandem_coop_fp64(item, dp, rep, lam, mu1, mu2, mu3, n_clients, window, c3, rk, tab, out);
+    if (warp == 0) tandem_coop_fp64(item, lam, mu1, mu2, mu3, n_clients, window, row, rk, tab, out);
 }
 
 }  // namespace

@@ -2,6 +2,7 @@
 // device error flags, and the random-stream stage entry points
 // (mrip_philox, mrip_expo).
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -87,15 +88,19 @@ unsigned long long log_core(uint32_t mh, uint32_t ml, const LogSlice& e) {
     const uint64_t V = static_cast<uint64_t>(mh) * e.w + hi_u(ml, e.w);
     const int32_t a = static_cast<int32_t>(static_cast<uint32_t>(V >> 13));
     const uint32_t r2 = static_cast<uint32_t>(hi_s(a, a));
-    return e.lnw - V + hi_u(r2, static_cast<uint32_t>(hi_s(a, -174763)) + 0x80000004u);
+    const float f = static_cast<float>(a);
+    const float tail = std::fma(f * f * f, std::fma(f, kLogR4, kLogR3), kLogMagic);
+    uint32_t bits;
+    std::memcpy(&bits, &tail, sizeof(bits));
+    return e.lnw - V + ((r2 + (bits - kLogMagicBits)) >> 1);
 }
 
 // The slices' w_j and ln w_j from the host's long-double logarithm (64-bit or
 // wider mantissa).  w_j keeps |r| <= 2^-14 over its slice; among up to 49 such
 // 27-bit values around 1/c_j the one whose logarithm's rounding to 2^-58, about
-// the mean 0.3 of the truncations, is smallest.
+// the mean 0.05 of the truncations, is smallest.
 void build_log_slices(std::vector<LogSlice>& t) {
-    constexpr long double kMean = 0.3L;
+    constexpr long double kMean = 0.05L;
     t.resize(kLogSlices);
     for (int j = 0; j < kLogSlices; ++j) {
         const long double from = 1.0L + static_cast<long double>(j) / kLogSlices;
@@ -128,7 +133,7 @@ mrip_status log_table(LogTable* out) {
         // n ln2 2^58 rounded, from the 128-bit product n * round(ln2 2^64);
         // entry 64 makes K = 2^53 (M = 1 in slice 0) exactly 0
         const unsigned long long ln2_q64 = static_cast<unsigned long long>(ldexpl(logl(2.0L), 64) + 0.5L);
-        std::vector<unsigned long long> nln2(65);
+        std::vector<unsigned long long> nln2(kLogExponents);
         for (unsigned s = 0; s < 64; ++s) {
             const unsigned __int128 prod = static_cast<unsigned __int128>(s + 1) * ln2_q64 + 32u;
             nln2[s] = static_cast<unsigned long long>(prod >> 6);
@@ -149,6 +154,7 @@ mrip_status log_table(LogTable* out) {
     }
     out->slice = reinterpret_cast<const ulonglong2*>(reinterpret_cast<uintptr_t>(d.log_slices) -
                                                      kLogSlices * sizeof(LogSlice));
+    out->nln2_shared = 0;
     out->nln2 = reinterpret_cast<const unsigned long long*>(d.log_slices + kLogSlices);
     return MRIP_OK;
 }
@@ -190,7 +196,7 @@ __global__ void expo_kernel(const uint32_t* __restrict__ lo, const uint32_t* __r
     long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
     if (i >= n) return;
     if (u_out) u_out[i] = u53(lo[i], hi[i]);
-    if (e_out) e_out[i] = expo_fast(lo[i], hi[i], tab, 0x1p-58 / rate[i]);
+    if (e_out) e_out[i] = expo_fast<false>(lo[i], hi[i], tab, 0x1p-58 / rate[i]);
 }
 
 }  // namespace mrip
