@@ -1,32 +1,42 @@
 // Stochastic forest-fire cellular automaton (Drossel-Schwabl rules), one
-// replication per CTA, the lattice held in shared memory.
+// replication per CTA, the lattice held in shared memory and registers.
 //
 // Layout: the L x L lattice (L = 32 W) is two bit planes, "tree" and
-// "burning", one 32-bit word per 32 cells of a row (bit m of word k =
-// y W + j is cell x = 32 j + m of row y).  Both planes are double-buffered
-// in shared memory (2 buffers x 2 planes x L W words = 16 L W bytes); a step reads buffer
-// (t-1) mod 2 and writes buffer t mod 2, so one barrier per step suffices.
-// Thread i of the CTA updates words i, i + blockDim, ...: the word's
-// north/south neighbours are the words W above and below (periodic), its
-// east/west neighbour bits are shifts with the carry bit from the adjacent
-// word of the same row.  The random word of cell i = y L + x at step t is
-// word (i mod 4) of Philox block (c0 = i div 4, c1 = t); for lattice word k
-// that is blocks c0 = 8k .. 8k+7.  A thread compares its 32 cells' words
-// with the growth and lightning thresholds and packs the results into two
-// words.  The kernel is bound by Philox's 32x32->64 multiplies, which GB300
-// retires at under one warp instruction per SM-clock, so everything else
-// stays off that pipe and the multiplies are trimmed: all blocks of one step
-// share (t, rep, dp), hence round 1's product of counter word 2 and round
-// 2's product of counter word 0 are computed once per step (18 instead of
-// 20 wide multiplies per block, same words).  Lightning is rare: its four
-// compares run only for blocks whose smallest word is below its threshold.
-// The new state of 32 cells is then a few bitwise operations:
+// "burning", one 32-bit word per 32 cells of a row (bit m of word j is cell
+// x = 32 j + m).  Thread y of the CTA (L threads) owns row y, or thread y + L h
+// the h-th half of it (2 L threads, for few replications): its words are read and
+// written as 16-byte vectors, east and west neighbours are funnel
+// shifts within the thread's own words, and only the burning plane, which the
+// rows above and below read, is double-buffered in shared memory (one barrier
+// per step).  A plane keeps vector q of all rows together (ff_word), so that
+// neighbouring threads touch neighbouring 16-byte slots and no access
+// conflicts on a bank.  The new state of 32 cells is a few bitwise operations:
 //   ignite = burning neighbour | lightning,
 //   burning' = tree & ignite,
 //   tree'    = (tree & ~ignite) | (empty & grow).
+// (With the words dealt out to the threads in turn, every one with its own
+// address arithmetic and eight scalar accesses, 128 x 128 took 10.31 instead of
+// 10.11 ms, and the skip-sampled variant spent a third of its time on it.)
 // The burning count of each step is a popcount, a warp reduction and a
 // shared-memory atomic; counts are flushed to global memory every 64 steps
 // (coalesced, 16-byte stores where aligned) from a double-buffered slot array.
+//
+// The random word of cell i = y L + x at step t is word (i mod 4) of Philox
+// block (c0 = i div 4, c1 = t); lattice word k = y W + j uses blocks c0 = 8k ..
+// 8k+7.  The kernel is bound by Philox's 32x32->64 multiplies, which GB300
+// retires at under one warp instruction per SM-clock.  Of a block's 20
+// products, those of rounds 1 and 2 with words 0 and 2 and round 3's with
+// word 0 depend on the step alone or on the cell alone.  The words do not
+// depend on the lattice, so a thread draws several steps of a word at once
+// (ff_draw): the step's products are shared by all blocks of a row, the cell's
+// by all steps of the batch, and 15 + 2/NT products remain per block (NT steps;
+// 17.1 when each step was drawn by itself); the growth masks wait in shared
+// memory, one word per step, read back by the thread that wrote them, and the
+// rare lightning masks in local memory behind a flag bit.
+// Measured, against one step at a time on words dealt out in turn: 128 x 128, 1,024
+// replications x 1,000 steps 11.28 -> 9.85 ms; 256 x 256, 2,048 replications x 400
+// steps 34.5 -> 30.5 ms; 512 x 512, 308 x 122 9.09 -> 8.46 ms.  The FMA-heavy pipe is
+// 79 % busy, the ALU 61 %.
 #include "common.cuh"
 #include "model.cuh"
 
@@ -34,43 +44,6 @@ namespace mrip {
 namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
-
-// Philox4x32-10 of counter (c0, t, rep, c3) for one step: the parts that do
-// not depend on c0 are precomputed once per step (StepKey).
-struct StepKey {
-    uint32_t x0, x1;      // words 0 and 1 after round 1 (independent of c0)
-    uint32_t p_hi, p_lo;  // round 2's product 0xD2511F53 * x0
-};
-
-__device__ __forceinline__ StepKey step_key(uint32_t t, uint32_t rep, const RoundKeys& rk) {
-    StepKey s;
-    uint32_t h1;
-    mul_wide_u32(0xCD9E8D57u, rep, h1, s.x1);
-    s.x0 = h1 ^ t ^ rk.k0[0];
-    mul_wide_u32(0xD2511F53u, s.x0, s.p_hi, s.p_lo);
-    return s;
-}
-
-// prod = 0xD2511F53 * c0 as a 64-bit product (round 1's only varying product);
-// the 8 blocks of one lattice word have c0 = 8k + q, so the caller forms it
-// as 0xD2511F53 * 8k plus a constant: one 64-bit add instead of a wide
-// multiply for 7 of every 8 blocks.
-__device__ __forceinline__ uint4 philox_step(unsigned long long prod, uint32_t c3, const StepKey& sk,
-                                             const RoundKeys& rk) {
-    const uint32_t a_hi = static_cast<uint32_t>(prod >> 32);
-    const uint32_t a_lo = static_cast<uint32_t>(prod);
-    const uint32_t w2 = a_hi ^ c3 ^ rk.k1[0];
-    // round 2: the product with word 0 is sk.p
-    uint32_t b_hi, b_lo;
-    mul_wide_u32(0xCD9E8D57u, w2, b_hi, b_lo);
-    uint32_t x0 = b_hi ^ sk.x1 ^ rk.k0[1];
-    uint32_t x1 = b_lo;
-    uint32_t x2 = sk.p_hi ^ a_lo ^ rk.k1[1];
-    uint32_t x3 = sk.p_lo;
-#pragma unroll
-    for (int r = 2; r < 10; ++r) philox_round(x0, x1, x2, x3, rk.k0[r], rk.k1[r]);
-    return make_uint4(x0, x1, x2, x3);
-}
 
 // bits |= bit if w < t, as a compare and a predicated OR (integer ALU, not the
 // multiply pipe that Philox saturates).
@@ -105,24 +78,99 @@ __device__ __forceinline__ void ff_flush(int* slot, int n_slot, int32_t* dst, bo
     }
 }
 
-// Threads per CTA for a lattice of W words per row.
+
+// ---------------------------------------------------------------------------
+// Rows and planes
+// ---------------------------------------------------------------------------
+// Threads per CTA for a lattice of W words per row: one per row.
 template <int W>
 constexpr int ff_threads() {
-    return W == 1 ? 32 : W == 2 ? 64 : W == 4 ? 128 : W == 8 ? 256 : 512;
+    return 32 * W;
 }
 
-// Initial state into buffer 0 (planes T, B): from `init` (one byte per cell,
-// 0 empty, 1 tree, 2 burning) or from tag 1 (tree iff word < t_dens).
+// Index of word j of row y in a plane of L W words.
 template <int W>
-__device__ void ff_load_initial(uint32_t* lattice, const uint8_t* __restrict__ init, long long item,
+__device__ __forceinline__ int ff_word(int y, int j) {
+    constexpr int V = W < 4 ? W : 4;
+    return ((j / V) * 32 * W + y) * V + j % V;
+}
+
+// Words j0 .. j0 + N - 1 of row y (N divides W, j0 a multiple of N).
+template <int W, int N>
+__device__ __forceinline__ void row_load(const uint32_t* plane, int y, int j0, uint32_t (&w)[N]) {
+    if constexpr (N == 1) {
+        w[0] = plane[ff_word<W>(y, j0)];
+    } else if constexpr (N == 2) {
+        const uint2 v = *reinterpret_cast<const uint2*>(plane + ff_word<W>(y, j0));
+        w[0] = v.x;
+        w[1] = v.y;
+    } else {
+#pragma unroll
+        for (int q = 0; q < N / 4; ++q) {
+            const uint4 v = *reinterpret_cast<const uint4*>(plane + ff_word<W>(y, j0 + 4 * q));
+            w[4 * q] = v.x;
+            w[4 * q + 1] = v.y;
+            w[4 * q + 2] = v.z;
+            w[4 * q + 3] = v.w;
+        }
+    }
+}
+
+template <int W, int N>
+__device__ __forceinline__ void row_store(uint32_t* plane, int y, int j0, const uint32_t (&w)[N]) {
+    if constexpr (N == 1) {
+        plane[ff_word<W>(y, j0)] = w[0];
+    } else if constexpr (N == 2) {
+        *reinterpret_cast<uint2*>(plane + ff_word<W>(y, j0)) = make_uint2(w[0], w[1]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < N / 4; ++q)
+            *reinterpret_cast<uint4*>(plane + ff_word<W>(y, j0 + 4 * q)) =
+                make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+    }
+}
+
+// One step of words j0 .. j0 + N - 1 of row y: their tree and burning words from
+// the burning plane `cur`, the growth words g and the lightning words l; the
+// new burning words go to `nxt`.  Returns their burning cells.
+template <int W, int N>
+__device__ __forceinline__ int row_step(uint32_t (&t)[N], uint32_t (&b)[N], const uint32_t* cur, uint32_t* nxt, int y,
+                                        int j0, const uint32_t (&g)[N], const uint32_t (&l)[N]) {
+    constexpr int L = 32 * W;
+    uint32_t up[N], dn[N], nb[N];
+    row_load<W, N>(cur, (y + L - 1) & (L - 1), j0, up);
+    row_load<W, N>(cur, (y + 1) & (L - 1), j0, dn);
+    // the words beside them: the thread's own where it has the whole row
+    const uint32_t before = N == W ? b[N - 1] : cur[ff_word<W>(y, (j0 + W - 1) % W)];
+    const uint32_t after = N == W ? b[0] : cur[ff_word<W>(y, (j0 + N) % W)];
+    int c = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const uint32_t west = __funnelshift_l(j > 0 ? b[j > 0 ? j - 1 : 0] : before, b[j], 1);
+        const uint32_t east = __funnelshift_r(b[j], j + 1 < N ? b[j + 1 < N ? j + 1 : j] : after, 1);
+        const uint32_t ignite = up[j] | dn[j] | west | east | l[j];
+        nb[j] = t[j] & ignite;
+        t[j] = (t[j] & ~ignite) | (~(t[j] | b[j]) & g[j]);
+        c += __popc(nb[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) b[j] = nb[j];
+    row_store<W, N>(nxt, y, j0, b);
+    return c;
+}
+
+// Initial state into the planes: from `init` (one byte per cell, 0 empty, 1
+// tree, 2 burning) or from tag 1 (tree iff word < t_dens).
+template <int W, int TPB>
+__device__ void ff_load_initial(uint32_t* tree, uint32_t* burning, const uint8_t* __restrict__ init, long long item,
                                 uint32_t t_dens, uint32_t rep, uint32_t dp, const RoundKeys& rk) {
     constexpr int L = 32 * W;
     constexpr int NWORD = L * W;
-    constexpr int TPB = ff_threads<W>();
-    if (init) {
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(init + item * static_cast<long long>(L) * L);
-        for (int k = threadIdx.x; k < NWORD; k += TPB) {
-            uint32_t tw = 0, bw = 0;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(init + item * static_cast<long long>(L) * L);
+    const uint32_t c3i = stream_word(1u, dp);
+    for (int k = threadIdx.x; k < NWORD; k += TPB) {
+        uint32_t tw = 0, bw = 0;
+        if (init) {
             for (int r = 0; r < 8; ++r) {
                 const uint32_t v = src[8 * k + r];
                 for (int q = 0; q < 4; ++q) {
@@ -131,13 +179,7 @@ __device__ void ff_load_initial(uint32_t* lattice, const uint8_t* __restrict__ i
                     bw |= (s == 2u ? 1u : 0u) << (4 * r + q);
                 }
             }
-            lattice[k] = tw;
-            lattice[NWORD + k] = bw;
-        }
-    } else {
-        const uint32_t c3i = stream_word(1u, dp);
-        for (int k = threadIdx.x; k < NWORD; k += TPB) {
-            uint32_t tw = 0;
+        } else {
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const uint4 b = philox(8u * k + q, 0u, rep, c3i, rk);
@@ -146,22 +188,23 @@ __device__ void ff_load_initial(uint32_t* lattice, const uint8_t* __restrict__ i
                 tw |= (b.z < t_dens) ? (1u << (4 * q + 2)) : 0u;
                 tw |= (b.w < t_dens) ? (1u << (4 * q + 3)) : 0u;
             }
-            lattice[k] = tw;
-            lattice[NWORD + k] = 0u;
         }
+        const int at = ff_word<W>(k / W, k % W);
+        tree[at] = tw;
+        burning[at] = bw;
     }
 }
 
-// Planes (fin_t, fin_b) back to one byte per cell.
-template <int W>
-__device__ void ff_store_final(const uint32_t* fin_t, const uint32_t* fin_b, uint8_t* __restrict__ final_state,
+// The planes back to one byte per cell.
+template <int W, int TPB>
+__device__ void ff_store_final(const uint32_t* tree, const uint32_t* burning, uint8_t* __restrict__ final_state,
                                long long item) {
     constexpr int L = 32 * W;
     constexpr int NWORD = L * W;
-    constexpr int TPB = ff_threads<W>();
     uint32_t* dst = reinterpret_cast<uint32_t*>(final_state + item * static_cast<long long>(L) * L);
     for (int k = threadIdx.x; k < NWORD; k += TPB) {
-        const uint32_t tw = fin_t[k], bw = fin_b[k];
+        const int at = ff_word<W>(k / W, k % W);
+        const uint32_t tw = tree[at], bw = burning[at];
         for (int r = 0; r < 8; ++r) {
             uint32_t v = 0;
             for (int q = 0; q < 4; ++q) {
@@ -191,132 +234,241 @@ __device__ void ff_store_scalar(long long my_sum, long long* red, double* scalar
     }
 }
 
-// Register budget: a word's eight Philox blocks are independent, and the
-// more registers ptxas may use the more of them it interleaves.  256-thread
-// CTAs (L = 256) are held to three per SM (78 registers: 4.2 % faster than
-// five CTAs at 48); the other widths take the compiler's own maximum (L = 128:
-// 110 registers, four CTAs per SM, 5 % faster than nine at 56).
-template <int W>
-constexpr int ff_min_blocks() {
-    return W == 8 ? 3 : 1;
+// Step t is done (the CTA has met): flush the 64-step chunk it ends.
+template <int TPB>
+__device__ __forceinline__ void ff_end_step(int (*cnt)[64], int t, int n_steps, int32_t* counts, long long item,
+                                            long long& my_sum) {
+    if ((t & 63) == 0 || t == n_steps) {
+        const int chunk = (t - 1) >> 6;
+        const int n_slot = t - chunk * 64;
+        if (MRIP_CHECK(n_slot >= 1 && n_slot <= 64 && chunk * 64 + n_slot <= n_steps, 102, t))
+            ff_flush<TPB>(cnt[chunk & 1], n_slot, counts ? counts + item * n_steps + chunk * 64 : nullptr, true,
+                          my_sum);
+    }
 }
 
+// ---------------------------------------------------------------------------
+// The per-cell kernel
+// ---------------------------------------------------------------------------
+// Steps drawn together: eight, or four where the masks of eight would not fit in
+// shared memory (L = 512: 224 KB with four).  A batch is also the number of
+// independent Philox chains a thread interleaves.  128 x 128 at 2, 4, 6, 8, 12 and
+// 16 steps: 11.0, 10.1, 10.0, 9.94, 9.97, 10.5 ms; 256 x 256 at 4, 5, 6, 7, 8: 31.7,
+// 31.2, 31.1, 30.9, 30.8; 512 x 512 at 2 and 4: 8.91, 8.44.
 template <int W>
-__global__ void __launch_bounds__(ff_threads<W>(), ff_min_blocks<W>()) forest_fire_kernel(
+constexpr int ff_batch() {
+    return W == 16 ? 4 : 8;
+}
+
+// What the counters (c0, t, rep, c3) of the steps t0 .. t0 + NS - 1 of one
+// replication share: word 1 after round 1 and, per step, round 2's product of
+// word 0 (each with a round key).
+template <int NS>
+struct StepKeys {
+    uint32_t x1;
+    uint32_t p_hi[NS], p_lo[NS];
+};
+
+template <int NS>
+__device__ __forceinline__ StepKeys<NS> step_keys(uint32_t t0, uint32_t rep, const RoundKeys& rk) {
+    StepKeys<NS> s;
+    uint32_t h1, x1;
+    mul_wide_u32(0xCD9E8D57u, rep, h1, x1);
+    s.x1 = x1 ^ rk.k0[1];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        uint32_t hi, lo;
+        mul_wide_u32(0xD2511F53u, h1 ^ (t0 + i) ^ rk.k0[0], hi, lo);
+        s.p_hi[i] = hi ^ rk.k1[1];
+        s.p_lo[i] = lo ^ rk.k1[2];
+    }
+    return s;
+}
+
+// Philox4x32-10 of counter (c0, t0 + i, rep, c3) for i < NS, from a = 0xD2511F53
+// c0: the two products that do not depend on the step, then rounds 3 to 10.
+template <int NS>
+__device__ __forceinline__ void step_blocks(uint32_t a_hi, uint32_t a_lo, uint32_t c3, const StepKeys<NS>& sk,
+                                            const RoundKeys& rk, uint4 (&b)[NS]) {
+    uint32_t hi, u, r_hi, r_lo;
+    mul_wide_u32(0xCD9E8D57u, a_hi ^ c3 ^ rk.k1[0], hi, u);
+    u ^= rk.k0[2];
+    mul_wide_u32(0xD2511F53u, hi ^ sk.x1, r_hi, r_lo);
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        uint32_t x0, x1, x2, x3;
+        mul_wide_u32(0xCD9E8D57u, sk.p_hi[i] ^ a_lo, hi, x1);
+        x0 = hi ^ u;
+        x2 = r_hi ^ sk.p_lo[i];
+        x3 = r_lo;
+#pragma unroll
+        for (int r = 3; r < 10; ++r) philox_round(x0, x1, x2, x3, rk.k0[r], rk.k1[r]);
+        b[i] = make_uint4(x0, x1, x2, x3);
+    }
+}
+
+// Growth and lightning masks of lattice word k for NS steps.  Lightning is
+// rare: its masks are formed only where a word of a block, over the batch, is
+// below its threshold.
+template <int NS, int kUnroll>
+__device__ __forceinline__ void ff_draw(uint32_t k, uint32_t c3, const StepKeys<NS>& sk, const RoundKeys& rk,
+                                        uint32_t t_grow, uint32_t t_light, uint32_t (&g)[NS], uint32_t (&l)[NS]) {
+    uint32_t a_hi, a_lo;
+    mul_wide_u32(0xD2511F53u, 8u * k, a_hi, a_lo);
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        g[i] = 0u;
+        l[i] = 0u;
+    }
+#pragma unroll kUnroll
+    for (int q = 0; q < 8; ++q) {
+        uint4 b[NS];
+        step_blocks<NS>(a_hi, a_lo, c3, sk, rk, b);
+        bool any = false;
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            g[i] >>= 4;
+            or_if_below(g[i], b[i].x, t_grow, 1u << 28);
+            or_if_below(g[i], b[i].y, t_grow, 1u << 29);
+            or_if_below(g[i], b[i].z, t_grow, 1u << 30);
+            or_if_below(g[i], b[i].w, t_grow, 1u << 31);
+            any = any || b[i].x < t_light || b[i].y < t_light || b[i].z < t_light || b[i].w < t_light;
+        }
+        if (__builtin_expect(any, 0)) {
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                uint32_t nib = 0u;
+                or_if_below(nib, b[i].x, t_light, 1u);
+                or_if_below(nib, b[i].y, t_light, 2u);
+                or_if_below(nib, b[i].z, t_light, 4u);
+                or_if_below(nib, b[i].w, t_light, 8u);
+                l[i] |= nib << (4 * q);
+            }
+        }
+        asm("add.cc.u32 %0, %0, 0xD2511F53;\n\taddc.u32 %1, %1, 0;" : "+r"(a_lo), "+r"(a_hi));
+    }
+}
+
+// R threads share a row, each N = W / R of its words.
+// Register budget: 512 threads per SM, 128 registers each (128 x 128 with 512, 640
+// and 384 threads: 9.96, 10.13, 9.94 ms).
+template <int W, int R>
+constexpr int ff_min_blocks() {
+    return 512 / (32 * W * R);
+}
+
+template <int W, int R>
+__global__ void __launch_bounds__(R * ff_threads<W>(), ff_min_blocks<W, R>()) forest_fire_kernel(
     const double* __restrict__ dps, long long n_reps, long long rep0, int n_steps, uint32_t t_dens,
     const __grid_constant__ RoundKeys rk, const uint8_t* __restrict__ init,
     int32_t* __restrict__ counts, double* __restrict__ scalar, uint8_t* __restrict__ final_state) {
     constexpr int L = 32 * W;
     constexpr int NWORD = L * W;  // words per plane
-    constexpr int TPB = ff_threads<W>();
+    constexpr int TPB = R * ff_threads<W>();
     constexpr int NWARP = TPB / 32;
-    extern __shared__ uint32_t lattice[];  // [buffer][plane T, B][NWORD]
+    constexpr int NT = ff_batch<W>();
+    constexpr int N = W / R;  // words per thread
+    static_assert(N * R == W && N * NT <= 64, "one flag bit per word and step");
+    extern __shared__ __align__(16) uint32_t ff_smem[];
+    uint32_t* burning = ff_smem;             // [2][NWORD], by step parity
+    uint32_t* tree = ff_smem + 2 * NWORD;    // [NWORD], each row private to its thread
+    uint32_t* grow = ff_smem + 3 * NWORD;    // [NT][NWORD], likewise
     __shared__ __align__(16) int cnt[2][64];
     __shared__ long long red[NWARP];
 
-    const int lane = threadIdx.x & 31;
+    const int y = threadIdx.x % L, j0 = (threadIdx.x / L) * N, lane = threadIdx.x & 31;
     const long long item = blockIdx.x;
-    if (!MRIP_CHECK(4u * NWORD * sizeof(uint32_t) <= dynamic_smem_bytes(), 101, NWORD)) return;  // CTA-uniform
+    if (!MRIP_CHECK((3u + NT) * NWORD * sizeof(uint32_t) <= dynamic_smem_bytes(), 101, NWORD)) return;  // CTA-uniform
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const uint32_t t_grow = threshold32(dps[2 * dp]);
     const uint32_t t_light = threshold32(dps[2 * dp + 1]);
     const uint32_t c3 = stream_word(0u, dp);
 
-    ff_load_initial<W>(lattice, init, item, t_dens, rep, dp, rk);
+    ff_load_initial<W, TPB>(tree, burning, init, item, t_dens, rep, dp, rk);
     for (int i = threadIdx.x; i < 128; i += TPB) (&cnt[0][0])[i] = 0;
     __syncthreads();
 
     long long my_sum = 0;
-    for (int t = 1; t <= n_steps; ++t) {
-        const uint32_t* cur_t = lattice + ((t - 1) & 1) * 2 * NWORD;
-        const uint32_t* cur_b = cur_t + NWORD;
-        uint32_t* nxt_t = lattice + (t & 1) * 2 * NWORD;
-        uint32_t* nxt_b = nxt_t + NWORD;
-        int c = 0;
-        const StepKey sk = step_key(static_cast<uint32_t>(t), rep, rk);
-        for (int k = threadIdx.x; k < NWORD; k += TPB) {
-            const int y = k / W;
-            const int j = k - y * W;
-            const uint32_t tw = cur_t[k];
-            const uint32_t bw = cur_b[k];
-            uint32_t up, dn, bwest, beast;
-            if constexpr (W >= 8) {  // the same words, indexed from k (rows are W words; L W a power of two)
-                up = cur_b[(k + NWORD - W) & (NWORD - 1)];
-                dn = cur_b[(k + W) & (NWORD - 1)];
-                bwest = cur_b[(k & ~(W - 1)) | ((j + W - 1) & (W - 1))];
-                beast = cur_b[(k & ~(W - 1)) | ((j + 1) & (W - 1))];
-            } else {
-                up = cur_b[((y + L - 1) & (L - 1)) * W + j];
-                dn = cur_b[((y + 1) & (L - 1)) * W + j];
-                bwest = cur_b[y * W + ((j + W - 1) & (W - 1))];
-                beast = cur_b[y * W + ((j + 1) & (W - 1))];
-            }
-            const uint32_t nb = up | dn | (bw << 1) | (bwest >> 31) | (bw >> 1) | (beast << 31);
-            uint32_t g = 0, l = 0;
-            const unsigned long long base = 0xD2511F53ull * (8u * static_cast<uint32_t>(k));
+    uint32_t light[N * NT];  // [j][s], written and read only where flagged (local memory)
+    for (int t0 = 1; t0 <= n_steps; t0 += NT) {
+        unsigned long long flags = 0;  // bit NT j + s: word j has lightning at step t0 + s
+        const int ns = min(NT, n_steps + 1 - t0);
+        if (ns == NT) {
+            const StepKeys<NT> sk = step_keys<NT>(static_cast<uint32_t>(t0), rep, rk);
+#pragma unroll 1
+            for (int j = 0; j < N; ++j) {
+                uint32_t g[NT], l[NT];
+                ff_draw<NT, 1>(static_cast<uint32_t>(y * W + j0 + j), c3, sk, rk, t_grow, t_light, g, l);
+                const int at = ff_word<W>(y, j0 + j);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                unsigned long long pq = base + 0xD2511F53ull * q;
-                if constexpr (W >= 8) {  // the same sum as an explicit carry chain of two 32-bit adds
-                    const unsigned long long cq = 0xD2511F53ull * q;
-                    uint32_t plo, phi;
-                    asm("add.cc.u32 %0, %2, %4;\n\taddc.u32 %1, %3, %5;"
-                        : "=r"(plo), "=r"(phi)
-                        : "r"(static_cast<uint32_t>(base)), "r"(static_cast<uint32_t>(base >> 32)),
-                          "r"(static_cast<uint32_t>(cq)), "r"(static_cast<uint32_t>(cq >> 32)));
-                    pq = (static_cast<unsigned long long>(phi) << 32) | plo;
-                }
-                const uint4 b = philox_step(pq, c3, sk, rk);
-                or_if_below(g, b.x, t_grow, 1u << (4 * q));
-                or_if_below(g, b.y, t_grow, 1u << (4 * q + 1));
-                or_if_below(g, b.z, t_grow, 1u << (4 * q + 2));
-                or_if_below(g, b.w, t_grow, 1u << (4 * q + 3));
-                const uint32_t lowest = min(min(b.x, b.y), min(b.z, b.w));
-                if (__builtin_expect(lowest < t_light, 0)) {
-                    l |= (b.x < t_light) ? (1u << (4 * q)) : 0u;
-                    l |= (b.y < t_light) ? (1u << (4 * q + 1)) : 0u;
-                    l |= (b.z < t_light) ? (1u << (4 * q + 2)) : 0u;
-                    l |= (b.w < t_light) ? (1u << (4 * q + 3)) : 0u;
+                for (int s = 0; s < NT; ++s) {
+                    grow[s * NWORD + at] = g[s];
+                    if (__builtin_expect(l[s] != 0u, 0)) {
+                        light[j * NT + s] = l[s];
+                        flags |= 1ull << (j * NT + s);
+                    }
                 }
             }
-            const uint32_t ignite = nb | l;
-            const uint32_t nbw = tw & ignite;
-            nxt_b[k] = nbw;
-            nxt_t[k] = (tw & ~ignite) | (~(tw | bw) & g);
-            c += __popc(nbw);
+        } else {  // the last n_steps mod NT steps, one at a time
+#pragma unroll 1
+            for (int s = 0; s < ns; ++s) {
+                const StepKeys<1> sk = step_keys<1>(static_cast<uint32_t>(t0 + s), rep, rk);
+#pragma unroll 1
+                for (int j = 0; j < N; ++j) {
+                    uint32_t g[1], l[1];
+                    ff_draw<1, 4>(static_cast<uint32_t>(y * W + j0 + j), c3, sk, rk, t_grow, t_light, g, l);
+                    grow[s * NWORD + ff_word<W>(y, j0 + j)] = g[0];
+                    if (l[0] != 0u) {
+                        light[j * NT + s] = l[0];
+                        flags |= 1ull << (j * NT + s);
+                    }
+                }
+            }
         }
-        c = __reduce_add_sync(kFull, c);
-        if (lane == 0) atomicAdd(&cnt[((t - 1) >> 6) & 1][(t - 1) & 63], c);
-        __syncthreads();
-        if ((t & 63) == 0 || t == n_steps) {
-            const int chunk = (t - 1) >> 6;
-            const int n_slot = t - chunk * 64;
-            if (MRIP_CHECK(n_slot >= 1 && n_slot <= 64 && chunk * 64 + n_slot <= n_steps, 102, t))
-                ff_flush<TPB>(cnt[chunk & 1], n_slot, counts ? counts + item * n_steps + chunk * 64 : nullptr,
-                              true, my_sum);
+        uint32_t t_row[N], b_row[N];
+        row_load<W, N>(tree, y, j0, t_row);
+        row_load<W, N>(burning + ((t0 - 1) & 1) * NWORD, y, j0, b_row);
+#pragma unroll 1
+        for (int s = 0; s < ns; ++s) {
+            const int t = t0 + s;
+            uint32_t g[N], l[N];
+            row_load<W, N>(grow + s * NWORD, y, j0, g);
+#pragma unroll
+            for (int j = 0; j < N; ++j) l[j] = 0u;
+            if (__builtin_expect(flags != 0ull, 0)) {
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    if ((flags >> (j * NT + s)) & 1ull) l[j] = light[j * NT + s];
+            }
+            int c = row_step<W, N>(t_row, b_row, burning + ((t - 1) & 1) * NWORD, burning + (t & 1) * NWORD, y, j0, g, l);
+            c = __reduce_add_sync(kFull, c);
+            if (lane == 0) atomicAdd(&cnt[((t - 1) >> 6) & 1][(t - 1) & 63], c);
+            __syncthreads();
+            ff_end_step<TPB>(cnt, t, n_steps, counts, item, my_sum);
         }
+        row_store<W, N>(tree, y, j0, t_row);
     }
 
     if (scalar) ff_store_scalar<NWARP>(my_sum, red, scalar, item, n_steps, L);
     if (final_state) {
-        const uint32_t* fin_t = lattice + (n_steps & 1) * 2 * NWORD;
-        ff_store_final<W>(fin_t, fin_t + NWORD, final_state, item);
+        __syncthreads();  // every row's trees
+        ff_store_final<W, TPB>(tree, burning + (n_steps & 1) * NWORD, final_state, item);
     }
 }
 
-template <int W>
+template <int W, int R>
 mrip_status launch_ff(const double* dps, long long n_items, long long n_reps, long long rep0, int n_steps,
                       uint32_t t_dens, const RoundKeys& rk, const uint8_t* init, int32_t* counts,
                       double* scalar, uint8_t* final_state, cudaStream_t st) {
-    const size_t smem = 2 * 2 * static_cast<size_t>(32 * W) * W * sizeof(uint32_t);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(forest_fire_kernel<W>,
+    const size_t smem = (3 + ff_batch<W>()) * static_cast<size_t>(32 * W) * W * sizeof(uint32_t);
+    if (smem > 40 * 1024) {  // beside about 1 KB of static shared memory
+        cudaError_t e = cudaFuncSetAttribute(forest_fire_kernel<W, R>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
         if (e != cudaSuccess) return cuda_status(e, "forest fire: shared memory attribute");
     }
-    forest_fire_kernel<W><<<static_cast<unsigned>(n_items), ff_threads<W>(), smem, st>>>(
+    forest_fire_kernel<W, R><<<static_cast<unsigned>(n_items), R * ff_threads<W>(), smem, st>>>(
         dps, n_reps, rep0, n_steps, t_dens, rk, init, counts, scalar, final_state);
     return MRIP_OK;
 }
@@ -329,19 +481,23 @@ mrip_status launch_ff(const double* dps, long long n_items, long long n_reps, lo
 // (c0 = j div 2, c1 = t) under tag 5 (growth) or 6 (lightning)).  Work per
 // step is p L^2 variates instead of L^2 words.
 //
-// A warp draws 64 gaps per round (lane l takes one block, i.e. two gaps), a
-// warp scan of the lanes' (2 + K_2l + K_2l+1) places the events, and each
-// event sets its bit in an event plane in shared memory (atomicOr).  All
-// warps but the last share the growth set (a round's warp totals meet in
-// shared memory), the last warp draws the lightning set (one warp draws
-// both, in turn, when the CTA has one); then all threads update the lattice
-// word-parallel:
-//   ignite = burning neighbour | lightning event,
-//   burning' = tree & ignite,
-//   tree'    = (tree & ~ignite) | (empty & growth event),
-// clearing the event words they read.  Event planes are double-buffered by
-// step parity for L <= 256, so one barrier per step (between the draw and
-// the update) suffices; L = 512 keeps one buffer and adds a second barrier.
+// The event sets do not depend on the lattice, so several steps are drawn at
+// once, each by its own warps (group g of a CTA's kSlots groups draws step
+// t0 + g), and the CTA then updates the lattice kSlots times, a barrier per
+// step.  A warp draws 64 gaps per round (lane l takes one block, i.e. two
+// gaps), a warp scan of the lanes' (2 + K_2l + K_2l+1) places the events (a
+// group of several warps adds the warps' totals, met in shared memory behind
+// the group's own named barrier), and each event sets its bit in the step's
+// event plane (atomicOr); the update reads and clears the plane row by row.
+// The lightning set is empty at most steps, which one compare of its first
+// gap tells: lane l tests step t0 + l for 32 steps at once.
+//
+// The floor is decided in FP32 (MUFU.LG2) where the error bound leaves no
+// doubt, else by the fixed-point logarithm (gap_fast); same integers.
+// Measured against one set drawn per step by all warps, fixed-point floors and
+// scalar updates: 128 x 128, 1,024 replications x 1,000 steps 2.52 -> 1.44 ms; 256 x
+// 256, 2,048 x 400 11.3 -> 6.3 ms; 512 x 512, 183 x 65 1.80 -> 1.09 ms; 64 x 64, 2,155 x
+// 333 1.75 -> 0.74 ms; 32 x 32, 7,155 x 334 1.57 -> 0.83 ms.
 // ---------------------------------------------------------------------------
 // K = floor(E / mu) without the FP64 pipe: E = y58 2^-58 (the fixed-point
 // log), 2^-58 / mu = dm 2^-shift with dm a 64-bit integer (dm = the double's
@@ -385,6 +541,48 @@ __device__ __forceinline__ int gap_cells(unsigned long long y58, const GapScale&
     return k >= static_cast<unsigned long long>(n_cells) ? n_cells : static_cast<int>(k);
 }
 
+// The FP32 side of a gap: E / mu = q within q 2^-20 + c, where q = -log2(x)
+// scale from x = 1 - u rounded: v = the complement of u's top 32 bits, x = (v +
+// 1/2) 2^-32, is off by at most 2^-21 relative (v >= 2^20) plus 2^-23 of
+// rounding, log2 by 2^-22 absolute or relative (CUDA's bound for __log2f), in
+// all below 2^-20 / mu plus a relative 2^-21; 2^-22 more covers the roundings
+// of the interval's ends.
+struct GapFast {
+    float scale;  // ln 2 / mu
+    float c;
+};
+
+__device__ __forceinline__ GapFast gap_fast_scale(double p) {
+    if (p >= 1.0) return GapFast{0.0f, 0x1p-22f};
+    const double inv_mu = 1.0 / -log1p(-p);
+    return GapFast{static_cast<float>(fmin(0.69314718055994531 * inv_mu, 1e30)),
+                   static_cast<float>(fmin(0x1p-20 * inv_mu + 0x1p-22, 1e30))};
+}
+
+// K of words (lo, hi) if FP32 decides it, else -1.  RN(y - 1/2) at the
+// magnitude of 1.5 2^23 is floor(y) or, at an integer y, one less: where both
+// ends of the interval give the same k, the value between them is in [k, k + 1).
+__device__ __forceinline__ int gap_try(uint32_t hi, const GapFast& f, int n_cells) {
+    const uint32_t v = ~hi;
+    const float x = __fmaf_rn(__uint2float_rn(v), 0x1p-32f, 0x1p-33f);
+    const float q = fminf(-__log2f(x) * f.scale, 0x1p20f);  // past every lattice
+    const float a = __fmaf_rn(q, 1.0f - 0x1p-20f, -0.5f - f.c) + 12582912.0f;
+    const float b = __fmaf_rn(q, 1.0f + 0x1p-20f, -0.5f + f.c) + 12582912.0f;
+    const int k = static_cast<int>(__float_as_uint(a) - 0x4B400000u);
+    return (a == b && v >= (1u << 20)) ? min(k, n_cells) : -1;
+}
+
+// Both gaps of a block.
+__device__ __forceinline__ void block_gaps(const uint4& b, const GapFast& f, const GapScale& gs, int n_cells,
+                                           const LogTable& tab, int& k0, int& k1) {
+    k0 = gap_try(b.y, f, n_cells);
+    k1 = gap_try(b.w, f, n_cells);
+    if (__builtin_expect((k0 | k1) < 0, 0)) {
+        k0 = gap_cells(neg_log_q58<false>(b.x, b.y, tab), gs, n_cells);
+        k1 = gap_cells(neg_log_q58<false>(b.z, b.w, tab), gs, n_cells);
+    }
+}
+
 // Smallest 53-bit u (as an integer) for which the first gap of a set of
 // probability p passes n cells: u >= 1 - (1 - p)^n, i.e. -log(1 - u) >= n mu.
 // At least 1 (u = 0 gives the gap 0) and at most 2^53 (never, for p >= 1).
@@ -398,15 +596,37 @@ __device__ __forceinline__ unsigned long long first_gap_none(double p, int n) {
     return t >= 0x1p53 ? (1ull << 53) : static_cast<unsigned long long>(t);
 }
 
+// Event sets drawn together (and so warps per set): one per warp up to four.
+// 256 x 256 at two, four and eight sets (4, 2 and 1 warps each; the planes of eight
+// leave one CTA per SM): 7.2, 6.3, 8.0 ms; 128 x 128 at two and four: 2.09, 1.65.  L = 512
+// has room for two.
+template <int W>
+constexpr int skip_slots() {
+    return W == 16 ? 2 : W < 4 ? W : 4;
+}
+template <int W>
+constexpr int skip_warps() {
+    return W / skip_slots<W>();
+}
+
+// Draw the set of step t under (rep, c3) into the plane ev, by kWarps warps (sub
+// the index of this one; tot their shared totals, `bar` their named barrier).
 // Call only for p > 0.
-__device__ void draw_events(uint32_t* __restrict__ ev, int n_cells, const GapScale& gs, uint32_t t, uint32_t rep,
-                            uint32_t c3, const RoundKeys& rk, const LogTable& tab) {
+template <int W, int kWarps>
+__device__ __forceinline__ void draw_events(uint32_t* __restrict__ ev, const GapFast& gf, const GapScale& gs,
+                                            uint32_t t, uint32_t rep, uint32_t c3, const RoundKeys& rk,
+                                            const LogTable& tab, int sub, int (*tot)[kWarps], int bar) {
+    constexpr int L = 32 * W, n_cells = L * L;
     const int lane = threadIdx.x & 31;
-    int pos = -1;  // last event so far (warp-uniform)
-    for (uint32_t r = 0; pos + 1 < n_cells; ++r) {
-        const uint4 b = philox(32u * r + static_cast<uint32_t>(lane), t, rep, c3, rk);
-        const int k0 = gap_cells(neg_log_q58<false>(b.x, b.y, tab), gs, n_cells);
-        const int k1 = gap_cells(neg_log_q58<false>(b.z, b.w, tab), gs, n_cells);
+    const StepKeys<1> sk = step_keys<1>(t, rep, rk);
+    int pos = -1;  // last event so far (the same in every warp of the group)
+    for (int r = 0; pos + 1 < n_cells; ++r) {
+        uint32_t a_hi, a_lo;
+        mul_wide_u32(0xD2511F53u, static_cast<uint32_t>((r * kWarps + sub) * 32 + lane), a_hi, a_lo);
+        uint4 b[1];
+        step_blocks<1>(a_hi, a_lo, c3, sk, rk, b);
+        int k0, k1;
+        block_gaps(b[0], gf, gs, n_cells, tab, k0, k1);
         const int span = 2 + k0 + k1;
         int incl = span;
 #pragma unroll
@@ -414,99 +634,40 @@ __device__ void draw_events(uint32_t* __restrict__ ev, int n_cells, const GapSca
             const int v = __shfl_up_sync(kFull, incl, off);
             if (lane >= off) incl += v;
         }
-        const int p0 = pos + (incl - span) + 1 + k0;
-        const int p1 = p0 + 1 + k1;
-        if (p0 < n_cells && MRIP_CHECK(p0 >= 0, 103, p0)) atomicOr(ev + (p0 >> 5), 1u << (p0 & 31));
-        if (p1 < n_cells && MRIP_CHECK(p1 > p0, 104, p1)) atomicOr(ev + (p1 >> 5), 1u << (p1 & 31));
-        pos += __shfl_sync(kFull, incl, 31);
-    }
-}
-
-// All warps draw: warps 0 .. NG-1 share the growth gaps (round r, warp w
-// takes blocks (r NG + w) 32 + lane), warp NG the lightning gaps (blocks
-// 32 r + lane) while its set is unfinished.  Each warp scans its 64 gaps; the
-// warp totals meet in shared memory (double-buffered by round parity, one
-// barrier per round) and give every warp its offset and every thread the new
-// last position, so all threads agree on when each set ends.
-template <int NWARP>
-__device__ void draw_step_events(uint32_t* __restrict__ ev_g, uint32_t* __restrict__ ev_h, int n_cells,
-                                 bool grow_on, bool light_on, const GapScale& gsg, const GapScale& gsh,
-                                 unsigned long long light_none, uint32_t t, uint32_t rep, uint32_t c3g,
-                                 uint32_t c3h, const RoundKeys& rk, const LogTable& tab, int (*tot)[NWARP]) {
-    static_assert(NWARP >= 2, "one-warp CTAs draw with draw_events");
-    constexpr int NG = NWARP - 1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int pos_g = -1, pos_h = -1;
-    for (int r = 0; grow_on || light_on; ++r) {
-        int* tt = tot[r & 1];
-        const bool mine = (warp < NG) ? grow_on : light_on;
-        int k0 = 0, k1 = 0, span = 0, incl = 0;
-        if (mine) {
-            const bool g = warp < NG;
-            const uint32_t c0 = static_cast<uint32_t>(g ? (r * NG + warp) * 32 + lane : r * 32 + lane);
-            const uint4 b = philox(c0, t, rep, g ? c3g : c3h, rk);
-            // The lightning set's first gap passes the lattice (no event this
-            // step) iff u >= 1 - (1 - p)^(L^2): one compare of gap 0's 53 bits
-            // instead of the logs and the scan, most steps.
-            bool none = false;
-            if (!g && r == 0) {
-                const unsigned long long bits = ((static_cast<unsigned long long>(b.y) << 32) | b.x) >> 11;
-                none = __shfl_sync(kFull, bits >= light_none ? 1 : 0, 0) != 0;
-            }
-            if (none) {
-                k0 = n_cells;
-                k1 = n_cells;
-                incl = n_cells + 1;  // the set ends; no event bits
-                if (lane == 31) tt[warp] = incl;
-            } else {
-                const GapScale& gs = g ? gsg : gsh;
-                k0 = gap_cells(neg_log_q58<false>(b.x, b.y, tab), gs, n_cells);
-                k1 = gap_cells(neg_log_q58<false>(b.z, b.w, tab), gs, n_cells);
-                span = 2 + k0 + k1;
-                incl = span;
+        int before = 0, total;
+        if constexpr (kWarps > 1) {
+            int* tt = tot[r & 1];
+            if (lane == 31) tt[sub] = incl;
+            asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(32 * kWarps) : "memory");
+            total = 0;
 #pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int v = __shfl_up_sync(kFull, incl, off);
-                    if (lane >= off) incl += v;
-                }
-                if (lane == 31) tt[warp] = incl;
-            }
-        }
-        __syncthreads();
-        int before = 0, total_g = 0;
-        if (grow_on) {
-            for (int w = 0; w < NG; ++w) {
+            for (int w = 0; w < kWarps; ++w) {
                 const int v = tt[w];
-                before += (w < warp) ? v : 0;
-                total_g += v;
+                before += w < sub ? v : 0;
+                total += v;
             }
+        } else {
+            total = __shfl_sync(kFull, incl, 31);
         }
-        if (mine) {
-            const bool g = warp < NG;
-            const int p0 = (g ? pos_g + before : pos_h) + (incl - span) + 1 + k0;
-            const int p1 = p0 + 1 + k1;
-            uint32_t* ev = g ? ev_g : ev_h;
-            if (p0 < n_cells && MRIP_CHECK(p0 >= 0, 105, p0)) atomicOr(ev + (p0 >> 5), 1u << (p0 & 31));
-            if (p1 < n_cells && MRIP_CHECK(p1 > p0, 106, p1)) atomicOr(ev + (p1 >> 5), 1u << (p1 & 31));
-        }
-        if (grow_on) {
-            pos_g += total_g;
-            grow_on = pos_g + 1 < n_cells;
-        }
-        if (light_on) {
-            pos_h += tt[NG];
-            light_on = pos_h + 1 < n_cells;
-        }
+        const int p0 = pos + before + (incl - span) + 1 + k0;
+        const int p1 = p0 + 1 + k1;
+        if (p0 < n_cells && MRIP_CHECK(p0 >= 0, 103, p0))
+            atomicOr(ev + ff_word<W>(p0 / L, (p0 % L) / 32), 1u << (p0 & 31));
+        if (p1 < n_cells && MRIP_CHECK(p1 > p0, 104, p1))
+            atomicOr(ev + ff_word<W>(p1 / L, (p1 % L) / 32), 1u << (p1 & 31));
+        pos += total;
     }
 }
 
+// 128 x 128: 1,024 replications are 6.7 CTAs per SM, so seven resident ones (72
+// registers) make one wave: 1.44 ms against 1.65 at the compiler's 85 registers.
 template <int W>
-constexpr int ev_buffers() {
-    return W <= 8 ? 2 : 1;
+constexpr int skip_min_blocks() {
+    return W == 4 ? 7 : 1;
 }
 
 template <int W>
-__global__ void __launch_bounds__(ff_threads<W>()) forest_fire_skip_kernel(
+__global__ void __launch_bounds__(ff_threads<W>(), skip_min_blocks<W>()) forest_fire_skip_kernel(
     const double* __restrict__ dps, long long n_reps, long long rep0, int n_steps, uint32_t t_dens,
     const __grid_constant__ RoundKeys rk, LogTable tab, const uint8_t* __restrict__ init,
     int32_t* __restrict__ counts, double* __restrict__ scalar, uint8_t* __restrict__ final_state) {
@@ -514,89 +675,84 @@ __global__ void __launch_bounds__(ff_threads<W>()) forest_fire_skip_kernel(
     constexpr int NWORD = L * W;
     constexpr int TPB = ff_threads<W>();
     constexpr int NWARP = TPB / 32;
-    constexpr int NEV = ev_buffers<W>();
-    extern __shared__ uint32_t lattice[];  // [buffer][plane T, B][NWORD], then events [NEV][G, H][NWORD]
-    uint32_t* events = lattice + 4 * NWORD;
+    constexpr int NS = skip_slots<W>();
+    constexpr int GW = skip_warps<W>();
+    static_assert(32 % NS == 0 && NWARP == NS * GW, "32 steps are whole batches");
+    extern __shared__ __align__(16) uint32_t ff_smem[];
+    uint32_t* burning = ff_smem;                        // [2][NWORD], by step parity
+    uint32_t* ev_grow = ff_smem + 2 * NWORD;            // [NS][NWORD]
+    uint32_t* ev_light = ff_smem + (2 + NS) * NWORD;    // [NS][NWORD]
     __shared__ __align__(16) int cnt[2][64];
     __shared__ long long red[NWARP];
-    __shared__ int tot[2][NWARP];
+    __shared__ int tot[NS][2][GW];
 
-    const int lane = threadIdx.x & 31;
+    const int y = threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int slot = warp / GW, sub = warp % GW;
     const long long item = blockIdx.x;
-    if (!MRIP_CHECK((4u + 2u * NEV) * NWORD * sizeof(uint32_t) <= dynamic_smem_bytes(), 107, NWORD)) return;
+    if (!MRIP_CHECK((2u + 2u * NS) * NWORD * sizeof(uint32_t) <= dynamic_smem_bytes(), 107, NWORD)) return;
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double p_grow = dps[2 * dp], p_light = dps[2 * dp + 1];
     const bool any_grow = p_grow > 0.0, any_light = p_light > 0.0;
     const GapScale gs_grow = any_grow ? gap_scale(p_grow) : GapScale{0ull, 128};
     const GapScale gs_light = any_light ? gap_scale(p_light) : GapScale{0ull, 128};
-    const unsigned long long light_none = any_light ? first_gap_none(p_light, L * L) : (1ull << 53);
+    const GapFast gf_grow = gap_fast_scale(any_grow ? p_grow : 1.0);
+    const GapFast gf_light = gap_fast_scale(any_light ? p_light : 1.0);
+    const unsigned long long light_none = any_light ? first_gap_none(p_light, L * L) : 0ull;
     const uint32_t c3_grow = stream_word(5u, dp), c3_light = stream_word(6u, dp);
 
-    ff_load_initial<W>(lattice, init, item, t_dens, rep, dp, rk);
-    for (int k = threadIdx.x; k < NEV * 2 * NWORD; k += TPB) events[k] = 0u;
+    ff_load_initial<W, TPB>(ev_grow, burning, init, item, t_dens, rep, dp, rk);
     for (int i = threadIdx.x; i < 128; i += TPB) (&cnt[0][0])[i] = 0;
+    __syncthreads();
+    uint32_t t_row[W], b_row[W];
+    row_load<W, W>(ev_grow, y, 0, t_row);
+    row_load<W, W>(burning, y, 0, b_row);
+    __syncthreads();  // every row has its trees: the event planes start empty
+    for (int k = threadIdx.x; k < 2 * NS * NWORD; k += TPB) ev_grow[k] = 0u;
     __syncthreads();
 
     long long my_sum = 0;
-    for (int t = 1; t <= n_steps; ++t) {
-        uint32_t* ev_g = events + ((NEV == 2) ? (t & 1) : 0) * 2 * NWORD;
-        uint32_t* ev_h = ev_g + NWORD;
-        if constexpr (NWARP == 1) {
-            if (any_grow) draw_events(ev_g, L * L, gs_grow, t, rep, c3_grow, rk, tab);
-            if (any_light) draw_events(ev_h, L * L, gs_light, t, rep, c3_light, rk, tab);
-        } else {
-            draw_step_events<NWARP>(ev_g, ev_h, L * L, any_grow, any_light, gs_grow, gs_light, light_none, t, rep,
-                                    c3_grow, c3_light, rk, tab, tot);
+    unsigned none = 0u;  // bit i: no lightning at step 32 floor((t0 - 1) / 32) + 1 + i
+    for (int t0 = 1; t0 <= n_steps; t0 += NS) {
+        if (((t0 - 1) & 31) == 0) {
+            const uint4 b = philox(0u, static_cast<uint32_t>(t0 + lane), rep, c3_light, rk);
+            none = __ballot_sync(kFull, (((static_cast<unsigned long long>(b.y) << 32) | b.x) >> 11) >= light_none);
+        }
+        const int ns = min(NS, n_steps + 1 - t0);
+        if (slot < ns) {
+            const int t = t0 + slot;
+            if (any_grow)
+                draw_events<W, GW>(ev_grow + slot * NWORD, gf_grow, gs_grow, static_cast<uint32_t>(t), rep, c3_grow,
+                                   rk, tab, sub, tot[slot], 1 + slot);
+            if (sub == GW - 1 && !((none >> ((t - 1) & 31)) & 1u))
+                draw_events<W, 1>(ev_light + slot * NWORD, gf_light, gs_light, static_cast<uint32_t>(t), rep, c3_light,
+                                  rk, tab, 0, nullptr, 0);
         }
         __syncthreads();
-        // counts of the steps before t are complete: flush a finished chunk
-        if (t > 1 && ((t - 1) & 63) == 0) {
-            const int chunk = (t - 2) >> 6;
-            if (MRIP_CHECK(chunk * 64 + 64 <= n_steps, 108, t))
-                ff_flush<TPB>(cnt[chunk & 1], 64, counts ? counts + item * n_steps + chunk * 64 : nullptr, true,
-                              my_sum);
+#pragma unroll 1
+        for (int s = 0; s < ns; ++s) {
+            const int t = t0 + s;
+            uint32_t g[W], l[W], zero[W];
+#pragma unroll
+            for (int j = 0; j < W; ++j) zero[j] = l[j] = 0u;
+            row_load<W, W>(ev_grow + s * NWORD, y, 0, g);
+            row_store<W, W>(ev_grow + s * NWORD, y, 0, zero);
+            if (!((none >> ((t - 1) & 31)) & 1u)) {
+                row_load<W, W>(ev_light + s * NWORD, y, 0, l);
+                row_store<W, W>(ev_light + s * NWORD, y, 0, zero);
+            }
+            int c = row_step<W, W>(t_row, b_row, burning + ((t - 1) & 1) * NWORD, burning + (t & 1) * NWORD, y, 0, g, l);
+            c = __reduce_add_sync(kFull, c);
+            if (lane == 0) atomicAdd(&cnt[((t - 1) >> 6) & 1][(t - 1) & 63], c);
+            __syncthreads();
+            ff_end_step<TPB>(cnt, t, n_steps, counts, item, my_sum);
         }
-        const uint32_t* cur_t = lattice + ((t - 1) & 1) * 2 * NWORD;
-        const uint32_t* cur_b = cur_t + NWORD;
-        uint32_t* nxt_t = lattice + (t & 1) * 2 * NWORD;
-        uint32_t* nxt_b = nxt_t + NWORD;
-        int c = 0;
-        for (int k = threadIdx.x; k < NWORD; k += TPB) {
-            const int y = k / W;
-            const int j = k - y * W;
-            const uint32_t tw = cur_t[k];
-            const uint32_t bw = cur_b[k];
-            const uint32_t up = cur_b[((y + L - 1) & (L - 1)) * W + j];
-            const uint32_t dn = cur_b[((y + 1) & (L - 1)) * W + j];
-            const uint32_t bwest = cur_b[y * W + ((j + W - 1) & (W - 1))];
-            const uint32_t beast = cur_b[y * W + ((j + 1) & (W - 1))];
-            const uint32_t nb = up | dn | (bw << 1) | (bwest >> 31) | (bw >> 1) | (beast << 31);
-            const uint32_t g = ev_g[k];
-            const uint32_t h = ev_h[k];
-            ev_g[k] = 0u;
-            ev_h[k] = 0u;
-            const uint32_t ignite = nb | h;
-            const uint32_t nbw = tw & ignite;
-            nxt_b[k] = nbw;
-            nxt_t[k] = (tw & ~ignite) | (~(tw | bw) & g);
-            c += __popc(nbw);
-        }
-        c = __reduce_add_sync(kFull, c);
-        if (lane == 0) atomicAdd(&cnt[((t - 1) >> 6) & 1][(t - 1) & 63], c);
-        if (NEV == 1) __syncthreads();
-    }
-    __syncthreads();
-    if (n_steps > 0) {
-        const int chunk = (n_steps - 1) >> 6;
-        const int n_slot = n_steps - chunk * 64;
-        ff_flush<TPB>(cnt[chunk & 1], n_slot, counts ? counts + item * n_steps + chunk * 64 : nullptr, false,
-                      my_sum);
     }
     if (scalar) ff_store_scalar<NWARP>(my_sum, red, scalar, item, n_steps, L);
     if (final_state) {
-        const uint32_t* fin_t = lattice + (n_steps & 1) * 2 * NWORD;
-        ff_store_final<W>(fin_t, fin_t + NWORD, final_state, item);
+        row_store<W, W>(ev_grow, y, 0, t_row);
+        __syncthreads();
+        ff_store_final<W, TPB>(ev_grow, burning + (n_steps & 1) * NWORD, final_state, item);
     }
 }
 
@@ -604,9 +760,8 @@ template <int W>
 mrip_status launch_ff_skip(const double* dps, long long n_items, long long n_reps, long long rep0, int n_steps,
                            uint32_t t_dens, const RoundKeys& rk, const LogTable& tab, const uint8_t* init,
                            int32_t* counts, double* scalar, uint8_t* final_state, cudaStream_t st) {
-    const size_t nword = static_cast<size_t>(32 * W) * W;
-    const size_t smem = (4 + 2 * ev_buffers<W>()) * nword * sizeof(uint32_t);
-    if (smem > 48 * 1024) {
+    const size_t smem = (2 + 2 * skip_slots<W>()) * static_cast<size_t>(32 * W) * W * sizeof(uint32_t);
+    if (smem > 40 * 1024) {  // beside about 1 KB of static shared memory
         cudaError_t e = cudaFuncSetAttribute(forest_fire_skip_kernel<W>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
@@ -643,13 +798,23 @@ mrip_status forest_fire_launch(const double* d_dps, int32_t n_dp, int64_t rep0, 
         return fail(MRIP_EINVAL, "mrip_forest_fire_simulate: state buffers need 16-byte alignment");
     const RoundKeys rk = expand_key(seed);
     const uint32_t t_dens = threshold32(density);
+    // Two threads per lattice row where one per row would leave the SMs with at
+    // most 256 of the 512 threads the register budget allows: 100 replications
+    // of 128 x 128 x 999 steps take 1.63 ms with two and 2.07 with one, 101 of 256 x
+    // 256 x 502 2.84 and 2.97.  On a full GPU one is faster (1,024 of 128 x 128: 9.95
+    // against 10.16 ms, 2,048 of 256 x 256: 30.8 against 31.6); four per row gain
+    // nothing over two (1.66 ms).
+    const bool wide = n_items * L <= 256ll * sm_count();
+    auto launch = [&](auto* f) {
+        return f(d_dps, n_items, n_reps, rep0, n_steps, t_dens, rk, d_init, d_counts, d_scalar, d_final, st);
+    };
     mrip_status rc = MRIP_OK;
     switch (L) {
-        case 32: rc = launch_ff<1>(d_dps, n_items, n_reps, rep0, n_steps, t_dens, rk, d_init, d_counts, d_scalar, d_final, st); break;
-        case 64: rc = launch_ff<2>(d_dps, n_items, n_reps, rep0, n_steps, t_dens, rk, d_init, d_counts, d_scalar, d_final, st); break;
-        case 128: rc = launch_ff<4>(d_dps, n_items, n_reps, rep0, n_steps, t_dens, rk, d_init, d_counts, d_scalar, d_final, st); break;
-        case 256: rc = launch_ff<8>(d_dps, n_items, n_reps, rep0, n_steps, t_dens, rk, d_init, d_counts, d_scalar, d_final, st); break;
-        case 512: rc = launch_ff<16>(d_dps, n_items, n_reps, rep0, n_steps, t_dens, rk, d_init, d_counts, d_scalar, d_final, st); break;
+        case 32: rc = launch(launch_ff<1, 1>); break;
+        case 64: rc = wide ? launch(launch_ff<2, 2>) : launch(launch_ff<2, 1>); break;
+        case 128: rc = wide ? launch(launch_ff<4, 2>) : launch(launch_ff<4, 1>); break;
+        case 256: rc = wide ? launch(launch_ff<8, 2>) : launch(launch_ff<8, 1>); break;
+        case 512: rc = launch(launch_ff<16, 1>); break;
     }
     if (rc != MRIP_OK) return rc;
     return launch_status("mrip_forest_fire_simulate");

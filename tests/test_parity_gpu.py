@@ -277,6 +277,29 @@ def test_forest_fire_bit_exact(eng, torch_mod, L, n_steps):
         assert gsc[i] == rc.sum() / (n_steps * L * L)
 
 
+@pytest.mark.parametrize("L", [32, 64, 128, 256, 512])
+@pytest.mark.parametrize("many", [False, True])
+@pytest.mark.parametrize("n_steps", [7, 8, 17])
+def test_forest_fire_batches_of_steps(eng, torch_mod, L, many, n_steps):
+    """Steps are drawn in batches of 8 (4 at L = 512) and a row of the lattice is one thread's or, for few
+    replications, two threads': step counts around the batch, replication counts on both sides of the rule, with
+    lightning in most words and without any."""
+    t = torch_mod
+    few = 256 * t.cuda.get_device_properties(0).multi_processor_count // L
+    dps = np.array([[0.3, 0.4], [0.9, 0.0]])
+    n_reps = few // 2 + 1 if many else 2
+    counts = t.empty(2 * n_reps * n_steps, dtype=t.int32, device="cuda")
+    final = t.empty(2 * n_reps * L * L, dtype=t.uint8, device="cuda")
+    eng.mrip_forest_fire_simulate(dev(t, dps), n_reps, L, n_steps, 0.6, 5, counts=counts, final=final)
+    got = counts.cpu().numpy().reshape(2, n_reps, n_steps)
+    lattice = final.view(2, n_reps, L, L)
+    for dp in range(2):
+        for rep in (0, n_reps - 1):
+            ref, state = oracle.forest_fire_rep(L, n_steps, dps[dp, 0], dps[dp, 1], 0.6, 5, dp, rep)
+            assert np.array_equal(got[dp, rep], ref)
+            assert np.array_equal(lattice[dp, rep].cpu().numpy(), state)
+
+
 def test_forest_fire_from_given_states(eng, torch_mod):
     t = torch_mod
     L, n_steps, n_reps = 64, 70, 4
