@@ -11,6 +11,11 @@
 //               entry wait, and each lane then replays its segment with the
 //               plain recurrence.  The tandem does the same with 3-station
 //               max-plus maps (lower-triangular 3x3 matrix plus constants).
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace mrip {
@@ -38,7 +43,6 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // are summed in FP64 from the same log values, where a variate's relative
 // precision matters.
 // ---------------------------------------------------------------------------
-constexpr int kFixBits = 48;
 constexpr long long kFixGuard = 1LL << 60;
 constexpr long long kFixNegInf = -(1LL << 62);  // "empty" state: v - A stays above -2^63
 
@@ -113,11 +117,15 @@ __device__ __forceinline__ void mm1_client(uint32_t n, const RowKey& row, double
     a = expo_fast<kShared>(b.z, b.w, tab, inv_lam);
 }
 
-// (A minimum of four CTAs per SM; 1, 3, 6 and 8 take the same time, 0.569 ms
-// for 2^16 replications of 1,000 clients before the FP32 tail of the
-// logarithm: 13.5 warps per SM are latency-bound at any budget.)
+// Clients whose variates are drawn together: 2^16 replications are 13.5 warps
+// per SM, too few to hide one client's chain of Philox rounds and logarithms
+// behind other warps.  2^16 replications x 1,000 clients at 1, 2, 3 and 4 clients:
+// 561, 526, 504, 500 us (the last with 114 registers; a minimum of three CTAs per
+// SM leaves them).
+constexpr uint32_t kMm1Group = 4;
+
 template <bool kLane0Only>
-__global__ void __launch_bounds__(128, 4) mm1_serial_kernel(const double* __restrict__ dps, long long n_items,
+__global__ void __launch_bounds__(128, 3) mm1_serial_kernel(const double* __restrict__ dps, long long n_items,
                                   long long n_reps, long long rep0, long long n_clients,
                                   const __grid_constant__ RoundKeys rk, LogTable tab, Mm1Out out) {
     __shared__ unsigned long long nln2[kLogExponents];
@@ -142,21 +150,36 @@ __global__ void __launch_bounds__(128, 4) mm1_serial_kernel(const double* __rest
         bool overflow = false;
         // (client indices are 32-bit: n_clients < 2^32, the counter word c1)
         const uint32_t nc = static_cast<uint32_t>(n_clients);
-        for (uint32_t n = 0; n < nc; ++n) {
-            const uint4 b = philox_row(row, static_cast<uint32_t>(n), rk);
-            const long long s_ = to_fix(neg_log_q58<true>(b.x, b.y, tab), cmu);
-            const long long a_ = to_fix(neg_log_q58<true>(b.z, b.w, tab), cl);
-            sw.add(wf);
-            const long long v = wf + s_;
-            sv.add(v);
-            const long long t = v - a_;
-            wf = relu64(t);
-            si.add(wf - t);  // max(0, -t)
-            if (wf >= kFixGuard) {
-                overflow = true;
-                break;
+        // kMm1Group clients' variates at a time: their Philox rounds and
+        // logarithms are independent chains, the Lindley steps follow.  The
+        // guard is tested per group: a wait below 2^60 grows by less than 2^59.3
+        // a client, so nothing overflows before the test.
+        auto clients = [&](uint32_t n, auto count) {
+            constexpr int kCount = decltype(count)::value;
+            long long s_[kCount], a_[kCount];
+#pragma unroll
+            for (int i = 0; i < kCount; ++i) {
+                const uint4 b = philox_row(row, n + i, rk);
+                s_[i] = to_fix(neg_log_q58<true>(b.x, b.y, tab), cmu);
+                a_[i] = to_fix(neg_log_q58<true>(b.z, b.w, tab), cl);
             }
-        }
+            long long any = 0;
+#pragma unroll
+            for (int i = 0; i < kCount; ++i) {
+                sw.add(wf);
+                const long long v = wf + s_[i];
+                sv.add(v);
+                const long long t = v - a_[i];
+                wf = relu64(t);
+                si.add(wf - t);  // max(0, -t)
+                any |= wf;
+            }
+            return any < kFixGuard;
+        };
+        uint32_t n = 0;
+        for (; nc - n >= kMm1Group && !overflow; n += kMm1Group)
+            overflow = !clients(n, std::integral_constant<int, kMm1Group>{});
+        for (; n < nc && !overflow; ++n) overflow = !clients(n, std::integral_constant<int, 1>{});
         if (!overflow) {
             if (out.wait) out.wait[item] = sw.to_double() / inv;
             if (out.idle) out.idle[item] = si.to_double() / inv;
@@ -514,19 +537,52 @@ __device__ __forceinline__ FTMap ftmap_identity() {
 
 __device__ __forceinline__ long long lmax(long long x, long long y) { return x > y ? x : y; }
 
+// f followed by one client, without saturation: each of the nine grows or
+// shrinks by less than four variates.
 __device__ __forceinline__ FTMap ftmap_push(const FTMap& f, long long a, long long s1, long long s2, long long s3) {
     const long long e1 = s1 - a, e2 = s2 - a, e3 = s3 - a;
     FTMap r;
-    r.c1 = lmax(s1, sat61(f.c1 + e1));
-    r.d11 = sat61(f.d11 + e1);
-    r.c2 = sat61(lmax(f.c2 + e2, r.c1 + s2));
-    r.d21 = sat61(lmax(f.d21 + e2, r.d11 + s2));
-    r.d22 = sat61(f.d22 + e2);
-    r.c3 = sat61(lmax(f.c3 + e3, r.c2 + s3));
-    r.d31 = sat61(lmax(f.d31 + e3, r.d21 + s3));
-    r.d32 = sat61(lmax(f.d32 + e3, r.d22 + s3));
-    r.d33 = sat61(f.d33 + e3);
+    r.c1 = lmax(s1, f.c1 + e1);
+    r.d11 = f.d11 + e1;
+    r.c2 = lmax(f.c2 + e2, r.c1 + s2);
+    r.d21 = lmax(f.d21 + e2, r.d11 + s2);
+    r.d22 = f.d22 + e2;
+    r.c3 = lmax(f.c3 + e3, r.c2 + s3);
+    r.d31 = lmax(f.d31 + e3, r.d21 + s3);
+    r.d32 = lmax(f.d32 + e3, r.d22 + s3);
+    r.d33 = f.d33 + e3;
     return r;
+}
+
+__device__ __forceinline__ void ftmap_saturate(FTMap& f) {
+    f.c1 = sat61(f.c1);
+    f.c2 = sat61(f.c2);
+    f.c3 = sat61(f.c3);
+    f.d11 = sat61(f.d11);
+    f.d21 = sat61(f.d21);
+    f.d22 = sat61(f.d22);
+    f.d31 = sat61(f.d31);
+    f.d32 = sat61(f.d32);
+    f.d33 = sat61(f.d33);
+}
+
+// Clients between two saturations.  A variate is below 36.8 / rate time units:
+// for rates of at least 1/4 that is 2^55.3 units of 2^-48, so 8 clients move a
+// saturated map by less than 2^60.3 and nothing leaves 63 bits; for the
+// slowest rates (2^-6) it is 2^59.3 and every client saturates.  (16 replications x
+// 100,000 clients on 64 SMs: 134.8 us, 143.7 when every client saturates.)
+__device__ __forceinline__ uint32_t saturation_mask(double r0, double r1, double r2, double r3) {
+    return fmin(fmin(r0, r1), fmin(r2, r3)) >= 0.25 ? 7u : 0u;
+}
+
+// State after the clients of f, from state v.
+__device__ __forceinline__ void ftmap_apply(const FTMap& f, long long& v1, long long& v2, long long& v3) {
+    const long long w1 = lmax(f.c1, sat61(v1 + f.d11));
+    const long long w2 = lmax(f.c2, sat61(lmax(v1 + f.d21, v2 + f.d22)));
+    const long long w3 = lmax(f.c3, sat61(lmax(v1 + f.d31, lmax(v2 + f.d32, v3 + f.d33))));
+    v1 = w1;
+    v2 = w2;
+    v3 = w3;
 }
 
 __device__ __forceinline__ FTMap ftmap_compose(const FTMap& f, const FTMap& g) {  // g after f
@@ -661,6 +717,7 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
         const unsigned long long cl = fix_scale(lam), c1 = fix_scale(mu1), c2 = fix_scale(mu2),
                                  c3f = fix_scale(mu3);
         FTMap f = ftmap_identity();
+        const uint32_t every = saturation_mask(lam, mu1, mu2, mu3);
         for (long long n = lo; n < hi; ++n) {
             uint4 b0, b1;
             philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
@@ -668,7 +725,9 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
                            to_fix(neg_log_q58<false>(b0.z, b0.w, tab), c1),
                            to_fix(neg_log_q58<false>(b1.x, b1.y, tab), c2),
                            to_fix(neg_log_q58<false>(b1.z, b1.w, tab), c3f));
+            if ((static_cast<uint32_t>(n - lo) & every) == every) ftmap_saturate(f);
         }
+        ftmap_saturate(f);
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const FTMap prev = ftmap_shfl_up(f, off);
@@ -741,11 +800,15 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
 }
 
 // ---------------------------------------------------------------------------
-// M/M/1, one replication per CTA (few replications of a latency-bound
-// length): thread i takes the contiguous clients [i k, (i+1) k).  Pass 1
+// M/M/1, one replication per CTA or cluster of CTAs (few replications of a
+// latency-bound length; cta_shape): thread i takes the contiguous clients
+// [i k, (i+1) k).  Pass 1
 // composes each thread's Lindley maps W -> max(c, W + d); a block scan (warp
 // shuffles, then the warp totals in shared memory) gives every thread the
 // map of all clients before it, whose value at W_0 = 0 is its entry wait;
+// in a cluster the maps of the earlier CTAs, read over distributed shared
+// memory, carry W_0 = 0 to the CTA's first client (14 replications x 100,003
+// clients 201 -> 47 us, 32 x 10,000 36 -> 21 us);
 // pass 2 replays the thread's clients with the plain recurrence.  Times run
 // in the 48-bit fixed point of the tandem, so composition is exact and the
 // sums are exact integers (order-free); c and d saturate at +-2^61, which
@@ -775,10 +838,10 @@ __device__ __forceinline__ Map shfl_up_map(const Map& m, int off) {
 }
 
 // Exclusive block scan of per-thread maps (thread order); `identity` for
-// thread 0.  smem: one Map per warp.
+// thread 0.  smem: one Map per warp.  *total (by the last thread): all of them.
 template <class Map, class Compose>
-__device__ Map block_exclusive_map(Map f, Map identity, Map* smem, Compose compose) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+__device__ Map block_exclusive_map(Map f, Map identity, Map* smem, Map* total, Compose compose) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     Map incl = f;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -789,6 +852,7 @@ __device__ Map block_exclusive_map(Map f, Map identity, Map* smem, Compose compo
     __syncthreads();
     Map before = identity;  // maps of the earlier warps, composed in order
     for (int w = 0; w < warp; ++w) before = compose(before, smem[w]);
+    if (threadIdx.x == blockDim.x - 1) *total = compose(before, incl);
     Map excl = shfl_up_map(incl, 1);
     if (lane == 0) excl = identity;
     __syncthreads();  // smem reusable
@@ -800,24 +864,36 @@ struct Mm1Sums {
 };
 
 
+template <bool kCluster>
 __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict__ dps, long long n_reps,
                                                        long long rep0, long long n_clients, bool staged,
                                                        const __grid_constant__ RoundKeys rk, LogTable tab,
                                                        Mm1Out out) {
+    namespace cg = cooperative_groups;
     extern __shared__ long long fix_stage[];  // [client - lo][thread] x (S, A) when staged
     __shared__ FixMap fmaps[32];
     __shared__ DblMap dmaps[32];
     __shared__ U96 part[3][32];
     __shared__ double dpart[3][32];
+    __shared__ DblMap dtotal;
+    __shared__ struct {
+        FixMap map;  // all clients of this CTA
+        U96 sum[3];
+        int bad;
+    } mine;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int ctas = kCluster ? static_cast<int>(cluster.num_blocks()) : 1;
+    const int rank = kCluster ? static_cast<int>(cluster.block_rank()) : 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const long long item = blockIdx.x;
+    const long long item = blockIdx.x / ctas;
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double lam = dps[2 * dp], mu = dps[2 * dp + 1];
     const RowKey row = row_key(rep, stream_word(0u, dp), rk);
-    const long long k = (n_clients + blockDim.x - 1) / blockDim.x;
-    const long long lo = min(static_cast<long long>(threadIdx.x) * k, n_clients);
-    const long long hi = min(lo + k, n_clients);
+    const long long threads = static_cast<long long>(ctas) * blockDim.x;
+    const long long k = (n_clients + threads - 1) / threads;
+    long long lo = min((static_cast<long long>(rank) * blockDim.x + threadIdx.x) * k, n_clients);
+    long long hi = min(lo + k, n_clients);
     const double inv_n = static_cast<double>(n_clients);
     // (debug build: a stage larger than the launch's shared memory is
     // recorded and the variates recomputed)
@@ -847,9 +923,16 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
             }
             f = fcompose(f, FixMap{0, sv - av});
         }
-        const FixMap pre = block_exclusive_map(f, FixMap{-kSat, 0}, fmaps, fcompose);
-        long long w = pre.c > pre.d ? pre.c : pre.d;  // map at W_0 = 0
-        if (threadIdx.x == 0) w = 0;
+        const FixMap pre = block_exclusive_map(f, FixMap{-kSat, 0}, fmaps, &mine.map, fcompose);
+        long long w = 0;  // W_0
+        if constexpr (kCluster) {
+            cluster.sync();
+            for (int r = 0; r < rank; ++r) {
+                const FixMap e = *cluster.map_shared_rank(&mine.map, r);
+                w = max(e.c, sat61(w + e.d));
+            }
+        }
+        if (threadIdx.x > 0) w = max(pre.c, sat61(w + pre.d));
         bool bad = w >= kFixGuard;
         Mm1Sums sm;
         for (long long n = lo; n < hi && !bad; ++n) {
@@ -870,30 +953,49 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
             sm.i.add(w - t);  // max(0, -t)
             bad = w >= kFixGuard;
         }
-        fixed_ok = !__syncthreads_or(bad);
-        if (fixed_ok) {
+        const bool cta_bad = __syncthreads_or(bad) != 0;
+        fixed_ok = !cta_bad;
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                add_u96(sm.w, shfl_down_u96(sm.w, off));
-                add_u96(sm.i, shfl_down_u96(sm.i, off));
-                add_u96(sm.v, shfl_down_u96(sm.v, off));
+        for (int off = 16; off > 0; off >>= 1) {
+            add_u96(sm.w, shfl_down_u96(sm.w, off));
+            add_u96(sm.i, shfl_down_u96(sm.i, off));
+            add_u96(sm.v, shfl_down_u96(sm.v, off));
+        }
+        if (lane == 0) {
+            part[0][warp] = sm.w;
+            part[1][warp] = sm.i;
+            part[2][warp] = sm.v;
+        }
+        __syncthreads();
+        U96 tot;
+        if (threadIdx.x < 3)
+            for (int x = 0; x < nwarp; ++x) add_u96(tot, part[threadIdx.x][x]);
+        if constexpr (kCluster) {
+            if (threadIdx.x < 3) mine.sum[threadIdx.x] = tot;
+            if (threadIdx.x == 0) mine.bad = cta_bad ? 1 : 0;
+            cluster.sync();
+            if (rank == 0) {
+                for (int r = 1; r < ctas; ++r) {
+                    fixed_ok = fixed_ok && *cluster.map_shared_rank(&mine.bad, r) == 0;
+                    if (threadIdx.x < 3) add_u96(tot, cluster.map_shared_rank(&mine.sum[0], r)[threadIdx.x]);
+                }
             }
-            if (lane == 0) {
-                part[0][warp] = sm.w;
-                part[1][warp] = sm.i;
-                part[2][warp] = sm.v;
-            }
-            __syncthreads();
+            cluster.sync();  // the first CTA has read the others' shared memory
+        }
+        if (rank != 0) return;
+        if (fixed_ok) {
             if (threadIdx.x < 3) {
-                U96 tot;
-                for (int x = 0; x < nwarp; ++x) add_u96(tot, part[threadIdx.x][x]);
                 double* dst = threadIdx.x == 0 ? out.wait : threadIdx.x == 1 ? out.idle : out.system;
                 if (dst) dst[item] = tot.to_double() / inv_n;
             }
             return;
         }
     }
-    // FP64: the same passes with doubles
+    if (rank != 0) return;
+    // FP64: the same passes with doubles, by the first CTA alone
+    const long long k1 = (n_clients + blockDim.x - 1) / blockDim.x;
+    lo = min(static_cast<long long>(threadIdx.x) * k1, n_clients);
+    hi = min(lo + k1, n_clients);
     const double inv_lam = 0x1p-58 / lam, inv_mu = 0x1p-58 / mu;
     DblMap f{-INFINITY, 0.0};
     for (long long n = lo; n < hi; ++n) {
@@ -901,7 +1003,7 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
         mm1_client<false>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, sv, av);
         f = dcompose(f, DblMap{0.0, sv - av});
     }
-    const DblMap pre = block_exclusive_map(f, DblMap{-INFINITY, 0.0}, dmaps, dcompose);
+    const DblMap pre = block_exclusive_map(f, DblMap{-INFINITY, 0.0}, dmaps, &dtotal, dcompose);
     double w = pre.c > pre.d ? pre.c : pre.d;
     if (threadIdx.x == 0) w = 0.0;
     double sw = 0.0, si = 0.0, sv_sum = 0.0;
@@ -941,37 +1043,61 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
 }
 
 // ---------------------------------------------------------------------------
-// Tandem, one replication per CTA (few replications of a long horizon): thread
-// i takes the contiguous clients [i k, (i+1) k); its fixed-point max-plus map
-// (FTMap) is composed in pass 1, a block scan (warp shuffles, then the warp
-// totals in order) gives every thread the map of all clients before it, and
-// pass 2 replays its clients from that entry state.  Sojourn sums are exact
-// 96-bit integers; the early-window sums FP64 in a fixed order.  Rates
-// outside the fixed-point range or a sojourn past 2^12 hand the replication
-// to the FP64 warp scan (warp 0).
+// Tandem, one replication per CTA or cluster of CTAs (few replications of a
+// long horizon): thread i of the cluster takes the contiguous clients
+// [i k, (i+1) k); its fixed-point max-plus map (FTMap) is composed in pass 1, a
+// block scan (warp shuffles, then the warp totals in order) gives every thread
+// the map of the CTA's clients before it, the maps of the earlier CTAs (read
+// over distributed shared memory) applied to the empty state give the CTA's
+// entry state, and pass 2 replays the thread's clients from there.  Sojourn
+// sums are exact integers; the early-window sums FP64 in a fixed order.  Rates
+// outside the fixed-point range or a sojourn past 2^12 hand the replication to
+// the FP64 warp scan (the first CTA's warp 0).
+//
+// One CTA per replication leaves the SMs without one idle, so few replications
+// are split over clusters of up to 8 CTAs (cta_shape): 16 x 100,000 clients run on
+// 112 SMs instead of 16, 439 -> 102 us.  At most 512 threads per CTA: at 1,024 the 64
+// registers of a thread spill (33 replications x 50,021 clients in clusters: 86 us,
+// at 640, 768 and 1,024 threads 94, 104, 119); 256 where there are more replications
+// than SMs, so that several CTAs share one (333 x 5,021 clients: 91 .. 98 us at 256
+// threads, 123 at 384, 133 at 512, 186 at the former 1,024).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restrict__ dps, long long n_reps,
+constexpr int kTandemThreads = 512;
+template <bool kCluster>
+__global__ void __launch_bounds__(kTandemThreads) tandem3_cta_kernel(const double* __restrict__ dps, long long n_reps,
                                                            long long rep0, long long n_clients, long long window,
                                                            uint32_t tag, const __grid_constant__ RoundKeys rk,
                                                            LogTable tab, TandemOut out) {
+    namespace cg = cooperative_groups;
     __shared__ FTMap wmap[32];
     __shared__ U96 wy[32];
     __shared__ double wsum[4][32];
+    __shared__ struct {
+        FTMap map;     // all clients of this CTA
+        U96 y;
+        double sum[4];
+        int bad;
+    } mine;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int ctas = kCluster ? static_cast<int>(cluster.num_blocks()) : 1;
+    const int rank = kCluster ? static_cast<int>(cluster.block_rank()) : 0;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarp = blockDim.x >> 5;
-    const long long item = blockIdx.x;
+    const long long item = blockIdx.x / ctas;
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
     const double lam = dps[4 * dp], mu1 = dps[4 * dp + 1], mu2 = dps[4 * dp + 2], mu3 = dps[4 * dp + 3];
     const RowKey row = row_key(rep, stream_word(tag, dp), rk);
     const long long w_len = (n_clients < window) ? n_clients : window;
-    const long long k = (n_clients + blockDim.x - 1) / blockDim.x;
-    const long long lo = min(static_cast<long long>(t) * k, n_clients);
+    const long long threads = static_cast<long long>(ctas) * blockDim.x;
+    const long long k = (n_clients + threads - 1) / threads;
+    const long long lo = min((static_cast<long long>(rank) * blockDim.x + t) * k, n_clients);
     const long long hi = min(lo + k, n_clients);
 
     if (fix_rate_ok(lam) && fix_rate_ok(mu1) && fix_rate_ok(mu2) && fix_rate_ok(mu3)) {
         const unsigned long long cl = fix_scale(lam), c1 = fix_scale(mu1), c2 = fix_scale(mu2),
                                  c3f = fix_scale(mu3);
         FTMap f = ftmap_identity();
+        const uint32_t every = saturation_mask(lam, mu1, mu2, mu3);
         for (long long n = lo; n < hi; ++n) {
             uint4 b0, b1;
             philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
@@ -979,7 +1105,9 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
                            to_fix(neg_log_q58<false>(b0.z, b0.w, tab), c1),
                            to_fix(neg_log_q58<false>(b1.x, b1.y, tab), c2),
                            to_fix(neg_log_q58<false>(b1.z, b1.w, tab), c3f));
+            if ((static_cast<uint32_t>(n - lo) & every) == every) ftmap_saturate(f);
         }
+        ftmap_saturate(f);
         // block exclusive scan of the maps
         FTMap incl = f;
 #pragma unroll
@@ -991,10 +1119,16 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
         __syncthreads();
         FTMap pre = ftmap_identity();
         for (int w = 0; w < warp; ++w) pre = ftmap_compose(pre, wmap[w]);
+        if (kCluster && t == blockDim.x - 1) mine.map = ftmap_compose(pre, incl);
         FTMap excl = ftmap_shfl_up(incl, 1);
         if (lane == 0) excl = ftmap_identity();
         pre = ftmap_compose(pre, excl);
-        long long v1 = pre.c1, v2 = pre.c2, v3 = pre.c3;  // -2^61 for the first thread: empty
+        long long v1 = -kSat, v2 = -kSat, v3 = -kSat;  // empty
+        if constexpr (kCluster) {
+            cluster.sync();
+            for (int r = 0; r < rank; ++r) ftmap_apply(*cluster.map_shared_rank(&mine.map, r), v1, v2, v3);
+        }
+        ftmap_apply(pre, v1, v2, v3);
         bool bad = v3 >= kFixGuard;
         U96 sy;
         double wa = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
@@ -1017,7 +1151,9 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
             }
             bad = v3 >= kFixGuard;
         }
-        if (!__syncthreads_or(bad)) {
+        const bool cta_bad = __syncthreads_or(bad) != 0;
+        bool any_bad = cta_bad;
+        if (!cta_bad) {
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {  // lane-ordered tree (integers: exact)
                 const U96 oy = shfl_down_u96(sy, off);
@@ -1040,36 +1176,137 @@ __global__ void __launch_bounds__(1024) tandem3_cta_kernel(const double* __restr
                 wsum[2][warp] = w2;
                 wsum[3][warp] = w3;
             }
-            __syncthreads();
-            if (t == 0) {
-                U96 ty;
-                double sa = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+        }
+        __syncthreads();
+        if (t == 0) {
+            U96 ty;
+            double sum[4] = {0.0, 0.0, 0.0, 0.0};
+            if (!cta_bad) {
                 for (int w = 0; w < nwarp; ++w) {
                     add_u96(ty, wy[w]);
-                    sa += wsum[0][w];
-                    s1 += wsum[1][w];
-                    s2 += wsum[2][w];
-                    s3 += wsum[3][w];
-                }
-                out.y[item] = ty.to_double() / static_cast<double>(n_clients);
-                if (out.feat) {
-                    const double wl = static_cast<double>(w_len);
-                    double* fo = out.feat + item;
-                    const long long p = out.plane;
-                    fo[0] = lam;
-                    fo[p] = mu1;
-                    fo[2 * p] = mu2;
-                    fo[3 * p] = mu3;
-                    fo[4 * p] = sa / wl;
-                    fo[5 * p] = s1 / wl;
-                    fo[6 * p] = s2 / wl;
-                    fo[7 * p] = s3 / wl;
+                    for (int q = 0; q < 4; ++q) sum[q] += wsum[q][w];
                 }
             }
-            return;
+            mine.y = ty;
+            for (int q = 0; q < 4; ++q) mine.sum[q] = sum[q];
+            mine.bad = cta_bad ? 1 : 0;
+        }
+        if constexpr (kCluster) {
+            cluster.sync();
+            if (rank == 0)
+                for (int r = 1; r < ctas; ++r) any_bad = any_bad || *cluster.map_shared_rank(&mine.bad, r) != 0;
+        }
+        if (rank == 0 && t == 0 && !any_bad) {
+            U96 ty = mine.y;
+            double sum[4] = {mine.sum[0], mine.sum[1], mine.sum[2], mine.sum[3]};
+            for (int r = 1; r < ctas; ++r) {
+                add_u96(ty, *cluster.map_shared_rank(&mine.y, r));
+                for (int q = 0; q < 4; ++q) sum[q] += cluster.map_shared_rank(&mine.sum[0], r)[q];
+            }
+            out.y[item] = ty.to_double() / static_cast<double>(n_clients);
+            if (out.feat) {
+                const double wl = static_cast<double>(w_len);
+                double* fo = out.feat + item;
+                const long long p = out.plane;
+                fo[0] = lam;
+                fo[p] = mu1;
+                fo[2 * p] = mu2;
+                fo[3 * p] = mu3;
+                for (int q = 0; q < 4; ++q) fo[(4 + q) * p] = sum[q] / wl;
+            }
+        }
+        if constexpr (kCluster) cluster.sync();  // the first CTA has read the others' shared memory
+        if (!any_bad) return;
+    }
+    if (rank == 0 && warp == 0)
+        tandem_coop_fp64(item, lam, mu1, mu2, mu3, n_clients, window, row, rk, tab, out);
+}
+
+}  // namespace
+}  // namespace mrip
+
+namespace mrip {
+namespace {
+
+// Launch shape of a CTA-mapped queue kernel: CTAs per replication (a cluster),
+// threads per CTA, dynamic shared memory.
+struct CtaShape {
+    unsigned ctas = 1, threads = 32;
+    size_t smem = 0;
+    bool staged = false;
+};
+
+void cluster_config(long long n_items, const CtaShape& s, cudaStream_t st, cudaLaunchConfig_t* cfg,
+                    cudaLaunchAttribute* attr) {
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3(static_cast<unsigned>(n_items * s.ctas));
+    cfg->blockDim = dim3(s.threads);
+    cfg->dynamicSmemBytes = s.smem;
+    cfg->stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = s.ctas;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = s.ctas > 1 ? 1 : 0;
+}
+
+// About 4 clients per thread, 32 .. `most` threads per CTA.  Where one CTA would
+// leave its threads more than 4, the clients are split over the largest
+// cluster of 2 .. 8 CTAs per replication that still leaves every replication
+// running at once (the driver says how many clusters fit: on 152 SMs 36 of four
+// CTAs with an SM each, 15 of eight).  stage: the
+// variates of the first pass are kept in shared memory when they fit 96 KiB.
+template <class Kernel>
+mrip_status cta_shape(Kernel one, Kernel many, long long n_items, long long n_clients, int most, bool stage, CtaShape* out) {
+    auto shape_of = [&](unsigned ctas) {
+        CtaShape s;
+        s.ctas = ctas;
+        const long long part = (n_clients + ctas - 1) / ctas;
+        const long long threads = ((part + 3) / 4 + 31) / 32 * 32;
+        s.threads = static_cast<unsigned>(threads < 32 ? 32 : (threads > most ? most : threads));
+        const long long all = static_cast<long long>(s.threads) * ctas;
+        const size_t bytes = static_cast<size_t>(s.threads * ((n_clients + all - 1) / all)) * 2 * sizeof(long long);
+        s.staged = stage && bytes <= 96 * 1024;
+        s.smem = s.staged ? bytes : 0;
+        return s;
+    };
+    *out = shape_of(1);
+    const long long sms = sm_count();
+    const long long wanted = std::min<long long>(8, (n_clients + 4ll * most - 1) / (4ll * most));
+    for (unsigned ctas = static_cast<unsigned>(wanted); ctas > 1; --ctas) {
+        if (n_items * ctas > sms) continue;
+        const CtaShape s = shape_of(ctas);
+        if (s.smem > 40 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(many, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+            if (e != cudaSuccess) return cuda_status(e, "queues: shared memory attribute");
+        }
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        cluster_config(n_items, s, nullptr, &cfg, &attr);
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, many, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (fit >= n_items) {
+            *out = s;
+            return MRIP_OK;
         }
     }
-    if (warp == 0) tandem_coop_fp64(item, lam, mu1, mu2, mu3, n_clients, window, row, rk, tab, out);
+    if (out->smem > 40 * 1024) {  // plus ~3.3 KB of static shared memory
+        cudaError_t e = cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+        if (e != cudaSuccess) return cuda_status(e, "queues: shared memory attribute");
+    }
+    return MRIP_OK;
+}
+
+template <class... P, class... A>
+mrip_status launch_ctas(void (*kernel)(P...), long long n_items, const CtaShape& s, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config(n_items, s, st, &cfg, &attr);
+    return cuda_status(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...), "queues: launch");
 }
 
 }  // namespace
@@ -1102,20 +1339,12 @@ extern "C" mrip_status mrip_mm1_simulate(const double* d_dps, int32_t n_dp, int6
             d_dps, n_items, n_reps, rep0, n_clients, rk, tab, out);
     } else if (mapping == MRIP_MAP_CTA) {
         if (n_items > 0x7FFFFFFFll) return fail(MRIP_EINVAL, "mrip_mm1_simulate: too many replications for CTA");
-        // about 4 clients per thread, 32 .. 1024 threads; fixed-point variates
-        // staged in shared memory between the passes when they fit 96 KiB
-        long long threads = ((n_clients + 3) / 4 + 31) / 32 * 32;
-        threads = threads < 32 ? 32 : (threads > 1024 ? 1024 : threads);
-        const long long per_thread = (n_clients + threads - 1) / threads;
-        const size_t stage = static_cast<size_t>(threads * per_thread) * 2 * sizeof(long long);
-        const bool staged = stage <= 96 * 1024;  // plus ~3.3 KB of static shared memory
-        if (staged && stage > 40 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(mm1_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 96 * 1024);
-            if (e != cudaSuccess) return cuda_status(e, "mrip_mm1_simulate: shared memory attribute");
-        }
-        mm1_cta_kernel<<<static_cast<unsigned>(n_items), static_cast<unsigned>(threads), staged ? stage : 0, st>>>(
-            d_dps, n_reps, rep0, n_clients, staged, rk, tab, out);
+        CtaShape shape;
+        mrip_status cs = cta_shape(mm1_cta_kernel<false>, mm1_cta_kernel<true>, n_items, n_clients, 1024, true, &shape);
+        if (cs != MRIP_OK) return cs;
+        cs = launch_ctas(shape.ctas > 1 ? mm1_cta_kernel<true> : mm1_cta_kernel<false>, n_items, shape, st, d_dps, static_cast<long long>(n_reps),
+                         static_cast<long long>(rep0), static_cast<long long>(n_clients), shape.staged, rk, tab, out);
+        if (cs != MRIP_OK) return cs;
     } else if (mapping == MRIP_MAP_WARP_COOP) {
         const long long seg = (n_clients + 31) / 32;
         const size_t per_warp = static_cast<size_t>(seg) * 32 * 2 * sizeof(double);
@@ -1168,11 +1397,14 @@ extern "C" mrip_status mrip_tandem3_simulate(const double* d_dps, int32_t n_dp, 
             d_dps, n_items, n_reps, rep0, n_clients, window, tag, rk, tab, out);
     } else if (mapping == MRIP_MAP_CTA) {
         if (n_items > 0x7FFFFFFFll) return fail(MRIP_EINVAL, "mrip_tandem3_simulate: too many replications for CTA");
-        // about 4 clients per thread, 32 .. 1024 threads
-        long long threads = ((n_clients + 3) / 4 + 31) / 32 * 32;
-        threads = threads < 32 ? 32 : (threads > 1024 ? 1024 : threads);
-        tandem3_cta_kernel<<<static_cast<unsigned>(n_items), static_cast<unsigned>(threads), 0, st>>>(
-            d_dps, n_reps, rep0, n_clients, window, tag, rk, tab, out);
+        CtaShape shape;
+        mrip_status cs = cta_shape(tandem3_cta_kernel<false>, tandem3_cta_kernel<true>, n_items, n_clients,
+                                   n_items > sm_count() ? kTandemThreads / 2 : kTandemThreads, false, &shape);
+        if (cs != MRIP_OK) return cs;
+        cs = launch_ctas(shape.ctas > 1 ? tandem3_cta_kernel<true> : tandem3_cta_kernel<false>, n_items, shape, st, d_dps, static_cast<long long>(n_reps),
+                         static_cast<long long>(rep0), static_cast<long long>(n_clients),
+                         static_cast<long long>(window), tag, rk, tab, out);
+        if (cs != MRIP_OK) return cs;
     } else {
         return fail(MRIP_EINVAL, "mrip_tandem3_simulate: mapping must be THREAD, WARP_1LANE, WARP_COOP or CTA");
     }

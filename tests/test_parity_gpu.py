@@ -249,6 +249,27 @@ def test_tandem_workload_full(eng, torch_mod):
     np.testing.assert_allclose(gf, rf, rtol=REL)
 
 
+@pytest.mark.parametrize("n_items", [1, 5, 16, 40, 153])
+def test_cta_mapping_clusters(eng, torch_mod, n_items):
+    """CTA mapping of few replications: clusters of 2 to 8 CTAs (16 replications take 7), one CTA beyond, ragged
+    client counts, both rate ranges (the slowest saturate every client) and the FP64 fallback of a whole cluster."""
+    t = torch_mod
+    for n_clients, tdp, mdp in ((4099, [0.9, 1.0, 1.1, 1.2], [0.9, 1.0]), (20011, [0.02, 0.03, 0.021, 4.0], [0.02, 0.03]),
+                                (9001, [4.0, 1.0, 1.1, 1.2], [4.0, 1.0]), (9001, [0.01, 1.0, 1.0, 1.0], [0.01, 1.0])):
+        dps = np.array([tdp])
+        items = oracle.all_items(1, n_items)
+        y = t.empty(n_items, dtype=t.float64, device="cuda")
+        f = t.empty(8 * n_items, dtype=t.float64, device="cuda")
+        eng.mrip_tandem3_simulate(dev(t, dps), 0, n_items, n_clients, 100, 3, 0, eng.MRIP_MAP_CTA, y, f)
+        ry, rf = oracle.tandem3(dps, *items, n_clients, 3, window=100, threads=threads())
+        np.testing.assert_allclose(y.cpu().numpy(), ry, rtol=REL)
+        np.testing.assert_allclose(f.cpu().numpy().reshape(8, n_items).T, rf, rtol=REL)
+        out = [t.empty(n_items, dtype=t.float64, device="cuda") for _ in range(3)]
+        eng.mrip_mm1_simulate(dev(t, np.array([mdp])), n_items, n_clients, 3, eng.MRIP_MAP_CTA, *out)
+        for g, r in zip(out, oracle.mm1(np.array([mdp]), *items, n_clients, 3, threads=threads())):
+            np.testing.assert_allclose(g.cpu().numpy(), r, rtol=REL, atol=1e-300)
+
+
 # ------------------------------------------------------------------ forest fire
 @pytest.mark.parametrize("L", [32, 64, 128, 256, 512])
 @pytest.mark.parametrize("n_steps", [1, 64, 130])
