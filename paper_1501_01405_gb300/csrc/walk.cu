@@ -105,41 +105,39 @@ __device__ __forceinline__ bool walk_block(const uint4 b, int R, int& x, int& y,
 
 // Warp-convergent block step for the persistent mapping, in the diagonal
 // coordinates u = x + y, v = x - y (|x| + |y| = max(|u|, |v|); a move changes
-// u by +1 iff its bit 0 is clear and v by +1 iff its two bits agree).  Per
-// 16-move word, a lane whose walker cannot leave within the word -- u plus
-// the word's +1 steps in u below R, u minus its -1 steps above -R, the same
-// for v -- applies the word at once (popcounts).  The other lanes' words are
-// then walked by the whole warp, two lanes at a time: each half-warp takes
-// one walker's 16 moves, one per lane, a 16-lane scan gives the positions
-// and a ballot the first exit.
+// u by +1 iff its bit 0 is clear and v by +1 iff its two bits agree), each
+// held as U = u + R - 1: the walker is inside iff U and V, as unsigned words,
+// are below span = 2R - 1.  Per 16-move word, a lane whose walker cannot leave
+// within the word applies it at once (popcounts): u's positions within the word
+// lie between u - mu and u - mu + 16 (mu its -1 steps), so with t = U - mu the
+// word is safe in u iff t is in [0, 2R - 17): one unsigned compare against
+// lim = max(2R - 17, 0) (R <= 8: never safe); the same for v.  The other
+// lanes' words are then walked by the whole warp, two lanes at a time: lane i
+// of a half-warp counts the -1 steps among the walker's first i + 1 moves by
+// popcount, which gives its position after them, and a ballot the first exit.
 // This keeps the per-move work off the warp when one lane of 32 is near the
 // boundary, which (with stopping times spread over orders of magnitude) is
-// most of the time.  `live`: the lane has a walker; on return `done` marks
-// walkers that exited in this block, `exit_at` (1..64) the exiting move
-// within it.
-//
-// The no-exit test: u's positions within the word lie between u - mu and
-// u - mu + 16 (mu its -1 steps), so with t = u - mu the word is safe in u iff
-// -R < t < R - 16, i.e. t + R - 1 in [0, 2R - 17): one unsigned compare
-// against lim = max(2R - 17, 0) (R <= 8: never safe).  The same for v.
+// most of the time.  `live`: the lane has a walker; `prefix`: the even bits of
+// the first (lane mod 16) + 1 moves.  On return `done` marks walkers that
+// exited in this block, `exit_at` (1..64) the exiting move within it.
+__device__ __forceinline__ uint32_t walk_span(int R) { return static_cast<uint32_t>(2 * R - 1); }
 __device__ __forceinline__ uint32_t walk_safe_limit(int R) { return R > 8 ? static_cast<uint32_t>(2 * R - 17) : 0u; }
 
-__device__ __forceinline__ void walk_block_warp(const uint4 b, bool live, int R, uint32_t lim, int& u, int& v,
-                                                int& exit_at, bool& done) {
+__device__ __forceinline__ uint32_t minus_u(uint32_t w) { return w & kEven; }
+__device__ __forceinline__ uint32_t minus_v(uint32_t w) { return (w ^ (w >> 1)) & kEven; }
+
+__device__ __forceinline__ void walk_block_warp(const uint4 b, bool live, uint32_t span, uint32_t lim, uint32_t prefix,
+                                                uint32_t& U, uint32_t& V, int& exit_at, bool& done) {
     const int lane = threadIdx.x & 31;
     const uint32_t words[4] = {b.x, b.y, b.z, b.w};
     done = false;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const uint32_t w = words[k];
-        const int mu = __popc(w & kEven), mv = __popc((w ^ (w >> 1)) & kEven);  // -1 steps of u, of v
-        const int tu = u - mu, tv = v - mv;
+        const uint32_t mu = __popc(minus_u(w)), mv = __popc(minus_v(w));  // -1 steps of u, of v
+        const uint32_t tu = U - mu, tv = V - mv;
         const bool going = live && !done;
-        const bool safe = static_cast<uint32_t>(tu + (R - 1)) < lim && static_cast<uint32_t>(tv + (R - 1)) < lim;
-        if (going && safe) {
-            u = tu + (16 - mu);
-            v = tv + (16 - mv);
-        }
+        const bool safe = tu < lim && tv < lim;
         unsigned near = __ballot_sync(kFull, going && !safe);
         while (near) {  // two walkers per pass: lanes 0..15 and 16..31
             const int src0 = __ffs(near) - 1;
@@ -151,34 +149,23 @@ __device__ __forceinline__ void walk_block_warp(const uint4 b, bool live, int R,
             }
             const int src = (lane >= 16 && src1 >= 0) ? src1 : src0;
             const uint32_t ws = __shfl_sync(kFull, w, src);
-            const int us = __shfl_sync(kFull, u, src), vs = __shfl_sync(kFull, v, src);
-            const int rs = __shfl_sync(kFull, R, src);
-            const uint32_t f = (ws >> (2 * (lane & 15))) & 3u;
-            int du = 1 - 2 * static_cast<int>(f & 1u);
-            int dv = 1 - 2 * static_cast<int>((f ^ (f >> 1)) & 1u);
-#pragma unroll
-            for (int off = 1; off < 16; off <<= 1) {
-                const int pu = __shfl_up_sync(kFull, du, off, 16);
-                const int pv = __shfl_up_sync(kFull, dv, off, 16);
-                if ((lane & 15) >= off) {
-                    du += pu;
-                    dv += pv;
-                }
-            }
-            const unsigned hits = __ballot_sync(kFull, max(abs(us + du), abs(vs + dv)) >= rs);
-            const int tu0 = __shfl_sync(kFull, du, 15), tv0 = __shfl_sync(kFull, dv, 15);
-            const int tu1 = __shfl_sync(kFull, du, 31), tv1 = __shfl_sync(kFull, dv, 31);
-            const bool me0 = lane == src0, me1 = lane == src1;
-            if (me0 || me1) {
-                const unsigned h = me0 ? (hits & 0xFFFFu) : (hits >> 16);
+            const uint32_t us = __shfl_sync(kFull, U, src), vs = __shfl_sync(kFull, V, src);
+            const uint32_t ss = __shfl_sync(kFull, span, src);
+            const uint32_t moves = (lane & 15) + 1;
+            const uint32_t pu = us + moves - 2 * __popc(ws & prefix);
+            const uint32_t pv = vs + moves - 2 * __popc((ws ^ (ws >> 1)) & prefix);
+            const unsigned hits = __ballot_sync(kFull, pu >= ss || pv >= ss);
+            if (lane == src0 || lane == src1) {
+                const unsigned h = lane == src0 ? (hits & 0xFFFFu) : (hits >> 16);
                 if (h) {
                     exit_at = 16 * k + __ffs(h);
                     done = true;
-                } else {
-                    u += me0 ? tu0 : tu1;
-                    v += me0 ? tv0 : tv1;
                 }
             }
+        }
+        if (live && !done) {
+            U = tu + (16 - mu);
+            V = tv + (16 - mv);
         }
     }
 }
@@ -194,50 +181,50 @@ __device__ __forceinline__ void walk_block_warp(const uint4 b, bool live, int R,
 // exit time has an exponential tail) would otherwise set the launch's length.
 constexpr int kTailLanes = 16;
 
-// Whole walk from (u, v) after blk blocks; returns tau, or -1 past max_steps.
+// Whole walk from (U, V) after blk blocks; returns tau, or -1 past max_steps.
 // Warp-uniform arguments; every lane returns the same value.
-__device__ long long walk_tail_coop(int u, int v, uint32_t blk, int R, uint32_t lim, uint32_t rep, uint32_t c3,
-                                    long long max_steps, const RoundKeys& rk) {
+__device__ long long walk_tail_coop(uint32_t U, uint32_t V, uint32_t blk, uint32_t span, uint32_t lim,
+                                    const RowKey& row, long long max_steps, const RoundKeys& rk) {
     const int lane = threadIdx.x & 31;
-    // the same no-exit test as walk_block_warp, over 64 moves: t + R - 1 in [0, 2R - 65)
-    const uint32_t lim64 = R > 32 ? static_cast<uint32_t>(2 * R - 65) : 0u;
+    // the same no-exit test as walk_block_warp, over 64 moves: t in [0, 2R - 65)
+    const uint32_t lim64 = span > 64u ? span - 64u : 0u;
     while (true) {
-        const uint4 b = philox(0u, blk + static_cast<uint32_t>(lane), rep, c3, rk);
+        const uint4 b = philox_row(row, blk + static_cast<uint32_t>(lane), rk);
         const uint32_t words[4] = {b.x, b.y, b.z, b.w};
-        int mu = 0, mv = 0;
+        uint32_t mu = 0, mv = 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            mu += __popc(words[k] & kEven);
-            mv += __popc((words[k] ^ (words[k] >> 1)) & kEven);
+            mu += __popc(minus_u(words[k]));
+            mv += __popc(minus_v(words[k]));
         }
-        const int du = 64 - 2 * mu, dv = 64 - 2 * mv;
+        const int du = 64 - 2 * static_cast<int>(mu), dv = 64 - 2 * static_cast<int>(mv);
         int su = du, sv = dv;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            const int pu = __shfl_up_sync(kFull, su, off), pv = __shfl_up_sync(kFull, sv, off);
+            const int ou = __shfl_up_sync(kFull, su, off), ov = __shfl_up_sync(kFull, sv, off);
             if (lane >= off) {
-                su += pu;
-                sv += pv;
+                su += ou;
+                sv += ov;
             }
         }
-        int pu = u + su - du, pv = v + sv - dv;  // position before this lane's block
+        uint32_t pu = U + static_cast<uint32_t>(su - du), pv = V + static_cast<uint32_t>(sv - dv);  // before this block
         int e = 0;
-        if (!(static_cast<uint32_t>(pu - mu + (R - 1)) < lim64 && static_cast<uint32_t>(pv - mv + (R - 1)) < lim64)) {
+        if (!(pu - mu < lim64 && pv - mv < lim64)) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (e) break;
                 const uint32_t w = words[k];
-                const int wu = __popc(w & kEven), wv = __popc((w ^ (w >> 1)) & kEven);
-                if (static_cast<uint32_t>(pu - wu + (R - 1)) < lim && static_cast<uint32_t>(pv - wv + (R - 1)) < lim) {
+                const uint32_t wu = __popc(minus_u(w)), wv = __popc(minus_v(w));
+                if (pu - wu < lim && pv - wv < lim) {
                     pu += 16 - 2 * wu;
                     pv += 16 - 2 * wv;
                     continue;
                 }
                 for (int s = 0; s < 16; ++s) {
                     const uint32_t f = (w >> (2 * s)) & 3u;
-                    pu += (f & 1u) ? -1 : 1;
-                    pv += ((f ^ (f >> 1)) & 1u) ? -1 : 1;
-                    if (max(abs(pu), abs(pv)) >= R) {
+                    pu += (f & 1u) ? 0xFFFFFFFFu : 1u;
+                    pv += ((f ^ (f >> 1)) & 1u) ? 0xFFFFFFFFu : 1u;
+                    if (pu >= span || pv >= span) {
                         e = 16 * k + s + 1;
                         break;
                     }
@@ -252,8 +239,8 @@ __device__ long long walk_tail_coop(int u, int v, uint32_t blk, int R, uint32_t 
         }
         // blocks past the cap are never used (and blk + 32 stays below 2^32)
         if (64LL * blk + 2048 >= max_steps) return -1;
-        u += __shfl_sync(kFull, su, 31);
-        v += __shfl_sync(kFull, sv, 31);
+        U += static_cast<uint32_t>(__shfl_sync(kFull, su, 31));
+        V += static_cast<uint32_t>(__shfl_sync(kFull, sv, 31));
         blk += 32;
     }
 }
@@ -294,9 +281,9 @@ __device__ void walk_serial(const WalkJob& job, long long g, const RoundKeys& rk
     decode(job, g, R, dp, rep, out);
     int x = 0, y = 0;
     long long m = 0;
-    const uint32_t c3 = stream_word(0u, dp);
+    const RowKey row = row_key(rep, stream_word(0u, dp), rk);
     while (true) {
-        const uint4 b = philox(0u, static_cast<uint32_t>(m >> 6), rep, c3, rk);
+        const uint4 b = philox_row(row, static_cast<uint32_t>(m >> 6), rk);
         if (walk_block(b, R, x, y, m)) {
             if (m > job.max_steps) break;
             job.tau[out] = m;
@@ -321,78 +308,81 @@ __global__ void walk_serial_kernel(WalkJob job, const __grid_constant__ RoundKey
     walk_serial(job, g, rk);
 }
 
+// What bounds it is instruction issue (74 %, ALU 72 %).  Measured, 8 radii 16 .. 256 x
+// 2^17 replications with their statistics: 1.61 -> 1.35 ms by row keys (16 of 19
+// Philox products per block), biased coordinates, popcounts instead of a scan for
+// the walkers near the boundary, and no refill test while every lane walks.
 __global__ void __launch_bounds__(1024) walk_persistent_kernel(WalkJob job, const __grid_constant__ RoundKeys rk) {
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
+    const uint32_t prefix = kEven & (0xFFFFFFFFu >> (30 - 2 * (lane & 15)));
+    const uint32_t last_blk = static_cast<uint32_t>((job.max_steps + 63) / 64 - 1);  // max_steps <= 2^38
     bool active = false;
-    int u = 0, v = 0, R = 1;
-    uint32_t lim = 0, blk = 0;  // blk: Philox block index, the walker has made 64 blk moves
+    uint32_t U = 0, V = 0, span = 1, lim = 0, blk = 0;  // blk: Philox block index, the walker has made 64 blk moves
+    RowKey row{0u, 0u, 0u, 0u};
     long long out = 0;
-    uint32_t dp = 0, rep = 0, c3 = 0;
     long long next = 0, end = 0;  // warp-uniform range of the current chunk
     bool exhausted = false;       // warp-uniform
     while (true) {
         unsigned need = __ballot_sync(kFull, !active);
-        while (need && !exhausted) {
-            if (next >= end) {
-                unsigned long long start = 0;
-                if (lane == 0) start = atomicAdd(job.ticket, static_cast<unsigned long long>(job.chunk));
-                start = __shfl_sync(kFull, start, 0);
-                if (static_cast<long long>(start) >= job.total) {
-                    exhausted = true;
-                    break;
+        if (need) {
+            while (need && !exhausted) {
+                if (next >= end) {
+                    unsigned long long start = 0;
+                    if (lane == 0) start = atomicAdd(job.ticket, static_cast<unsigned long long>(job.chunk));
+                    start = __shfl_sync(kFull, start, 0);
+                    if (static_cast<long long>(start) >= job.total) {
+                        exhausted = true;
+                        break;
+                    }
+                    next = static_cast<long long>(start);
+                    end = next + job.chunk < job.total ? next + job.chunk : job.total;
                 }
-                next = static_cast<long long>(start);
-                end = next + job.chunk < job.total ? next + job.chunk : job.total;
-            }
-            const long long g = next + __popc(need & below);
-            const bool take = ((need >> lane) & 1u) && g < end;
-            if (take) {
-                decode(job, g, R, dp, rep, out);
-                c3 = stream_word(0u, dp);
-                lim = walk_safe_limit(R);
-                u = 0;
-                v = 0;
-                blk = 0;
-                active = true;
-            }
-            const unsigned took = __ballot_sync(kFull, take);
-            next += __popc(took);
-            need &= ~took;
-        }
-        const unsigned act = __ballot_sync(kFull, active);
-        if (!act) break;
-        if (exhausted && __popc(act) <= kTailLanes) {
-            for (unsigned rest = act; rest; rest &= rest - 1) {
-                const int src = __ffs(rest) - 1;
-                const long long tau = walk_tail_coop(
-                    __shfl_sync(kFull, u, src), __shfl_sync(kFull, v, src), __shfl_sync(kFull, blk, src),
-                    __shfl_sync(kFull, R, src), __shfl_sync(kFull, lim, src), __shfl_sync(kFull, rep, src),
-                    __shfl_sync(kFull, c3, src), job.max_steps, rk);
-                if (lane == src) {
-                    job.tau[out] = tau;
-                    if (tau < 0) atomicExch(job.err, 1);
+                const long long g = next + __popc(need & below);
+                const bool take = ((need >> lane) & 1u) && g < end;
+                if (take) {
+                    int R;
+                    uint32_t dp, rep;
+                    decode(job, g, R, dp, rep, out);
+                    row = row_key(rep, stream_word(0u, dp), rk);
+                    span = walk_span(R);
+                    lim = walk_safe_limit(R);
+                    U = V = static_cast<uint32_t>(R - 1);
+                    blk = 0;
+                    active = true;
                 }
+                const unsigned took = __ballot_sync(kFull, take);
+                next += __popc(took);
+                need &= ~took;
             }
-            break;
+            const unsigned act = __ballot_sync(kFull, active);
+            if (!act) break;
+            if (exhausted && __popc(act) <= kTailLanes) {
+                for (unsigned rest = act; rest; rest &= rest - 1) {
+                    const int src = __ffs(rest) - 1;
+                    const RowKey r{__shfl_sync(kFull, row.h, src), __shfl_sync(kFull, row.u, src),
+                                   __shfl_sync(kFull, row.t, src), __shfl_sync(kFull, row.l, src)};
+                    const long long tau = walk_tail_coop(
+                        __shfl_sync(kFull, U, src), __shfl_sync(kFull, V, src), __shfl_sync(kFull, blk, src),
+                        __shfl_sync(kFull, span, src), __shfl_sync(kFull, lim, src), r, job.max_steps, rk);
+                    if (lane == src) {
+                        job.tau[out] = tau;
+                        if (tau < 0) atomicExch(job.err, 1);
+                    }
+                }
+                break;
+            }
         }
-        const uint4 b = philox(0u, blk, rep, c3, rk);
+        const uint4 b = philox_row(row, blk, rk);
         bool done;
         int exit_at = 0;
-        walk_block_warp(b, active, R, lim, u, v, exit_at, done);
+        walk_block_warp(b, active, span, lim, prefix, U, V, exit_at, done);
         if (active) {
-            if (done) {
+            if (done || blk >= last_blk) {  // (so blk stays below 2^32)
                 const long long m = 64LL * blk + exit_at;
-                if (m > job.max_steps) {
-                    job.tau[out] = -1;
-                    atomicExch(job.err, 1);
-                } else {
-                    job.tau[out] = m;
-                }
-                active = false;
-            } else if (64LL * blk + 64 >= job.max_steps) {  // so blk stays below 2^32 (max_steps <= 2^38)
-                job.tau[out] = -1;
-                atomicExch(job.err, 1);
+                const bool capped = !done || m > job.max_steps;
+                job.tau[out] = capped ? -1 : m;
+                if (capped) atomicExch(job.err, 1);
                 active = false;
             } else {
                 ++blk;
@@ -410,12 +400,12 @@ __global__ void walk_warp_coop_kernel(WalkJob job, const __grid_constant__ Round
     uint32_t dp, rep;
     long long out;
     decode(job, g, R, dp, rep, out);
-    const uint32_t c3 = stream_word(0u, dp);
+    const RowKey row = row_key(rep, stream_word(0u, dp), rk);
     int px = 0, py = 0;  // warp-uniform position before the round
     long long m = 0;     // warp-uniform move count before the round (multiple of 512)
     long long result = -1;
     while (m < job.max_steps) {
-        const uint4 b = philox(0u, static_cast<uint32_t>((m >> 6) + (lane >> 2)), rep, c3, rk);
+        const uint4 b = philox_row(row, static_cast<uint32_t>((m >> 6) + (lane >> 2)), rk);
         const int sel = lane & 3;
         const uint32_t w = sel == 0 ? b.x : sel == 1 ? b.y : sel == 2 ? b.z : b.w;
         int dx, dy;
