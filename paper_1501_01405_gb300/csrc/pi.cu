@@ -2,11 +2,11 @@
 // square counted when they fall in the quarter disc.  Draw k of replication
 // `rep` uses words 2(k mod 2), 2(k mod 2)+1 of Philox block (c0 = 0,
 // c1 = k div 2) as integer coordinates x, y in [0, 2^32); it is inside iff
-// x^2 + y^2 < 2^64, tested exactly as x^2 <= (2^64 - 1) - y^2.
+// x^2 + y^2 < 2^64, tested exactly as the absence of a carry out of 64 bits.
 //
-// Draws are independent, so a replication is split over CTAs of 2^16 draws
-// (a 10^7-draw replication spreads over ~150 CTAs, i.e. the whole GPU even
-// for one replication); each CTA reduces its count (warp reduction, then
+// Draws are independent, so a replication is split over CTAs of up to 2^16
+// draws, fewer (down to 2^12) while that leaves fewer than eight CTAs per SM: a
+// 10^7-draw replication fills the whole GPU by itself; each CTA reduces its count (warp reduction, then
 // shared memory) and adds it to the replication's counter with one 64-bit
 // atomic -- integer addition, so the result does not depend on the order.
 #include "common.cuh"
@@ -15,35 +15,52 @@ namespace mrip {
 namespace {
 
 constexpr int kPiThreads = 256;
-constexpr long long kPiChunk = 1LL << 16;  // draws per CTA (even)
+constexpr long long kPiChunk = 1LL << 16, kPiLeast = 1LL << 12;  // most and least draws per CTA (even)
 
-__device__ __forceinline__ uint32_t inside(uint32_t x, uint32_t y) {
-    const unsigned long long x2 = static_cast<unsigned long long>(x) * x;
-    const unsigned long long y2 = static_cast<unsigned long long>(y) * y;
-    return x2 <= ~y2 ? 1u : 0u;
+// outside += 1 if x^2 + y^2 >= 2^64: the carry out of the 64-bit sum, taken by
+// the multiply that adds y^2 to x^2 (two multiplies and an add; comparing x^2
+// with the complement of y^2 took four instructions more).
+__device__ __forceinline__ void add_outside(uint32_t x, uint32_t y, uint32_t& outside) {
+    uint32_t hi, lo;
+    [[maybe_unused]] uint32_t s0, s1;
+    mul_wide_u32(x, x, hi, lo);
+    asm("mad.lo.cc.u32 %0, %3, %3, %4;\n\tmadc.hi.cc.u32 %1, %3, %3, %5;\n\taddc.u32 %2, %2, 0;"
+        : "=r"(s0), "=r"(s1), "+r"(outside)
+        : "r"(y), "r"(lo), "r"(hi));
 }
 
-__global__ void __launch_bounds__(kPiThreads) pi_kernel(long long n_draws, long long chunks, long long rep0,
+// What bounds it is the FMA-heavy pipe (16 widening multiplies of Philox per
+// block of two draws and 4 of the squares, 4.2 cycles each: 84 of the 87 cycles a
+// warp takes).  Measured, 64 replications x 10^7 draws: 0.921 -> 0.700 ms (row keys
+// alone 0.809); one replication 29.0 -> 17.7 us,
+// 3 x 200,001 draws 23 -> 9.8 us.  The test in FP32 with an exact second look needs two multiplies less but four conversions more: 0.717 ms.
+__global__ void __launch_bounds__(kPiThreads) pi_kernel(long long n_draws, long long chunk, long long chunks, long long rep0,
                                                         const __grid_constant__ RoundKeys rk,
                                                         unsigned long long* __restrict__ hits) {
     __shared__ uint32_t part[kPiThreads / 32];
     const long long rep = blockIdx.x / chunks;
-    const long long start = (blockIdx.x - rep * chunks) * kPiChunk;
-    const long long end = min(start + kPiChunk, n_draws);
-    const uint32_t c3 = stream_word(0u, 0u);
-    uint32_t cnt = 0;
-    for (long long b = start / 2 + threadIdx.x; 2 * b < end; b += kPiThreads) {
-        const uint4 w = philox(0u, static_cast<uint32_t>(b), static_cast<uint32_t>(rep0 + rep), c3, rk);
-        cnt += inside(w.x, w.y);
-        if (2 * b + 1 < end) cnt += inside(w.z, w.w);
+    const long long start = (blockIdx.x - rep * chunks) * chunk;
+    const uint32_t draws = static_cast<uint32_t>(min(chunk, n_draws - start));
+    const RowKey row = row_key(static_cast<uint32_t>(rep0 + rep), stream_word(0u, 0u), rk);
+    const uint32_t first = static_cast<uint32_t>(start / 2), pairs = draws / 2;  // whole blocks
+    uint32_t outside = 0;
+#pragma unroll 2
+    for (uint32_t b = threadIdx.x; b < pairs; b += kPiThreads) {
+        const uint4 w = philox_row(row, first + b, rk);
+        add_outside(w.x, w.y, outside);
+        add_outside(w.z, w.w, outside);
     }
-    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = cnt;
+    if ((draws & 1u) && threadIdx.x == 0) {  // the last draw of an odd number
+        const uint4 w = philox_row(row, first + pairs, rk);
+        add_outside(w.x, w.y, outside);
+    }
+    outside = __reduce_add_sync(0xFFFFFFFFu, outside);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = outside;
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long tot = 0;
+        uint32_t tot = 0;
         for (int i = 0; i < kPiThreads / 32; ++i) tot += part[i];
-        atomicAdd(hits + rep, tot);
+        atomicAdd(hits + rep, static_cast<unsigned long long>(draws - tot));
     }
 }
 
@@ -63,9 +80,12 @@ extern "C" mrip_status mrip_pi_simulate(int64_t rep0, int64_t n_reps, int64_t n_
     cudaError_t e = cudaMemsetAsync(d_hits, 0, static_cast<size_t>(n_reps) * sizeof(int64_t), st);
     if (e != cudaSuccess) return cuda_status(e, "mrip_pi_simulate: clear");
     if (n_draws == 0) return MRIP_OK;
-    const long long chunks = (n_draws + kPiChunk - 1) / kPiChunk;
+    long long chunk = kPiChunk;
+    auto ctas = [&]() { return (n_draws + chunk - 1) / chunk; };
+    while (chunk > kPiLeast && ctas() * n_reps < 8ll * sm_count()) chunk /= 2;
+    const long long chunks = ctas();
     if (chunks * n_reps > 0x7FFFFFFFll) return fail(MRIP_EINVAL, "mrip_pi_simulate: too many draws in total");
     pi_kernel<<<static_cast<unsigned>(chunks * n_reps), kPiThreads, 0, st>>>(
-        n_draws, chunks, rep0, expand_key(seed), reinterpret_cast<unsigned long long*>(d_hits));
+        n_draws, chunk, chunks, rep0, expand_key(seed), reinterpret_cast<unsigned long long*>(d_hits));
     return launch_status("mrip_pi_simulate");
 }
