@@ -76,6 +76,27 @@ def test_forward(env, d_in, n):
     np.testing.assert_allclose(got, ref, rtol=2e-2, atol=2e-3 * np.abs(ref).max())
 
 
+@pytest.mark.parametrize("d_in", [1, 5, 8])
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 70001])
+def test_forward_tiles(env, d_in, n):
+    """Edges of the 128-sample tiles and more tiles than resident CTAs: a sample's
+    output does not depend on where it stands, so copies of 61 rows in any
+    order give the 61 outputs bit for bit (61 rows against the oracle)."""
+    eng, torch = env
+    theta = _seeded_net(d_in, 3)
+    X = omlp.f32(mrip_inputs.random_matrix((61, d_in), 4))
+
+    def run(rows):
+        out = torch.full((len(rows),), np.nan, dtype=torch.float32, device="cuda")
+        eng.mrip_mlp_forward(f32dev(torch, theta), d_in, f32dev(torch, X[rows].T.copy()), out)
+        return out.cpu().numpy()
+    base = run(np.arange(61))
+    ref, _ = omlp.forward(theta, X, d_in)
+    assert np.linalg.norm(base - ref) / np.linalg.norm(ref) < 1e-3
+    rows = np.random.default_rng(n).integers(0, 61, n)
+    assert np.array_equal(run(rows), base[rows])
+
+
 @pytest.mark.parametrize("d_in,n,B", [(8, 3000, 1024), (6, 500, 500), (8, 100, 33)])
 def test_loss_and_gradient(env, d_in, n, B):
     eng, torch = env
