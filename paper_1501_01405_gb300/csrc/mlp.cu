@@ -22,7 +22,9 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <numeric>
 #include <vector>
 
@@ -47,9 +49,6 @@ __host__ __device__ constexpr long long off_b3(int d) { return off_w3(d) + H; }
 __host__ __device__ constexpr long long n_params(int d) { return off_b3(d) + 1; }
 
 __device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-
-// W1 element (unit u, input k); W1 is stored row-major [u][k].
-__device__ __forceinline__ float theta_w1(const float* theta, int d_in, int u, int k) { return theta[u * d_in + k]; }
 
 // He-uniform weights from stream tag 3: element e of (W1, W2, W3) reads words
 // 2(e mod 2), 2(e mod 2)+1 of block (c0 = e div 2, c1 = 0, rep 0, dp 0).
@@ -405,59 +404,154 @@ struct TrainArgs {
 };
 
 // ---------------------------------------------------------------------------
-// Training with the four 64-wide contractions on the tensor cores (tcgen05,
-// FP32 accumulators in tensor memory).  A cluster of kTcCluster CTAs of 512
-// threads holds the FP32 parameters in every CTA's shared memory; per step
-// each CTA takes 1/kTcCluster of the minibatch in tiles of 128 samples
-// (sample m = TMEM lane m, its 64 columns split over 4 threads):
+// Training with the five contractions of a step on the tensor cores (tcgen05,
+// FP32 accumulators in tensor memory).  A cluster of kTcCluster CTAs keeps the
+// BF16 operands of the weights in every CTA's shared memory and the FP32
+// parameters with Adam's moments in registers, spread over the cluster; per
+// step each CTA takes 1/kTcCluster of the minibatch in tiles of 128 samples
+// (sample m = TMEM lane m, its 64 columns split over 4 of the 512 workers):
 //   Z1  = X~ W1~^T        (M 128, N 64, K 16: the d_in features, zero-padded)
 //   Z2  = H1~ W2~^T       (K 64)
-//   dH1 = dZ2~ W2~        (K 64, B = W2~ transposed)
-//   dW2 = dZ2~^T H1~      (M 128 with rows 64..127 zero, K = the 128 samples)
-//   dW1 = dZ1~^T X~       (M 128 with rows 64..127 zero, N 16, K = the 128 samples)
-// Each thread turns its 16 columns of a row of Z1 / Z2 / dH1 into
-// activations, residual and deltas (FP32, rounded to BF16 where the next
-// contraction reads them) and writes them in the operands' core-matrix
-// layouts (16-byte stores where a row's 8 columns are contiguous); the bias
-// and W3 gradients are FP32 column sums over the tile in a fixed order
-// (chunks of 16 samples, then the chunks in order).  After a cluster barrier CTA r owns the r-th slice of the
-// parameters: it adds that slice of every CTA's gradient in rank order over
-// distributed shared memory, applies Adam and writes the new values into
-// every CTA's copy; a second barrier ends the step.  Same arithmetic as
-// mlp_step (BF16 operands, FP32 sums; only the order of the sums differs).
-// Every MMA completion is awaited with an
-// iteration limit; on a timeout the CTA stops issuing MMAs, runs on to the
-// same barriers (so no peer waits forever) and reports it in *err.
+//   dH1 = dZ2~ W2~        (K 64, W2~ read MN-major)
+//   dW2 = dZ2~^T H1~      (K = the 128 samples, both read MN-major)
+//   dW1 = dZ1~^T X~       (N 16, likewise)
+// Activations and deltas are written once, as rows (16-byte stores), and read
+// by the tensor cores along either index; the last two products are taken at
+// M = 128, whose rows 64.. read neighbouring bytes and are not used.  Each
+// worker turns its 16 columns of a row of Z1 / Z2 / dH1 into activations,
+// residual and deltas (FP32, rounded to BF16 where the next contraction reads
+// them; a unit counts as on where its BF16 activation is not zero, so for
+// pre-activations above 2^-134).  The bias and W3 gradients are FP32 column
+// sums over the tile in a fixed order (chunks of 16 samples, then the chunks
+// in order), taken while the products run.  Four more warps: one issues the
+// products, one adds the output deltas and the squared residuals one after
+// the other, two fetch samples.
+//
+// CTA r owns hidden units 8r .. 8r + 7 of both layers: a CTA's gradient lies in
+// shared memory as one block per owner and is sent to the owners' shared memory
+// as bulk copies that complete on the owner's mbarrier; a thread of the owner adds its
+// one word over the 8 CTAs in rank order, applies Adam and writes the new value
+// as the operand it is used as, again into one block, which is sent to the other
+// CTAs in the same way.  No cluster barrier is needed in a step: an owner sends
+// the weights of a step only once every CTA's gradient has arrived, so nothing of
+// the old weights is still read, and a CTA starts the next step only once every
+// owner's weights have arrived, so nothing of its gradient or of the owners'
+// receive buffers is still read.
+//
+// What bounds it: a step is a chain of latencies on 8 SMs (three products, one
+// after the other, and two exchanges in the cluster; the gradient of a step
+// needs the weights of the one before, and the order of additions is kept, so
+// more SMs would not shorten it), so everything that can leaves the chain: the
+// samples are copied behind the products (loads into registers were waited for
+// at the next loop), the sums run behind the products, the next tile's operand
+// is built while the weights are under way.  The kernel before, at 13.0 us a
+// step, held two transposed operand copies (4,000 of 24,000 cycles), additions of
+// the gradient in shared memory with 32-way bank conflicts (2,600), rounding of
+// all weights by every CTA (1,850), remote loads and stores of single words and
+// two cluster barriers (6,500), the samples' loads (2,500) and a serial sum
+// (1,900).  Measured, 94,208 samples of 8 inputs in minibatches of 1,024 and 12,288
+// validation samples, one epoch: 1.21 -> 0.63 ms (6.5 us a step).
+//
+// Every wait has an iteration limit; on a timeout a thread stops waiting, no
+// more products are issued, everything runs on to the same barriers (so no peer
+// waits forever), waits once more, with the limit, for what is in flight, and
+// *err reports it.
 // ---------------------------------------------------------------------------
 constexpr int kTcCluster = 8;
-constexpr int kTcThreads = 512;  // 4 threads per sample row, 16 columns each
+constexpr int kTcWorkers = 512;              // 4 threads per sample row, 16 columns each
+constexpr int kTcThreads = kTcWorkers + 128;  // and the issuing, the adding and two fetching warps
 constexpr int kTcRows = 128;
-constexpr int kTcChunks = kTcThreads / H;  // row chunks of the column sums
+constexpr int kTcChunks = kTcWorkers / H;    // row chunks of the column sums
 constexpr int kTcWait = 1 << 22;
+constexpr int kTcUnits = H / kTcCluster;     // hidden units per owner
+constexpr int kRowF = H + 4, kRowB = H + 8;  // row strides of the FP32 and BF16 tiles: 16-byte stores of
+                                             // eight neighbouring rows fall on different banks
+static_assert(kTcUnits == 8, "an owner's rows are one group of core matrices");
+
+// An owner's part of the weights, as it is used.
+struct TcWeights {
+    unsigned char w2[kTcUnits * H * 2];   // W2~ [v][u], one row group of core matrices
+    unsigned char w1[kTcUnits * 16 * 2];  // W1~ [u][k], k padded to 16
+    float b1[kTcUnits], b2[kTcUnits];
+    float w3[kTcUnits];                   // rounded to BF16
+    float b3;                             // (owner 0)
+    float pad[7];
+};
+constexpr uint32_t kWStride = sizeof(TcWeights);
+static_assert(kWStride == 1408 && kWStride % 128 == 0, "row groups of the weight operands lie kWStride apart");
+
+// An owner's part of the gradient: W2 as 8 rows of 65 words, W1 as 8 rows of
+// d + 1 (odd strides: the rows of a warp's lanes fall on different banks, also
+// across owners, kGradWords being 8 modulo 32), b1, b2, W3, then (owner 0) b3
+// and the sum of squared residuals.
+constexpr int kGradWords = 648;
+__host__ __device__ constexpr int grad_w1() { return kTcUnits * (H + 1); }
+__host__ __device__ constexpr int grad_b1(int d) { return grad_w1() + kTcUnits * (d + 1); }
+__host__ __device__ constexpr int grad_b3(int d) { return grad_b1(d) + 3 * kTcUnits; }
+__host__ __device__ constexpr int grad_loss(int d) { return grad_b3(d) + 1; }
+static_assert(grad_loss(kMaxIn) < kGradWords && grad_loss(kMaxIn) <= kTcThreads, "a block, and the threads, hold its words");
 
 struct TcSmem {
-    alignas(1024) unsigned char a1[kTcRows * 16 * 2];      // X~ tile, K = 16
-    alignas(1024) unsigned char w1b[H * 16 * 2];           // W1~ as B, K = 16
-    alignas(1024) unsigned char a2[kTcRows * H * 2];       // H1~ rows, K = 64
-    alignas(1024) unsigned char w2b[H * H * 2];            // W2~ [v][u] as B
-    alignas(1024) unsigned char w2tb[H * H * 2];           // W2~ [u][v] as B
-    alignas(1024) unsigned char h1tt[H * kTcRows * 2];     // H1~ transposed [u][m], K = 128
-    alignas(1024) unsigned char a3[kTcRows * H * 2];       // dZ2~ rows, K = 64
-    alignas(1024) unsigned char dz2tt[kTcRows * kTcRows * 2];  // dZ2~, then dZ1~, transposed [v][m]; rows 64.. zero
-    alignas(1024) unsigned char xtt[16 * kTcRows * 2];     // X~ transposed [k][m], K = 128; rows d_in.. zero
-    float f32[kTcRows][H + 1];                             // dZ2, then dZ1 (FP32)
-    __nv_bfloat16 h2t[kTcRows][H + 2];                     // H2~ rows (for dW3)
+    alignas(1024) unsigned char a1[kTcRows * 16 * 2];      // X~ rows, 16 columns
+    alignas(1024) unsigned char a2[kTcRows * H * 2];       // H1~ rows
+    alignas(1024) unsigned char a3[kTcRows * H * 2];       // dZ2~ rows
+    alignas(1024) unsigned char a4[kTcRows * H * 2];       // dZ1~ rows
+    alignas(128) TcWeights w[kTcCluster];
+    alignas(16) float dz1[kTcRows][kRowF];                 // dZ1, FP32
+    alignas(16) __nv_bfloat16 h2t[kTcRows][kRowB];         // H2~ rows (for dW3)
+    alignas(16) float part[kTcCluster][kGradWords];        // this CTA's gradient, by owner
+    alignas(16) float recv[kTcCluster][kGradWords];        // this owner's gradient, by CTA
     float ypart[4][kTcRows];                               // output partials per column block
     float colpart[3][kTcChunks][H];                        // column sums per row chunk
-    float dy[kTcRows], r2[kTcRows];
-    float w3[H], b1[H], b2[H];
-    float b3;
-    uint64_t bar;
+    alignas(16) float dy[kTcRows];
+    alignas(16) float r2[kTcRows];
+    float vsum;                                            // validation: this CTA's squared residuals
+    uint64_t bar, bar_w2, bar_grad, bar_weights;
+    float rows[4][kMaxIn + 1][kTcRows];                    // samples fetched: features, target; two tiles of
+                                                           // a step and two of the validation samples
+    float bc[2][2];                                        // Adam's bias corrections of this step and the next
     uint32_t tmem;
 };
+static_assert(sizeof(TcSmem) <= 227 * 1024, "fits a CTA's shared memory");
 
-__device__ __forceinline__ void put_bf16(unsigned char* tile, uint32_t off, float v) {
-    *reinterpret_cast<__nv_bfloat16*>(tile + off) = __float2bfloat16_rn(v);
+// What word e of owner r's gradient block belongs to: the parameter's index (-1:
+// padding), the byte it is used at within TcWeights and how.
+enum ParamUse { kUseBf16, kUseRounded, kUseFp32 };
+__device__ __forceinline__ int owned_param(int e, int r, int d, uint32_t& at, ParamUse& use) {
+    at = 0;
+    use = kUseBf16;
+    if (e < grad_w1()) {
+        const int row = e / (H + 1), u = e % (H + 1);
+        if (u == H) return -1;
+        at = static_cast<uint32_t>(offsetof(TcWeights, w2)) + tc::core_offset(row, u, H);
+        return static_cast<int>(off_w2(d)) + (kTcUnits * r + row) * H + u;
+    }
+    if (e < grad_b1(d)) {
+        const int row = (e - grad_w1()) / (d + 1), k = (e - grad_w1()) % (d + 1);
+        if (k == d) return -1;
+        at = static_cast<uint32_t>(offsetof(TcWeights, w1)) + tc::core_offset(row, k, 16);
+        return (kTcUnits * r + row) * d + k;
+    }
+    use = kUseFp32;
+    if (e < grad_b3(d)) {
+        const int i = e - grad_b1(d), unit = i % kTcUnits;
+        const int which = i / kTcUnits;
+        at = static_cast<uint32_t>(which == 0 ? offsetof(TcWeights, b1) : which == 1 ? offsetof(TcWeights, b2)
+                                                                                     : offsetof(TcWeights, w3)) +
+             4u * unit;
+        if (which == 2) use = kUseRounded;
+        return static_cast<int>(which == 0 ? off_b1(d) : which == 1 ? off_b2(d) : off_w3(d)) + kTcUnits * r + unit;
+    }
+    at = static_cast<uint32_t>(offsetof(TcWeights, b3));
+    return e == grad_b3(d) && r == 0 ? static_cast<int>(off_b3(d)) : -1;
+}
+
+__device__ __forceinline__ void put_weight(TcWeights& w, uint32_t at, ParamUse use, float v) {
+    unsigned char* dst = reinterpret_cast<unsigned char*>(&w) + at;
+    if (use == kUseBf16)
+        *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(v);
+    else
+        *reinterpret_cast<float*>(dst) = use == kUseRounded ? bf(v) : v;
 }
 
 // Eight FP32 values rounded to BF16 (nearest even), the first at the lowest
@@ -479,63 +573,75 @@ __global__ void __cluster_dims__(kTcCluster, 1, 1) __launch_bounds__(kTcThreads,
     extern __shared__ __align__(1024) unsigned char tc_raw[];
     TcSmem& S = *reinterpret_cast<TcSmem*>(tc_raw);
     const int d_in = ta.d_in;
-    const int P = static_cast<int>(n_params(d_in));
-    const int P4 = (P + 1 + 3) & ~3;
-    float* th = reinterpret_cast<float*>(tc_raw + sizeof(TcSmem));
-    float* part = th + P4;
-    const int slice = (P + kTcCluster - 1) / kTcCluster;
-    float* mom = part + P4;
-    float* vel = mom + slice;
     const int rank = static_cast<int>(cluster.block_rank());
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int quarter = warp & 3, cb = warp >> 2;  // TMEM lane quarter, column block
-    const int m = 32 * quarter + lane;              // this thread's sample row / TMEM lane
+    const int t = threadIdx.x, lane = t & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, t >> 5, 0);  // (known to be the same in a warp)
+    const bool worker = t < kTcWorkers;
+    const bool issuer = warp == kTcWorkers / 32;    // the warp that issues products
+    const bool sends = warp < kTcCluster && warp != rank && lane == 0;  // blocks to CTA `warp` (a warp each: 60 cycles)
+    const bool fetcher = warp >= kTcWorkers / 32 + 2;  // the two warps that fetch samples
+    const bool summer = warp == kTcWorkers / 32 + 1 && lane < 2;  // lane 0 adds the outputs' deltas, 1 the squared residuals
+    const int quarter = warp & 3, cb = warp >> 2;   // TMEM lane quarter, column block
+    const int m = 32 * quarter + lane;              // this worker's sample row / TMEM lane
     const int c0 = 16 * cb;                         // its 16 columns
-    const int p_lo = rank * slice, p_hi = min(P, p_lo + slice);
     constexpr uint32_t kIdesc = tc::idesc_bf16(kTcRows, H);
-    constexpr uint32_t kIdescW1 = tc::idesc_bf16(kTcRows, 16);
+    constexpr uint32_t kIdescH1 = tc::idesc_bf16(kTcRows, H, false, true);
+    constexpr uint32_t kIdescW2 = tc::idesc_bf16(kTcRows, H, true, true);
+    constexpr uint32_t kIdescW1 = tc::idesc_bf16(kTcRows, 16, true, true);
     // (debug build: the layout must fit the launch's shared memory; every CTA
-    // of the cluster computes the same sizes, so all leave together, before
-    // any cluster barrier or tensor-memory allocation)
-    if (!MRIP_CHECK(sizeof(TcSmem) + (2ull * P4 + 2ull * slice) * sizeof(float) <= dynamic_smem_bytes(), 402, P)) {
+    // of the cluster leaves together, before any cluster barrier or
+    // tensor-memory allocation)
+    if (!MRIP_CHECK(sizeof(TcSmem) <= dynamic_smem_bytes(), 402, sizeof(TcSmem))) {
         if (t == 0 && rank == 0) atomicExch(err, 1);
         return;
     }
 
     if (warp == 0) tc::tmem_alloc(&S.tmem, 256);
-    if (t == 0) tc::mbar_init(&S.bar);
-    const float* th_src = ta.theta_in ? ta.theta_in : ta.theta;
-    for (int i = t; i < P; i += kTcThreads) th[i] = th_src[i];
-    for (int i = t; i < slice; i += kTcThreads) {
-        const int p = p_lo + i;
-        mom[i] = (ta.m_in && p < P) ? ta.m_in[p] : 0.0f;
-        vel[i] = (ta.v_in && p < P) ? ta.v_in[p] : 0.0f;
+    if (t == 0) {
+        tc::mbar_init(&S.bar);
+        tc::mbar_init(&S.bar_w2);
+        tc::mbar_init(&S.bar_grad);
+        tc::mbar_init(&S.bar_weights);
     }
-    for (int i = t; i < kTcRows * kTcRows * 2 / 16; i += kTcThreads)
-        reinterpret_cast<uint4*>(S.dz2tt)[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = t; i < kTcRows * 16 * 2 / 16; i += kTcThreads) {
+    for (int i = t; i < kTcRows * 16 * 2 / 16; i += kTcThreads)
         reinterpret_cast<uint4*>(S.a1)[i] = make_uint4(0u, 0u, 0u, 0u);
-        reinterpret_cast<uint4*>(S.xtt)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = t; i < static_cast<int>(sizeof(S.w) / 16); i += kTcThreads)
+        reinterpret_cast<uint4*>(S.w)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    const float* th_src = ta.theta_in ? ta.theta_in : ta.theta;
+    for (int i = t; i < kTcCluster * grad_loss(d_in); i += kTcThreads) {
+        uint32_t at;
+        ParamUse use;
+        const int r = i / grad_loss(d_in);
+        const int p = owned_param(i - r * grad_loss(d_in), r, d_in, at, use);
+        if (p >= 0) put_weight(S.w[r], at, use, th_src[p]);
     }
+    // this thread's parameter: word t of the owner's block
+    uint32_t at = 0;
+    ParamUse use = kUseFp32;
+    const int par = t <= grad_b3(d_in) ? owned_param(t, rank, d_in, at, use) : -1;
+    float th = par >= 0 ? th_src[par] : 0.0f;
+    float mom = (ta.m_in && par >= 0) ? ta.m_in[par] : 0.0f;
+    float vel = (ta.v_in && par >= 0) ? ta.v_in[par] : 0.0f;
+    tc::fence_smem_async();
     tc::fence_before_sync();
     cluster.sync();
     tc::fence_after_sync();
     const uint32_t tm = S.tmem;
     const uint32_t lane_base = static_cast<uint32_t>(32 * quarter) << 16;
-    uint32_t phase = 0;
-    bool ok = true;
+    uint32_t phase = 0, phase_w2 = 0, phase_grad = 0, phase_weights = 0;
+    bool ok = true;  // of this thread
 
-    // one MMA group's completion: every thread polls; ok stays CTA-uniform
-    auto wait_mma = [&]() {
-        bool mine = ok ? tc::mbar_wait(&S.bar, phase, kTcWait) : false;
-        phase ^= 1u;
-        tc::fence_before_sync();
-        const bool all = __syncthreads_and(mine) != 0;
-        tc::fence_after_sync();
-        if (ok && !all) {
+    auto wait_on = [&](uint64_t* bar, uint32_t& ph) {
+        if (ok && !tc::mbar_wait(bar, ph, kTcWait)) {
             ok = false;
-            if (t == 0) atomicExch(err, 1);
+            atomicExch(err, 1);
         }
+        ph ^= 1u;
+    };
+    auto wait_mma = [&]() {
+        wait_on(&S.bar, phase);
+        tc::fence_after_sync();
     };
     auto sync_for_mma = [&]() {
         tc::fence_smem_async();
@@ -543,327 +649,492 @@ __global__ void __cluster_dims__(kTcCluster, 1, 1) __launch_bounds__(kTcThreads,
         __syncthreads();
         tc::fence_after_sync();
     };
-    // BF16 operands (and FP32 biases) of the current parameters th; every
-    // thread packs 8 consecutive K elements of one operand row into one
-    // 16-byte store (a core-matrix row)
-    auto stage_weights = [&]() {
-        if (t < 2 * H) {  // W1~ as B: row u, K = the 16 (zero-padded) inputs
-            const int u = t >> 1, k0 = 8 * (t & 1);
-            float w[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) w[q] = k0 + q < d_in ? theta_w1(th, d_in, u, k0 + q) : 0.0f;
-            *reinterpret_cast<uint4*>(S.w1b + tc::core_offset(u, k0, 16)) = pack_bf16x8(w);
-        }
-        {   // W2~ [v][u] as B of Z2 (K = u): row v, columns 8j .. 8j + 7
-            const int v = t >> 3, j = t & 7;
-            const float4* src = reinterpret_cast<const float4*>(th + off_w2(d_in) + v * H + 8 * j);
-            const float4 a = src[0], b = src[1];
-            const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-            *reinterpret_cast<uint4*>(S.w2b + tc::core_offset(v, 8 * j, H)) = pack_bf16x8(w);
-        }
-        {   // W2~ transposed [u][v] as B of dH1 (K = v): row u, columns 8j .. 8j + 7
-            const int u = t & (H - 1), j = t >> 6;
-            float w[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) w[q] = th[off_w2(d_in) + (8 * j + q) * H + u];
-            *reinterpret_cast<uint4*>(S.w2tb + tc::core_offset(u, 8 * j, H)) = pack_bf16x8(w);
-        }
-        for (int i = t; i < H; i += kTcThreads) {
-            S.w3[i] = bf(th[off_w3(d_in) + i]);
-            S.b1[i] = th[off_b1(d_in) + i];
-            S.b2[i] = th[off_b2(d_in) + i];
-        }
-        if (t == 0) S.b3 = th[off_b3(d_in)];
+    // the same without the fetching warps, which may be waiting for memory
+    auto sync_for_mma_tile = [&]() {
+        tc::fence_smem_async();
+        tc::fence_before_sync();
+        tc::sync_threads(2, kTcThreads - 64);
+        tc::fence_after_sync();
     };
-    // Forward pass of one tile: row m is sample smp of the planes Xs (n_total
-    // samples each) when valid, else zero.  Leaves H1~ (rows and transposed),
-    // H2~ rows and X~ in shared memory and the ReLU masks of this thread's 16
-    // columns in mask1 / mask2; returns the output of row m without b3.
-    auto forward_tile = [&](const float* Xs, long long n_total, long long smp, bool valid, uint32_t& mask1,
-                            uint32_t& mask2) -> float {
-        for (int k = 2 * cb; k < 2 * cb + 2 && k < d_in; ++k) {  // features 2cb, 2cb + 1 of row m
-            const float x = valid ? bf(Xs[k * n_total + smp]) : 0.0f;
-            put_bf16(S.a1, tc::core_offset(m, k, 16), x);
-            put_bf16(S.xtt, tc::core_offset(k, m, kTcRows), x);
+    bool pending = false;  // weights on their way
+    auto settle = [&]() {
+        if (pending) wait_on(&S.bar_weights, phase_weights);
+        pending = false;
+    };
+    // a block of this CTA to `dst` in CTA `to`, completing on its mbarrier `bar`
+    auto send = [&](const void* src, uint32_t bytes, const void* dst, uint64_t* bar, int to) {
+        tc::bulk_to_cta(tc::cluster_addr(tc::smem_addr(dst), to), tc::smem_addr(src), bytes,
+                        tc::cluster_addr(tc::smem_addr(bar), to));
+    };
+
+    // Sample smp into column `col` of S.rows[buf], asynchronously (zeros if !valid).
+    auto copy_row = [&](int buf, int col, const float* Xs, const float* Ys, long long n_total, long long smp, bool valid) {
+        const float* x = valid ? Xs + smp : Xs;
+        for (int k = 0; k < d_in; ++k, x += valid ? n_total : 0) tc::copy4(tc::smem_addr(&S.rows[buf][k][col]), x, valid);
+        tc::copy4(tc::smem_addr(&S.rows[buf][kMaxIn][col]), valid ? Ys + smp : Ys, valid);
+    };
+    // this worker's 16 words of a per-unit array
+    auto units16 = [&](const float* first, float (&v)[16]) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const float4 a = *reinterpret_cast<const float4*>(
+                reinterpret_cast<const unsigned char*>(first) + (2 * cb + (g >> 1)) * kWStride + 16 * (g & 1));
+            v[4 * g] = a.x;
+            v[4 * g + 1] = a.y;
+            v[4 * g + 2] = a.z;
+            v[4 * g + 3] = a.w;
         }
-        sync_for_mma();
-        if (t == 0 && ok) {
+    };
+    // v = 0 for the units whose activations, two times eight at h0 and h1, are zero
+    auto zero_where_off = [&](const void* h0, const void* h1, float (&v)[16]) {
+        const uint4 p = *static_cast<const uint4*>(h0), q = *static_cast<const uint4*>(h1);
+        const uint32_t w[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) {
+            v[j] = (w[j / 2] & 0xFFFFu) ? v[j] : 0.0f;
+            v[j + 1] = (w[j / 2] & 0xFFFF0000u) ? v[j + 1] : 0.0f;
+        }
+    };
+    auto store16 = [&](float (*tile)[kRowF], const float (&v)[16]) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+            *reinterpret_cast<float4*>(&tile[m][c0 + 4 * g]) =
+                make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+    };
+    auto store16_bf = [&](unsigned char* operand, const float (&v)[16]) {
+        *reinterpret_cast<uint4*>(operand + tc::core_offset(m, c0, H)) = pack_bf16x8(v);
+        *reinterpret_cast<uint4*>(operand + tc::core_offset(m, c0 + 8, H)) = pack_bf16x8(v + 8);
+    };
+
+    // Forward pass of the tile in S.rows[buf] (not the fetching warps).  Leaves X~,
+    // H1~ and H2~ rows in shared memory (zero exactly where the unit is off: the
+    // ReLU masks); returns the output of row m without b3 (workers).
+    auto forward_tile = [&](int buf) -> float {
+        if (worker) {
+            const float x0 = 2 * cb < d_in ? S.rows[buf][2 * cb][m] : 0.0f;
+            const float x1 = 2 * cb + 1 < d_in ? S.rows[buf][2 * cb + 1][m] : 0.0f;
+            *reinterpret_cast<__nv_bfloat162*>(S.a1 + tc::core_offset(m, 2 * cb, 16)) = __floats2bfloat162_rn(x0, x1);
+        }
+        settle();
+        sync_for_mma_tile();
+        if (issuer && __all_sync(0xFFFFFFFFu, ok)) {
             tc::mma_bf16(tm, tc::smem_desc(tc::smem_addr(S.a1), 128, 256),
-                         tc::smem_desc(tc::smem_addr(S.w1b), 128, 256), kIdesc, false);
+                         tc::smem_desc(tc::smem_addr(S.w[0].w1), 128, kWStride), kIdesc, false);
             tc::mma_commit(&S.bar);
         }
-        wait_mma();
-        // layer 1 epilogue: h1 = relu(z1 + b1) on columns c0 .. c0 + 15
-        mask1 = 0u;
-        {
-            float z[16];
+        if (worker) {
+            wait_mma();
+            // layer 1 epilogue: h1 = relu(z1 + b1) on columns c0 .. c0 + 15
+            float z[16], b[16];
+            units16(S.w[0].b1, b);
             tc::tmem_ld16(tm + lane_base + c0, z);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int u = c0 + j;
-                const float h = fmaxf(z[j] + S.b1[u], 0.0f);
-                if (h > 0.0f) mask1 |= 1u << j;
-                z[j] = bf(h);
-                put_bf16(S.h1tt, tc::core_offset(u, m, kTcRows), z[j]);
-            }
-            *reinterpret_cast<uint4*>(S.a2 + tc::core_offset(m, c0, H)) = pack_bf16x8(z);
-            *reinterpret_cast<uint4*>(S.a2 + tc::core_offset(m, c0 + 8, H)) = pack_bf16x8(z + 8);
+            for (int j = 0; j < 16; ++j) z[j] = fmaxf(z[j] + b[j], 0.0f);
+            store16_bf(S.a2, z);
         }
-        sync_for_mma();
-        if (t == 0 && ok) {
+        sync_for_mma_tile();
+        if (issuer && __all_sync(0xFFFFFFFFu, ok)) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
                 tc::mma_bf16(tm + 64, tc::smem_desc(tc::smem_addr(S.a2) + 256 * ks, 128, 1024),
-                             tc::smem_desc(tc::smem_addr(S.w2b) + 256 * ks, 128, 1024), kIdesc, ks > 0);
+                             tc::smem_desc(tc::smem_addr(S.w[0].w2) + 256 * ks, 128, kWStride), kIdesc, ks > 0);
             tc::mma_commit(&S.bar);
         }
-        wait_mma();
-        // layer 2 epilogue: h2 and this block's share of the output
-        mask2 = 0u;
-        {
-            float z[16], yp = 0.0f;
+        if (worker) {
+            float z[16], b[16], yp = 0.0f;
+            units16(S.w[0].b2, b);
+            wait_mma();
+            // layer 2 epilogue: h2 and this block's share of the output
             tc::tmem_ld16(tm + lane_base + 64 + c0, z);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int v = c0 + j;
-                const float h = fmaxf(z[j] + S.b2[v], 0.0f);
-                if (h > 0.0f) mask2 |= 1u << j;
-                const float hb = bf(h);
-                S.h2t[m][v] = __float2bfloat16_rn(hb);
-                yp = fmaf(hb, S.w3[v], yp);
+            for (int j = 0; j < 16; ++j) z[j] = fmaxf(z[j] + b[j], 0.0f);
+            units16(S.w[0].w3, b);
+            const uint4 packed[2] = {pack_bf16x8(z), pack_bf16x8(z + 8)};
+            const uint32_t* word = &packed[0].x;
+#pragma unroll
+            for (int j = 0; j < 16; j += 2) {
+                yp = fmaf(__uint_as_float(word[j / 2] << 16), b[j], yp);
+                yp = fmaf(__uint_as_float(word[j / 2] & 0xFFFF0000u), b[j + 1], yp);
             }
+            *reinterpret_cast<uint4*>(&S.h2t[m][c0]) = packed[0];
+            *reinterpret_cast<uint4*>(&S.h2t[m][c0 + 8]) = packed[1];
             S.ypart[cb][m] = yp;
+            tc::sync_threads(1, kTcWorkers);
         }
-        __syncthreads();
-        return ((S.ypart[0][m] + S.ypart[1][m]) + S.ypart[2][m]) + S.ypart[3][m];
+        return worker ? ((S.ypart[0][m] + S.ypart[1][m]) + S.ypart[2][m]) + S.ypart[3][m] : 0.0f;
+    };
+    // sum += values[first .. first + 64) in order
+    auto add64 = [&](const float* values, int first, float& sum) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float4 v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = *reinterpret_cast<const float4*>(values + first + 32 * h + 4 * q);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                sum += v[q].x;
+                sum += v[q].y;
+                sum += v[q].z;
+                sum += v[q].w;
+            }
+        }
+    };
+
+    // x mod n by a 64-bit reciprocal
+    const unsigned long long n_mod = static_cast<unsigned long long>(ta.n_tr);
+    const unsigned long long n_inv = ~0ull / n_mod;
+    auto mod_n = [&](unsigned long long x) {
+        unsigned long long r = x - __umul64hi(x, n_inv) * n_mod;
+        if (r >= n_mod) r -= n_mod;  // (the quotient is at most 2 too small)
+        if (r >= n_mod) r -= n_mod;
+        return static_cast<long long>(r);
+    };
+    // positions lo .. hi - 1 of the minibatch of nb samples at `off` are this CTA's
+    auto split = [&](long long nb, long long& lo, long long& hi) {
+        const long long chunk = (nb + kTcCluster - 1) / kTcCluster;
+        lo = min(nb, rank * chunk);
+        hi = min(nb, lo + chunk);
+    };
+    long long full_lo, full_hi;
+    split(ta.B, full_lo, full_hi);
+    auto share = [&](long long off, long long& nb, long long& lo, long long& hi) {
+        if (off + ta.B <= ta.n_tr) {
+            nb = ta.B;
+            lo = full_lo;
+            hi = full_hi;
+        } else {
+            nb = ta.n_tr - off;
+            split(nb, lo, hi);
+        }
+    };
+    // the tile at position p0 of the minibatch at `off` into S.rows[buf], by the two fetching warps
+    auto fetch = [&](int buf, unsigned long long a, unsigned long long b, long long off, long long p0, long long hi) {
+        for (int col = t - (kTcThreads - 64); col < kTcRows; col += 64) {
+            bool valid = p0 + col < hi;
+            const long long smp = mod_n(a * static_cast<unsigned long long>(off + p0 + col) + b);
+            if (valid && !MRIP_CHECK(smp >= 0 && smp < ta.n_tr, 401, smp)) valid = false;
+            copy_row(buf, col, ta.X, ta.Y, ta.n_tr, smp, valid);
+        }
+    };
+    auto fetch_bc = [&](long long of) {
+        const int i = t - (kTcThreads - 64);
+        if (i < 2) tc::copy4(tc::smem_addr(&S.bc[of & 1][i]), ta.bc + 2 * of + i, true);
+    };
+    auto fetch_val = [&](int buf, long long p0, long long hi) {
+        for (int col = t - (kTcThreads - 64); col < kTcRows; col += 64)
+            copy_row(buf, col, ta.Xv, ta.Yv, ta.n_val, p0 + col, p0 + col < hi);
     };
 
     long long step = 0;
     bool stop = false;
     float best = ta.best0;
     int bad = ta.bad0, best_epoch = 0, epochs_run = 0;
+    unsigned long long oa = 0, ob = 0;  // this epoch's order (fetching warps)
+    if (fetcher) {
+        oa = ta.ab[0];
+        ob = ta.ab[1];
+    }
+    int buf = 0;  // of the next tile's samples
+    long long nb, lo, hi;
+    share(0, nb, lo, hi);
+    if (fetcher) {
+        fetch(buf, oa, ob, 0, lo, hi);
+        fetch_bc(0);
+        tc::copy_wait();
+    }
+    __syncthreads();
     for (int ep = 0; ep < ta.epochs && !stop; ++ep) {
-        const SampleMap map{nullptr, ta.ab[2 * ep], ta.ab[2 * ep + 1], static_cast<unsigned long long>(ta.n_tr), 0};
+        const bool more = ep + 1 < ta.epochs;
+        unsigned long long na = 0, nb_ = 0;
+        if (fetcher && more) {
+            na = ta.ab[2 * ep + 2];
+            nb_ = ta.ab[2 * ep + 3];
+        }
         for (long long off = 0; off < ta.n_tr; off += ta.B, ++step) {
             if (ta.max_steps > 0 && step >= ta.max_steps) {  // uniform across the cluster
                 stop = true;
                 break;
             }
-            const long long nb = (off + ta.B <= ta.n_tr) ? ta.B : ta.n_tr - off;
-            const long long chunk = (nb + kTcCluster - 1) / kTcCluster;
-            const long long lo = min(nb, rank * chunk), hi = min(nb, lo + chunk);
-            SampleMap smap = map;
-            smap.off = off;
-            stage_weights();
-            for (int i = t; i <= P; i += kTcThreads) part[i] = 0.0f;
+            share(off, nb, lo, hi);
+            // the tile after position p0's: this step's or the next one's
+            auto fetch_ahead = [&](long long p0) {
+                if (p0 + kTcRows < hi) {
+                    fetch(buf, oa, ob, off, p0 + kTcRows, hi);
+                } else if (off + ta.B < ta.n_tr || more) {
+                    const bool same = off + ta.B < ta.n_tr;
+                    const long long xoff = same ? off + ta.B : 0;
+                    long long xnb, xlo, xhi;
+                    share(xoff, xnb, xlo, xhi);
+                    fetch(buf, same ? oa : na, same ? ob : nb_, xoff, xlo, xhi);
+                    if (ta.max_steps <= 0 || step + 1 < ta.max_steps) fetch_bc(step + 1);
+                }
+            };
+            // the blocks of this step, from the 7 other CTAs (after settle())
+            auto expect = [&]() {
+                if (t == kTcWorkers) {
+                    tc::mbar_expect(&S.bar_grad, (kTcCluster - 1) * kGradWords * 4);
+                    tc::mbar_expect(&S.bar_weights, (kTcCluster - 1) * kWStride);
+                }
+            };
+            if (lo >= hi) {  // no sample of a small minibatch is this CTA's
+                settle();
+                expect();
+                for (int i = t; i < kTcCluster * kGradWords; i += kTcThreads) (&S.part[0][0])[i] = 0.0f;
+                if (fetcher) {
+                    fetch_ahead(lo);
+                    tc::copy_wait();
+                }
+            }
 
             for (long long p0 = lo; p0 < hi; p0 += kTcRows) {
-                const int n_valid = static_cast<int>(min(static_cast<long long>(kTcRows), hi - p0));
-                const bool valid = m < n_valid;
-                long long smp = valid ? sample_of(smap, p0 + m) : 0;
-                if (valid && !MRIP_CHECK(smp >= 0 && smp < ta.n_tr, 401, smp)) smp = 0;
-                const float y = valid ? ta.Y[smp] : 0.0f;
-                uint32_t mask1, mask2;
-                const float yhat = forward_tile(ta.X, ta.n_tr, smp, valid, mask1, mask2);
-                const float r = valid ? (yhat + S.b3) - y : 0.0f;
-                const float dyv = valid ? 2.0f * r / static_cast<float>(nb) : 0.0f;
-                if (cb == 0) {
-                    S.dy[m] = dyv;
-                    S.r2[m] = r * r;
-                }
-                {
-                    float db[16];
+                const bool first = p0 == lo;
+                // (adds to a tile's predecessor; the first tile starts from zero)
+                auto put = [&](float& dst, float v) {
+                    if (first)
+                        dst = 0.0f + v;
+                    else
+                        dst += v;
+                };
+                buf ^= 1;
+                if (fetcher) {
+                    settle();  // (then, behind the first product)
+                    fetch_ahead(p0);
+                    tc::copy_wait();
+                } else {
+                    const float yhat = forward_tile(buf ^ 1);
+                    if (first) expect();
+                    if (worker) {
+                        const bool valid = p0 + m < hi;
+                        const float r = valid ? (yhat + S.w[0].b3) - S.rows[buf ^ 1][kMaxIn][m] : 0.0f;
+                        const float dyv = valid ? 2.0f * r / static_cast<float>(nb) : 0.0f;
+                        if (cb == 0) {
+                            S.dy[m] = dyv;
+                            S.r2[m] = r * r;
+                        }
+                        float d[16];
+                        units16(S.w[0].w3, d);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int v = c0 + j;
-                        const float d = ((mask2 >> j) & 1u) ? dyv * S.w3[v] : 0.0f;
-                        S.f32[m][v] = d;
-                        db[j] = bf(d);
-                        put_bf16(S.dz2tt, tc::core_offset(v, m, kTcRows), db[j]);
+                        for (int j = 0; j < 16; ++j) d[j] = dyv * d[j];
+                        zero_where_off(&S.h2t[m][c0], &S.h2t[m][c0 + 8], d);
+                        store16_bf(S.a3, d);
                     }
-                    *reinterpret_cast<uint4*>(S.a3 + tc::core_offset(m, c0, H)) = pack_bf16x8(db);
-                    *reinterpret_cast<uint4*>(S.a3 + tc::core_offset(m, c0 + 8, H)) = pack_bf16x8(db + 8);
+                    sync_for_mma_tile();
+                    if (issuer && __all_sync(0xFFFFFFFFu, ok)) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)  // dH1 = dZ2~ W2~
+                            tc::mma_bf16(tm, tc::smem_desc(tc::smem_addr(S.a3) + 256 * ks, 128, 1024),
+                                         tc::smem_desc(tc::smem_addr(S.w[0].w2) + 2 * kWStride * ks, kWStride, 128),
+                                         kIdescH1, ks > 0);
+                        tc::mma_commit(&S.bar);
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks)  // dW2 = dZ2~^T H1~
+                            tc::mma_bf16(tm + 128, tc::smem_desc(tc::smem_addr(S.a3) + 2048 * ks, 1024, 128),
+                                         tc::smem_desc(tc::smem_addr(S.a2) + 2048 * ks, 1024, 128), kIdescW2, ks > 0);
+                        tc::mma_commit(&S.bar_w2);
+                    }
+                    if (worker) {
+                        // meanwhile: column sums of dZ2 (b2: dy w3 where h2~ is not zero) and, by
+                        // the odd column blocks' warps, of dy h2~ (W3); a chunk of 16 rows per
+                        // warp, two columns per lane
+                        const int chunk = 4 * (cb >> 1) + quarter, q0 = 16 * chunk;
+                        float2 a = make_float2(0.0f, 0.0f);
+                        float dy[16];
+                        uint32_t h[16];
+#pragma unroll
+                        for (int q = 0; q < 16; q += 4) {
+                            const float4 d = *reinterpret_cast<const float4*>(&S.dy[q0 + q]);
+                            dy[q] = d.x;
+                            dy[q + 1] = d.y;
+                            dy[q + 2] = d.z;
+                            dy[q + 3] = d.w;
+                        }
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) h[q] = *reinterpret_cast<const uint32_t*>(&S.h2t[q0 + q][2 * lane]);
+                        if ((cb & 1) == 0) {
+                            const float2 w3 = *reinterpret_cast<const float2*>(&S.w[lane / 4].w3[2 * (lane % 4)]);
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) {  // (no fma: dZ2 is rounded)
+                                a.x = __fadd_rn(a.x, (h[q] & 0xFFFFu) ? __fmul_rn(dy[q], w3.x) : 0.0f);
+                                a.y = __fadd_rn(a.y, (h[q] & 0xFFFF0000u) ? __fmul_rn(dy[q], w3.y) : 0.0f);
+                            }
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) {
+                                a.x = fmaf(dy[q], __uint_as_float(h[q] << 16), a.x);
+                                a.y = fmaf(dy[q], __uint_as_float(h[q] & 0xFFFF0000u), a.y);
+                            }
+                        }
+                        *reinterpret_cast<float2*>(&S.colpart[cb & 1][chunk][2 * lane]) = a;
+                        wait_mma();
+                        // dZ1 = dH1 [z1 > 0] (FP32 for b1, BF16 for dW1)
+                        float z[16];
+                        tc::tmem_ld16(tm + lane_base + c0, z);
+                        zero_where_off(S.a2 + tc::core_offset(m, c0, H), S.a2 + tc::core_offset(m, c0 + 8, H), z);
+                        store16_bf(S.a4, z);
+                        store16(S.dz1, z);
+                    } else if (summer) {
+                        float sum = 0.0f;
+                        add64(lane == 0 ? S.dy : S.r2, 0, sum);
+                        add64(lane == 0 ? S.dy : S.r2, 64, sum);
+                        put(S.part[0][lane == 0 ? grad_b3(d_in) : grad_loss(d_in)], sum);
+                    }
                 }
                 sync_for_mma();
-                if (t == 0 && ok) {
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)  // dH1 = dZ2~ W2~
-                        tc::mma_bf16(tm, tc::smem_desc(tc::smem_addr(S.a3) + 256 * ks, 128, 1024),
-                                     tc::smem_desc(tc::smem_addr(S.w2tb) + 256 * ks, 128, 1024), kIdesc, ks > 0);
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)  // dW2 = dZ2~^T H1~
-                        tc::mma_bf16(tm + 128, tc::smem_desc(tc::smem_addr(S.dz2tt) + 256 * ks, 128, 2048),
-                                     tc::smem_desc(tc::smem_addr(S.h1tt) + 256 * ks, 128, 2048), kIdesc, ks > 0);
-                    tc::mma_commit(&S.bar);
-                }
-                // meanwhile: column sums of dZ2 (b2) and dy h2~ (W3) per chunk of 16 rows
-                {
-                    const int v = t & (H - 1), ch = t / H;
-                    float a2 = 0.0f, a3 = 0.0f;
-                    for (int q = 16 * ch; q < 16 * ch + 16; ++q) {
-                        a2 += S.f32[q][v];
-                        a3 = fmaf(S.dy[q], __bfloat162float(S.h2t[q][v]), a3);
-                    }
-                    S.colpart[0][ch][v] = a2;
-                    S.colpart[1][ch][v] = a3;
-                }
-                wait_mma();  // includes the barrier that frees S.f32
-                if (t < H) {
-                    float a2 = 0.0f, a3 = 0.0f;
-                    for (int ch = 0; ch < kTcChunks; ++ch) {
-                        a2 += S.colpart[0][ch][t];
-                        a3 += S.colpart[1][ch][t];
-                    }
-                    part[off_b2(d_in) + t] += a2;
-                    part[off_w3(d_in) + t] += a3;
-                } else if (t == H) {
-                    float a = 0.0f, l = 0.0f;
-                    for (int q = 0; q < kTcRows; ++q) {
-                        a += S.dy[q];
-                        l += S.r2[q];
-                    }
-                    part[off_b3(d_in)] += a;
-                    part[P] += l;
-                }
-                // dZ1 = dH1 [z1 > 0] (FP32 for b1; BF16 transposed into the
-                // freed dZ2~ buffer for dW1); dW2 rows 0..63 (TMEM lanes 0..63)
-                // into the gradient
-                {
-                    float z[16];
-                    tc::tmem_ld16(tm + lane_base + c0, z);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float d = ((mask1 >> j) & 1u) ? z[j] : 0.0f;
-                        S.f32[m][c0 + j] = d;
-                        put_bf16(S.dz2tt, tc::core_offset(c0 + j, m, kTcRows), d);
-                    }
-                }
-                if (quarter < 2) {
-                    float z[16];
-                    tc::tmem_ld16(tm + lane_base + 128 + c0, z);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) part[off_w2(d_in) + m * H + c0 + j] += z[j];
-                }
-                sync_for_mma();
-                if (t == 0 && ok) {
+                if (issuer && __all_sync(0xFFFFFFFFu, ok)) {
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks)  // dW1 = dZ1~^T X~
-                        tc::mma_bf16(tm + 192, tc::smem_desc(tc::smem_addr(S.dz2tt) + 256 * ks, 128, 2048),
-                                     tc::smem_desc(tc::smem_addr(S.xtt) + 256 * ks, 128, 2048), kIdescW1, ks > 0);
+                        tc::mma_bf16(tm + 192, tc::smem_desc(tc::smem_addr(S.a4) + 2048 * ks, 1024, 128),
+                                     tc::smem_desc(tc::smem_addr(S.a1) + 512 * ks, 256, 128), kIdescW1, ks > 0);
                     tc::mma_commit(&S.bar);
                 }
-                // meanwhile: column sums of dZ1 (b1) per chunk
-                {
-                    const int u = t & (H - 1), ch = t / H;
-                    float a1 = 0.0f;
-                    for (int q = 16 * ch; q < 16 * ch + 16; ++q) a1 += S.f32[q][u];
-                    S.colpart[2][ch][u] = a1;
+                if (worker) {
+                    const int chunk = 2 * cb + (quarter & 1), q0 = 16 * chunk;
+                    // meanwhile: rows 0..63 (TMEM lanes 0..63) of dW2 and, by the
+                    // warps whose TMEM lanes hold no gradient, the column sums of dZ1 (b1)
+                    if (quarter < 2) {
+                        wait_on(&S.bar_w2, phase_w2);
+                        tc::fence_after_sync();
+                        float z[16];
+                        tc::tmem_ld16(tm + lane_base + 128 + c0, z);
+                        float* block = S.part[m / kTcUnits] + (m % kTcUnits) * (H + 1) + c0;
+                        if (first) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) block[j] = 0.0f + z[j];
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) block[j] += z[j];
+                        }
+                    } else {
+                        float2 a = make_float2(0.0f, 0.0f);
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) {
+                            const float2 d = *reinterpret_cast<const float2*>(&S.dz1[q0 + q][2 * lane]);
+                            a.x += d.x;
+                            a.y += d.y;
+                        }
+                        *reinterpret_cast<float2*>(&S.colpart[2][chunk][2 * lane]) = a;
+                    }
+                    tc::sync_threads(1, kTcWorkers);
+                    if (quarter >= 2) {  // the chunks of all three
+                        const int i = 32 * chunk + lane;
+                        if (i < 3 * H) {
+                            const int which = i / H, col = i & (H - 1);
+                            float s = 0.0f;
+#pragma unroll
+                            for (int c = 0; c < kTcChunks; ++c) s += S.colpart[which][c][col];
+                            const int order = which == 0 ? 1 : which == 1 ? 2 : 0;  // b2, W3, b1 -> b1, b2, W3
+                            put(S.part[col / kTcUnits][grad_b1(d_in) + kTcUnits * order + col % kTcUnits], s);
+                        }
+                    }
+                    wait_mma();
+                    if (quarter < 2 && 4 * cb < d_in) {  // rows 0..63 of dW1
+                        float z[4];
+                        tc::tmem_ld4(tm + lane_base + 192 + 4 * cb, z);
+                        float* block = S.part[m / kTcUnits] + grad_w1() + (m % kTcUnits) * (d_in + 1) + 4 * cb;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (4 * cb + k < d_in) put(block[k], z[k]);
+                    }
                 }
-                wait_mma();
-                if (t < H) {
-                    float a1 = 0.0f;
-                    for (int ch = 0; ch < kTcChunks; ++ch) a1 += S.colpart[2][ch][t];
-                    part[off_b1(d_in) + t] += a1;
-                }
-                if (quarter < 2 && cb == 0) {  // dW1 rows u = m < 64 (TMEM lanes 0..63), columns = inputs
-                    float z[16];
-                    tc::tmem_ld16(tm + lane_base + 192, z);
-                    for (int k = 0; k < d_in; ++k) part[m * d_in + k] += z[k];
-                }
-                tc::fence_before_sync();
-                __syncthreads();
-                tc::fence_after_sync();
             }
-            cluster.sync();  // every CTA's gradient is complete
-            const float bc1 = ta.bc[2 * step], bc2 = ta.bc[2 * step + 1];
-            for (int p = p_lo + t; p < p_hi; p += kTcThreads) {
-                float g = 0.0f;
-                for (int rr = 0; rr < kTcCluster; ++rr) g += cluster.map_shared_rank(part, rr)[p];
-                if (ta.grad) ta.grad[p] = g;
-                const int q = p - p_lo;
-                const float mi = ta.beta1 * mom[q] + (1.0f - ta.beta1) * g;
-                const float vi = ta.beta2 * vel[q] + (1.0f - ta.beta2) * g * g;
-                mom[q] = mi;
-                vel[q] = vi;
-                const float nv = th[p] - ta.lr * (mi / bc1) / (sqrtf(vi / bc2) + ta.eps);
-                for (int rr = 0; rr < kTcCluster; ++rr) cluster.map_shared_rank(th, rr)[p] = nv;
+            sync_for_mma();  // the gradient is complete
+            if (sends) send(S.part[warp], kGradWords * 4, S.recv[rank], &S.bar_grad, warp);
+            wait_on(&S.bar_grad, phase_grad);
+            float g = 0.0f;  // this thread's word, of all CTAs (word grad_loss: the squared residuals)
+#pragma unroll
+            for (int rr = 0; rr < kTcCluster; ++rr) g += rr == rank ? S.part[rr][t] : S.recv[rr][t];
+            if (par >= 0) {
+                if (ta.grad) ta.grad[par] = g;
+                mom = ta.beta1 * mom + (1.0f - ta.beta1) * g;
+                vel = ta.beta2 * vel + (1.0f - ta.beta2) * g * g;
+                th = th - ta.lr * (mom / S.bc[step & 1][0]) / (sqrtf(vel / S.bc[step & 1][1]) + ta.eps);
+                put_weight(S.w[rank], at, use, th);
             }
-            if (rank == 0 && t == 0) {
-                float l = 0.0f;
-                for (int rr = 0; rr < kTcCluster; ++rr) l += cluster.map_shared_rank(part, rr)[P];
-                if (ta.losses) ta.losses[step] = l / static_cast<float>(nb);
-            }
-            cluster.sync();
+            sync_for_mma();  // the owner's new weights are written, its receive buffers read
+            if (sends) send(&S.w[rank], kWStride, &S.w[rank], &S.bar_weights, warp);
+            if (rank == 0 && t == grad_loss(d_in) && ta.losses) ta.losses[step] = g / static_cast<float>(nb);
+            pending = true;
         }
         if (stop) break;
         ++epochs_run;
+        oa = na;
+        ob = nb_;
         if (ta.n_val > 0) {
             // validation loss of this epoch's parameters (each CTA a slice of
             // the validation samples, in order; the CTAs' sums added in rank
             // order, so every CTA computes the same value and takes the same
             // early-stopping decision)
-            stage_weights();
-            if (t == 0) part[P] = 0.0f;
-            __syncthreads();
             const long long vchunk = (ta.n_val + kTcCluster - 1) / kTcCluster;
             const long long vlo = min(ta.n_val, rank * vchunk), vhi = min(ta.n_val, vlo + vchunk);
-            for (long long p0 = vlo; p0 < vhi; p0 += kTcRows) {
-                const int n_valid = static_cast<int>(min(static_cast<long long>(kTcRows), vhi - p0));
-                const bool valid = m < n_valid;
-                const long long smp = valid ? p0 + m : 0;
-                uint32_t mask1, mask2;
-                const float yhat = forward_tile(ta.Xv, ta.n_val, smp, valid, mask1, mask2);
-                const float r = valid ? (yhat + S.b3) - ta.Yv[smp] : 0.0f;
-                if (cb == 0) S.r2[m] = r * r;
-                __syncthreads();
-                if (t == H) {
-                    float l = 0.0f;
-                    for (int q = 0; q < kTcRows; ++q) l += S.r2[q];
-                    part[P] += l;
+            float vsum = 0.0f;
+            int vbuf = 2;
+            if (fetcher) {
+                fetch_val(vbuf, vlo, vhi);
+                tc::copy_wait();
+            }
+            __syncthreads();
+            for (long long p0 = vlo; p0 < vhi; p0 += kTcRows, vbuf ^= 1) {
+                if (fetcher) {
+                    fetch_val(vbuf ^ 1, p0 + kTcRows, vhi);
+                    settle();
+                    tc::copy_wait();
+                } else {
+                    const float yhat = forward_tile(vbuf);
+                    if (worker && cb == 0) {
+                        const float r = p0 + m < vhi ? (yhat + S.w[0].b3) - S.rows[vbuf][kMaxIn][m] : 0.0f;
+                        S.r2[m] = r * r;
+                    }
                 }
                 __syncthreads();
+                if (summer && lane == 0) {
+                    float l = 0.0f;
+                    add64(S.r2, 0, l);
+                    add64(S.r2, 64, l);
+                    vsum += l;
+                }
             }
+            if (summer && lane == 0) S.vsum = vsum;
             cluster.sync();
             float vl = 0.0f;
-            for (int rr = 0; rr < kTcCluster; ++rr) vl += cluster.map_shared_rank(part, rr)[P];
+            for (int rr = 0; rr < kTcCluster; ++rr)
+                vl += tc::ld_cluster(tc::cluster_addr(tc::smem_addr(&S.vsum), rr));
             vl /= static_cast<float>(ta.n_val);
-            cluster.sync();  // every CTA has read the sums before part[] is cleared again
+            cluster.sync();  // every CTA has read the sums before they are written again
             if (rank == 0 && t == 0 && ta.val_losses) ta.val_losses[ep] = vl;
             if (vl < best) {
                 best = vl;
                 best_epoch = ep + 1;
                 bad = 0;
-                for (int p = p_lo + t; p < p_hi; p += kTcThreads) ta.theta[p] = th[p];
+                if (par >= 0) ta.theta[par] = th;
             } else if (ta.patience > 0 && ++bad >= ta.patience) {
                 stop = true;
             }
         }
     }
-    if (ta.n_val == 0)
-        for (int p = p_lo + t; p < p_hi; p += kTcThreads) ta.theta[p] = th[p];
-    if (ta.theta_last)
-        for (int p = p_lo + t; p < p_hi; p += kTcThreads) ta.theta_last[p] = th[p];
-    if (ta.m_out)
-        for (int p = p_lo + t; p < p_hi; p += kTcThreads) ta.m_out[p] = mom[p - p_lo];
-    if (ta.v_out)
-        for (int p = p_lo + t; p < p_hi; p += kTcThreads) ta.v_out[p] = vel[p - p_lo];
+    if (par >= 0) {
+        if (ta.n_val == 0) ta.theta[par] = th;
+        if (ta.theta_last) ta.theta_last[par] = th;
+        if (ta.m_out) ta.m_out[par] = mom;
+        if (ta.v_out) ta.v_out[par] = vel;
+    }
     if (rank == 0 && t == 0 && ta.info) {
         ta.info[0] = epochs_run;
         ta.info[1] = ta.n_val > 0 ? best_epoch : epochs_run;
         ta.info[2] = static_cast<int>(step);
     }
+    settle();
+    if (!ok) {  // (after a timeout: once more, with a limit, for what is still in flight)
+        if (worker) tc::mbar_wait(&S.bar, phase ^ 1u, kTcWait);
+        tc::mbar_wait(&S.bar_grad, phase_grad ^ 1u, kTcWait);
+        tc::mbar_wait(&S.bar_weights, phase_weights ^ 1u, kTcWait);
+    }
     tc::fence_before_sync();
-    __syncthreads();
+    cluster.sync();  // no CTA leaves while another may still copy from or to it
     tc::fence_after_sync();
     if (warp == 0) tc::tmem_free(tm, 256);
 }
 
-size_t mlp_train_tc_smem(int d_in) {
-    const int P = static_cast<int>(n_params(d_in));
-    const int P4 = (P + 1 + 3) & ~3;
-    const int slice = (P + kTcCluster - 1) / kTcCluster;
-    return sizeof(TcSmem) + (2 * static_cast<size_t>(P4) + 2 * slice) * sizeof(float);
-}
+size_t mlp_train_tc_smem() { return sizeof(TcSmem); }
 
 // Inference.  The two layers are FP32 products of BF16-rounded operands with a
 // prescribed order of additions (one chain per unit, inputs ascending), so
@@ -1134,31 +1405,29 @@ mrip_status mlp_train(const TrainSpec& sp, TrainInfo* info, cudaStream_t st) {
     if (sp.max_steps > 0 && sp.max_steps < n_steps) n_steps = sp.max_steps;
     // resuming at epoch epoch0: its order and Adam's step count continue
     const long long step0 = static_cast<long long>(sp.epoch0) * spe;
-    std::vector<unsigned long long> ab(2 * static_cast<size_t>(sp.epochs));
+    // one upload: [info 16 B, timeout flag 16 B, both zero][ab][bc]
+    const size_t ab_bytes = 2 * static_cast<size_t>(sp.epochs) * sizeof(unsigned long long);
+    const size_t bytes = 32 + ab_bytes + 2 * static_cast<size_t>(n_steps) * sizeof(float);
+    std::vector<unsigned long long> schedule((bytes + 7) / 8, 0ull);
+    unsigned long long* ab = schedule.data() + 4;
     for (int ep = 0; ep < sp.epochs; ++ep)
         epoch_affine(sp.order_seed, sp.epoch0 + ep, static_cast<unsigned long long>(sp.n), ab[2 * ep],
                      ab[2 * ep + 1]);
-    std::vector<float> bc(2 * static_cast<size_t>(n_steps));
+    float* bc = reinterpret_cast<float*>(ab + 2 * static_cast<size_t>(sp.epochs));
     for (long long k = 1; k <= n_steps; ++k) {
         const double kk = static_cast<double>(step0 + k);
         bc[2 * (k - 1)] = static_cast<float>(1.0 - std::pow(static_cast<double>(sp.beta1), kk));
         bc[2 * (k - 1) + 1] = static_cast<float>(1.0 - std::pow(static_cast<double>(sp.beta2), kk));
     }
-    // scratch: [info 16 B, timeout flag 16 B][ab][bc]
-    const size_t ab_bytes = ab.size() * sizeof(unsigned long long);
-    const size_t bytes = 32 + ab_bytes + bc.size() * sizeof(float);
     char* base = static_cast<char*>(scratch(bytes, 4));
     if (!base) return fail(MRIP_ENOMEM, "mlp train: scratch allocation failed");
     int* d_info = reinterpret_cast<int*>(base);
     int* flag = reinterpret_cast<int*>(base + 16);
     unsigned long long* d_ab = reinterpret_cast<unsigned long long*>(base + 32);
     float* d_bc = reinterpret_cast<float*>(base + 32 + ab_bytes);
-    cudaError_t e = cudaMemsetAsync(base, 0, 32, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_ab, ab.data(), ab_bytes, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_bc, bc.data(), bc.size() * sizeof(float), cudaMemcpyHostToDevice, st);
+    cudaError_t e = cudaMemcpyAsync(base, schedule.data(), bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_status(e, "mlp train: schedule upload");
-    const size_t smem = mlp_train_tc_smem(sp.d_in);
+    const size_t smem = mlp_train_tc_smem();
     e = cudaFuncSetAttribute(mlp_train_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return cuda_status(e, "mlp train: shared memory attribute");
     TrainArgs ta{sp.X, sp.Y, sp.n, sp.B, spe, sp.epochs, sp.d_in, d_ab, d_bc, sp.lr, sp.beta1, sp.beta2, sp.eps,

@@ -120,6 +120,15 @@ def test_training_steps_match_oracle(env, d_in, n, batch, steps):
         prev = dict(theta=r["theta"], m=r["m"], v=r["v"])
 
 
+@pytest.mark.parametrize("d_in,n,batch,steps", [
+    (2, 330, 33, 3),      # five rows per CTA, the seventh three, the last CTA none in any step
+    (3, 1057, 1024, 3),   # the same in a last minibatch only
+    (5, 9000, 4600, 3),   # five tiles per CTA, then a last minibatch of 4,400 (550 rows per CTA)
+])
+def test_uneven_shares_match_oracle(env, d_in, n, batch, steps):
+    test_training_steps_match_oracle(env, d_in, n, batch, steps)
+
+
 def _expected_stop(val, epochs, patience):
     best, best_e, bad = np.inf, 0, 0
     for e in range(1, epochs + 1):
