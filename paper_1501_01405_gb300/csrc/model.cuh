@@ -43,7 +43,23 @@ struct DevBuf {
     }
 };
 
+// Page-locked host memory the device can write.
+struct HostBuf {
+    void* p = nullptr;
+    ~HostBuf() {
+        if (p) cudaFreeHost(p);
+    }
+    bool ensure(size_t bytes) {
+        if (!p && cudaHostAlloc(&p, bytes, cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return p != nullptr;
+    }
+};
+
 struct mrip_model {
+    HostBuf back;  // a small run's moments and outputs (released after the device buffers, so after every run)
     int kind = 0;
     mrip_mm1_params mm1{};
     mrip_tandem3_params tandem{};
@@ -57,6 +73,8 @@ struct mrip_model {
     int64_t n_reps = 0;
     int64_t rep0 = 0;  // replication index of output column 0 (mrip_run_range)
     bool has_run = false;
+    bool back_valid = false;              // `back` holds the last run's results once back_stream is synchronised
+    cudaStream_t back_stream = nullptr;
     // the control variate's working buffers (kept between mrip_run_cv calls)
     // and the network of the last one
     struct {
@@ -73,6 +91,7 @@ struct mrip_model {
     int64_t g_n_reps = -1;
     int64_t g_rep0 = -1;
     uint64_t g_seed = 0;
+    bool g_back = false;  // the graph ends with the copy to `back`
     Plan g_plan;
     ~mrip_model() {
         if (exec) cudaGraphExecDestroy(exec);

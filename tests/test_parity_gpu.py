@@ -799,3 +799,32 @@ def test_every_stage_accepts_an_empty_batch(eng, torch_mod):
     zi = t.full((6,), 7.0, dtype=t.float64, device="cuda")
     eng.mrip_stats_reduce_i64(t.empty((2, 0), dtype=t.int64, device="cuda"), zi)
     assert z.cpu().tolist() == [0.0] * 9 and zi.cpu().tolist() == [0.0] * 6
+
+
+@pytest.mark.parametrize("kind,dp,kw,dtypes,largest", [
+    ("MM1", [0.9, 1.0], dict(n_clients=50), ["f8", "f8", "f8"], 169),      # 24 + 24 n bytes
+    ("TANDEM3", [0.8, 1.0, 1.1, 1.2], dict(n_clients=50, window=10), ["f8", "f8"], 56),  # 24 + 72 n
+    ("FOREST_FIRE", [0.01, 1e-4], dict(L=32, n_steps=3, density=0.5, window=2), ["i4", "f8"], 203),  # 24 + 20 n
+    ("WALK_L1_EXIT", [4.0], dict(max_steps=1 << 38), ["i8"], 509),                           # 24 + 8 n
+])
+def test_results_returned_with_a_small_run(eng, torch_mod, kind, dp, kw, dtypes, largest):
+    """Up to 4,096 bytes of moments and outputs come back with the run, one replication more does not: both equal
+    the planes read on the device, also after a second run and after a change of stream."""
+    t = torch_mod
+    m = eng.Model(getattr(eng, "MRIP_" + kind), **kw)
+    other = t.cuda.Stream()
+    for n, seed in ((largest, 1), (largest, 2), (largest + 1, 2), (1, 3), (largest, 2)):
+        m.set_stream(None)
+        m.run(np.array([dp]), n, seed)
+        for moved in (False, True):
+            for w, ty in enumerate(dtypes):
+                host = m.outputs(w, dtype=np.dtype(ty))
+                on_dev = t.empty(host.size, dtype={"f8": t.float64, "i4": t.int32, "i8": t.int64}[ty], device="cuda")
+                eng.mrip_outputs(m.h, w, on_dev)
+                assert np.array_equal(host, on_dev.cpu().numpy()), (n, seed, moved, w)
+            if kind != "FOREST_FIRE":
+                y = m.outputs(0, dtype=np.dtype(dtypes[0])).astype(np.float64)[:n]
+                np.testing.assert_allclose(m.moments()[0], [n, y.mean(), ((y - y.mean()) ** 2).sum()], rtol=1e-12, atol=1e-12)
+            t.cuda.synchronize()
+            m.set_stream(other)
+    m.close()
