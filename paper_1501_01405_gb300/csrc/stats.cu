@@ -49,13 +49,16 @@ __device__ __forceinline__ double total8(const double* g) {
 // the same moments but puts a dependent FP64 division on every element and
 // two on every tree level; on GB300's narrow FP64 pipe that chain was the
 // kernel's whole latency: 12.3k cycles for 32 values and 45k for 4,096,
-// against 4.8k and 11k for the two passes.)  With one slice out[dp] gets
+// against 4.8k and 11k for the two passes.)  That pipe is also why only the
+// warps that have elements add and one thread divides: with all eight warps
+// doing the same sums and the division the kernel took 7.2 us for 32 values,
+// 4.9 now.  With one slice out[dp] gets
 // (n, m + (sum d) / n, M2); otherwise part[dp][slice] gets the mean as the
 // unrounded pair (n, m, M2, (sum d) / n) for the slice merge.
 template <typename T>
 __global__ void __launch_bounds__(kStatsThreads) stats_kernel(const T* __restrict__ x, long long n_reps,
                                                               int slices, double* __restrict__ out) {
-    __shared__ double gsum[kGroups], gsq[kGroups], gdev[kGroups];
+    __shared__ double gsum[kGroups], gsq[kGroups], gdev[kGroups], gmean;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long dp = blockIdx.x / slices;
     const long long sl = blockIdx.x - dp * slices;
@@ -63,29 +66,36 @@ __global__ void __launch_bounds__(kStatsThreads) stats_kernel(const T* __restric
     const long long lo = sl * per;
     const long long hi = lo + per < n_reps ? lo + per : n_reps;
     const long long n = hi > lo ? hi - lo : 0;
-    const double inv_n = n > 0 ? 1.0 / static_cast<double>(n) : 0.0;
     const T* row = x + dp * n_reps;
     if (!MRIP_CHECK(lo >= 0 && hi <= n_reps, 701, sl)) return;  // CTA-uniform
+    const bool active = 32 * warp < n;  // the warp has an element
     double a = 0.0;
-    for (long long i = lo + threadIdx.x; i < hi; i += kStatsThreads) a += static_cast<double>(row[i]);
-    a = warp_sum(a);
+    if (active) {
+        for (long long i = lo + threadIdx.x; i < hi; i += kStatsThreads) a += static_cast<double>(row[i]);
+        a = warp_sum(a);
+    }
     if (lane == 0) gsum[warp] = a;
     __syncthreads();
-    const double mean = n > 0 ? total8(gsum) / static_cast<double>(n) : 0.0;
+    if (threadIdx.x == 0) gmean = n > 0 ? total8(gsum) / static_cast<double>(n) : 0.0;
+    __syncthreads();
+    const double mean = gmean;
     double q = 0.0, c = 0.0;
-    for (long long i = lo + threadIdx.x; i < hi; i += kStatsThreads) {
-        const double d = static_cast<double>(row[i]) - mean;
-        q += d * d;
-        c += d;
+    if (active) {
+        for (long long i = lo + threadIdx.x; i < hi; i += kStatsThreads) {
+            const double d = static_cast<double>(row[i]) - mean;
+            q += d * d;
+            c += d;
+        }
+        q = warp_sum(q);
+        c = warp_sum(c);
     }
-    q = warp_sum(q);
-    c = warp_sum(c);
     if (lane == 0) {
         gsq[warp] = q;
         gdev[warp] = c;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
+        const double inv_n = n > 0 ? 1.0 / static_cast<double>(n) : 0.0;
         const double sd = total8(gdev);
         double m2 = total8(gsq) - sd * sd * inv_n;
         if (m2 < 0.0) m2 = 0.0;

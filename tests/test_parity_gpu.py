@@ -801,6 +801,12 @@ def test_every_stage_accepts_an_empty_batch(eng, torch_mod):
     assert z.cpu().tolist() == [0.0] * 9 and zi.cpu().tolist() == [0.0] * 6
 
 
+@pytest.mark.parametrize("n_reps", [31, 32, 33, 63, 65, 256])
+def test_stats_reduce_few(eng, torch_mod, n_reps):
+    """Fewer values than the CTA has warps' worth: the warps without an element add nothing."""
+    test_stats_reduce(eng, torch_mod, n_reps)
+
+
 @pytest.mark.parametrize("kind,dp,kw,dtypes,largest", [
     ("MM1", [0.9, 1.0], dict(n_clients=50), ["f8", "f8", "f8"], 169),      # 24 + 24 n bytes
     ("TANDEM3", [0.8, 1.0, 1.1, 1.2], dict(n_clients=50, window=10), ["f8", "f8"], 56),  # 24 + 72 n
