@@ -808,7 +808,7 @@ __global__ void __launch_bounds__(128) tandem3_warp_coop_kernel(
 // map of all clients before it, whose value at W_0 = 0 is its entry wait;
 // in a cluster the maps of the earlier CTAs, read over distributed shared
 // memory, carry W_0 = 0 to the CTA's first client (14 replications x 100,003
-// clients 201 -> 47 us, 32 x 10,000 36 -> 21 us);
+// clients 201 -> 41 us, 32 x 10,000 36 -> 14.5 us);
 // pass 2 replays the thread's clients with the plain recurrence.  Times run
 // in the 48-bit fixed point of the tandem, so composition is exact and the
 // sums are exact integers (order-free); c and d saturate at +-2^61, which
@@ -864,11 +864,18 @@ struct Mm1Sums {
 };
 
 
+// Clients whose variates are drawn together, before the two multipliers of the
+// rates are needed (FP64 divisions on a slow pipe: two lanes of the last warp,
+// which has the fewest clients, compute them meanwhile for all), and the most
+// threads per CTA.  32 x 10,000 clients 20.9 -> 14.5 us, 1,024 x 1,000 26.7 -> 20.6, 14
+// x 100,003 47.2 -> 41.1; one client at a time 18.3, 22.0, 43.1; up to 1,024 threads
+// 18.4, 20.6, 42.8; 256 14.5, 20.6, 53.1.
+constexpr int kMm1CtaGroup = 2, kMm1CtaThreads = 512;
+
 template <bool kCluster>
-__global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict__ dps, long long n_reps,
-                                                       long long rep0, long long n_clients, bool staged,
-                                                       const __grid_constant__ RoundKeys rk, LogTable tab,
-                                                       Mm1Out out) {
+__global__ void __launch_bounds__(kMm1CtaThreads) mm1_cta_kernel(
+    const double* __restrict__ dps, long long n_reps, long long rep0, long long n_clients, bool staged,
+    const __grid_constant__ RoundKeys rk, LogTable tab, Mm1Out out) {
     namespace cg = cooperative_groups;
     extern __shared__ long long fix_stage[];  // [client - lo][thread] x (S, A) when staged
     __shared__ FixMap fmaps[32];
@@ -876,6 +883,7 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
     __shared__ U96 part[3][32];
     __shared__ double dpart[3][32];
     __shared__ DblMap dtotal;
+    __shared__ unsigned long long scale[2];
     __shared__ struct {
         FixMap map;  // all clients of this CTA
         U96 sum[3];
@@ -901,27 +909,47 @@ __global__ void __launch_bounds__(1024) mm1_cta_kernel(const double* __restrict_
 
     bool fixed_ok = fix_rate_ok(lam) && fix_rate_ok(mu);
     if (fixed_ok) {
-        // every thread needs the same two multipliers (FP64 divisions on a
-        // slow pipe): lane 0 of each warp computes them, a shuffle shares them
-        unsigned long long cl = 0, cmu = 0;
-        if (lane == 0) {
-            cl = fix_scale(lam);
-            cmu = fix_scale(mu);
-        }
-        cl = __shfl_sync(kFull, cl, 0);
-        cmu = __shfl_sync(kFull, cmu, 0);
         FixMap f{-kSat, 0};
         long long* st_s = fix_stage + threadIdx.x;
         long long* st_a = fix_stage + k * blockDim.x + threadIdx.x;
-        for (long long n = lo; n < hi; ++n) {
-            const uint4 b = philox_row(row, static_cast<uint32_t>(n), rk);
-            const long long sv = to_fix(neg_log_q58<false>(b.x, b.y, tab), cmu);
-            const long long av = to_fix(neg_log_q58<false>(b.z, b.w, tab), cl);
+        unsigned long long cl = 0, cmu = 0, ys[kMm1CtaGroup], ya[kMm1CtaGroup];
+        auto draw = [&](long long n0) {
+#pragma unroll
+            for (int g = 0; g < kMm1CtaGroup; ++g) {
+                const uint4 b = philox_row(row, static_cast<uint32_t>(n0 + g), rk);
+                ys[g] = neg_log_q58<false>(b.x, b.y, tab);
+                ya[g] = neg_log_q58<false>(b.z, b.w, tab);
+            }
+        };
+        auto use = [&](long long n, unsigned long long s58, unsigned long long a58) {
+            const long long sv = to_fix(s58, cmu);
+            const long long av = to_fix(a58, cl);
             if (staged) {
                 st_s[(n - lo) * blockDim.x] = sv;
                 st_a[(n - lo) * blockDim.x] = av;
             }
             f = fcompose(f, FixMap{0, sv - av});
+        };
+        const bool whole = lo + kMm1CtaGroup <= hi;
+        if (warp == nwarp - 1 && lane < 2) scale[lane] = fix_scale(lane == 0 ? lam : mu);
+        if (whole) draw(lo);
+        __syncthreads();
+        cl = scale[0];
+        cmu = scale[1];
+        long long n0 = lo;
+        if (whole) {
+#pragma unroll
+            for (int g = 0; g < kMm1CtaGroup; ++g) use(lo + g, ys[g], ya[g]);
+            n0 += kMm1CtaGroup;
+            for (; n0 + kMm1CtaGroup <= hi; n0 += kMm1CtaGroup) {
+                draw(n0);
+#pragma unroll
+                for (int g = 0; g < kMm1CtaGroup; ++g) use(n0 + g, ys[g], ya[g]);
+            }
+        }
+        for (; n0 < hi; ++n0) {
+            const uint4 b = philox_row(row, static_cast<uint32_t>(n0), rk);
+            use(n0, neg_log_q58<false>(b.x, b.y, tab), neg_log_q58<false>(b.z, b.w, tab));
         }
         const FixMap pre = block_exclusive_map(f, FixMap{-kSat, 0}, fmaps, &mine.map, fcompose);
         long long w = 0;  // W_0
@@ -1340,7 +1368,8 @@ extern "C" mrip_status mrip_mm1_simulate(const double* d_dps, int32_t n_dp, int6
     } else if (mapping == MRIP_MAP_CTA) {
         if (n_items > 0x7FFFFFFFll) return fail(MRIP_EINVAL, "mrip_mm1_simulate: too many replications for CTA");
         CtaShape shape;
-        mrip_status cs = cta_shape(mm1_cta_kernel<false>, mm1_cta_kernel<true>, n_items, n_clients, 1024, true, &shape);
+        mrip_status cs = cta_shape(mm1_cta_kernel<false>, mm1_cta_kernel<true>, n_items, n_clients, kMm1CtaThreads,
+                                   true, &shape);
         if (cs != MRIP_OK) return cs;
         cs = launch_ctas(shape.ctas > 1 ? mm1_cta_kernel<true> : mm1_cta_kernel<false>, n_items, shape, st, d_dps, static_cast<long long>(n_reps),
                          static_cast<long long>(rep0), static_cast<long long>(n_clients), shape.staged, rk, tab, out);

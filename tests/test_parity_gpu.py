@@ -801,6 +801,18 @@ def test_every_stage_accepts_an_empty_batch(eng, torch_mod):
     assert z.cpu().tolist() == [0.0] * 9 and zi.cpu().tolist() == [0.0] * 6
 
 
+@pytest.mark.parametrize("n_clients", [1, 2, 3, 127, 128, 257, 2047, 2049])
+def test_mm1_cta_few_clients(eng, torch_mod, n_clients):
+    """CTA mapping with fewer clients than two per thread, up to the first cluster of two; fixed-point and FP64 rates."""
+    t = torch_mod
+    dps = np.array([[0.9, 1.0], [0.01, 1.0], [4.0, 1.0]])
+    for i in range(3):
+        out = [t.empty(5, dtype=t.float64, device="cuda") for _ in range(3)]
+        eng.mrip_mm1_simulate(dev(t, dps[i:i + 1]), 5, n_clients, 3, eng.MRIP_MAP_CTA, *out)
+        for g, r in zip(out, oracle.mm1(dps[i:i + 1], *oracle.all_items(1, 5), n_clients, 3, threads=threads())):
+            np.testing.assert_allclose(g.cpu().numpy(), r, rtol=REL, atol=1e-14)
+
+
 @pytest.mark.parametrize("n_reps", [31, 32, 33, 63, 65, 256])
 def test_stats_reduce_few(eng, torch_mod, n_reps):
     """Fewer values than the CTA has warps' worth: the warps without an element add nothing."""
