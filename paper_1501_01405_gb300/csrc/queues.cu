@@ -1084,12 +1084,16 @@ __global__ void __launch_bounds__(kMm1CtaThreads) mm1_cta_kernel(
 //
 // One CTA per replication leaves the SMs without one idle, so few replications
 // are split over clusters of up to 8 CTAs (cta_shape): 16 x 100,000 clients run on
-// 112 SMs instead of 16, 439 -> 102 us.  At most 512 threads per CTA: at 1,024 the 64
-// registers of a thread spill (33 replications x 50,021 clients in clusters: 86 us,
-// at 640, 768 and 1,024 threads 94, 104, 119); 256 where there are more replications
-// than SMs, so that several CTAs share one (333 x 5,021 clients: 91 .. 98 us at 256
-// threads, 123 at 384, 133 at 512, 186 at the former 1,024).
-// ---------------------------------------------------------------------------
+// 112 SMs instead of 16, 439 -> 102 us.  FP64 is kept to the warps that need it
+// (its pipe takes a warp instruction every 16 cycles, however few lanes are
+// active): the four multipliers by four lanes for the CTA, the reciprocals and
+// the sums of the early window only in the warps that hold its clients: 90 us.
+// At most 512 threads per CTA (16 x 100,000 at 512, 768 and 1,024 threads: 90, 98, 111;
+// 33 replications x 50,021 clients 76, 84, 96: the scan grows with the warps); 256 where
+// there are more replications than SMs and 128 where more than twice as many,
+// so that several CTAs share one (333 x 5,021 clients at 128, 256, 384 threads: 85, 88,
+// 109 us; 1,400 x 2,000: 115, 136, 221).  Two clients drawn together gain nothing
+// (96 us: 16 warps of 128 registers hide the chains).
 constexpr int kTandemThreads = 512;
 template <bool kCluster>
 __global__ void __launch_bounds__(kTandemThreads) tandem3_cta_kernel(const double* __restrict__ dps, long long n_reps,
@@ -1100,6 +1104,7 @@ __global__ void __launch_bounds__(kTandemThreads) tandem3_cta_kernel(const doubl
     __shared__ FTMap wmap[32];
     __shared__ U96 wy[32];
     __shared__ double wsum[4][32];
+    __shared__ unsigned long long scale[4];
     __shared__ struct {
         FTMap map;     // all clients of this CTA
         U96 y;
@@ -1122,19 +1127,27 @@ __global__ void __launch_bounds__(kTandemThreads) tandem3_cta_kernel(const doubl
     const long long hi = min(lo + k, n_clients);
 
     if (fix_rate_ok(lam) && fix_rate_ok(mu1) && fix_rate_ok(mu2) && fix_rate_ok(mu3)) {
-        const unsigned long long cl = fix_scale(lam), c1 = fix_scale(mu1), c2 = fix_scale(mu2),
-                                 c3f = fix_scale(mu3);
-        FTMap f = ftmap_identity();
-        const uint32_t every = saturation_mask(lam, mu1, mu2, mu3);
-        for (long long n = lo; n < hi; ++n) {
+        // every thread needs the same four multipliers: one division each in
+        // four lanes (FP64 is a slow pipe, and a warp occupies it as long as one lane)
+        if (t < 4) scale[t] = fix_scale(t == 0 ? lam : t == 1 ? mu1 : t == 2 ? mu2 : mu3);
+        __syncthreads();
+        const unsigned long long cl = scale[0], c1 = scale[1], c2 = scale[2], c3f = scale[3];
+        struct Draw {
+            unsigned long long a, s1, s2, s3;
+        };
+        auto draw = [&](long long n) {
             uint4 b0, b1;
             philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
-            f = ftmap_push(f, to_fix(neg_log_q58<false>(b0.x, b0.y, tab), cl),
-                           to_fix(neg_log_q58<false>(b0.z, b0.w, tab), c1),
-                           to_fix(neg_log_q58<false>(b1.x, b1.y, tab), c2),
-                           to_fix(neg_log_q58<false>(b1.z, b1.w, tab), c3f));
+            return Draw{neg_log_q58<false>(b0.x, b0.y, tab), neg_log_q58<false>(b0.z, b0.w, tab),
+                        neg_log_q58<false>(b1.x, b1.y, tab), neg_log_q58<false>(b1.z, b1.w, tab)};
+        };
+        FTMap f = ftmap_identity();
+        const uint32_t every = saturation_mask(lam, mu1, mu2, mu3);
+        auto push = [&](long long n, const Draw& d) {
+            f = ftmap_push(f, to_fix(d.a, cl), to_fix(d.s1, c1), to_fix(d.s2, c2), to_fix(d.s3, c3f));
             if ((static_cast<uint32_t>(n - lo) & every) == every) ftmap_saturate(f);
-        }
+        };
+        for (long long n = lo; n < hi; ++n) push(n, draw(n));
         ftmap_saturate(f);
         // block exclusive scan of the maps
         FTMap incl = f;
@@ -1160,41 +1173,47 @@ __global__ void __launch_bounds__(kTandemThreads) tandem3_cta_kernel(const doubl
         bool bad = v3 >= kFixGuard;
         U96 sy;
         double wa = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
-        const double i_lam = 0x1p-58 / lam, i_mu1 = 0x1p-58 / mu1, i_mu2 = 0x1p-58 / mu2,
-                     i_mu3 = 0x1p-58 / mu3;
-        for (long long n = lo; n < hi && !bad; ++n) {
-            uint4 b0, b1;
-            philox_row2(row, static_cast<uint32_t>(n), rk, b0, b1);
-            const unsigned long long ya = neg_log_q58<false>(b0.x, b0.y, tab);
-            const unsigned long long y1 = neg_log_q58<false>(b0.z, b0.w, tab);
-            const unsigned long long y2 = neg_log_q58<false>(b1.x, b1.y, tab);
-            const unsigned long long y3 = neg_log_q58<false>(b1.z, b1.w, tab);
-            tandem_step(v1, v2, v3, to_fix(ya, cl), to_fix(y1, c1), to_fix(y2, c2), to_fix(y3, c3f));
+        double i_lam = 0.0, i_mu1 = 0.0, i_mu2 = 0.0, i_mu3 = 0.0;
+        const bool early = __any_sync(kFull, lo < w_len);  // the warp has clients of the early window
+        if (early) {
+            i_lam = 0x1p-58 / lam;
+            i_mu1 = 0x1p-58 / mu1;
+            i_mu2 = 0x1p-58 / mu2;
+            i_mu3 = 0x1p-58 / mu3;
+        }
+        auto step = [&](long long n, const Draw& d) {
+            tandem_step(v1, v2, v3, to_fix(d.a, cl), to_fix(d.s1, c1), to_fix(d.s2, c2), to_fix(d.s3, c3f));
             sy.add(v3);
             if (n < w_len) {
-                wa += __ull2double_rn(ya) * i_lam;
-                w1 += __ull2double_rn(y1) * i_mu1;
-                w2 += __ull2double_rn(y2) * i_mu2;
-                w3 += __ull2double_rn(y3) * i_mu3;
+                wa += __ull2double_rn(d.a) * i_lam;
+                w1 += __ull2double_rn(d.s1) * i_mu1;
+                w2 += __ull2double_rn(d.s2) * i_mu2;
+                w3 += __ull2double_rn(d.s3) * i_mu3;
             }
             bad = v3 >= kFixGuard;
-        }
+        };
+        for (long long n = lo; n < hi && !bad; ++n) step(n, draw(n));
         const bool cta_bad = __syncthreads_or(bad) != 0;
         bool any_bad = cta_bad;
         if (!cta_bad) {
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {  // lane-ordered tree (integers: exact)
                 const U96 oy = shfl_down_u96(sy, off);
-                const double oa = __shfl_down_sync(kFull, wa, off);
-                const double o1 = __shfl_down_sync(kFull, w1, off);
-                const double o2 = __shfl_down_sync(kFull, w2, off);
-                const double o3 = __shfl_down_sync(kFull, w3, off);
-                if ((lane & (2 * off - 1)) == 0) {
-                    add_u96(sy, oy);
-                    wa += oa;
-                    w1 += o1;
-                    w2 += o2;
-                    w3 += o3;
+                if ((lane & (2 * off - 1)) == 0) add_u96(sy, oy);
+            }
+            if (early) {
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const double oa = __shfl_down_sync(kFull, wa, off);
+                    const double o1 = __shfl_down_sync(kFull, w1, off);
+                    const double o2 = __shfl_down_sync(kFull, w2, off);
+                    const double o3 = __shfl_down_sync(kFull, w3, off);
+                    if ((lane & (2 * off - 1)) == 0) {
+                        wa += oa;
+                        w1 += o1;
+                        w2 += o2;
+                        w3 += o3;
+                    }
                 }
             }
             if (lane == 0) {
@@ -1427,8 +1446,10 @@ extern "C" mrip_status mrip_tandem3_simulate(const double* d_dps, int32_t n_dp, 
     } else if (mapping == MRIP_MAP_CTA) {
         if (n_items > 0x7FFFFFFFll) return fail(MRIP_EINVAL, "mrip_tandem3_simulate: too many replications for CTA");
         CtaShape shape;
-        mrip_status cs = cta_shape(tandem3_cta_kernel<false>, tandem3_cta_kernel<true>, n_items, n_clients,
-                                   n_items > sm_count() ? kTandemThreads / 2 : kTandemThreads, false, &shape);
+        const long long sms = sm_count();
+        const int most = n_items > 2 * sms ? kTandemThreads / 4 : n_items > sms ? kTandemThreads / 2 : kTandemThreads;
+        mrip_status cs = cta_shape(tandem3_cta_kernel<false>, tandem3_cta_kernel<true>, n_items, n_clients, most, false,
+                                   &shape);
         if (cs != MRIP_OK) return cs;
         cs = launch_ctas(shape.ctas > 1 ? tandem3_cta_kernel<true> : tandem3_cta_kernel<false>, n_items, shape, st, d_dps, static_cast<long long>(n_reps),
                          static_cast<long long>(rep0), static_cast<long long>(n_clients),
