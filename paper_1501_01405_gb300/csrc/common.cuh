@@ -259,8 +259,8 @@ struct __align__(16) LogSlice {
 };
 
 struct LogTable {
-    // entry kLogSlices + j is slice j (the pointer is kLogSlices entries
-    // before the first, so that the leading one need not be masked off)
+    // entry kLogSlices + j is slice j (the leading one need not be masked off),
+    // the entries before are zero
     const ulonglong2* slice;
     const unsigned long long* nln2;  // [s] = round((s + 1) ln 2 2^58), s = 0..63; [64] see neg_log_q58
     uint32_t nln2_shared;            // the same table in the CTA's shared memory (stage_nln2)
@@ -297,9 +297,12 @@ __device__ __forceinline__ uint32_t mad_hi_u32(uint32_t a, uint32_t b, uint32_t 
 }
 
 // -log(1 - u) * 2^58, u = top 53 bits of hi:lo times 2^-53.  kShared: n ln 2
-// from the copy stage_nln2 made.
-template <bool kShared>
-__device__ __forceinline__ unsigned long long neg_log_q58(uint32_t lo, uint32_t hi, const LogTable& tab) {
+// from the copy stage_nln2 made.  kRare: takes every u; otherwise *top is negative
+// for the 2^-32 of the words it does not (their result is meaningless, the
+// look-ups stay within the tables: s held to 64, any 14 bits).
+template <bool kShared, bool kRare>
+__device__ __forceinline__ unsigned long long neg_log_impl(uint32_t lo, uint32_t hi, const LogTable& tab, uint32_t* top) {
+    static_assert(kShared || kRare, "the global table has no look-up for s = -1");
     // K 2^11 = 2^64 - (hi:lo without its 11 lowest bits); 0 stands for K = 2^53
     const unsigned long long K = 0ull - ((static_cast<unsigned long long>(hi) << 32) | (lo & 0xFFFFF800u));
     const uint32_t kh = static_cast<uint32_t>(K >> 32), kl = static_cast<uint32_t>(K);
@@ -307,15 +310,19 @@ __device__ __forceinline__ unsigned long long neg_log_q58(uint32_t lo, uint32_t 
     asm("bfind.shiftamt.u32 %0, %1;" : "=r"(s) : "r"(kh));
     uint32_t mh = __funnelshift_lc(kl, kh, s);
     asm("shl.b32 %0, %1, %2;" : "=r"(ml) : "r"(kl), "r"(s));  // 0 for s >= 32
-    while (static_cast<int>(s) < 0) {  // kh = 0 (s = 2^32 - 1), once in 2^32 draws: one turn
-        s = 32u + static_cast<uint32_t>(__clz(kl));
-        mh = kl ? kl << (s & 31u) : 0x80000000u;  // K = 2^53: M = 1, s = 64
-        ml = 0u;
+    if constexpr (kRare) {
+        while (static_cast<int>(s) < 0) {  // kh = 0 (s = 2^32 - 1), once in 2^32 draws: one turn
+            s = 32u + static_cast<uint32_t>(__clz(kl));
+            mh = kl ? kl << (s & 31u) : 0x80000000u;  // K = 2^53: M = 1, s = 64
+            ml = 0u;
+        }
+    } else {
+        *top = s;
     }
     const ulonglong2 e = __ldg(tab.slice + (mh >> (31 - kLogSliceBits)));
     unsigned long long nln2;
     if constexpr (kShared)
-        asm("ld.shared.u64 %0, [%1];" : "=l"(nln2) : "r"(tab.nln2_shared + 8u * s));
+        asm("ld.shared.u64 %0, [%1];" : "=l"(nln2) : "r"(tab.nln2_shared + 8u * (kRare ? s : min(s, 64u))));
     else
         nln2 = __ldg(tab.nln2 + s);
     const uint32_t w = static_cast<uint32_t>(e.y);
@@ -327,6 +334,35 @@ __device__ __forceinline__ unsigned long long neg_log_q58(uint32_t lo, uint32_t 
     const float f = __int2float_rn(a);
     const float tail = __fmaf_rn(f * f * f, __fmaf_rn(f, kLogR4, kLogR3), kLogMagic);  // -2 r^3/3 + r^4/2
     return nln2 + e.x - V + ((r2 + (__float_as_uint(tail) - kLogMagicBits)) >> 1);
+}
+
+template <bool kShared>
+__device__ __forceinline__ unsigned long long neg_log_q58(uint32_t lo, uint32_t hi, const LogTable& tab) {
+    return neg_log_impl<kShared, true>(lo, hi, tab, nullptr);
+}
+
+// kN logarithms with one branch for the rare words of all: y[i] from words
+// (lo[i], hi[i]), n ln 2 from the copy stage_nln2 made.  It saves a branch with
+// its reconvergence, a compare and moves per logarithm, and keeps the words
+// alive: 65,536 M/M/1 replications x 1,000 clients 500 -> 475 us (eight at a
+// time).  The tandem's kernels, short of registers and bound by the multiply
+// pipe, gain nothing (119 ms) or lose 4 % (a replication per CTA).  s is held to 64
+// rather than the copy moved up by an entry for s = -1: any offset there cost the
+// tandem 0.3 % (this kernel 472 us).
+template <int kN>
+__device__ __forceinline__ void neg_log_many(const uint32_t (&lo)[kN], const uint32_t (&hi)[kN], const LogTable& tab,
+                                             unsigned long long (&y)[kN]) {
+    uint32_t rare = 0u;
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+        uint32_t top;
+        y[i] = neg_log_impl<true, false>(lo[i], hi[i], tab, &top);
+        rare |= top;
+    }
+    if (__builtin_expect(static_cast<int>(rare) < 0, 0)) {
+#pragma unroll
+        for (int i = 0; i < kN; ++i) y[i] = neg_log_q58<true>(lo[i], hi[i], tab);
+    }
 }
 
 // Exponential variate from words (lo, hi): -log(1 - u) * inv_rate_q58 where

@@ -120,8 +120,8 @@ __device__ __forceinline__ void mm1_client(uint32_t n, const RowKey& row, double
 // Clients whose variates are drawn together: 2^16 replications are 13.5 warps
 // per SM, too few to hide one client's chain of Philox rounds and logarithms
 // behind other warps.  2^16 replications x 1,000 clients at 1, 2, 3 and 4 clients:
-// 561, 526, 504, 500 us (the last with 114 registers; a minimum of three CTAs per
-// SM leaves them).
+// 561, 526, 504, 500 us, and 475 with one branch for the rare words of a group's
+// eight logarithms (128 registers: a minimum of three CTAs per SM leaves them).
 constexpr uint32_t kMm1Group = 4;
 
 template <bool kLane0Only>
@@ -157,11 +157,21 @@ __global__ void __launch_bounds__(128, 3) mm1_serial_kernel(const double* __rest
         auto clients = [&](uint32_t n, auto count) {
             constexpr int kCount = decltype(count)::value;
             long long s_[kCount], a_[kCount];
+            uint32_t lo[2 * kCount], hi[2 * kCount];
+            unsigned long long y[2 * kCount];
 #pragma unroll
             for (int i = 0; i < kCount; ++i) {
                 const uint4 b = philox_row(row, n + i, rk);
-                s_[i] = to_fix(neg_log_q58<true>(b.x, b.y, tab), cmu);
-                a_[i] = to_fix(neg_log_q58<true>(b.z, b.w, tab), cl);
+                lo[2 * i] = b.x;
+                hi[2 * i] = b.y;
+                lo[2 * i + 1] = b.z;
+                hi[2 * i + 1] = b.w;
+            }
+            neg_log_many<2 * kCount>(lo, hi, tab, y);
+#pragma unroll
+            for (int i = 0; i < kCount; ++i) {
+                s_[i] = to_fix(y[2 * i], cmu);
+                a_[i] = to_fix(y[2 * i + 1], cl);
             }
             long long any = 0;
 #pragma unroll
@@ -1084,7 +1094,7 @@ __global__ void __launch_bounds__(kMm1CtaThreads) mm1_cta_kernel(
 //
 // One CTA per replication leaves the SMs without one idle, so few replications
 // are split over clusters of up to 8 CTAs (cta_shape): 16 x 100,000 clients run on
-// 112 SMs instead of 16, 439 -> 102 us.  FP64 is kept to the warps that need it
+// 96 SMs instead of 16, 439 -> 102 us.  FP64 is kept to the warps that need it
 // (its pipe takes a warp instruction every 16 cycles, however few lanes are
 // active): the four multipliers by four lanes for the CTA, the reciprocals and
 // the sums of the early window only in the warps that hold its clients: 90 us.

@@ -139,6 +139,8 @@ mrip_status log_table(LogTable* out) {
             nln2[s] = static_cast<unsigned long long>(prod >> 6);
         }
         nln2[64] = 0ull - log_core(0x80000000u, 0u, t[0]);
+        // before the first slice stand zeros, for the look-ups of rare words (neg_log_impl)
+        t.insert(t.begin(), kLogSlices, LogSlice{0, 0, 0});
         const size_t slice_bytes = t.size() * sizeof(LogSlice);
         LogSlice* p = nullptr;
         cudaError_t e = cudaMalloc(&p, slice_bytes + nln2.size() * sizeof(unsigned long long));
@@ -152,10 +154,9 @@ mrip_status log_table(LogTable* out) {
         }
         d.log_slices = p;
     }
-    out->slice = reinterpret_cast<const ulonglong2*>(reinterpret_cast<uintptr_t>(d.log_slices) -
-                                                     kLogSlices * sizeof(LogSlice));
+    out->slice = reinterpret_cast<const ulonglong2*>(d.log_slices);
     out->nln2_shared = 0;
-    out->nln2 = reinterpret_cast<const unsigned long long*>(d.log_slices + kLogSlices);
+    out->nln2 = reinterpret_cast<const unsigned long long*>(d.log_slices + 2 * kLogSlices);
     return MRIP_OK;
 }
 

@@ -813,6 +813,22 @@ def test_mm1_cta_few_clients(eng, torch_mod, n_clients):
             np.testing.assert_allclose(g.cpu().numpy(), r, rtol=REL, atol=1e-14)
 
 
+@pytest.mark.parametrize("mapping", ["THREAD", "WARP_1LANE", "WARP_COOP", "CTA"])
+@pytest.mark.parametrize("n_clients", [549, 550, 551, 560])
+def test_mm1_rare_word(eng, torch_mod, mapping, n_clients):
+    """Client 549 of replication 2,479,712 under seed 3 draws an all-ones leading word (one in 2^32, the logarithm's
+    rare path); as no client, as the last one alone or in a group, and followed by others."""
+    assert oracle.stream_block(3, 0, 0, 2479712, 549, 0)[0][1] == 0xFFFFFFFF
+    m = eng.Model(eng.MRIP_MM1, n_clients=n_clients)
+    m.set_plan('{"mapping": %d}' % getattr(eng, "MRIP_MAP_" + mapping))
+    dps, lo, n = np.array([[0.9, 1.0]]), 2479700, 40
+    m.run_range(dps, lo, lo + n, 3)
+    dp, rep = oracle.all_items(1, n)
+    for w, r in enumerate(oracle.mm1(dps, dp, rep + lo, n_clients, 3, threads=threads())):
+        np.testing.assert_allclose(m.outputs(w), r, rtol=REL, atol=1e-14)
+    m.close()
+
+
 @pytest.mark.parametrize("n_reps", [31, 32, 33, 63, 65, 256])
 def test_stats_reduce_few(eng, torch_mod, n_reps):
     """Fewer values than the CTA has warps' worth: the warps without an element add nothing."""
