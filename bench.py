@@ -63,21 +63,20 @@ IMUL_PER_CLK_SM = 64      # 32-bit integer multiply / multiply-add results
 DFMA_PER_CLK_SM = 2       # FP64 fused multiply-add results (1.25 TFLOP/s nominal)
 INT_MULS_PER_PHILOX = 40  # 10 rounds x 2 products x (low + high half)
 # one gap of the skip-sampled lattice: half a Philox block (20) + the
-# fixed-point log's seven 64x64-bit products, each four 32-bit products (28)
-MULS_PER_GAP = 48
-# one exponential variate in 48-bit fixed point: the log's products (26: the
-# 64x64-bit m * 1/c and r^2, the 32-bit tail, n ln 2) + the 64x64-bit scaling
-# by 2^-9 / rate (8)
-MULS_PER_FIXED_VARIATE = 34
+# fixed-point log's products (4)
+MULS_PER_GAP = 24
+# one exponential variate in 48-bit fixed point: the log's products (4: the
+# mantissa's two words by 1/c, both halves of the first, and r^2's high half)
+# + the scaling by 2^-9 / rate (4: one product in full, two by their high halves)
+MULS_PER_FIXED_VARIATE = 8
 
 
 # DRAM bytes (read + write) per launch of a dominant kernel, from the ncu
 # capture summarised in profiles/ (None once the kernel changes).  The 256^2
 # kernel was captured on 4 of its 128 replications per design point (256 of
-# 8,192 CTAs: 37,888 B read, 0 written during the launch -- per-CTA design
-# points, constants and code; the counts stay in L2) and is scaled by the
-# replications of a full launch (x32).
-PROFILED_TRAFFIC = {"forest_fire_kernel<8>": 399360 * 32}
+# 8,192 CTAs: 2.07 MB read, 1.88 MB written during the launch, of 2.05 MB of
+# counts) and is scaled by the replications of a full launch (x32).
+PROFILED_TRAFFIC = {"forest_fire_kernel<8>": 3950000 * 32}
 
 
 # Issue slots: 4 schedulers per SM, one warp instruction each per clock.
@@ -86,7 +85,10 @@ ISSUE_PER_CLK_SM = 4
 # Philox4x32-10 block (15-20 integer instructions) plus the bit-parallel
 # rule (32 cells per word); the midpoint 17.5 is the algorithmic figure.
 FF_INSTR_PER_CELL = 17.5
-FF_MUL_WIDE_PER_WORD = 137  # widening multiplies per 32-cell lattice word and step
+# Widening multiplies per 32-cell lattice word and step, where what a step or
+# a word shares is computed once.  The kernel draws several steps at a time and
+# executes 122; the figure stays the one of a step by itself.
+FF_MUL_WIDE_PER_WORD = 137
 
 
 def issue_peak_g():
@@ -191,7 +193,7 @@ class ForestFire(Workload):
                     mul_wide=dict(work=cells * FF_MUL_WIDE_PER_WORD / 32.0 / 32.0,
                                   per_unit="%d widening multiplies per 32-cell word and step (8 "
                                            "Philox blocks x 17, two per-step products shared, "
-                                           "+ 1), 32 per warp instruction" % FF_MUL_WIDE_PER_WORD))
+                                           "+ 1; 122 are executed), 32 per warp instruction" % FF_MUL_WIDE_PER_WORD))
 
     def extra_rates(self, reps_per_s, torch):
         w = self.w
@@ -427,7 +429,7 @@ class Queue(Workload):
                     peak_source="nominal: %d SMs x %d int-mul/clk x %.0f MHz" % (
                         SMS, IMUL_PER_CLK_SM, SM_MAX_MHZ),
                     per_unit="%d int multiplies per client: %d Philox block(s) (40 each) + %d "
-                             "fixed-point variates (%d each: log 26, scaling 8)" % (
+                             "fixed-point variates (%d each: log 4, scaling 4)" % (
                                  per_client, blocks, logs, MULS_PER_FIXED_VARIATE))
 
     def make_model(self):

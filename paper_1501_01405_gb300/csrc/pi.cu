@@ -32,8 +32,9 @@ __device__ __forceinline__ void add_outside(uint32_t x, uint32_t y, uint32_t& ou
 // What bounds it is the FMA-heavy pipe (16 widening multiplies of Philox per
 // block of two draws and 4 of the squares, 4.2 cycles each: 84 of the 87 cycles a
 // warp takes).  Measured, 64 replications x 10^7 draws: 0.921 -> 0.700 ms (row keys
-// alone 0.809); one replication 29.0 -> 17.7 us,
-// 3 x 200,001 draws 23 -> 9.8 us.  The test in FP32 with an exact second look needs two multiplies less but four conversions more: 0.717 ms.
+// alone 0.809); one replication 29.0 -> 17.7 us, 3 x 200,001 draws 23 -> 9.8 us.  The
+// test in FP32 with an exact second look needs two multiplies less but four
+// conversions more: 0.717 ms.
 __global__ void __launch_bounds__(kPiThreads) pi_kernel(long long n_draws, long long chunk, long long chunks, long long rep0,
                                                         const __grid_constant__ RoundKeys rk,
                                                         unsigned long long* __restrict__ hits) {
