@@ -165,29 +165,37 @@ bool same_plan(const Plan& a, const Plan& b) {
            a.ctas_per_sm == b.ctas_per_sm && a.chunk == b.chunk;
 }
 
-// Size buffers and upload the per-shape tables; host_dps already validated.
+// Size the run's buffers; host_dps already validated.  The earlier run's
+// results are given up here: until the new run is launched there are none.
+// A buffer that grows moves, whether or not the call then succeeds, so the
+// graph that was captured with its address goes first.
 mrip_status prepare(mrip_model* m, int32_t n_dp, int64_t n_reps) {
     const size_t items = static_cast<size_t>(n_dp) * n_reps;
     m->n_dp = n_dp;
     m->n_reps = n_reps;
+    m->has_run = false;
     m->back_valid = false;
-    bool ok = m->dps.ensure(static_cast<size_t>(n_dp) * dp_dim(m->kind) * sizeof(double)) &&
-              m->nmm2.ensure(static_cast<size_t>(n_dp) * 3 * sizeof(double));
+    auto fit = [m](DevBuf& buf, size_t bytes) {
+        if (!buf.holds(bytes)) m->drop_graph();
+        return buf.ensure(bytes);
+    };
+    bool ok = fit(m->dps, static_cast<size_t>(n_dp) * dp_dim(m->kind) * sizeof(double)) &&
+              fit(m->nmm2, static_cast<size_t>(n_dp) * 3 * sizeof(double));
     const size_t spart = stats_scratch_bytes(n_dp, n_reps);
-    if (spart) ok = ok && m->spart.ensure(spart);
+    if (spart) ok = ok && fit(m->spart, spart);
     switch (m->kind) {
-        case MRIP_MM1: ok = ok && m->out0.ensure(3 * items * sizeof(double)); break;
+        case MRIP_MM1: ok = ok && fit(m->out0, 3 * items * sizeof(double)); break;
         case MRIP_TANDEM3:
-            ok = ok && m->out0.ensure(items * sizeof(double)) && m->out1.ensure(8 * items * sizeof(double));
+            ok = ok && fit(m->out0, items * sizeof(double)) && fit(m->out1, 8 * items * sizeof(double));
             break;
         case MRIP_FOREST_FIRE:
-            ok = ok && m->out0.ensure(items * m->ff.n_steps * sizeof(int32_t)) &&
-                 m->out1.ensure(items * sizeof(double));
+            ok = ok && fit(m->out0, items * m->ff.n_steps * sizeof(int32_t)) &&
+                 fit(m->out1, items * sizeof(double));
             break;
         case MRIP_WALK_L1_EXIT:
-            ok = ok && m->out0.ensure(items * sizeof(int64_t)) &&
-                 m->walk_tab.ensure(2 * static_cast<size_t>(n_dp) * sizeof(int32_t)) &&
-                 m->ticket.ensure(sizeof(unsigned long long));
+            ok = ok && fit(m->out0, items * sizeof(int64_t)) &&
+                 fit(m->walk_tab, 2 * static_cast<size_t>(n_dp) * sizeof(int32_t)) &&
+                 fit(m->ticket, sizeof(unsigned long long));
             break;
     }
     if (!ok) return fail(MRIP_ENOMEM, "mrip_run: device allocation failed");
@@ -210,10 +218,7 @@ mrip_status run_common(mrip_model* m, int32_t n_dp, int64_t n_reps, uint64_t see
     const bool reuse = m->exec && m->g_n_dp == n_dp && m->g_n_reps == n_reps && m->g_rep0 == m->rep0 &&
                        m->g_seed == seed && same_plan(m->g_plan, m->plan);
     if (!reuse) {
-        if (m->exec) {
-            cudaGraphExecDestroy(m->exec);
-            m->exec = nullptr;
-        }
+        m->drop_graph();
         // the stage launchers touch lazily created tables; create them before capture
         sm_count();
         LogTable tab;
@@ -485,9 +490,9 @@ extern "C" mrip_status mrip_run_range(mrip_model* m, const double* design_points
     const int64_t n_reps = rep_hi - rep_lo;
     mrip_status s = check_shape(m, n_dp, n_reps, rep_lo);
     if (s != MRIP_OK) return s;
-    m->rep0 = rep_lo;
     s = check_dps(m->kind, design_points, n_dp);
     if (s != MRIP_OK) return s;
+    m->rep0 = rep_lo;
     const size_t nval = static_cast<size_t>(n_dp) * dp_dim(m->kind);
     m->host_dps.assign(design_points, design_points + nval);
     s = prepare(m, n_dp, n_reps);
@@ -508,17 +513,19 @@ extern "C" mrip_status mrip_run_device(mrip_model* m, const double* d_design_poi
     if (!m || !d_design_points) return fail(MRIP_EINVAL, "mrip_run_device: null argument");
     mrip_status s = check_shape(m, n_dp, n_reps);
     if (s != MRIP_OK) return s;
-    m->rep0 = 0;
+    // validation, before anything of the handle changes, and the walk's
+    // processing order need the values on the host
     const size_t nval = static_cast<size_t>(n_dp) * dp_dim(m->kind);
-    s = prepare(m, n_dp, n_reps);
-    if (s != MRIP_OK) return s;
-    // validation and the walk's processing order need the values on the host
-    m->host_dps.resize(nval);
-    cudaError_t e = cudaMemcpyAsync(m->host_dps.data(), d_design_points, nval * sizeof(double),
-                                    cudaMemcpyDeviceToHost, m->stream);
+    std::vector<double> dps(nval);
+    cudaError_t e = cudaMemcpyAsync(dps.data(), d_design_points, nval * sizeof(double), cudaMemcpyDeviceToHost,
+                                    m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return cuda_status(e, "mrip_run_device: design point read");
-    s = check_dps(m->kind, m->host_dps.data(), n_dp);
+    s = check_dps(m->kind, dps.data(), n_dp);
+    if (s != MRIP_OK) return s;
+    m->rep0 = 0;
+    m->host_dps.swap(dps);
+    s = prepare(m, n_dp, n_reps);
     if (s != MRIP_OK) return s;
     e = cudaMemcpyAsync(m->dps.p, d_design_points, nval * sizeof(double), cudaMemcpyDeviceToDevice,
                         m->stream);

@@ -23,8 +23,9 @@ struct DevBuf {
     ~DevBuf() {
         if (p) cudaFree(p);
     }
+    bool holds(size_t bytes) const { return p && bytes <= cap; }
     bool ensure(size_t bytes) {
-        if (bytes <= cap && p) return true;
+        if (holds(bytes)) return true;
         if (p) {
             cudaFree(p);
             p = nullptr;
@@ -85,7 +86,8 @@ struct mrip_model {
     DevBuf cv_theta;
     std::vector<double> cv_norm;
     int cv_d_in = 0;
-    // graph cache
+    // graph cache: the graph holds the addresses of the buffers above and is
+    // dropped before one of them moves
     cudaGraphExec_t exec = nullptr;
     int32_t g_n_dp = -1;
     int64_t g_n_reps = -1;
@@ -93,9 +95,11 @@ struct mrip_model {
     uint64_t g_seed = 0;
     bool g_back = false;  // the graph ends with the copy to `back`
     Plan g_plan;
-    ~mrip_model() {
+    void drop_graph() {
         if (exec) cudaGraphExecDestroy(exec);
+        exec = nullptr;
     }
+    ~mrip_model() { drop_graph(); }
 };
 
 namespace mrip {

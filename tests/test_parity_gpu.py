@@ -862,3 +862,52 @@ def test_results_returned_with_a_small_run(eng, torch_mod, kind, dp, kw, dtypes,
             t.cuda.synchronize()
             m.set_stream(other)
     m.close()
+
+
+@pytest.mark.parametrize("kind,dp,kw,dtypes", [
+    ("MM1", [0.9, 1.0], dict(n_clients=50), ["f8", "f8", "f8"]),
+    ("TANDEM3", [0.8, 1.0, 1.1, 1.2], dict(n_clients=50, window=10), ["f8", "f8"]),
+    ("FOREST_FIRE", [0.01, 1e-4], dict(L=32, n_steps=3, density=0.5, window=2), ["i4", "f8"]),
+    ("WALK_L1_EXIT", [4.0], dict(max_steps=1 << 38), ["i8"]),
+])
+def test_run_after_a_refused_run(eng, torch_mod, kind, dp, kw, dtypes):
+    """A run that is refused between two runs of one shape and seed, by its design points (the earlier results
+    stay) or by a plane larger than the device (there are none then): the second run gives the first one's results,
+    on the host and on the device, whatever buffer moved in between."""
+    t = torch_mod
+    m = eng.Model(getattr(eng, "MRIP_" + kind), **kw)
+    with pytest.raises(eng.MripError) as e:
+        m.outputs(0)
+    assert e.value.code == 5  # ESTATE
+    dps = np.array([dp])
+
+    def results():
+        host = [m.outputs(w, dtype=np.dtype(ty)) for w, ty in enumerate(dtypes)]
+        for w, h in enumerate(host):
+            on_dev = t.empty(h.size, dtype={"f8": t.float64, "i4": t.int32, "i8": t.int64}[dtypes[w]], device="cuda")
+            eng.mrip_outputs(m.h, w, on_dev)
+            assert np.array_equal(h, on_dev.cpu().numpy())
+        return host + [m.moments()]
+
+    def equal(a, b):
+        return all(np.array_equal(x, y) for x, y in zip(a, b))
+
+    m.run(dps, 10, 3)
+    first = results()
+    with pytest.raises(eng.MripError) as e:
+        eng.mrip_run_device(m.h, dev(t, np.repeat(-dps, 2, axis=0)), 1 << 16, 3)
+    assert e.value.code == 1  # EINVAL
+    assert equal(results(), first)
+    m.run(dps, 10, 3)
+    assert equal(results(), first)
+    if kind == "MM1":  # 3 planes of 8 x (2^32 - 1) doubles, 824 GB
+        with pytest.raises(eng.MripError) as e:
+            eng.mrip_run(m.h, np.repeat(dps, 8, axis=0), 0xFFFFFFFF, 3)
+        assert e.value.code == 2  # ENOMEM
+        for call in (lambda: m.outputs(0), m.moments, m.stats):
+            with pytest.raises(eng.MripError) as e:
+                call()
+            assert e.value.code == 5  # ESTATE
+        m.run(dps, 10, 3)
+        assert equal(results(), first)
+    m.close()
