@@ -1441,7 +1441,7 @@ mrip_status mlp_train(const TrainSpec& sp, TrainInfo* info, cudaStream_t st) {
     e = cudaMemcpyAsync(h, base, 32, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // also: the host schedule dies at return
     if (e != cudaSuccess) return cuda_status(e, "mlp train (tensor cores)");
-    if (h[4]) return fail(MRIP_ECUDA, "mlp train: a tensor-core MMA did not complete in time");
+    if (h[4]) return fail(MRIP_ECUDA, "mlp train: a tensor-core product or an exchange between CTAs did not complete in time");
     if (info) {
         info->epochs_run = h[0];
         info->best_epoch = h[1];
