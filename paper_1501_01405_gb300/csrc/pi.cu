@@ -22,10 +22,9 @@ constexpr long long kPiChunk = 1LL << 16, kPiLeast = 1LL << 12;  // most and lea
 // with the complement of y^2 took four instructions more).
 __device__ __forceinline__ void add_outside(uint32_t x, uint32_t y, uint32_t& outside) {
     uint32_t hi, lo;
-    [[maybe_unused]] uint32_t s0, s1;
     mul_wide_u32(x, x, hi, lo);
-    asm("mad.lo.cc.u32 %0, %3, %3, %4;\n\tmadc.hi.cc.u32 %1, %3, %3, %5;\n\taddc.u32 %2, %2, 0;"
-        : "=r"(s0), "=r"(s1), "+r"(outside)
+    asm("{\n .reg .u32 sum;\n mad.lo.cc.u32 sum, %1, %1, %2;\n madc.hi.cc.u32 sum, %1, %1, %3;\n addc.u32 %0, %0, 0;\n}"
+        : "+r"(outside)
         : "r"(y), "r"(lo), "r"(hi));
 }
 

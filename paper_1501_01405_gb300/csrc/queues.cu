@@ -75,7 +75,10 @@ struct U96 {
     __device__ __forceinline__ void add(unsigned long long v) { add(v, 0u); }
     __device__ __forceinline__ void add(unsigned long long v, uint32_t v_hi) {
         uint32_t l0 = static_cast<uint32_t>(lo), l1 = static_cast<uint32_t>(lo >> 32);
-        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        // (the low words wait in registers of the statement's own: %0 and %1 may not
+        // change before every input has been read)
+        asm("{\n .reg .u32 a, b;\n add.cc.u32 a, %0, %3;\n addc.cc.u32 b, %1, %4;\n addc.u32 %2, %2, %5;\n"
+            " mov.u32 %0, a;\n mov.u32 %1, b;\n}"
             : "+r"(l0), "+r"(l1), "+r"(hi)
             : "r"(static_cast<uint32_t>(v)), "r"(static_cast<uint32_t>(v >> 32)), "r"(v_hi));
         lo = (static_cast<unsigned long long>(l1) << 32) | l0;
