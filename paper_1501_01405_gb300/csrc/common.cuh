@@ -322,7 +322,10 @@ __device__ __forceinline__ unsigned long long neg_log_impl(uint32_t lo, uint32_t
     const ulonglong2 e = __ldg(tab.slice + (mh >> (31 - kLogSliceBits)));
     unsigned long long nln2;
     if constexpr (kShared)
-        asm("ld.shared.u64 %0, [%1];" : "=l"(nln2) : "r"(tab.nln2_shared + 8u * (kRare ? s : min(s, 64u))));
+        asm volatile("ld.shared.u64 %0, [%1];"
+                     : "=l"(nln2)
+                     : "r"(tab.nln2_shared + 8u * (kRare ? s : min(s, 64u)))
+                     : "memory");  // (after stage_nln2's barrier)
     else
         nln2 = __ldg(tab.nln2 + s);
     const uint32_t w = static_cast<uint32_t>(e.y);

@@ -6,8 +6,8 @@ import re
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1501_01405_gb300", "csrc")
-# statements that order memory accesses, or make or take data of another thread or unit
-ORDERING = re.compile(r"mbarrier|barrier\.cta|bar\.sync|fence|cp\.async|tcgen05|ld\.shared::cluster")
+# statements that order memory accesses, or take data that another thread or unit made
+ORDERING = re.compile(r"mbarrier|barrier\.cta|bar\.sync|fence|cp\.async|tcgen05|\bld\.(?!param)")
 
 
 def statements():
