@@ -61,13 +61,18 @@ size_t plane_bytes(const mrip_model* m, int which) {
     return 0;
 }
 
-// Results of up to this many bytes return to the host with the run: the last
-// node of its graph writes the moments and the outputs to page-locked memory,
-// and mrip_stats, mrip_moments and mrip_outputs synchronise and read them
-// there.  A device-to-host copy per call, issued after the run, to pageable
-// memory, costs about 10 us each; the node costs about 2 us and grows by the
-// bytes, so the line is where it is still one small CTA's work.  M/M/1, 32 x 1,000
-// clients, run + interval + one output: 47.6 -> 34.6 us.
+// Results of up to this many bytes go to the host together, by a kernel that
+// writes the moments and all outputs to page-locked memory, where mrip_stats,
+// mrip_moments and mrip_outputs read them after a synchronisation.  A
+// device-to-host copy per call to pageable memory costs about 10 us each; the
+// kernel is one small CTA's work.  It is the last node of the run's graph until a
+// run of the handle goes unread by the host; from then on, and for the walk, the
+// first read after a run launches it.  M/M/1, 32 x 1,000 clients, run + interval +
+// one output: 48.2 us by copies, 32.0 with the node, 36.3 launched by the read.  The
+// run alone: 16.6 us with the node, 14.6 without; with a new seed, that has the graph
+// captured anew, 25.4 and 23.5.  A walk waits for the run before it (its table's
+// upload), so the node's time would always show: 400 walks to 16, run + output on
+// the device 86.6 us with it, 83.1 without.
 constexpr size_t kBackBytes = 4096;
 
 size_t moment_bytes(const mrip_model* m) { return static_cast<size_t>(m->n_dp) * 3 * sizeof(double); }
@@ -87,7 +92,7 @@ __global__ void __launch_bounds__(256) back_kernel(const uint32_t* __restrict__ 
         host[i] = i < na ? a[i] : i < na + nb ? b[i - na] : c[i - na - nb];
 }
 
-mrip_status enqueue_back(mrip_model* m) {
+mrip_status launch_back(mrip_model* m) {
     const bool two = m->kind == MRIP_TANDEM3 || m->kind == MRIP_FOREST_FIRE;  // planes in out0 and out1
     const size_t b0 = two ? plane_bytes(m, 0) : back_offset(m, 3) - moment_bytes(m);
     const size_t b1 = two ? plane_bytes(m, 1) : 0;
@@ -95,22 +100,35 @@ mrip_status enqueue_back(mrip_model* m) {
                                           m->out0.as<uint32_t>(), static_cast<uint32_t>(b0 / 4),
                                           m->out1.as<uint32_t>(), static_cast<uint32_t>(b1 / 4),
                                           static_cast<uint32_t*>(m->back.p));
-    return launch_status("mrip_run: results to the host");
+    return launch_status("results to the host");
 }
 
-// `bytes` of results at byte `at` of `back`, or at `src` on the device, to host memory.
+bool small_results(const mrip_model* m) { return back_offset(m, 3) <= kBackBytes; }
+
+// `bytes` of results at byte `at` of `back`, or at `src` on the device, to host
+// memory.  `back` serves only on the run's stream, where the read is behind the run
+// (on another one that is the caller's affair, and what is read may not be kept).
 mrip_status read_back(mrip_model* m, size_t at, const void* src, size_t bytes, void* dst, const char* what) {
-    bool here = m->back_valid && m->back_stream == m->stream;
+    bool here = small_results(m) && m->run_stream == m->stream;
     cudaPointerAttributes attr{};
     if (here && (cudaPointerGetAttributes(&attr, dst) != cudaSuccess || attr.type == cudaMemoryTypeDevice)) {
         cudaGetLastError();  // not host memory: the copy below refuses it
         here = false;
     }
+    here = here && m->back.ensure(kBackBytes);
+    if (here && !m->back_valid) {
+        mrip_status s = launch_back(m);
+        if (s != MRIP_OK) return s;
+    }
     cudaError_t e = cudaSuccess;
     if (!here) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return cuda_status(e, what);
-    if (here) std::memcpy(dst, static_cast<const char*>(m->back.p) + at, bytes);
+    if (here) {
+        m->back_valid = true;
+        std::memcpy(dst, static_cast<const char*>(m->back.p) + at, bytes);
+    }
+    m->unread = false;
     return MRIP_OK;
 }
 
@@ -215,7 +233,9 @@ mrip_status run_common(mrip_model* m, int32_t n_dp, int64_t n_reps, uint64_t see
         if (e != cudaSuccess) return cuda_status(e, "mrip_run: table upload");
         if (!device_error_flags()) return fail(MRIP_ENOMEM, "device error flags");
     }
-    const bool reuse = m->exec && m->g_n_dp == n_dp && m->g_n_reps == n_reps && m->g_rep0 == m->rep0 &&
+    m->back_on_read = m->back_on_read || m->unread;
+    const bool to_back = small_results(m) && m->kind != MRIP_WALK_L1_EXIT && !m->back_on_read && m->back.ensure(kBackBytes);
+    const bool reuse = m->exec && m->g_back == to_back && m->g_n_dp == n_dp && m->g_n_reps == n_reps && m->g_rep0 == m->rep0 &&
                        m->g_seed == seed && same_plan(m->g_plan, m->plan);
     if (!reuse) {
         m->drop_graph();
@@ -224,7 +244,6 @@ mrip_status run_common(mrip_model* m, int32_t n_dp, int64_t n_reps, uint64_t see
         LogTable tab;
         mrip_status ts = log_table(&tab);
         if (ts != MRIP_OK) return ts;
-        const bool to_back = back_offset(m, 3) <= kBackBytes && m->back.ensure(kBackBytes);
         cudaStream_t cap = m->stream;
         bool own = false;
         if (cap == nullptr) {  // the legacy stream cannot be captured
@@ -239,7 +258,7 @@ mrip_status run_common(mrip_model* m, int32_t n_dp, int64_t n_reps, uint64_t see
         mrip_status s = MRIP_OK;
         if (e == cudaSuccess) {
             s = enqueue_run(m, seed);
-            if (s == MRIP_OK && to_back) s = enqueue_back(m);
+            if (s == MRIP_OK && to_back) s = launch_back(m);
             cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
             if (s == MRIP_OK && e2 != cudaSuccess) s = cuda_status(e2, "mrip_run: capture");
         } else {
@@ -267,8 +286,9 @@ mrip_status run_common(mrip_model* m, int32_t n_dp, int64_t n_reps, uint64_t see
     cudaError_t e = cudaGraphLaunch(m->exec, m->stream);
     if (e != cudaSuccess) return cuda_status(e, "mrip_run: graph launch");
     m->has_run = true;
-    m->back_valid = m->g_back;
-    m->back_stream = m->stream;
+    m->run_stream = m->stream;
+    m->back_valid = to_back;
+    m->unread = true;
     return MRIP_OK;
 }
 
@@ -652,6 +672,7 @@ extern "C" mrip_status mrip_autotune(mrip_model* m, const double* design_points,
     }
     const std::vector<Plan> cands = candidates(m->kind);
     const Plan saved = m->plan;
+    const bool on_read = m->back_on_read || m->unread;  // (the trials' unread runs do not count)
     float best_ms = 1e30f;
     Plan best = saved;
     std::vector<char> ref, cur;
@@ -690,6 +711,8 @@ extern "C" mrip_status mrip_autotune(mrip_model* m, const double* design_points,
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    m->back_on_read = on_read;
+    m->unread = false;
     if (s != MRIP_OK) {
         m->plan = saved;
         return s;

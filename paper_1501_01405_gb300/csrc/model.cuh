@@ -74,8 +74,10 @@ struct mrip_model {
     int64_t n_reps = 0;
     int64_t rep0 = 0;  // replication index of output column 0 (mrip_run_range)
     bool has_run = false;
-    bool back_valid = false;              // `back` holds the last run's results once back_stream is synchronised
-    cudaStream_t back_stream = nullptr;
+    bool back_valid = false;             // `back` holds the last run's results once run_stream is synchronised
+    cudaStream_t run_stream = nullptr;   // the last run's
+    bool unread = false;                 // the host has read nothing of the last run
+    bool back_on_read = false;           // a run went unread: `back` is written by the first read, not by the run
     // the control variate's working buffers (kept between mrip_run_cv calls)
     // and the network of the last one
     struct {
@@ -93,8 +95,8 @@ struct mrip_model {
     int64_t g_n_reps = -1;
     int64_t g_rep0 = -1;
     uint64_t g_seed = 0;
-    bool g_back = false;  // the graph ends with the copy to `back`
     Plan g_plan;
+    bool g_back = false;  // the graph ends with the copy to `back`
     void drop_graph() {
         if (exec) cudaGraphExecDestroy(exec);
         exec = nullptr;

@@ -911,3 +911,34 @@ def test_run_after_a_refused_run(eng, torch_mod, kind, dp, kw, dtypes):
         m.run(dps, 10, 3)
         assert equal(results(), first)
     m.close()
+
+
+@pytest.mark.parametrize("unread", [False, True])
+def test_small_results_read_on_another_stream(eng, torch_mod, unread):
+    """A run read first on another stream, then on its own, and by moments, statistics and outputs in any order, on a
+    handle whose every run is read (by a node of the run's graph) and on one with unread runs (by the read)."""
+    t = torch_mod
+    m = eng.Model(eng.MRIP_TANDEM3, n_clients=60, window=10)
+    own, other = t.cuda.Stream(), t.cuda.Stream()
+    reads = {"moments": m.moments, "stats": lambda: np.array([list(d.values()) for d in m.stats()]),
+             "y": lambda: m.outputs(0), "features": lambda: m.outputs(1)}
+    seen = []
+    for seed, streams, order in ((3, (own, own), ("moments", "stats", "y", "features")),
+                                 (3, (other, own), ("features", "y", "stats", "moments")),
+                                 (3, (own, other), ("y", "moments", "features", "stats")),
+                                 (4, (other, own), ("stats", "features", "moments", "y"))):
+        m.set_stream(own)
+        if unread:
+            m.run(np.array([[0.7, 1.0, 1.1, 1.2]]), 20, seed)
+        m.run(np.array([[0.8, 1.0, 1.1, 1.2]]), 20, seed)
+        t.cuda.synchronize()
+        got = []
+        for st in streams:
+            m.set_stream(st)
+            got.append({k: reads[k]() for k in order})
+        assert all(np.array_equal(got[0][k], got[1][k]) for k in order)
+        seen.append(got[0])
+    for k in reads:
+        assert np.array_equal(seen[0][k], seen[1][k]) and np.array_equal(seen[0][k], seen[2][k])
+        assert not np.array_equal(seen[0][k], seen[3][k])
+    m.close()
