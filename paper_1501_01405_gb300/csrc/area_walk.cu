@@ -7,9 +7,10 @@
 // the walker's area grows by one.  Outputs: final area and 30 visit counts.
 //
 // Mappings:
-//   THREAD      one replication per thread; a table of every cell's four
-//               successors and one histogram per thread ([area][thread]: the
-//               per-move scatter never conflicts on a bank) in shared memory;
+//   THREAD      one replication per thread; one histogram per thread
+//               ([area][thread]: the per-move scatter never conflicts on a bank)
+//               and, from 64 moves, a table of every cell's four successors in
+//               shared memory;
 //   WARP_1LANE  one replication per warp, lane 0 only (the paper's WLP);
 //   WARP_COOP   one replication per warp: a round covers 512 moves, lane l
 //               takes moves 16l .. 16l+15, a warp scan of the 16-move
@@ -36,6 +37,44 @@ __device__ __forceinline__ void move(uint32_t f, int& x, int& y) {
     }
 }
 
+// THREAD and WARP_1LANE, walks of fewer than kTableMoves moves: two coordinates,
+// and the area by division.  The table below costs a CTA 3,000 entries and 61 KB before
+// its first move, which short walks do not earn back.  300,000 replications x 1,
+// 10, 30, 63 moves: 8.5, 9.8, 16.4, 26.8 us here, 18.6, 20.6, 24.7, 30.8 with the
+// table; x 64 28 and 24.  16,384 replications by one lane per warp x 1, 30, 63 moves: 8.7,
+// 24.4, 41.2 and 30.9, 39.1, 49.3; x 64 45 and 37.
+constexpr int kTableMoves = 64;
+
+template <bool kLane0Only>
+__global__ void __launch_bounds__(kThreads) area_walk_short_kernel(long long rep0, long long n_reps, int n_steps,
+                                                                   const __grid_constant__ RoundKeys rk,
+                                                                   int32_t* __restrict__ final_area,
+                                                                   int32_t* __restrict__ visits) {
+    constexpr int kWalkers = kLane0Only ? kThreads / 32 : kThreads;
+    static_assert(kTableMoves <= 64, "the moves of one Philox block");
+    __shared__ uint32_t hist[kAreas][kWalkers];
+    if (kLane0Only && (threadIdx.x & 31) != 0) return;
+    const int slot = kLane0Only ? threadIdx.x >> 5 : threadIdx.x;
+    const long long item = blockIdx.x * static_cast<long long>(kWalkers) + slot;
+    if (item >= n_reps) return;
+    for (int a = 0; a < kAreas; ++a) hist[a][slot] = 0u;
+    int x = kW / 2, y = kH / 2;
+    const uint4 b = philox(0u, 0u, static_cast<uint32_t>(rep0 + item), stream_word(0u, 0u), rk);
+    const uint32_t words[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t w = words[k];
+        for (int s = 16 * k; s < min(16 * k + 16, n_steps); ++s, w >>= 2) {
+            move(w & 3u, x, y);
+            const int a = area_of(x, y);
+            if (MRIP_CHECK(a >= 0 && a < kAreas, 604, a)) hist[a][slot] += 1u;
+        }
+    }
+    final_area[item] = area_of(x, y);
+    if (visits)
+        for (int a = 0; a < kAreas; ++a) visits[a * n_reps + item] = static_cast<int32_t>(hist[a][slot]);
+}
+
 // THREAD and WARP_1LANE.  A move is one table look-up: cell c of area a has the
 // code 128 a + c, and next[code] holds the codes (times 8) of its four
 // successors, so the walker's state is e = 8 code, 16 bits; e | 2 f is the byte
@@ -46,8 +85,8 @@ __device__ __forceinline__ void move(uint32_t f, int& x, int& y) {
 // 38).  What bounds it is shared memory: the look-ups of 32 walkers conflict
 // on about 3.4 banks.  The counter's own column makes the addition race-free, but
 // the one-way atomic beats a load, an add and a store (53 us).  Measured, 65,536
-// replications x 1,000 moves: 102.4 -> 43.1 us; 300,001 x 701: 254 -> 117; 500 x
-// 1,013: 47 -> 29.
+// replications x 1,000 moves: 102.7 -> 43.2 us, x 100 14.4 -> 10.4; 300,000 x 300 112 ->
+// 55.5; 16,384 x 1,000 by one lane per warp 596 -> 152.
 constexpr int kSerialThreads = 256;
 constexpr int kCodes = 128 * kAreas;
 static_assert(4 * kSerialThreads == 1024, "a histogram row is 1 << 10 bytes: the area bits of e");
@@ -104,9 +143,10 @@ __global__ void __launch_bounds__(kSerialThreads) area_walk_serial_kernel(long l
                 for (int s = 1; s < 16; ++s) step(words[k] >> (2 * s - 1));
             }
         } else {
-            for (int s = 0; s < n_steps - m0; ++s) {
-                const uint32_t w = (s >> 4) == 0 ? b.x : (s >> 4) == 1 ? b.y : (s >> 4) == 2 ? b.z : b.w;
-                step(((w >> (2 * (s & 15))) & 3u) << 1);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                uint32_t w = words[k];
+                for (int s = m0 + 16 * k; s < min(m0 + 16 * k + 16, n_steps); ++s, w >>= 2) step(w << 1);
             }
         }
     }
@@ -170,11 +210,21 @@ __global__ void __launch_bounds__(kThreads) area_walk_coop_kernel(long long rep0
     if (visits && lane < kAreas) visits[lane * n_reps + item] = static_cast<int32_t>(hist[warp][lane]);
 }
 
-template <class Kernel>
-mrip_status serial_smem(Kernel kernel) {
-    return cuda_status(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            static_cast<int>(sizeof(SerialSmem))),
-                       "mrip_area_walk_simulate: shared memory attribute");
+template <bool kLane0Only>
+mrip_status launch_serial(int64_t rep0, int64_t n_reps, int32_t n_steps, const RoundKeys& rk, int32_t* d_final_area,
+                          int32_t* d_visits, cudaStream_t st) {
+    const int64_t threads = kLane0Only ? n_reps * 32 : n_reps;
+    if (n_steps < kTableMoves) {
+        area_walk_short_kernel<kLane0Only><<<ceil_div_u(threads, kThreads), kThreads, 0, st>>>(rep0, n_reps, n_steps, rk,
+                                                                                             d_final_area, d_visits);
+        return MRIP_OK;
+    }
+    cudaError_t e = cudaFuncSetAttribute(area_walk_serial_kernel<kLane0Only>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(sizeof(SerialSmem)));
+    if (e != cudaSuccess) return cuda_status(e, "mrip_area_walk_simulate: shared memory attribute");
+    area_walk_serial_kernel<kLane0Only><<<ceil_div_u(threads, kSerialThreads), kSerialThreads, sizeof(SerialSmem), st>>>(
+        rep0, n_reps, n_steps, rk, d_final_area, d_visits);
+    return MRIP_OK;
 }
 
 }  // namespace
@@ -194,15 +244,11 @@ extern "C" mrip_status mrip_area_walk_simulate(int64_t rep0, int64_t n_reps, int
     const RoundKeys rk = expand_key(seed);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (mapping == MRIP_MAP_AUTO || mapping == MRIP_MAP_THREAD) {
-        const mrip_status s = serial_smem(area_walk_serial_kernel<false>);
+        const mrip_status s = launch_serial<false>(rep0, n_reps, n_steps, rk, d_final_area, d_visits, st);
         if (s != MRIP_OK) return s;
-        area_walk_serial_kernel<false><<<ceil_div_u(n_reps, kSerialThreads), kSerialThreads, sizeof(SerialSmem), st>>>(
-            rep0, n_reps, n_steps, rk, d_final_area, d_visits);
     } else if (mapping == MRIP_MAP_WARP_1LANE) {
-        const mrip_status s = serial_smem(area_walk_serial_kernel<true>);
+        const mrip_status s = launch_serial<true>(rep0, n_reps, n_steps, rk, d_final_area, d_visits, st);
         if (s != MRIP_OK) return s;
-        area_walk_serial_kernel<true><<<ceil_div_u(n_reps * 32, kSerialThreads), kSerialThreads, sizeof(SerialSmem), st>>>(
-            rep0, n_reps, n_steps, rk, d_final_area, d_visits);
     } else if (mapping == MRIP_MAP_WARP_COOP) {
         area_walk_coop_kernel<<<ceil_div_u(n_reps * 32, kThreads), kThreads, 0, st>>>(rep0, n_reps, n_steps, rk,
                                                                                      d_final_area, d_visits);

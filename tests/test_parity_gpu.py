@@ -942,3 +942,18 @@ def test_small_results_read_on_another_stream(eng, torch_mod, unread):
         assert np.array_equal(seen[0][k], seen[1][k]) and np.array_equal(seen[0][k], seen[2][k])
         assert not np.array_equal(seen[0][k], seen[3][k])
     m.close()
+
+
+@pytest.mark.parametrize("mapping", ["THREAD", "WARP_1LANE"])
+@pytest.mark.parametrize("n_steps", [0, 1, 16, 17, 63, 64, 65])
+def test_area_walk_short(eng, torch_mod, mapping, n_steps):
+    """Walks on both sides of the line from which a move is a table look-up (64), with replications on both sides of a
+    CTA's walkers."""
+    t = torch_mod
+    for n in (1, 4, 129, 300):
+        fa = t.full((n,), -1, dtype=t.int32, device="cuda")
+        vis = t.full((30, n), -1, dtype=t.int32, device="cuda")
+        eng.mrip_area_walk_simulate(n, n_steps, 9, getattr(eng, "MRIP_MAP_" + mapping), fa, vis, rep0=77)
+        ref_f, ref_v = oracle.area_walk(77 + np.arange(n), n_steps, 9, threads=threads())
+        assert np.array_equal(fa.cpu().numpy(), ref_f)
+        assert np.array_equal(vis.cpu().numpy().T, ref_v)
