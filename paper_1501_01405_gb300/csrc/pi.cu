@@ -9,6 +9,8 @@
 // 10^7-draw replication fills the whole GPU by itself; each CTA reduces its count (warp reduction, then
 // shared memory) and adds it to the replication's counter with one 64-bit
 // atomic -- integer addition, so the result does not depend on the order.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace mrip {
@@ -16,6 +18,7 @@ namespace {
 
 constexpr int kPiThreads = 256;
 constexpr long long kPiChunk = 1LL << 16, kPiLeast = 1LL << 12;  // most and least draws per CTA (even)
+constexpr long long kPiFew = 768;
 
 // outside += 1 if x^2 + y^2 >= 2^64: the carry out of the 64-bit sum, taken by
 // the multiply that adds y^2 to x^2 (two multiplies and an add; comparing x^2
@@ -34,10 +37,13 @@ __device__ __forceinline__ void add_outside(uint32_t x, uint32_t y, uint32_t& ou
 // alone 0.809); one replication 29.0 -> 17.7 us, 3 x 200,001 draws 23 -> 9.8 us.  The
 // test in FP32 with an exact second look needs two multiplies less but four
 // conversions more: 0.717 ms.
+// kFew: any number of threads up to kPiThreads.
+template <bool kFew>
 __global__ void __launch_bounds__(kPiThreads) pi_kernel(long long n_draws, long long chunk, long long chunks, long long rep0,
                                                         const __grid_constant__ RoundKeys rk,
                                                         unsigned long long* __restrict__ hits) {
     __shared__ uint32_t part[kPiThreads / 32];
+    const uint32_t threads = kFew ? blockDim.x : kPiThreads;
     const long long rep = blockIdx.x / chunks;
     const long long start = (blockIdx.x - rep * chunks) * chunk;
     const uint32_t draws = static_cast<uint32_t>(min(chunk, n_draws - start));
@@ -45,7 +51,7 @@ __global__ void __launch_bounds__(kPiThreads) pi_kernel(long long n_draws, long 
     const uint32_t first = static_cast<uint32_t>(start / 2), pairs = draws / 2;  // whole blocks
     uint32_t outside = 0;
 #pragma unroll 2
-    for (uint32_t b = threadIdx.x; b < pairs; b += kPiThreads) {
+    for (uint32_t b = threadIdx.x; b < pairs; b += threads) {
         const uint4 w = philox_row(row, first + b, rk);
         add_outside(w.x, w.y, outside);
         add_outside(w.z, w.w, outside);
@@ -59,7 +65,7 @@ __global__ void __launch_bounds__(kPiThreads) pi_kernel(long long n_draws, long 
     __syncthreads();
     if (threadIdx.x == 0) {
         uint32_t tot = 0;
-        for (int i = 0; i < kPiThreads / 32; ++i) tot += part[i];
+        for (uint32_t i = 0; i < threads / 32; ++i) tot += part[i];
         atomicAdd(hits + rep, static_cast<unsigned long long>(draws - tot));
     }
 }
@@ -85,7 +91,15 @@ extern "C" mrip_status mrip_pi_simulate(int64_t rep0, int64_t n_reps, int64_t n_
     while (chunk > kPiLeast && ctas() * n_reps < 8ll * sm_count()) chunk /= 2;
     const long long chunks = ctas();
     if (chunks * n_reps > 0x7FFFFFFFll) return fail(MRIP_EINVAL, "mrip_pi_simulate: too many draws in total");
-    pi_kernel<<<static_cast<unsigned>(chunks * n_reps), kPiThreads, 0, st>>>(
+    // Replications of fewer than kPiFew draws spread them evenly over as many threads
+    // as one or two rounds need: 100,000 replications of 1, 100, 300, 600 draws take 57, 57,
+    // 107, 148 us so and 86, 96, 120, 164 with 256 threads; of 1,000 (the loop's stride is no
+    // constant here) 226 and 205.
+    const long long pairs = std::max<long long>(1, n_draws / 2), rounds = (pairs + kPiThreads - 1) / kPiThreads;
+    const bool few = n_draws < kPiFew;
+    const unsigned threads = few ? static_cast<unsigned>(((pairs + rounds - 1) / rounds + 31) / 32 * 32) : kPiThreads;
+    auto* kernel = few ? pi_kernel<true> : pi_kernel<false>;
+    kernel<<<static_cast<unsigned>(chunks * n_reps), threads, 0, st>>>(
         n_draws, chunk, chunks, rep0, expand_key(seed), reinterpret_cast<unsigned long long*>(d_hits));
     return launch_status("mrip_pi_simulate");
 }

@@ -957,3 +957,12 @@ def test_area_walk_short(eng, torch_mod, mapping, n_steps):
         ref_f, ref_v = oracle.area_walk(77 + np.arange(n), n_steps, 9, threads=threads())
         assert np.array_equal(fa.cpu().numpy(), ref_f)
         assert np.array_equal(vis.cpu().numpy().T, ref_v)
+
+
+@pytest.mark.parametrize("n_draws", [1, 2, 3, 63, 64, 65, 66, 130, 511, 512, 513, 515, 766, 767, 768])
+def test_pi_few_draws(eng, torch_mod, n_draws):
+    """Few draws: CTAs of 32 threads and up, one and two rounds, up to the line (768) of the full CTA."""
+    t = torch_mod
+    hits = t.full((70,), -1, dtype=t.int64, device="cuda")
+    eng.mrip_pi_simulate(70, n_draws, 5, hits, rep0=11)
+    assert np.array_equal(hits.cpu().numpy(), oracle.pi_hits(11 + np.arange(70), n_draws, 5, threads=threads()))
