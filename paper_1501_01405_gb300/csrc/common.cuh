@@ -302,7 +302,6 @@ __device__ __forceinline__ uint32_t mad_hi_u32(uint32_t a, uint32_t b, uint32_t 
 // look-ups stay within the tables: s held to 64, any 14 bits).
 template <bool kShared, bool kRare>
 __device__ __forceinline__ unsigned long long neg_log_impl(uint32_t lo, uint32_t hi, const LogTable& tab, uint32_t* top) {
-    static_assert(kShared || kRare, "the global table has no look-up for s = -1");
     // K 2^11 = 2^64 - (hi:lo without its 11 lowest bits); 0 stands for K = 2^53
     const unsigned long long K = 0ull - ((static_cast<unsigned long long>(hi) << 32) | (lo & 0xFFFFF800u));
     const uint32_t kh = static_cast<uint32_t>(K >> 32), kl = static_cast<uint32_t>(K);
@@ -327,7 +326,7 @@ __device__ __forceinline__ unsigned long long neg_log_impl(uint32_t lo, uint32_t
                      : "r"(tab.nln2_shared + 8u * (kRare ? s : min(s, 64u)))
                      : "memory");  // (after stage_nln2's barrier)
     else
-        nln2 = __ldg(tab.nln2 + s);
+        nln2 = __ldg(tab.nln2 + (kRare ? s : min(s, 64u)));
     const uint32_t w = static_cast<uint32_t>(e.y);
     uint32_t v_hi, v_lo;
     mul_wide_u32(mh, w, v_hi, v_lo);
@@ -345,26 +344,26 @@ __device__ __forceinline__ unsigned long long neg_log_q58(uint32_t lo, uint32_t 
 }
 
 // kN logarithms with one branch for the rare words of all: y[i] from words
-// (lo[i], hi[i]), n ln 2 from the copy stage_nln2 made.  It saves a branch with
+// (lo[i], hi[i]); kShared: n ln 2 from the copy stage_nln2 made.  It saves a branch with
 // its reconvergence, a compare and moves per logarithm, and keeps the words
 // alive: 65,536 M/M/1 replications x 1,000 clients 500 -> 475 us (eight at a
 // time).  The tandem's kernels, short of registers and bound by the multiply
 // pipe, gain nothing (119 ms) or lose 4 % (a replication per CTA).  s is held to 64
 // rather than the copy moved up by an entry for s = -1: any offset there cost the
 // tandem 0.3 % (this kernel 472 us).
-template <int kN>
+template <int kN, bool kShared>
 __device__ __forceinline__ void neg_log_many(const uint32_t (&lo)[kN], const uint32_t (&hi)[kN], const LogTable& tab,
                                              unsigned long long (&y)[kN]) {
     uint32_t rare = 0u;
 #pragma unroll
     for (int i = 0; i < kN; ++i) {
         uint32_t top;
-        y[i] = neg_log_impl<true, false>(lo[i], hi[i], tab, &top);
+        y[i] = neg_log_impl<kShared, false>(lo[i], hi[i], tab, &top);
         rare |= top;
     }
     if (__builtin_expect(static_cast<int>(rare) < 0, 0)) {
 #pragma unroll
-        for (int i = 0; i < kN; ++i) y[i] = neg_log_q58<true>(lo[i], hi[i], tab);
+        for (int i = 0; i < kN; ++i) y[i] = neg_log_q58<kShared>(lo[i], hi[i], tab);
     }
 }
 

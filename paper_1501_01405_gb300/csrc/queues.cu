@@ -120,6 +120,29 @@ __device__ __forceinline__ void mm1_client(uint32_t n, const RowKey& row, double
     a = expo_fast<kShared>(b.z, b.w, tab, inv_lam);
 }
 
+// Clients n .. n + kCount - 1 in FP64, their logarithms with one branch for the rare words.
+template <int kCount>
+__device__ __forceinline__ void mm1_clients(uint32_t n, const RowKey& row, double inv_lam, double inv_mu,
+                                            const RoundKeys& rk, const LogTable& tab, double (&s)[kCount],
+                                            double (&a)[kCount]) {
+    uint32_t lo[2 * kCount], hi[2 * kCount];
+    unsigned long long y[2 * kCount];
+#pragma unroll
+    for (int i = 0; i < kCount; ++i) {
+        const uint4 b = philox_row(row, n + i, rk);
+        lo[2 * i] = b.x;
+        hi[2 * i] = b.y;
+        lo[2 * i + 1] = b.z;
+        hi[2 * i + 1] = b.w;
+    }
+    neg_log_many<2 * kCount, false>(lo, hi, tab, y);
+#pragma unroll
+    for (int i = 0; i < kCount; ++i) {
+        s[i] = __ull2double_rn(y[2 * i]) * inv_mu;
+        a[i] = __ull2double_rn(y[2 * i + 1]) * inv_lam;
+    }
+}
+
 // Clients whose variates are drawn together: 2^16 replications are 13.5 warps
 // per SM, too few to hide one client's chain of Philox rounds and logarithms
 // behind other warps.  2^16 replications x 1,000 clients at 1, 2, 3 and 4 clients:
@@ -170,7 +193,7 @@ __global__ void __launch_bounds__(128, 3) mm1_serial_kernel(const double* __rest
                 lo[2 * i + 1] = b.z;
                 hi[2 * i + 1] = b.w;
             }
-            neg_log_many<2 * kCount>(lo, hi, tab, y);
+            neg_log_many<2 * kCount, true>(lo, hi, tab, y);
 #pragma unroll
             for (int i = 0; i < kCount; ++i) {
                 s_[i] = to_fix(y[2 * i], cmu);
@@ -230,7 +253,13 @@ __device__ __forceinline__ MaxPlus compose(MaxPlus f, MaxPlus g) {
     return r;
 }
 
-// One warp per replication; clients staged in shared memory when kStage.
+// One warp per replication; clients staged in shared memory when kStage.  What bounds
+// it is the latency of a client's chain (few warps per SM, and the staged slices leave
+// its L1 little room for the logarithm's 128 KB table), so kMm1WarpGroup clients are
+// drawn together: 500 x 1,000 clients 46.0 -> 41.2 us, 32 x 1,000 43.4 -> 39.2, 150 x 5,000
+// 185 -> 169 (four together 43.2, 39.2, 165, but 1,500 x 150 20.6 instead of 18.6).
+constexpr int kMm1WarpGroup = 2;
+
 template <bool kStage>
 __global__ void mm1_warp_coop_kernel(const double* __restrict__ dps, long long n_items,
                                      long long n_reps, long long rep0, long long n_clients,
@@ -255,18 +284,31 @@ __global__ void mm1_warp_coop_kernel(const double* __restrict__ dps, long long n
     const bool staged =
         kStage && MRIP_CHECK((warp_in_cta + 1ull) * 2 * seg * 32 * sizeof(double) <= dynamic_smem_bytes(), 201, seg);
 
+    auto for_clients = [&](long long from, long long to, auto use) {
+        long long n = from;
+        for (; n + kMm1WarpGroup <= to; n += kMm1WarpGroup) {
+            double s[kMm1WarpGroup], a[kMm1WarpGroup];
+            mm1_clients<kMm1WarpGroup>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, s, a);
+#pragma unroll
+            for (int i = 0; i < kMm1WarpGroup; ++i) use(n + i, s[i], a[i]);
+        }
+        for (; n < to; ++n) {
+            double s, a;
+            mm1_client<false>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, s, a);
+            use(n, s, a);
+        }
+    };
+
     // pass 1: the segment's composed map
     MaxPlus f{-INFINITY, 0.0};
-    for (long long n = lo; n < hi; ++n) {
-        double s, a;
-        mm1_client<false>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, s, a);
+    auto map = [&](long long n, double s, double a) {
         if (staged) {
             s_buf[(n - lo) * 32 + lane] = s;
             a_buf[(n - lo) * 32 + lane] = a;
         }
-        MaxPlus step{0.0, s - a};
-        f = compose(f, step);
-    }
+        f = compose(f, MaxPlus{0.0, s - a});
+    };
+    for_clients(lo, hi, map);
     // inclusive scan of maps over lanes (earlier lanes first), then shift
     MaxPlus acc = f;
 #pragma unroll
@@ -284,20 +326,18 @@ __global__ void mm1_warp_coop_kernel(const double* __restrict__ dps, long long n
 
     // pass 2: replay the segment with the plain recurrence
     double sum_w = 0.0, sum_i = 0.0, sum_v = 0.0;
-    for (long long n = lo; n < hi; ++n) {
-        double s, a;
-        if (staged) {
-            s = s_buf[(n - lo) * 32 + lane];
-            a = a_buf[(n - lo) * 32 + lane];
-        } else {
-            mm1_client<false>(static_cast<uint32_t>(n), row, inv_lam, inv_mu, rk, tab, s, a);
-        }
+    auto replay = [&](long long, double s, double a) {
         sum_w += w;
         const double v = w + s;
         sum_v += v;
         const double t = v - a;
         sum_i += (t < 0.0) ? -t : 0.0;
         w = (t > 0.0) ? t : 0.0;
+    };
+    if (staged) {
+        for (long long n = lo; n < hi; ++n) replay(n, s_buf[(n - lo) * 32 + lane], a_buf[(n - lo) * 32 + lane]);
+    } else {
+        for_clients(lo, hi, replay);
     }
     // fixed-order (lane-ordered tree) reduction of the three sums
 #pragma unroll
@@ -1409,8 +1449,13 @@ extern "C" mrip_status mrip_mm1_simulate(const double* d_dps, int32_t n_dp, int6
     } else if (mapping == MRIP_MAP_WARP_COOP) {
         const long long seg = (n_clients + 31) / 32;
         const size_t per_warp = static_cast<size_t>(seg) * 32 * 2 * sizeof(double);
+        // Staged where the slices leave an SM enough warps (24 KB: nine) or all of its
+        // replications fit it at once; else the second pass draws again.  Staged and not:
+        // 1,500 x 5,000 clients 742 and 307 us, 500 x 5,000 304 and 181, 5,000 x 2,000 484 and
+        // 381; 1,500 x 1,000 67 and 80, 700 x 2,000 80 and 105.
         const int warps = 1;
-        if (per_warp * warps <= 96 * 1024) {
+        const long long per_sm = (n_items + sm_count() - 1) / sm_count();
+        if (per_warp <= 24 * 1024 || (per_warp <= 96 * 1024 && per_warp * per_sm <= 220 * 1024)) {
             const size_t smem = per_warp * warps;
             if (smem > 48 * 1024)
                 cudaFuncSetAttribute(mm1_warp_coop_kernel<true>,

@@ -966,3 +966,23 @@ def test_pi_few_draws(eng, torch_mod, n_draws):
     hits = t.full((70,), -1, dtype=t.int64, device="cuda")
     eng.mrip_pi_simulate(70, n_draws, 5, hits, rep0=11)
     assert np.array_equal(hits.cpu().numpy(), oracle.pi_hits(11 + np.arange(70), n_draws, 5, threads=threads()))
+
+
+@pytest.mark.parametrize("n_clients", [767, 768, 769, 1025, 3073])
+def test_mm1_warp_staging(eng, torch_mod, n_clients):
+    """Warp mapping on both sides of the rule that keeps the variates of the first pass (slices of 24 KB, or as many
+    replications as fit an SM): the oracle's numbers from many replications and from one at a time."""
+    t = torch_mod
+    dps, n = np.array([[0.9, 1.0]]), 1600
+
+    def run(n, rep0):
+        out = [t.empty(n, dtype=t.float64, device="cuda") for _ in range(3)]
+        eng.mrip_mm1_simulate(dev(t, dps), n, n_clients, 3, eng.MRIP_MAP_WARP_COOP, *out, rep0=rep0)
+        return np.stack([o.cpu().numpy() for o in out])
+    many = run(n, 0)
+    some = np.arange(0, n, 50)
+    ref = oracle.mm1(dps, np.zeros(some.size, dtype=np.int32), some, n_clients, 3, threads=threads())
+    one = np.stack([run(1, r)[:, 0] for r in some[:6]], axis=1)
+    for g, h, r in zip(many[:, some], one, ref):
+        np.testing.assert_allclose(g, r, rtol=REL, atol=1e-14)
+        np.testing.assert_allclose(h, r[:6], rtol=REL, atol=1e-14)
