@@ -986,3 +986,11 @@ def test_mm1_warp_staging(eng, torch_mod, n_clients):
     for g, h, r in zip(many[:, some], one, ref):
         np.testing.assert_allclose(g, r, rtol=REL, atol=1e-14)
         np.testing.assert_allclose(h, r[:6], rtol=REL, atol=1e-14)
+
+
+@pytest.mark.parametrize("L", [32, 64, 128, 256, 512])
+@pytest.mark.parametrize("many", [False, True])
+@pytest.mark.parametrize("n_steps", [2, 3, 5, 11])
+def test_forest_fire_steps_beside_a_batch(eng, torch_mod, L, many, n_steps):
+    """The steps that do not fill a batch, an even and an odd number of them."""
+    test_forest_fire_batches_of_steps(eng, torch_mod, L, many, n_steps)
