@@ -696,18 +696,40 @@ __global__ void __launch_bounds__(ff_threads<W>(), skip_min_blocks<W>()) forest_
     if (!MRIP_CHECK((2u + 2u * NS) * NWORD * sizeof(uint32_t) <= dynamic_smem_bytes(), 107, NWORD)) return;
     const uint32_t dp = static_cast<uint32_t>(item / n_reps);
     const uint32_t rep = static_cast<uint32_t>(rep0 + item % n_reps);
+    // The scales of both sets by lanes 0 and 1 of the first warp and the lightning's
+    // threshold by the last one: logarithms and divisions in FP64, whose pipe a warp
+    // occupies as long as one lane does.  (By every thread for itself, 300 replications
+    // of 1 step took 130 us at L = 512, 53.5 at 256 and 26 at 128, and take 74, 24.7 and 14.4;
+    // 1,024 of 128 x 128 x 1,000 1.446 -> 1.406 ms.)  A CTA of one warp computes them in every
+    // lane: it has nothing to share out, and its rounds are up to 8 % faster so.
+    __shared__ GapScale gs[2];
+    __shared__ GapFast gf[2];
+    __shared__ unsigned long long none_from;
     const double p_grow = dps[2 * dp], p_light = dps[2 * dp + 1];
     const bool any_grow = p_grow > 0.0, any_light = p_light > 0.0;
-    const GapScale gs_grow = any_grow ? gap_scale(p_grow) : GapScale{0ull, 128};
-    const GapScale gs_light = any_light ? gap_scale(p_light) : GapScale{0ull, 128};
-    const GapFast gf_grow = gap_fast_scale(any_grow ? p_grow : 1.0);
-    const GapFast gf_light = gap_fast_scale(any_light ? p_light : 1.0);
-    const unsigned long long light_none = any_light ? first_gap_none(p_light, L * L) : 0ull;
+    if (W > 1 && warp == 0 && lane < 2) {
+        const double p = lane == 0 ? p_grow : p_light;
+        gs[lane] = p > 0.0 ? gap_scale(p) : GapScale{0ull, 128};
+        gf[lane] = gap_fast_scale(p > 0.0 ? p : 1.0);
+    }
+    if (W > 1 && warp == NWARP - 1 && lane == 0) none_from = any_light ? first_gap_none(p_light, L * L) : 0ull;
     const uint32_t c3_grow = stream_word(5u, dp), c3_light = stream_word(6u, dp);
 
     ff_load_initial<W, TPB>(ev_grow, burning, init, item, t_dens, rep, dp, rk);
     for (int i = threadIdx.x; i < 128; i += TPB) (&cnt[0][0])[i] = 0;
     __syncthreads();
+    GapScale gs_grow, gs_light;
+    GapFast gf_grow, gf_light;
+    unsigned long long light_none;
+    if constexpr (W == 1) {
+        gs_grow = any_grow ? gap_scale(p_grow) : GapScale{0ull, 128};
+        gs_light = any_light ? gap_scale(p_light) : GapScale{0ull, 128};
+        gf_grow = gap_fast_scale(any_grow ? p_grow : 1.0);
+        gf_light = gap_fast_scale(any_light ? p_light : 1.0);
+        light_none = any_light ? first_gap_none(p_light, L * L) : 0ull;
+    } else {
+        gs_grow = gs[0], gs_light = gs[1], gf_grow = gf[0], gf_light = gf[1], light_none = none_from;
+    }
     uint32_t t_row[W], b_row[W];
     row_load<W, W>(ev_grow, y, 0, t_row);
     row_load<W, W>(burning, y, 0, b_row);
