@@ -663,8 +663,13 @@ __device__ __forceinline__ void draw_events(uint32_t* __restrict__ ev, const Gap
     }
 }
 
-// 128 x 128: 1,024 replications are 6.7 CTAs per SM, so seven resident ones (72
-// registers) make one wave: 1.44 ms against 1.65 at the compiler's 85 registers.
+// Resident CTAs asked for at L = 128: seven (72 registers) are a compromise over the
+// replications.  200 steps of 100, 800, 1,024, 2,000, 10,000 replications take 148, 264, 300, 557,
+// 2,421 us with seven, 144, 255, 352, 565, 2,447 with the compiler's six (85 registers), 150,
+// 267, 302, 547, 2,368 with eight: six are 3 % faster while they hold every replication and
+// 15 % slower just beyond.  L = 64 and 32 take the compiler's choice: sixteen CTAs of 64 x
+// 64 gain 2 % from 4,000 replications (12 % where 2,000 just need them) and lose 2 to 6 %
+// below, more of 32 x 32 lose 3 to 5 % throughout.  From L = 256 shared memory holds two.
 template <int W>
 constexpr int skip_min_blocks() {
     return W == 4 ? 7 : 1;

@@ -53,6 +53,15 @@ constexpr long long kFixNegInf = -(1LL << 62);  // "empty" state: v - A stays ab
 // 3 is added instead of 2: the variate is then within one unit (2^-48) of
 // y58 2^-10 / rate.  cm < 2^62 keeps the sum of the middle halves (below
 // 1.15 2^31 + 2^30 + 4) in 32 bits, so the first additions ride on the multiplies.
+//
+// This rounding, not the logarithm, is the M/M/1 outputs' error.  With cl the low
+// word of cm, 1 + cl 2^-33 units are missing on average (a half where cl is 0), so a
+// variate is (1/2 - cl 2^-33)/4 of a unit too large on average, 1/4 where cl is 0 (mu = 1),
+// and S - A drifts by the difference within a busy period.  The error of one rate
+// therefore depends on the bits of its multiplier: mean waits of 400 random rates x
+// 32 replications x 1,000 clients are off by 3.3e-15 rms (relative, against 64-bit mantissas),
+// 3.2e-15 when a variate was (hi(y57 cm) + 3) >> 2 with cm = round(2^57 / rate); single
+// rates differ by a factor of two either way.
 __device__ __forceinline__ bool fix_rate_ok(double rate) { return rate >= 0x1p-6 && rate <= 0x1p4; }
 
 __device__ __forceinline__ unsigned long long fix_scale(double rate) {
@@ -143,11 +152,14 @@ __device__ __forceinline__ void mm1_clients(uint32_t n, const RowKey& row, doubl
     }
 }
 
-// Clients whose variates are drawn together: 2^16 replications are 13.5 warps
-// per SM, too few to hide one client's chain of Philox rounds and logarithms
-// behind other warps.  2^16 replications x 1,000 clients at 1, 2, 3 and 4 clients:
-// 561, 526, 504, 500 us, and 475 with one branch for the rare words of a group's
-// eight logarithms (128 registers: a minimum of three CTAs per SM leaves them).
+// Clients whose variates are drawn together: a thread per replication gives an SM too
+// few warps (13.5 at 2^16 replications) to hide one client's chain of Philox rounds and
+// logarithms behind other warps.  2^16 x 1,000 clients at 1, 2, 3 and 4 clients: 561, 526,
+// 504, 500 us, and 475 with one branch for the rare words of a group's eight
+// logarithms (128 registers: a minimum of three CTAs per SM leaves them).  The choice holds
+// over the range: 1,000, 16,384, 65,536, 262,144, 10^6 replications x 400 clients take 80, 80,
+// 198, 648, 2,350 us, with two clients and four CTAs 82, 82, 200, 647, 2,344, with one and six
+// 116, 115, 220, 672, 2,392.
 constexpr uint32_t kMm1Group = 4;
 
 template <bool kLane0Only>
