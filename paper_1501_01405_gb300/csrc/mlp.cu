@@ -420,8 +420,7 @@ struct TrainArgs {
 // M = 128, whose rows 64.. read neighbouring bytes and are not used.  Each
 // worker turns its 16 columns of a row of Z1 / Z2 / dH1 into activations,
 // residual and deltas (FP32, rounded to BF16 where the next contraction reads
-// them; a unit counts as on where its BF16 activation is not zero, so for
-// pre-activations above 2^-134).  The bias and W3 gradients are FP32 column
+// them; a unit is off where its BF16 activation has its sign set, see relu_signed).  The bias and W3 gradients are FP32 column
 // sums over the tile in a fixed order (chunks of 16 samples, then the chunks
 // in order), taken while the products run.  Four more warps: one issues the
 // products, one adds the output deltas and the squared residuals one after
@@ -554,6 +553,10 @@ __device__ __forceinline__ void put_weight(TcWeights& w, uint32_t at, ParamUse u
         *reinterpret_cast<float*>(dst) = use == kUseRounded ? bf(v) : v;
 }
 
+// max(x, 0), zero with a sign where the unit is off: BF16 rounds 0 < x <= 2^-134 to zero
+// too, but such a unit is on.
+__device__ __forceinline__ float relu_signed(float x) { return x > 0.0f ? x : -0.0f; }
+
 // Eight FP32 values rounded to BF16 (nearest even), the first at the lowest
 // address: one core-matrix row of 16 bytes.
 __device__ __forceinline__ uint4 pack_bf16x8(const float* w) {
@@ -685,14 +688,14 @@ __global__ void __cluster_dims__(kTcCluster, 1, 1) __launch_bounds__(kTcThreads,
             v[4 * g + 3] = a.w;
         }
     };
-    // v = 0 for the units whose activations, two times eight at h0 and h1, are zero
+    // v = 0 for the units that are off, by the signs of their activations, two times eight at h0 and h1
     auto zero_where_off = [&](const void* h0, const void* h1, float (&v)[16]) {
         const uint4 p = *static_cast<const uint4*>(h0), q = *static_cast<const uint4*>(h1);
         const uint32_t w[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
 #pragma unroll
         for (int j = 0; j < 16; j += 2) {
-            v[j] = (w[j / 2] & 0xFFFFu) ? v[j] : 0.0f;
-            v[j + 1] = (w[j / 2] & 0xFFFF0000u) ? v[j + 1] : 0.0f;
+            v[j] = (w[j / 2] & 0x8000u) ? 0.0f : v[j];
+            v[j + 1] = (w[j / 2] & 0x80000000u) ? 0.0f : v[j + 1];
         }
     };
     auto store16 = [&](float (*tile)[kRowF], const float (&v)[16]) {
@@ -707,8 +710,7 @@ __global__ void __cluster_dims__(kTcCluster, 1, 1) __launch_bounds__(kTcThreads,
     };
 
     // Forward pass of the tile in S.rows[buf] (not the fetching warps).  Leaves X~,
-    // H1~ and H2~ rows in shared memory (zero exactly where the unit is off: the
-    // ReLU masks); returns the output of row m without b3 (workers).
+    // H1~ and H2~ rows in shared memory (their signs are the ReLU masks); returns the output of row m without b3 (workers).
     auto forward_tile = [&](int buf) -> float {
         if (worker) {
             const float x0 = 2 * cb < d_in ? S.rows[buf][2 * cb][m] : 0.0f;
@@ -729,7 +731,7 @@ __global__ void __cluster_dims__(kTcCluster, 1, 1) __launch_bounds__(kTcThreads,
             units16(S.w[0].b1, b);
             tc::tmem_ld16(tm + lane_base + c0, z);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] = fmaxf(z[j] + b[j], 0.0f);
+            for (int j = 0; j < 16; ++j) z[j] = relu_signed(z[j] + b[j]);
             store16_bf(S.a2, z);
         }
         sync_for_mma_tile();
@@ -747,7 +749,7 @@ __global__ void __cluster_dims__(kTcCluster, 1, 1) __launch_bounds__(kTcThreads,
             // layer 2 epilogue: h2 and this block's share of the output
             tc::tmem_ld16(tm + lane_base + 64 + c0, z);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] = fmaxf(z[j] + b[j], 0.0f);
+            for (int j = 0; j < 16; ++j) z[j] = relu_signed(z[j] + b[j]);
             units16(S.w[0].w3, b);
             const uint4 packed[2] = {pack_bf16x8(z), pack_bf16x8(z + 8)};
             const uint32_t* word = &packed[0].x;
@@ -933,7 +935,7 @@ __global__ void __cluster_dims__(kTcCluster, 1, 1) __launch_bounds__(kTcThreads,
                         tc::mma_commit(&S.bar_w2);
                     }
                     if (worker) {
-                        // meanwhile: column sums of dZ2 (b2: dy w3 where h2~ is not zero) and, by
+                        // meanwhile: column sums of dZ2 (b2: dy w3 where the unit is on) and, by
                         // the odd column blocks' warps, of dy h2~ (W3); a chunk of 16 rows per
                         // warp, two columns per lane
                         const int chunk = 4 * (cb >> 1) + quarter, q0 = 16 * chunk;
@@ -954,8 +956,8 @@ __global__ void __cluster_dims__(kTcCluster, 1, 1) __launch_bounds__(kTcThreads,
                             const float2 w3 = *reinterpret_cast<const float2*>(&S.w[lane / 4].w3[2 * (lane % 4)]);
 #pragma unroll
                             for (int q = 0; q < 16; ++q) {  // (no fma: dZ2 is rounded)
-                                a.x = __fadd_rn(a.x, (h[q] & 0xFFFFu) ? __fmul_rn(dy[q], w3.x) : 0.0f);
-                                a.y = __fadd_rn(a.y, (h[q] & 0xFFFF0000u) ? __fmul_rn(dy[q], w3.y) : 0.0f);
+                                a.x = __fadd_rn(a.x, (h[q] & 0x8000u) ? 0.0f : __fmul_rn(dy[q], w3.x));
+                                a.y = __fadd_rn(a.y, (h[q] & 0x80000000u) ? 0.0f : __fmul_rn(dy[q], w3.y));
                             }
                         } else {
 #pragma unroll

@@ -129,6 +129,25 @@ def test_uneven_shares_match_oracle(env, d_in, n, batch, steps):
     test_training_steps_match_oracle(env, d_in, n, batch, steps)
 
 
+def test_units_barely_on_match_oracle(env):
+    """A unit is on for every pre-activation above zero, also one that BF16 rounds to zero: units without weights of
+    their own and biases of 2^-149, 2^-134 (the largest such), the next larger number, 0 and below."""
+    eng, torch = env
+    d_in, n = 4, 700
+    X, y, theta = _data(d_in, n, 5)
+    W1, b1, W2, b2, _, _ = omlp.unpack(theta, d_in)  # views
+    edges = [2.0**-149, 2.0**-134, 2.0**-134 + 2.0**-149, 0.0, -2.0**-149]
+    for W, b in ((W1, b1), (W2, b2)):
+        W[:5], b[:5] = 0.0, edges
+    r = _run(eng, torch, d_in, X, y, theta, n, 1, 3, 1)
+    ref = omlp.unpack(omlp.loss_and_grad(theta, X, y, d_in)[1], d_in)
+    got = omlp.unpack(r["grad"], d_in)
+    for layer in (1, 3):
+        bound = 1e-3 * np.linalg.norm(ref[layer]) + 1e-7  # the whole gradient's above, for every unit
+        assert np.all(np.abs(ref[layer][:3]) > 5 * bound) and np.all(ref[layer][3:5] == 0.0)
+        assert np.all(np.abs(got[layer] - ref[layer]) <= bound)
+
+
 def _expected_stop(val, epochs, patience):
     best, best_e, bad = np.inf, 0, 0
     for e in range(1, epochs + 1):
