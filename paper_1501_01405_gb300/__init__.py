@@ -431,22 +431,25 @@ class Model:
     def set_stream(self, stream):
         mrip_set_stream(self.h, stream)
 
+    # n_dp sizes the arrays that mrip_stats and mrip_moments fill with the
+    # handle's design points, so it changes only with the handle's run
+
     def run(self, design_points, n_reps, seed):
         dp = np.asarray(design_points, dtype=np.float64)
-        self.n_dp = dp.shape[0] if dp.ndim > 1 else dp.size
         mrip_run(self.h, dp, n_reps, seed)
+        self.n_dp = dp.shape[0] if dp.ndim > 1 else dp.size
 
     def run_range(self, design_points, rep_lo, rep_hi, seed):
         dp = np.asarray(design_points, dtype=np.float64)
-        self.n_dp = dp.shape[0] if dp.ndim > 1 else dp.size
         mrip_run_range(self.h, dp, rep_lo, rep_hi, seed)
+        self.n_dp = dp.shape[0] if dp.ndim > 1 else dp.size
 
     def moments(self):
         return mrip_moments(self.h, self.n_dp)
 
     def run_device(self, d_design_points, n_reps, seed):
-        self.n_dp = d_design_points.shape[0]
         mrip_run_device(self.h, d_design_points, n_reps, seed)
+        self.n_dp = d_design_points.shape[0]
 
     def stats(self, conf=0.95):
         return mrip_stats(self.h, self.n_dp, conf)
@@ -467,7 +470,9 @@ class Model:
         mrip_autotune(self.h, design_points, n_reps, seed, trials, cache_path)
 
     def run_cv(self, design_points, n_reps, seed, **kw):
-        return mrip_run_cv(self.h, design_points, n_reps, seed, **kw)
+        result = mrip_run_cv(self.h, design_points, n_reps, seed, **kw)
+        self.n_dp = len(result[0])
+        return result
 
     def cv_network(self):
         return mrip_cv_network(self.h, 8 if self.kind == MRIP_TANDEM3 else 6)

@@ -200,3 +200,29 @@ def test_debug_variant_builds_and_exports_every_symbol():
     exported = set(l.split()[-1] for l in out.splitlines() if " T " in l)
     assert not [n for n in _declared() if n not in exported]
     eng.load_library(path)  # loads beside the release library
+
+
+def test_a_refused_run_keeps_the_design_points(monkeypatch):
+    """A refused run leaves the handle its earlier run, and with it the number of design points that statistics and
+    moments are read for (the library fills as many)."""
+    eng = _engine()
+    m = eng.Model(eng.MRIP_MM1, n_clients=10)
+    m.n_dp = 5  # as after a run of five
+    calls = [lambda: m.run(np.array([[-1.0, 1.0]] * 2), 10, 1), lambda: m.run_range(np.array([[-1.0, 1.0]] * 2), 0, 10, 1)]
+    for call in calls:
+        with pytest.raises(eng.MripError) as e:
+            call()
+        assert e.value.code == 1 and m.n_dp == 5
+
+    def refuse(*args, **kw):
+        raise eng.MripError(1, "refused")
+    monkeypatch.setattr(eng, "mrip_run_device", refuse)
+    monkeypatch.setattr(eng, "mrip_run_cv", refuse)
+    for call in (lambda: m.run_device(np.ones((2, 2)), 10, 1), lambda: m.run_cv(np.ones((2, 2)), 10, 1)):
+        with pytest.raises(eng.MripError):
+            call()
+        assert m.n_dp == 5
+    monkeypatch.setattr(eng, "mrip_run_cv", lambda *a, **k: ([{}, {}], [{}, {}], {}))
+    m.run_cv(np.ones((2, 2)), 10, 1)
+    assert m.n_dp == 2
+    m.close()
