@@ -61,13 +61,17 @@ SMS = 152
 SM_MAX_MHZ = 2070.0
 IMUL_PER_CLK_SM = 64      # 32-bit integer multiply / multiply-add results
 DFMA_PER_CLK_SM = 2       # FP64 fused multiply-add results (1.25 TFLOP/s nominal)
-INT_MULS_PER_PHILOX = 40  # 10 rounds x 2 products x (low + high half)
-# one gap of the skip-sampled lattice: half a Philox block (20) + the
-# fixed-point log's products (4)
-MULS_PER_GAP = 24
+# The multiplies below are the ones the kernels execute, a widening product counted
+# as two (low and high half): a Philox4x32-10 block has 20 products, of which the
+# kernels compute what a replication, a step or a lattice word shares once.
+INT_MULS_PER_BLOCK = 32       # 16 products per block of one replication's running counter
+INT_MULS_PER_BLOCK_PAIR = 62  # the pair of blocks of a tandem client shares one more
+# one gap of the skip-sampled lattice: half a block of 18 products (its floor is decided
+# in FP32 but for a few in ten thousand)
+MULS_PER_GAP = 18
 # one exponential variate in 48-bit fixed point: the log's products (4: the
 # mantissa's two words by 1/c, both halves of the first, and r^2's high half)
-# + the scaling by 2^-9 / rate (4: one product in full, two by their high halves)
+# + the scaling by 2^-10 / rate (4: one product in full, two by their high halves)
 MULS_PER_FIXED_VARIATE = 8
 
 
@@ -81,14 +85,14 @@ PROFILED_TRAFFIC = {"forest_fire_kernel<8>": 3950000 * 32}
 
 # Issue slots: 4 schedulers per SM, one warp instruction each per clock.
 ISSUE_PER_CLK_SM = 4
-# Integer instructions per forest-fire cell-update: a quarter of a
-# Philox4x32-10 block (15-20 integer instructions) plus the bit-parallel
-# rule (32 cells per word); the midpoint 17.5 is the algorithmic figure.
-FF_INSTR_PER_CELL = 17.5
-# Widening multiplies per 32-cell lattice word and step, where what a step or
-# a word shares is computed once.  The kernel draws several steps at a time and
-# executes 122; the figure stays the one of a step by itself.
+# Warp instructions per 32 cell-updates of the forest fire, as executed (ncu's
+# smsp__inst_executed, profiles/current_kernels.md: 12.5 at 128 x 128, 12.4 at 256 x 256).
+FF_INSTR_PER_CELL = 12.4
+# Widening multiplies per 32-cell lattice word and step: of a step drawn by itself, what
+# a step or a word shares computed once, and as executed, several steps at a time (8
+# blocks of 15 products and 2 per batch of 8 steps).
 FF_MUL_WIDE_PER_WORD = 137
+FF_MUL_WIDE_EXECUTED = 122
 
 
 def issue_peak_g():
@@ -178,22 +182,22 @@ class ForestFire(Workload):
         w = self.w
         cells = w["L"] * w["L"] * w["n_steps"] * self.units()
         alt = dict(unit="Gop/s (32-bit integer multiply)",
-                   work=cells * INT_MULS_PER_PHILOX / 4.0, peak=imul_peak_gops(),
+                   work=cells * FF_MUL_WIDE_EXECUTED * 2 / 32.0, peak=imul_peak_gops(),
                    peak_source="nominal: %d SMs x %d int-mul/clk x %.0f MHz" % (
                        SMS, IMUL_PER_CLK_SM, SM_MAX_MHZ),
-                   per_unit="10 int multiplies per cell-update (1/4 Philox block)")
+                   per_unit="%.3f int multiplies executed per cell-update" % (FF_MUL_WIDE_EXECUTED * 2 / 32.0))
         return dict(kernel="forest_fire_kernel<%d>" % (w["L"] // 32), bound="alu",
                     unit="G warp-instructions/s",
                     work=cells * FF_INSTR_PER_CELL / 32.0, peak=issue_peak_g(),
                     peak_source="issue slots: %d SMs x %d warp-instr/clk x %.0f MHz" % (
                         SMS, ISSUE_PER_CLK_SM, SM_MAX_MHZ),
-                    per_unit="%.1f integer instructions per cell-update (1/4 Philox4x32-10 "
+                    per_unit="%.1f instructions executed per cell-update (1/4 Philox4x32-10 "
                              "block + the bit-parallel rule), 32 per warp instruction"
                              % FF_INSTR_PER_CELL, alt=alt,
-                    mul_wide=dict(work=cells * FF_MUL_WIDE_PER_WORD / 32.0 / 32.0,
-                                  per_unit="%d widening multiplies per 32-cell word and step (8 "
-                                           "Philox blocks x 17, two per-step products shared, "
-                                           "+ 1; 122 are executed), 32 per warp instruction" % FF_MUL_WIDE_PER_WORD))
+                    mul_wide=dict(work=cells * FF_MUL_WIDE_EXECUTED / 32.0 / 32.0,
+                                  per_unit="%d widening multiplies executed per 32-cell word and step "
+                                           "(%d for a step drawn by itself), 32 per warp instruction"
+                                           % (FF_MUL_WIDE_EXECUTED, FF_MUL_WIDE_PER_WORD)))
 
     def extra_rates(self, reps_per_s, torch):
         w = self.w
@@ -255,7 +259,7 @@ class ForestFireSkip(ForestFire):
                     work=gaps * MULS_PER_GAP, peak=imul_peak_gops(),
                     peak_source="nominal: %d SMs x %d int-mul/clk x %.0f MHz" % (
                         SMS, IMUL_PER_CLK_SM, SM_MAX_MHZ),
-                    per_unit="%d int multiplies per gap (half a Philox block + the fixed-point log); "
+                    per_unit="%d int multiplies executed per gap (half a Philox block); "
                              "(p_grow + p_light) L^2 + 2 gaps per step" % MULS_PER_GAP)
 
     def make_model(self):
@@ -318,9 +322,9 @@ class Walk(Workload):
         for R in mrip_inputs.WALK_RADII:
             moves += self.w["n_reps"] * (2.0 / 3.0) * R * R
         return dict(kernel="walk_persistent_kernel", bound="alu",
-                    unit="Gop/s (32-bit integer multiply)", work=moves / 64.0 * INT_MULS_PER_PHILOX,
+                    unit="Gop/s (32-bit integer multiply)", work=moves / 64.0 * INT_MULS_PER_BLOCK,
                     peak=imul_peak_gops(), peak_source="nominal int-mul rate",
-                    per_unit="40 int multiplies per 64 moves (one Philox block); E[tau] ~ 2R^2/3")
+                    per_unit="32 int multiplies executed per 64 moves (one Philox block); E[tau] ~ 2R^2/3")
 
     def make_model(self):
         return self.eng.Model(self.eng.MRIP_WALK_L1_EXIT, max_steps=1 << 38)
@@ -420,7 +424,8 @@ class Queue(Workload):
         clients = self.units() * w["n_clients"]
         blocks = 2 if self.key == "tandem" else 1
         logs = 4 if self.key == "tandem" else 2
-        per_client = blocks * INT_MULS_PER_PHILOX + logs * MULS_PER_FIXED_VARIATE
+        philox = INT_MULS_PER_BLOCK_PAIR if self.key == "tandem" else INT_MULS_PER_BLOCK
+        per_client = philox + logs * MULS_PER_FIXED_VARIATE
         kernel = {"mm1_32": "mm1_cta_kernel (graph with the statistics kernel)",
                   "mm1_64k": "mm1_serial_kernel", "tandem": "tandem3_serial_kernel"}[self.key]
         return dict(kernel=kernel, bound="alu",
@@ -428,9 +433,9 @@ class Queue(Workload):
                     peak=imul_peak_gops(),
                     peak_source="nominal: %d SMs x %d int-mul/clk x %.0f MHz" % (
                         SMS, IMUL_PER_CLK_SM, SM_MAX_MHZ),
-                    per_unit="%d int multiplies per client: %d Philox block(s) (40 each) + %d "
+                    per_unit="%d int multiplies executed per client: %d for %d Philox block(s), %d "
                              "fixed-point variates (%d each: log 4, scaling 4)" % (
-                                 per_client, blocks, logs, MULS_PER_FIXED_VARIATE))
+                                 per_client, philox, blocks, logs, MULS_PER_FIXED_VARIATE))
 
     def make_model(self):
         w = self.w
@@ -497,9 +502,9 @@ class AreaWalk(Workload):
     def roofline_work(self):
         moves = float(self.w["n_reps"]) * self.w["n_steps"]
         return dict(kernel="area_walk_serial_kernel", bound="alu", unit="Gop/s (32-bit integer multiply)",
-                    work=moves / 64.0 * INT_MULS_PER_PHILOX, peak=imul_peak_gops(),
+                    work=moves / 64.0 * INT_MULS_PER_BLOCK, peak=imul_peak_gops(),
                     peak_source="nominal int-mul rate",
-                    per_unit="40 int multiplies per 64 moves (one Philox block)")
+                    per_unit="32 int multiplies executed per 64 moves (one Philox block)")
 
     def make_model(self):
         return None
@@ -548,9 +553,9 @@ class MonteCarloPi(Workload):
     def roofline_work(self):
         draws = float(self.w["n_reps"]) * self.w["n_draws"]
         return dict(kernel="pi_kernel", bound="alu", unit="Gop/s (32-bit integer multiply)",
-                    work=draws * (INT_MULS_PER_PHILOX + 4) / 2.0, peak=imul_peak_gops(),
+                    work=draws * (INT_MULS_PER_BLOCK + 8) / 2.0, peak=imul_peak_gops(),
                     peak_source="nominal int-mul rate",
-                    per_unit="22 int multiplies per draw (half a Philox block + two 32x32->64 squares)")
+                    per_unit="20 int multiplies executed per draw (half a Philox block + two 32x32->64 squares)")
 
     def make_model(self):
         return None
