@@ -47,10 +47,9 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// bits |= bit if w < t, as a compare and a predicated OR.  Where the bit is a
-// constant known to be clear the assembler makes it an addition on the multiply
-// pipe, which then carries 165 instructions per word and step; variable bits keep
-// it on the ALU (136) and were 6 % slower (128 x 128: 9.84 and 10.48 ms): the ALU and
+// bits |= bit if w < t, as a compare and a predicated OR.  With constant bits the
+// multiply pipe carries 165 instructions per word and step (ncu's pipe counter), with
+// variable ones 136, but those are 6 % slower (128 x 128: 9.84 and 10.48 ms): the ALU and
 // the issue slots are as near their limits.
 __device__ __forceinline__ void or_if_below(uint32_t& bits, uint32_t w, uint32_t t, uint32_t bit) {
     asm("{\n .reg .pred p;\n setp.lt.u32 p, %1, %2;\n @p or.b32 %0, %0, %3;\n}\n"

@@ -1149,7 +1149,7 @@ size_t mlp_train_tc_smem() { return sizeof(TcSmem); }
 // pass through shared memory ([unit][sample], so stores and loads are 16-byte
 // and conflict-free); the output layer is one chain per sample.  As many CTAs
 // as fit at once walk the tiles, so the weights are staged once per CTA.
-// Measured, 942,080 samples of 8 inputs: 281 -> 182 us (8.8 GFLOP, 48 of the
+// Measured, 942,080 samples of 8 inputs: 286 -> 187 us (8.8 GFLOP, 47 of the
 // 80 TFLOP/s of FP32); 100,001 of 6 inputs 42 -> 31; 5,003 of 8 16.5 -> 10.3.
 constexpr int kFwdThreads = 128;
 constexpr int kFwdTile = 128;   // samples per tile

@@ -58,9 +58,8 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// D (TMEM) = A B^T (+ D if accumulate).  The whole warp calls and one elected
-// thread issues: descriptors stay in uniform registers, where a branch on the
-// thread moves every operand there first.
+// D (TMEM) = A B^T (+ D if accumulate).  The whole warp calls, with the same
+// operands, and one elected thread issues.
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                          bool accumulate) {
     asm volatile(
