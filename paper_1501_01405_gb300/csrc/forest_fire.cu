@@ -312,9 +312,9 @@ __device__ __forceinline__ void step_blocks(uint32_t a_hi, uint32_t a_lo, uint32
 }
 
 // Growth and lightning masks of lattice word k for NS steps.  Lightning is
-// rare: its masks are formed only where a word of a block, over the batch, is
-// below its threshold.
-template <int NS, int kUnroll>
+// rare: its masks are formed only where a word of a block, over kTest steps of the
+// batch, is below its threshold.
+template <int NS, int kUnroll, int kTest>
 __device__ __forceinline__ void ff_draw(uint32_t k, uint32_t c3, const StepKeys<NS>& sk, const RoundKeys& rk,
                                         uint32_t t_grow, uint32_t t_light, uint32_t (&g)[NS], uint32_t (&l)[NS]) {
     uint32_t a_hi, a_lo;
@@ -328,25 +328,28 @@ __device__ __forceinline__ void ff_draw(uint32_t k, uint32_t c3, const StepKeys<
     for (int q = 0; q < 8; ++q) {
         uint4 b[NS];
         step_blocks<NS>(a_hi, a_lo, c3, sk, rk, b);
-        bool any = false;
 #pragma unroll
-        for (int i = 0; i < NS; ++i) {
-            g[i] >>= 4;
-            or_if_below(g[i], b[i].x, t_grow, 1u << 28);
-            or_if_below(g[i], b[i].y, t_grow, 1u << 29);
-            or_if_below(g[i], b[i].z, t_grow, 1u << 30);
-            or_if_below(g[i], b[i].w, t_grow, 1u << 31);
-            any = any || b[i].x < t_light || b[i].y < t_light || b[i].z < t_light || b[i].w < t_light;
-        }
-        if (__builtin_expect(any, 0)) {
+        for (int i0 = 0; i0 < NS; i0 += kTest) {
+            bool any = false;
 #pragma unroll
-            for (int i = 0; i < NS; ++i) {
-                uint32_t nib = 0u;
-                or_if_below(nib, b[i].x, t_light, 1u);
-                or_if_below(nib, b[i].y, t_light, 2u);
-                or_if_below(nib, b[i].z, t_light, 4u);
-                or_if_below(nib, b[i].w, t_light, 8u);
-                l[i] |= nib << (4 * q);
+            for (int i = i0; i < i0 + kTest; ++i) {
+                g[i] >>= 4;
+                or_if_below(g[i], b[i].x, t_grow, 1u << 28);
+                or_if_below(g[i], b[i].y, t_grow, 1u << 29);
+                or_if_below(g[i], b[i].z, t_grow, 1u << 30);
+                or_if_below(g[i], b[i].w, t_grow, 1u << 31);
+                any = any || b[i].x < t_light || b[i].y < t_light || b[i].z < t_light || b[i].w < t_light;
+            }
+            if (__builtin_expect(any, 0)) {
+#pragma unroll
+                for (int i = i0; i < i0 + kTest; ++i) {
+                    uint32_t nib = 0u;
+                    or_if_below(nib, b[i].x, t_light, 1u);
+                    or_if_below(nib, b[i].y, t_light, 2u);
+                    or_if_below(nib, b[i].z, t_light, 4u);
+                    or_if_below(nib, b[i].w, t_light, 8u);
+                    l[i] |= nib << (4 * q);
+                }
             }
         }
         asm("add.cc.u32 %0, %0, 0xD2511F53;\n\taddc.u32 %1, %1, 0;" : "+r"(a_lo), "+r"(a_hi));
@@ -398,14 +401,16 @@ __global__ void __launch_bounds__(R * ff_threads<W>(), ff_min_blocks<W, R>()) fo
     for (int t0 = 1; t0 <= n_steps; t0 += NT) {
         unsigned long long flags = 0;  // bit NT j + s: word j has lightning at step t0 + s
         const int ns = min(NT, n_steps + 1 - t0);
-        // masks of steps t0 + s .. t0 + s + K - 1
+        // masks of steps t0 + s .. t0 + s + K - 1 (L = 32 tests a batch for lightning by halves:
+        // at p_lightning = 10^-3 most warps find some in a whole one.  1,000 replications x 100
+        // steps 105 -> 101 us there, 92.5 at 10^-5 either way; 128 x 128 loses 0.7 % at 10^-5)
         auto draw = [&](int s, auto steps, auto unroll) {
             constexpr int K = decltype(steps)::value;
             const StepKeys<K> sk = step_keys<K>(static_cast<uint32_t>(t0 + s), rep, rk);
 #pragma unroll 1
             for (int j = 0; j < N; ++j) {
                 uint32_t g[K], l[K];
-                ff_draw<K, decltype(unroll)::value>(static_cast<uint32_t>(y * W + j0 + j), c3, sk, rk, t_grow, t_light, g, l);
+                ff_draw<K, decltype(unroll)::value, (W == 1 && K > 4 ? K / 2 : K)>(static_cast<uint32_t>(y * W + j0 + j), c3, sk, rk, t_grow, t_light, g, l);
                 const int at = ff_word<W>(y, j0 + j);
 #pragma unroll
                 for (int i = 0; i < K; ++i) {
