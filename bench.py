@@ -86,7 +86,7 @@ PROFILED_TRAFFIC = {"forest_fire_kernel<8>": 3950000 * 32}
 # Issue slots: 4 schedulers per SM, one warp instruction each per clock.
 ISSUE_PER_CLK_SM = 4
 # Warp instructions per 32 cell-updates of the forest fire, as executed (ncu's
-# smsp__inst_executed, profiles/current_kernels.md: 12.5 at 128 x 128, 12.4 at 256 x 256).
+# smsp__inst_executed, under profiles/: 12.5 at 128 x 128, 12.4 at 256 x 256).
 FF_INSTR_PER_CELL = 12.4
 # Widening multiplies per 32-cell lattice word and step: of a step drawn by itself, what
 # a step or a word shares computed once, and as executed, several steps at a time (8

@@ -141,7 +141,9 @@ mrip_status mrip_set_stream(mrip_model *model, void *cuda_stream);
  * work is enqueued (the replay of a CUDA graph captured on first use for this
  * shape).  Per-replication outputs stay on the device (mrip_outputs).
  * The scalar per replication is: MM1 mean wait; TANDEM3 mean sojourn;
- * FOREST_FIRE mean burning fraction sum_t burning_t / (T L^2); WALK tau. */
+ * FOREST_FIRE mean burning fraction sum_t burning_t / (T L^2); WALK tau.
+ * A design point or shape that is refused leaves the results of the run before;
+ * after a later failure there are none (MRIP_ESTATE) until the next run. */
 mrip_status mrip_run(mrip_model *model, const double *design_points, int32_t n_dp,
                      int64_t n_reps, uint64_t seed);
 
